@@ -104,9 +104,9 @@ METRIC = "keys/sec and % HBM roofline, 2^28 int32; learned/batched vs plain, bit
 # routing pass reads every key and writes it once (8 B); the bucket sort reads
 # and writes every key once (8 B).  With 4-byte payloads both double.
 PHASES = ["sample", "sample_sort", "splitters", "route", "bucket_sort"]
-PHASE_KERNEL = {("route", False): "route_keys_kernel", ("bucket_sort", False): "bucket_keys32_kernel",
+PHASE_KERNEL = {("route", False): "route_keys_kernel", ("bucket_sort", False): "bucket_count_kernel",
                 ("route", True): "route_kernel", ("bucket_sort", True): "bucket_sort_kernel"}
-PHASE_KERNEL_F64 = {"bucket_sort": "bucket_keys_kernel"}
+PHASE_KERNEL_F64 = {"bucket_sort": "bucket_count_kernel"}
 # the variant timed beside a workload: (label, the parameters that change)
 COMPARE = {"tree": ("tree", dict(classify=0)), "sort": ("bucket_sort_final_step", dict(final_step=0)),
            "tags": ("with_duplicate_handling", dict(duplicates=0))}
@@ -120,7 +120,6 @@ COMPARE = {"tree": ("tree", dict(classify=0)), "sort": ("bucket_sort_final_step"
 # (bytes per key, source hash, payloads) of each capture; the segment copy's
 # from the 2^26-pair Zipf capture (4096 buckets of 16-key segments, as at 2^28)
 NCU_TRAFFIC = {"route_keys_kernel": ((271.608576e6 + 223.674880e6) / (1 << 26), "8baca4c618da453f", False),
-               "bucket_keys32_kernel": ((537.268992e6 + 486.783232e6) / (1 << 27), "b2f4fe6e7d92e3af", False),
                "segment_copy_kernel": ((617.909248e6 + 494.979328e6) / (1 << 26), "333c4e171f9cd65e", True)}
 KERNEL_SOURCE = {"route_kernel": ["paper_1408_6729_gb300/csrc/route.cu"],
                  "segment_copy_kernel": ["paper_1408_6729_gb300/csrc/merge.cu"],
@@ -129,12 +128,9 @@ KERNEL_SOURCE = {"route_kernel": ["paper_1408_6729_gb300/csrc/route.cu"],
                                        "paper_1408_6729_gb300/csrc/kernels.cuh"],
                  "bucket_sort_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
                                         "paper_1408_6729_gb300/csrc/segsort.cuh"],
-                 "bucket_keys_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
-                                        "paper_1408_6729_gb300/csrc/segsort_keys.cuh"],
-                 "bucket_keys32_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
-                                          "paper_1408_6729_gb300/csrc/bucket_keys32.cuh",
-                                          "paper_1408_6729_gb300/csrc/segsort_keys.cuh",
-                                          "paper_1408_6729_gb300/csrc/radix.cuh"]}
+                 "bucket_count_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
+                                         "paper_1408_6729_gb300/csrc/countsort.cuh",
+                                         "paper_1408_6729_gb300/csrc/radix.cuh"]}
 
 
 def peaks():

@@ -1,20 +1,16 @@
 // bucket.cu -- final sort of every bucket (Fig. 2 step 12 / Fig. 3 step 14):
 // the keys a bucket received, in input order, are sorted stably and written
-// to the bucket's place in the output.  Each sub-bucket is sorted on chip by
-// one thread-block cluster, in up to three tiers:
-//   1. keys only: the throughput sort of segsort_keys.cuh (unstable ranks,
-//      which equal keys cannot reveal) -- for 8-byte keys in two capacities,
-//      two CTAs per SM for the sub-buckets that fit, then one CTA per SM
-//      holding twice the keys for the larger ones; with payloads: sub-buckets
-//      of one key value are copied as they stand;
+// to the bucket's place in the output, in up to three tiers:
+//   1. keys only: the streamed counting sort of countsort.cuh (unstable ranks,
+//      which equal keys cannot reveal), one CTA or several per sub-bucket; with
+//      payloads: sub-buckets of one key value are copied as they stand;
 //   2. the other sub-buckets with payloads, or what tier 1 gives back: the
 //      stable cluster sort of segsort.cuh over a list;
 //   3. sub-buckets larger than a cluster's shared memory: an out-of-core
 //      radix sort in global memory.
 #include "kernels.cuh"
 #include "segsort.cuh"
-#include "segsort_keys.cuh"
-#include "bucket_keys32.cuh"
+#include "countsort.cuh"
 
 namespace bsps {
 
@@ -34,8 +30,7 @@ template <typename K> struct BucketArgs {
     uint32_t *retry_list;
     const uint32_t *only;     // tier 2 over a list (nullable: every sub-bucket)
     const int32_t *only_count;
-    int64_t defer_above;      // tier 1: sub-buckets above this many keys are left to the larger tier 1
-    int64_t take_above;       // larger tier 1: only sub-buckets above this many keys
+    int64_t slow_above;       // keys a cluster of the stable sort holds
     int one_value_done;       // sub-buckets of one key value are already in the output
 };
 
@@ -67,8 +62,8 @@ bucket_sort_kernel(const BucketArgs<typename KeyTraits<DT>::T> a) {
         };
         const bool done = SS::run(sm, buf, slots, cnt, [&](int64_t e) { return src[e]; }, emit);
         if (!done && blockIdx.x % CL == 0 && threadIdx.x == 0) {
-            const int slot = atomicAdd(&a.st->slow_buckets, 1);
-            a.slow_list[slot] = (uint32_t)v;
+            atomicAdd(&a.st->slow_buckets, 1);
+            a.slow_list[atomicAdd(&a.st->slow_count, 1)] = (uint32_t)v;
         }
         // the next sub-bucket reuses every CTA's shared memory
         if (a.only) cg::this_cluster().sync();
@@ -106,74 +101,36 @@ __global__ void __launch_bounds__(kCopyThreads) bucket_copy_kernel(const BucketA
     }
 }
 
-// Tier 1 (keys only): one cluster per sub-bucket; its bounds are the two
-// splitters around it (the smallest and largest key for the end buckets).
-template <int DT, int CL, int ITEMS>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(512, ITEMS > kKeysItems64 ? 1 : 2)
-bucket_keys_kernel(const BucketArgs<typename KeyTraits<DT>::T> a) {
+// Tier 1 (keys only): G CTAs per sub-bucket, the streamed counting sort of
+// countsort.cuh; its bounds are the two splitters around it (the smallest and
+// largest key for the end buckets).
+template <int DT, int SIZE>
+__global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
+bucket_count_kernel(const BucketArgs<typename KeyTraits<DT>::T> a, int G) {
     using K = typename KeyTraits<DT>::T;
-    using SS = SegSortKeys<K, CL, ITEMS, false>;
+    using CS = typename CountShape<SIZE>::template Sort<K>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t v = blockIdx.x / CL;
+    const int64_t v = blockIdx.x / G;
+    const int g = (int)(blockIdx.x % G);
     const int64_t cnt = imin64(a.vsize[v], a.cap);
-    if (cnt == 0 || cnt > a.defer_above || cnt <= a.take_above) return;
+    if (cnt == 0) return;
     const K lo = v > 0 ? a.vphi[v - 1] : (K)~a.st->ext_min_inv;
     const K hi = v < a.P - 1 ? a.vphi[v] : (K)a.st->ext_max;
     K *out_k = a.out_keys + a.voff[v];
+    bool done = true;
     if (lo == hi) {  // one key value: nothing to read
         const K x = KeyTraits<DT>::inv(lo);
-        const int64_t share = (cnt + CL - 1) / CL, e0 = (int64_t)(blockIdx.x % CL) * share;
-        const int64_t e1 = imin64(cnt, e0 + share);
+        const int64_t share = (cnt + G - 1) / G, e0 = g * share, e1 = imin64(cnt, e0 + share);
 #pragma unroll 4
         for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) out_k[e] = x;
-        return;
+    } else {
+        done = CS::run(smem_raw, a.reg_keys + v * a.cap, (int)cnt, lo, hi, out_k, g, G, [](K k) { return k; },
+                       [](K k) { return KeyTraits<DT>::inv(k); });
+        // larger than a cluster of the stable sort holds: sorted out of core, part by part
+        if (done && cnt > a.slow_above && g == 0 && threadIdx.x == 0) atomicAdd(&a.st->slow_buckets, 1);
     }
-    auto emit = [&](uint32_t pos, K key) { out_k[pos] = KeyTraits<DT>::inv(key); };
-    if (!SS::run(smem_raw, a.reg_keys + v * a.cap, cnt, lo, hi, emit) && threadIdx.x == 0) {
-        if (atomicExch(&a.retry_flag[v], 1u) == 0u) {
-            const int slot = atomicAdd(&a.st->retry_count, 1);
-            a.retry_list[slot] = (uint32_t)v;
-        }
-    }
-}
-
-// Tier 1 for 32-bit keys: the same cluster per sub-bucket, with the lean
-// split / exchange / count sort of bucket_keys32.cuh.
-template <int DT, int CL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(512, 2)
-bucket_keys32_kernel(const BucketArgs<uint32_t> a) {
-    using SS = BucketKeys32<CL>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t v = blockIdx.x / CL;
-    const int64_t cnt = imin64(a.vsize[v], a.cap);
-    if (cnt == 0) return;
-    const uint32_t lo = v > 0 ? a.vphi[v - 1] : (uint32_t)~a.st->ext_min_inv;
-    const uint32_t hi = v < a.P - 1 ? a.vphi[v] : (uint32_t)a.st->ext_max;
-    uint32_t *out_k = a.out_keys + a.voff[v];
-    if (lo == hi) {  // one key value: nothing to read
-        const uint32_t x = KeyTraits<DT>::inv(lo);
-        const int64_t share = (cnt + CL - 1) / CL, e0 = (int64_t)(blockIdx.x % CL) * share;
-        const int64_t e1 = imin64(cnt, e0 + share);
-#pragma unroll 4
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) out_k[e] = x;
-        return;
-    }
-    auto emit = [&](uint32_t pos, uint32_t key) { out_k[pos] = KeyTraits<DT>::inv(key); };
-    typename SS::Smem &sm = *reinterpret_cast<typename SS::Smem *>(smem_raw);
-    if (threadIdx.x == 0) sm.stalled = 0;
-    __syncthreads();
-    bool done = SS::run(smem_raw, a.reg_keys + v * a.cap, cnt, lo, hi, emit, a.st);
-    __syncthreads();
-    if (sm.stalled) {  // the staged load's wait ran out: wait for the copy once more, give the sub-bucket back
-        SS::wait_staged(sm, kSpinLimit);
-        done = false;
-    }
-    if (!done && threadIdx.x == 0) {
-        if (atomicExch(&a.retry_flag[v], 1u) == 0u) {
-            const int slot = atomicAdd(&a.st->retry_count, 1);
-            a.retry_list[slot] = (uint32_t)v;
-        }
-    }
+    if (!done && threadIdx.x == 0 && atomicExch(&a.retry_flag[v], 1u) == 0u)
+        a.retry_list[atomicAdd(&a.st->retry_count, 1)] = (uint32_t)v;
 }
 
 // ---------------------------------------------------------------------------
@@ -190,7 +147,7 @@ __global__ void __launch_bounds__(kSlowThreads) bucket_slow_kernel(BucketArgs<ty
     __shared__ typename Rank::Smem rsm;
     __shared__ uint32_t hist[256], run[256], tmp[40];
     __shared__ K red[2];
-    const int nslow = a.st->slow_buckets;
+    const int nslow = a.st->slow_count;
     for (int idx = blockIdx.x; idx < nslow; idx += gridDim.x) {
         const int64_t v = a.slow_list[idx];
         const int64_t cnt = imin64(a.vsize[v], a.cap);
@@ -290,31 +247,15 @@ static cudaError_t launch_cluster(const Ctx &c, const BucketArgs<typename KeyTra
     return cudaGetLastError();
 }
 
-template <int DT, int CL, int ITEMS>
+template <int DT, int SIZE>
 static cudaError_t launch_keys(const Ctx &c, const BucketArgs<typename KeyTraits<DT>::T> &a) {
-    using K = typename KeyTraits<DT>::T;
-    if constexpr (sizeof(K) == 4) {
-        using SS = BucketKeys32<CL>;
-        static_assert(2 * (SS::smem_bytes() + 1024) <= 228 * 1024, "two CTAs per SM");
-        const size_t smem = SS::smem_bytes();
-        auto kern = bucket_keys32_kernel<DT, CL>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)(c.pl.P * CL), 512, smem, c.stream>>>(a);
-        return cudaGetLastError();
-    } else {
-        using SS = SegSortKeys<K, CL, ITEMS, false>;
-        // two CTAs per SM (228 KB of shared memory per SM, 1 KB of it reserved
-        // per CTA), or one for the larger tier
-        static_assert(2 * (SS::smem_bytes() + 1024) <= 228 * 1024 || ITEMS > kKeysItems64, "two CTAs per SM");
-        static_assert(SS::smem_bytes() + 1024 <= 228 * 1024, "one CTA per SM");
-        const size_t smem = SS::smem_bytes();
-        auto kern = bucket_keys_kernel<DT, CL, ITEMS>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)(c.pl.P * CL), 512, smem, c.stream>>>(a);
-        return cudaGetLastError();
-    }
+    using CS = typename CountShape<SIZE>::template Sort<typename KeyTraits<DT>::T>;
+    auto kern = bucket_count_kernel<DT, SIZE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS::smem_bytes());
+    if (e != cudaSuccess) return e;
+    const int G = count_sort_ctas<SIZE>(c.pl.P, c.pl.n / c.pl.P);
+    kern<<<(unsigned)(c.pl.P * G), CountShape<SIZE>::T, CS::smem_bytes(), c.stream>>>(a, G);
+    return cudaGetLastError();
 }
 
 template <int DT, bool PAIRS> static cudaError_t launch_bucket_t(const Ctx &c) {
@@ -335,34 +276,16 @@ template <int DT, bool PAIRS> static cudaError_t launch_bucket_t(const Ctx &c) {
     a.retry_list = c.ly.retry_list;
     a.only = nullptr;
     a.only_count = nullptr;
-    a.defer_above = INT64_MAX;
-    a.take_above = 0;
+    a.slow_above = (int64_t)8 * 1024 * (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32);
     a.one_value_done = c.pl.seg_route;
     constexpr int IT = PAIRS ? (sizeof(K) == 8 ? kPairItems64 : kPairItems32)
                              : (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32);
     cudaError_t e = cudaSuccess;
     if constexpr (!PAIRS) {
-        constexpr int KIT = sizeof(K) == 8 ? kKeysItems64 : kKeysItems32;
-        if constexpr (sizeof(K) == 8) {
-            // sub-buckets beyond the two-per-SM clusters: clusters of 8 CTAs
-            // holding twice the keys each, before anything is given back
-            a.defer_above = (int64_t)c.pl.bucket_cl * 512 * KIT;
-            if (a.defer_above < (int64_t)8 * 512 * kKeysItems64Large && c.pl.cap > a.defer_above) {
-                BucketArgs<K> big = a;
-                big.defer_above = INT64_MAX;
-                big.take_above = a.defer_above;
-                e = launch_keys<DT, 8, kKeysItems64Large>(c, big);
-                if (e != cudaSuccess) return e;
-            } else {
-                a.defer_above = INT64_MAX;
-            }
-        }
-        switch (c.pl.bucket_cl) {
-        case 1: e = launch_keys<DT, 1, KIT>(c, a); break;
-        case 2: e = launch_keys<DT, 2, KIT>(c, a); break;
-        case 4: e = launch_keys<DT, 4, KIT>(c, a); break;
-        case 8: e = launch_keys<DT, 8, KIT>(c, a); break;
-        default: return cudaErrorInvalidValue;
+        switch (count_sort_size(c.pl.n / c.pl.P, sizeof(K))) {
+        case kCountSmall: e = launch_keys<DT, kCountSmall>(c, a); break;
+        case kCountMedium: e = launch_keys<DT, kCountMedium>(c, a); break;
+        default: e = launch_keys<DT, kCountLarge>(c, a); break;
         }
         if (e != cudaSuccess) return e;
         // what tier 1 gave back: the stable cluster sort over the list

@@ -1,0 +1,622 @@
+// countsort.cuh -- keys-only sort of one segment by one CTA (or by several that
+// share its output): the bucket sort of Fig. 2 step 12 and the block sort of
+// Fig. 1 step 3 where no payload moves.  Equal keys cannot be told apart, so no
+// rank needs to be stable.
+//
+// The segment's keys lie in [lo, hi].  It stays in global memory (L2 after the
+// first pass) and is streamed, so its size is not bounded by shared memory:
+//   1. every key is counted in one of up to NBMAX bins, (key - lo) >> shift,
+//      with one shared-memory reduction (bins b and b + nb/2 are the halves of
+//      one word);
+//   2. a scan turns the counts into the bins' first positions.  The positions
+//      are cut into parts that the stage holds, at multiples of 256 bins;
+//   3. per part, the keys are read again and each key of the part is stored at
+//      its bin's next position of a shared-memory stage (one atomic);
+//   4. the stage is now sorted up to the order inside each bin.  A bin of at
+//      most kEdge keys is finished in registers: a warp takes 256 consecutive
+//      positions, eight to a lane, sorts them by a network inside the lanes and
+//      across their borders (odd-even transposition rounds where a bin needs
+//      more) and writes the middle 224 with 16-byte stores; every bin touching
+//      those lies inside the 256.  Longer bins (skewed or repeated keys) are
+//      listed by the scan and sorted in the stage first: not at all when all
+//      their keys are equal, else by a bitonic network.
+// Per key that is two shared-memory atomics and one shared store, and no
+// exchange between CTAs.
+//
+// A narrow stage holds only the low half of key - lo (16 bits of 32, 32 of 64),
+// so twice the keys: a 65,536-key bucket of 32-bit keys is one part, read twice
+// instead of three times.  The rest follows from the position: key - lo is cut
+// into units of 2^(half - 1) values, every unit is a range of bins, and the
+// scan records the position where it starts.  A window of at most two units is
+// put in order and rebuilt from the half words alone.  It is taken when the
+// units are few and long (ranges up to 2^23 values at 65,536 keys).
+//
+// Several CTAs (G of them) may take one segment: each counts all of it and
+// takes every G-th part.  Every decision is a function of the segment alone,
+// so the CTAs agree without talking to each other.
+#pragma once
+
+#include <type_traits>
+
+#include "radix.cuh"
+
+namespace bsps {
+
+template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
+    using S = typename std::conditional<sizeof(K) == 8, uint32_t, uint16_t>::type;  // word of a narrow stage
+    static constexpr int UB = sizeof(K) == 8 ? 31 : 15;  // bits of a unit
+    static constexpr int W = T / 32;
+    static constexpr int V = 16 / (int)sizeof(K);    // keys per 16-byte access
+    static constexpr int kSegBins = 256;             // bins per scan step of a warp
+    static constexpr int kSegs = NBMAX / kSegBins;
+    static constexpr int kWin = 256, kEdge = 16, kStep = kWin - 2 * kEdge;
+    static constexpr int kPer = kWin / 32;           // keys of a window per lane
+    static constexpr int kLongMax = NBMAX / 16;      // listed long bins
+    static constexpr int kWarpBin = 1024;            // long bins up to this size are sorted by one warp
+    static constexpr int kPartsMax = 32;
+    static constexpr int kUnits = 256;               // units of a narrow stage
+    static constexpr uint32_t kUseWide = STAGE / sizeof(K) - 8, kUseNarrow = STAGE / sizeof(S) - 8;
+    static_assert(NBMAX % 512 == 0 && kSegs <= 128 && NBMAX <= 65536, "the segments are scanned by one warp, four to a lane");
+    static_assert(kUseWide < 65528 && STAGE % 16 == 0, "16-bit positions inside a part");
+
+    struct Smem {
+        uint32_t seg[kSegs + 1];              // first position of every segment of 256 bins
+        uint32_t pseg[kPartsMax + 1];         // first segment of every part
+        uint32_t unit[kUnits + 2];            // first position of every unit (narrow stage)
+        uint32_t longs[kLongMax];             // bin | length << 16
+        uint32_t nlong, nparts, bad, half;
+    };
+    static constexpr size_t kHead = (sizeof(Smem) + 15) & ~size_t(15);
+    static constexpr size_t smem_bytes() { return kHead + (size_t)NBMAX * 2 + STAGE; }
+
+    // f(key) for every key of the segment; xf maps a loaded word to the key
+    template <typename Xf, typename F>
+    __device__ static void for_each(const K *__restrict__ src, int n, Xf xf, F f) {
+        const int tid = threadIdx.x;
+        if (((uintptr_t)src & 15) == 0) {
+            const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
+            const int nq = n / V;
+            auto take = [&](const uint4 &w) {
+                if constexpr (sizeof(K) == 4) {
+                    f(xf(w.x)); f(xf(w.y)); f(xf(w.z)); f(xf(w.w));
+                } else {
+                    f(xf((uint64_t)w.y << 32 | w.x)); f(xf((uint64_t)w.w << 32 | w.z));
+                }
+            };
+            int q = tid;
+            for (; q + 3 * T < nq; q += 4 * T) {
+                uint4 w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = s4[q + j * T];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) take(w[j]);
+            }
+            for (; q < nq; q += T) take(s4[q]);
+            const int e = nq * V + tid;
+            if (e < n) f(xf(src[e]));
+        } else {
+            int e = tid;
+            for (; e + 3 * T < n; e += 4 * T) {
+                K w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = src[e + j * T];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) f(xf(w[j]));
+            }
+            for (; e < n; e += T) f(xf(src[e]));
+        }
+    }
+
+    // Ascending bitonic network over a[0..len) by `size` threads, this one
+    // being `rank`; every comparator puts the larger key higher, so positions
+    // past len act as keys above all others and are never touched.
+    template <typename E, typename Sync>
+    __device__ static void bitonic(E *a, int len, int rank, int size, Sync sync) {
+        int n2 = 1;
+        while (n2 < len) n2 <<= 1;
+        auto step = [&](int i, int l) {
+            if (l < len) {
+                const E x = a[i], y = a[l];
+                if (x > y) {
+                    a[i] = y;
+                    a[l] = x;
+                }
+            }
+        };
+        for (int h = 1; h < n2; h <<= 1) {  // runs of h sorted: merge pairs of them
+            for (int t = rank; t < (n2 >> 1); t += size) {
+                const int b = (t & ~(h - 1)) * 2, o = t & (h - 1);
+                step(b + o, b + 2 * h - 1 - o);
+            }
+            sync();
+            for (int j = h >> 1; j > 0; j >>= 1) {
+                for (int t = rank; t < (n2 >> 1); t += size) {
+                    const int i = 2 * t - (t & (j - 1));
+                    step(i, i + j);
+                }
+                sync();
+            }
+        }
+    }
+
+    // The long bins inside bins [b0, b0 + bn), each unsorted in the len slots
+    // that end at its cursor.
+    template <typename E, typename End>
+    __device__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, End end_of) {
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        const uint32_t nl = sm.nlong;
+        for (uint32_t i = warp; i < nl; i += W) {
+            const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
+            if (b - b0 >= bn || len > (uint32_t)kWarpBin) continue;
+            E *a = stage + (end_of(b) - len);
+            bool differ = false;
+            const E first = a[0];
+            for (uint32_t e = lane; e < len; e += 32) differ |= a[e] != first;
+            if (__any_sync(0xffffffffu, differ)) bitonic(a, (int)len, lane, 32, [] { __syncwarp(); });
+        }
+        for (uint32_t i = 0; i < nl; ++i) {
+            const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
+            if (b - b0 >= bn || len <= (uint32_t)kWarpBin) continue;  // uniform
+            E *a = stage + (end_of(b) - len);
+            bool differ = false;
+            const E first = a[0];
+            for (uint32_t e = tid; e < len; e += T) differ |= a[e] != first;
+            if (__syncthreads_or(differ)) bitonic(a, (int)len, tid, T, [] { __syncthreads(); });
+        }
+    }
+
+    template <typename E> __device__ static void order(E &a, E &b) {
+        const E x = a, y = b;
+        a = x < y ? x : y;
+        b = x < y ? y : x;
+    }
+
+    // A window in order: the eight words of every lane (19 comparators), then a
+    // bin across the border of two lanes -- my upper four words and the next
+    // lane's lower four merge, each lane computing its own side -- then odd-even
+    // transposition rounds until nothing is out of order (rarely any).
+    template <typename E> __device__ static void sort_window(E (&x)[kPer]) {
+        const int lane = threadIdx.x & 31;
+        order(x[0], x[2]); order(x[1], x[3]); order(x[4], x[6]); order(x[5], x[7]);
+        order(x[0], x[4]); order(x[1], x[5]); order(x[2], x[6]); order(x[3], x[7]);
+        order(x[0], x[1]); order(x[2], x[3]); order(x[4], x[5]); order(x[6], x[7]);
+        order(x[2], x[4]); order(x[3], x[5]);
+        order(x[1], x[4]); order(x[3], x[6]);
+        order(x[1], x[2]); order(x[3], x[4]); order(x[5], x[6]);
+        E nx[4], pv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            nx[j] = __shfl_down_sync(0xffffffffu, x[j], 1);
+            pv[j] = __shfl_up_sync(0xffffffffu, x[4 + j], 1);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (lane < 31) x[4 + j] = nx[3 - j] < x[4 + j] ? nx[3 - j] : x[4 + j];
+            if (lane > 0) x[j] = pv[3 - j] > x[j] ? pv[3 - j] : x[j];
+        }
+        order(x[4], x[6]); order(x[5], x[7]); order(x[4], x[5]); order(x[6], x[7]);
+        order(x[0], x[2]); order(x[1], x[3]); order(x[0], x[1]); order(x[2], x[3]);
+        for (;;) {
+            bool bad = false;
+#pragma unroll
+            for (int j = 0; j + 1 < kPer; ++j) bad |= x[j + 1] < x[j];
+            const E nxt = __shfl_down_sync(0xffffffffu, x[0], 1);
+            bad |= lane < 31 && nxt < x[kPer - 1];
+            if (!__any_sync(0xffffffffu, bad)) break;
+#pragma unroll
+            for (int j = 0; j + 1 < kPer; j += 2) order(x[j], x[j + 1]);
+            const E up = __shfl_up_sync(0xffffffffu, x[kPer - 1], 1), dn = __shfl_down_sync(0xffffffffu, x[0], 1);
+#pragma unroll
+            for (int j = 1; j + 1 < kPer; j += 2) order(x[j], x[j + 1]);
+            if (lane > 0) x[0] = up > x[0] ? up : x[0];
+            if (lane < 31) x[kPer - 1] = dn < x[kPer - 1] ? dn : x[kPer - 1];
+        }
+    }
+
+    // Writes a lane's keys key(j) to ob[at + j]; at the ends of a part only
+    // those inside [pad, end).
+    template <typename Key>
+    __device__ static void put(K *ob, int at, bool inner, int pad, int end, Key key) {
+#pragma unroll
+        for (int j = 0; j < kPer / V; ++j) {
+            const int o = at + j * V;
+            if (inner) {
+                uint4 w;
+                if constexpr (sizeof(K) == 4) {
+                    w = make_uint4(key(j * 4), key(j * 4 + 1), key(j * 4 + 2), key(j * 4 + 3));
+                } else {
+                    const uint64_t a = key(j * 2), b = key(j * 2 + 1);
+                    w = make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+                }
+                *reinterpret_cast<uint4 *>(ob + o) = w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < V; ++e)
+                    if (o + e >= pad && o + e < end) ob[o + e] = key(j * V + e);
+            }
+        }
+    }
+
+    // A part of np keys at stage[pad..): its windows, written to out[0..np)
+    // (out + j and stage[pad + j] have the same 16-byte alignment).
+    template <typename Inv>
+    __device__ static void emit_wide(const K *stage, int pad, int np, K *out, Inv inv) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, end = pad + np;
+        for (int w0 = warp * kStep; w0 < end; w0 += W * kStep) {
+            const int at = w0 - kEdge + lane * kPer;
+            const bool inner = w0 - kEdge >= pad && w0 + kWin - kEdge <= end;  // the whole window
+            K x[kPer];
+            if (inner) {
+#pragma unroll
+                for (int j = 0; j < kPer / V; ++j) {
+                    const uint4 w = *reinterpret_cast<const uint4 *>(stage + at + j * V);
+                    if constexpr (sizeof(K) == 4) {
+                        x[j * 4] = w.x; x[j * 4 + 1] = w.y; x[j * 4 + 2] = w.z; x[j * 4 + 3] = w.w;
+                    } else {
+                        x[j * 2] = (uint64_t)w.y << 32 | w.x;
+                        x[j * 2 + 1] = (uint64_t)w.w << 32 | w.z;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kPer; ++j)
+                    x[j] = at + j < pad ? K(0) : (at + j < end ? stage[at + j] : all_ones<K>());
+            }
+            sort_window(x);
+            if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
+                put(out - pad, at, inner, pad, end, [&](int j) { return inv(x[j]); });
+        }
+    }
+
+    // The same from a narrow stage, whose first slot (pad) is position p0.
+    template <typename Inv>
+    __device__ static void emit_narrow(const Smem &sm, const S *stage, int pad, int np, uint32_t p0, uint32_t nunits, K lo,
+                                       K *out, Inv inv) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, end = pad + np;
+        for (int w0 = warp * kStep; w0 < end; w0 += W * kStep) {
+            const int at = w0 - kEdge + lane * kPer;
+            // the unit of the window's first position: the last one starting at or before it
+            const uint32_t first = p0 + (uint32_t)(max(w0 - kEdge, pad) - pad);
+            const uint32_t last = p0 + (uint32_t)(min(w0 + kWin - kEdge, end) - 1 - pad);
+            uint32_t u0 = 0;
+            for (uint32_t b = 0; b < nunits; b += 32) {
+                const uint32_t below = __ballot_sync(0xffffffffu, b + lane < nunits && sm.unit[b + lane] <= first);
+                u0 += (uint32_t)__popc(below);
+                if (below != 0xffffffffu) break;
+            }
+            --u0;
+            const bool inner = w0 - kEdge >= pad && w0 + kWin - kEdge <= end;  // the whole window
+            const bool two = sm.unit[u0 + 2] > last;  // at most two units: offsets from the first fit a half word
+            // an offset from unit u0: half word minus u0 << UB, which flips its top bit when u0 is odd
+            const uint32_t flip = two && (u0 & 1u) ? (sizeof(K) == 4 ? 0x80008000u : 0x80000000u) : 0u;
+            uint32_t s[kPer];
+            if (inner) {
+                uint4 w = *reinterpret_cast<const uint4 *>(stage + at);
+                w = make_uint4(w.x ^ flip, w.y ^ flip, w.z ^ flip, w.w ^ flip);
+                if constexpr (sizeof(K) == 4) {
+                    s[0] = w.x & 0xffffu; s[1] = w.x >> 16; s[2] = w.y & 0xffffu; s[3] = w.y >> 16;
+                    s[4] = w.z & 0xffffu; s[5] = w.z >> 16; s[6] = w.w & 0xffffu; s[7] = w.w >> 16;
+                } else {
+                    const uint4 y = *reinterpret_cast<const uint4 *>(stage + at + 4);
+                    s[0] = w.x; s[1] = w.y; s[2] = w.z; s[3] = w.w;
+                    s[4] = y.x ^ flip; s[5] = y.y ^ flip; s[6] = y.z ^ flip; s[7] = y.w ^ flip;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < kPer; ++j)
+                    s[j] = at + j < pad ? 0u : (at + j < end ? (uint32_t)(S)(stage[at + j] ^ (S)flip) : 0xffffffffu);
+            }
+            if (two) {
+                sort_window(s);
+                const K base = lo + ((K)u0 << UB);
+                if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
+                    put(out - pad, at, inner, pad, end, [&](int j) { return inv(base + s[j]); });
+            } else {
+                K x[kPer];
+#pragma unroll
+                for (int j = 0; j < kPer; ++j) {
+                    if (at + j < pad) x[j] = K(0);
+                    else if (at + j >= end) x[j] = all_ones<K>();
+                    else {
+                        uint32_t u = u0;
+                        while (sm.unit[u + 1] <= p0 + (uint32_t)(at + j - pad)) ++u;
+                        x[j] = lo + (((K)u << UB) | (s[j] & ((1u << UB) - 1u)));
+                    }
+                }
+                sort_window(x);
+                if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
+                    put(out - pad, at, inner, pad, end, [&](int j) { return inv(x[j]); });
+            }
+        }
+    }
+
+    // Smallest and largest key of the segment (n >= 1), for every thread.
+    template <typename Xf>
+    __device__ static void bounds(unsigned char *smem, const K *__restrict__ src, int n, Xf xf, K &lo, K &hi) {
+        K *red = reinterpret_cast<K *>(smem);
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        K mn = all_ones<K>(), mx = K(0);
+        for_each(src, n, xf, [&](K k) {
+            mn = k < mn ? k : mn;
+            mx = k > mx ? k : mx;
+        });
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const K a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+            mn = a < mn ? a : mn;
+            mx = b > mx ? b : mx;
+        }
+        if (lane == 0) {
+            red[warp] = mn;
+            red[W + warp] = mx;
+        }
+        __syncthreads();
+        lo = red[0];
+        hi = red[W];
+        for (int w = 1; w < W; ++w) {
+            lo = red[w] < lo ? red[w] : lo;
+            hi = red[W + w] > hi ? red[W + w] : hi;
+        }
+        __syncthreads();
+    }
+
+    // Sorts the n keys at src into out[0..n), as CTA g of G.  Returns false
+    // (in every CTA of the segment alike, with nothing written) when a run of
+    // 256 bins holds more keys than a part or there are too many long bins.
+    template <typename Xf, typename Inv>
+    __device__ static bool run(unsigned char *smem, const K *__restrict__ src, int n, K lo, K hi, K *out, int g, int G,
+                               Xf xf, Inv inv) {
+        Smem &sm = *reinterpret_cast<Smem *>(smem);
+        uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + kHead);
+        unsigned char *stage = smem + kHead + (size_t)NBMAX * 2;
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        // bins: a power of two about the number of keys
+        int nbl = 9;
+        while ((1 << nbl) < NBMAX && (1 << nbl) < n) ++nbl;
+        const K range = hi - lo;
+        const int bits = bit_length<K>(range);
+        const int shift = bits > nbl ? bits - nbl : 0;
+        const uint32_t nb = 1u << nbl, nseg = nb / kSegBins, hseg = nseg / 2, wmask = nb / 2 - 1;
+        // a narrow stage where a wide one would need more parts (or, of 64-bit
+        // keys, wherever it can be: its windows sort half words)
+        const K nu = (range >> UB) + 1;
+        const bool narrow = (sizeof(K) == 8 || (uint32_t)n > kUseWide) && shift + 3 <= UB && nu <= (K)kUnits &&
+                            (nu <= 2 || (uint64_t)nu * kWin <= (uint64_t)n);
+        const uint32_t nunits = (uint32_t)nu;
+        for (uint32_t q = tid; q < nb / 8; q += T) reinterpret_cast<uint4 *>(cnt)[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid == 0) {
+            sm.nlong = 0;
+            sm.bad = 0;
+        }
+        __syncthreads();
+        // keys outside [lo, hi] (a region that overflowed, which is reported) stay in bounds
+        auto bin_of = [&](K v) { return min((uint32_t)(v >> shift), nb - 1u); };
+        for_each(src, n, xf, [&](K k) {
+            const uint32_t b = bin_of(k - lo);
+            atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u);
+        });
+        __syncthreads();
+        // a warp takes 256 words: 256 bins in the low halves, 256 in the high ones
+        auto load8 = [&](uint32_t s, uint32_t (&w)[8]) {
+            const uint4 a = reinterpret_cast<const uint4 *>(cnt)[s * 64 + lane * 2];
+            const uint4 b = reinterpret_cast<const uint4 *>(cnt)[s * 64 + lane * 2 + 1];
+            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+            w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+        };
+        for (uint32_t s = warp; s < hseg; s += W) {
+            uint32_t w[8], l = 0, h = 0;
+            load8(s, w);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                l += w[j] & 0xffffu;
+                h += w[j] >> 16;
+            }
+            l = __reduce_add_sync(0xffffffffu, l);
+            h = __reduce_add_sync(0xffffffffu, h);
+            if (lane == 0) {
+                sm.seg[s] = l;
+                sm.seg[hseg + s] = h;
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t v[4], loc = 0, mx = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t s = lane * 4 + j;
+                v[j] = s < nseg ? sm.seg[s] : 0u;
+                loc += v[j];
+                mx = max(mx, v[j]);
+            }
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            uint32_t tot;
+            uint32_t at = warp_excl_scan(loc, &tot);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t s = lane * 4 + j;
+                if (s < nseg) sm.seg[s] = at;
+                at += v[j];
+            }
+            if (lane == 31) sm.seg[nseg] = tot;
+            __syncwarp();
+            // One part when the stage holds the segment.  Its positions are 16
+            // bits wide, counted from the middle bin's in the upper half of
+            // the bins.  Otherwise a part starts at the first segment at or
+            // past a multiple of target, so it holds at most target + mx keys,
+            // and its positions count from its start.  (A bin count past 16
+            // bits shows in the total.)
+            const uint32_t use = narrow ? kUseNarrow : kUseWide, mid = sm.seg[hseg];
+            uint32_t np = 1, half = mid;
+            bool ok = tot == (uint32_t)n;
+            if ((uint32_t)n > use || G > 1 || mid > 65000u || (uint32_t)n - mid > 65000u) {
+                const uint32_t most = min(use, 65528u);
+                ok = ok && mx < most;
+                np = ok ? ((uint32_t)n + (most - mx) - 1) / (most - mx) : 1u;
+                np = min(max(np, (uint32_t)G), max(np, nseg));
+                ok = ok && np <= (uint32_t)kPartsMax;
+                half = 0;
+            }
+            if (ok) {
+                const uint32_t target = ((uint32_t)n + np - 1) / np;
+                if (lane < (int)np) {  // part `lane` starts at the first segment at or past lane * target
+                    const uint32_t want = lane * target;
+                    uint32_t a = 0, b = nseg;
+                    while (a < b) {
+                        const uint32_t m = (a + b) >> 1;
+                        if (sm.seg[m] < want) a = m + 1;
+                        else b = m;
+                    }
+                    sm.pseg[lane] = a;
+                }
+                if (lane == 0) {
+                    sm.pseg[np] = nseg;
+                    sm.nparts = np;
+                    sm.half = half;
+                    sm.unit[nunits <= (uint32_t)kUnits ? nunits : 0] = 0xffffffffu;
+                    sm.unit[nunits <= (uint32_t)kUnits ? nunits + 1 : 0] = 0xffffffffu;
+                }
+            } else if (lane == 0) {
+                sm.bad = 1;
+            }
+        }
+        __syncthreads();
+        if (sm.bad) return false;
+        const uint32_t nparts = sm.nparts, half = sm.half;
+        // counts -> each bin's first slot inside its part; units and long bins recorded
+        for (uint32_t s = warp; s < hseg; s += W) {
+            uint32_t w[8], out_w[8];
+            load8(s, w);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) out_w[j] = 0;
+#pragma unroll
+            for (int hi_half = 0; hi_half < 2; ++hi_half) {
+                const uint32_t sg = s + hi_half * hseg;
+                uint32_t t = 0, m = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t c = (w[j] >> (16 * hi_half)) & 0xffffu;
+                    t += c;
+                    m = max(m, c);
+                }
+                uint32_t tot;
+                uint32_t p = warp_excl_scan(t, &tot) + sm.seg[sg];
+                uint32_t ps = 0;  // the part of this segment: the last one starting at or before it
+                for (uint32_t q = 1; q < nparts; ++q)
+                    if (sm.pseg[q] <= sg) ps = q;
+                const uint32_t bin0 = sg * kSegBins + lane * 8;
+                if (narrow && (bin0 & ((1u << (UB - shift)) - 1u)) == 0u && (bin0 >> (UB - shift)) < nunits)
+                    sm.unit[bin0 >> (UB - shift)] = p;
+                // relative to the part's start (or the middle) and the stage's pad
+                const uint32_t pstart = sm.seg[sm.pseg[ps]];
+                p += (uint32_t)(((uintptr_t)(out + pstart) / sizeof(K)) & (V - 1)) - pstart - (hi_half ? half : 0u);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    out_w[j] |= p << (16 * hi_half);
+                    p += (w[j] >> (16 * hi_half)) & 0xffffu;
+                }
+                if (shift > 0 && m > (uint32_t)kEdge) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t c = (w[j] >> (16 * hi_half)) & 0xffffu;
+                        if (c > (uint32_t)kEdge) {
+                            const uint32_t at = atomicAdd(&sm.nlong, 1u);
+                            if (at < (uint32_t)kLongMax) sm.longs[at] = (bin0 + j) | c << 16;
+                        }
+                    }
+                }
+            }
+            reinterpret_cast<uint4 *>(cnt)[s * 64 + lane * 2] = make_uint4(out_w[0], out_w[1], out_w[2], out_w[3]);
+            reinterpret_cast<uint4 *>(cnt)[s * 64 + lane * 2 + 1] = make_uint4(out_w[4], out_w[5], out_w[6], out_w[7]);
+        }
+        __syncthreads();
+        if (sm.nlong > (uint32_t)kLongMax) return false;
+        auto slot_of = [&](uint32_t b, uint32_t word) {
+            return b > wmask ? (word >> 16) + half : word & 0xffffu;
+        };
+        auto place = [&](uint32_t b, K v, K k) {
+            const uint32_t at = slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u));
+            if (narrow) reinterpret_cast<S *>(stage)[at] = (S)v;
+            else reinterpret_cast<K *>(stage)[at] = k;
+        };
+        for (uint32_t part = g; part < nparts; part += G) {
+            const uint32_t s0 = sm.pseg[part], s1 = sm.pseg[part + 1];
+            const uint32_t p0 = sm.seg[s0], np = sm.seg[s1] - p0;
+            if (np == 0) continue;  // uniform
+            const uint32_t b0 = s0 * kSegBins, bn = (s1 - s0) * kSegBins;
+            if (nparts == 1) {
+                if (narrow) {
+                    for_each(src, n, xf, [&](K k) {
+                        const K v = k - lo;
+                        const uint32_t b = bin_of(v);
+                        reinterpret_cast<S *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = (S)v;
+                    });
+                } else {
+                    for_each(src, n, xf, [&](K k) {
+                        const uint32_t b = bin_of(k - lo);
+                        reinterpret_cast<K *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = k;
+                    });
+                }
+            } else {
+                for_each(src, n, xf, [&](K k) {
+                    const K v = k - lo;
+                    const uint32_t b = bin_of(v);
+                    if (b - b0 < bn) place(b, v, k);
+                });
+            }
+            __syncthreads();
+            auto end_of = [&](uint32_t b) { return slot_of(b, cnt[b & wmask]); };
+            K *o = out + p0;
+            const int pad = (int)(((uintptr_t)o / sizeof(K)) & (V - 1));
+            if (narrow) {
+                if (sm.nlong) {
+                    sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, end_of);
+                    __syncthreads();
+                }
+                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, nunits, lo, o, inv);
+            } else {
+                if (sm.nlong) {
+                    sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, end_of);
+                    __syncthreads();
+                }
+                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, o, inv);
+            }
+            __syncthreads();  // the next part reuses the stage
+        }
+        return true;
+    }
+};
+
+// The shapes it runs in: one CTA of 1024 threads per SM, two of 512, or five
+// of 256 (228 KB of shared memory per SM, 1 KB of it reserved per CTA).
+enum { kCountSmall = 0, kCountMedium = 1, kCountLarge = 2 };
+template <int SIZE> struct CountShape {
+    static constexpr int T = SIZE == kCountLarge ? 1024 : SIZE == kCountMedium ? 512 : 256;
+    static constexpr int kPerSm = SIZE == kCountLarge ? 1 : SIZE == kCountMedium ? 2 : 5;
+    static constexpr int kBins = SIZE == kCountLarge ? 32768 : SIZE == kCountMedium ? 16384 : 4096;
+    static constexpr int kStageBytes = SIZE == kCountLarge ? 155648 : SIZE == kCountMedium ? 75776 : 32768;
+    template <typename K> using Sort = CountSort<K, T, kBins, kStageBytes>;
+    static_assert(kPerSm * (Sort<uint32_t>::smem_bytes() + 1024) <= 228 * 1024, "resident CTAs");
+    static_assert(kPerSm * (Sort<uint64_t>::smem_bytes() + 1024) <= 228 * 1024, "resident CTAs");
+};
+
+// The shape for segments of about `keys` keys: the smallest whose stage holds
+// one with room for uneven ones.
+inline int count_sort_size(int64_t keys, int key_bytes) {
+    if (keys * key_bytes <= CountShape<kCountSmall>::kStageBytes * 3 / 4) return kCountSmall;
+    if (keys * key_bytes <= CountShape<kCountMedium>::kStageBytes * 7 / 8) return kCountMedium;
+    return kCountLarge;
+}
+
+// CTAs per segment: one when the segments fill the GPU, else as many as keep it
+// full while each still places 1024 keys or more.
+template <int SIZE> int count_sort_ctas(int64_t segments, int64_t keys) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t slots = (int64_t)(sms > 0 ? sms : 1) * CountShape<SIZE>::kPerSm;
+    const int64_t g = segments > 0 ? slots / segments : 1;
+    return (int)imax64(1, imin64(imin64(g, keys / 1024), 16));
+}
+
+} // namespace bsps

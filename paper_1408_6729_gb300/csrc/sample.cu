@@ -4,7 +4,7 @@
 #include "mlp.cuh"
 #include "segsort.cuh"
 #include "segsort_keys.cuh"
-#include "bucket_keys32.cuh"
+#include "countsort.cuh"
 
 namespace bsps {
 
@@ -161,8 +161,8 @@ run_sample_keys_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, int64
 // ---------------------------------------------------------------------------
 // The same sample from the counting sort, when the sorted blocks of keys
 // without payloads are kept: a
-// block's 32-bit keys (their phi, as they load) are sorted by the keys-only
-// counting sort of bucket_keys32.cuh -- the bucket sort's own kernel -- into
+// block's 32-bit keys (their phi, as they load) are sorted by the streamed
+// counting sort of countsort.cuh -- the bucket sort's own -- into
 // the sorted block; run_sample_tags_kernel then reads the keys at the sampled
 // ranks and finds their tags (input positions).  Equal keys leave
 // the counting sort in no particular order, which neither the sorted block
@@ -174,18 +174,19 @@ template <int DT> struct PhiOf {
     __device__ uint32_t operator()(uint32_t u) const { return (uint32_t)KeyTraits<DT>::phi(u); }
 };
 
-template <int DT, int CL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(512, 2)
+template <int DT, int SIZE>
+__global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
 run_sample_count_kernel(const uint32_t *__restrict__ keys, int64_t n, int64_t m, int64_t M, int64_t s, int64_t x,
-                        uint32_t *sphi, uint32_t *stag, uint32_t *retry, uint32_t *runs, DevStatus *st) {
+                        uint32_t *sphi, uint32_t *stag, uint32_t *retry, uint32_t *runs, int G) {
     // (sphi, stag: the pads' records only; the keys' records come from run_sample_tags_kernel)
-    using SS = BucketKeys32<CL>;
+    using CS = typename CountShape<SIZE>::template Sort<uint32_t>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t k = blockIdx.x / CL;
+    const int64_t k = blockIdx.x / G;
+    const int g = (int)(blockIdx.x % G);
     const int64_t lo = k * m;
     const int64_t len = lo < n ? imin64(m, n - lo) : 0;
-    if (blockIdx.x % CL == 0) {  // pads: sorted positions len..M-1, in tag order
-        for (int64_t j = 1 + threadIdx.x; j <= s; j += blockDim.x) {
+    if (g == 0) {  // pads: sorted positions len..M-1, in tag order
+        for (int64_t j = imax64(1, (len + 1) / x) + threadIdx.x; j <= s; j += blockDim.x) {
             const int64_t pos = j * x - 1;
             if (pos >= len) {
                 sphi[k * s + (j - 1)] = 0xffffffffu;
@@ -196,7 +197,7 @@ run_sample_count_kernel(const uint32_t *__restrict__ keys, int64_t n, int64_t m,
     if (len == 0) return;
     {
         // many repeats among 64 evenly spaced keys: the few-values sampler
-        // (every CTA of the cluster reads the same keys and decides alike)
+        // (every CTA of the block reads the same keys and decides alike)
         __shared__ uint32_t probe[64];
         __shared__ int repeats;
         if (threadIdx.x < 64) probe[threadIdx.x] = keys[lo + threadIdx.x * len / 64];
@@ -213,17 +214,11 @@ run_sample_count_kernel(const uint32_t *__restrict__ keys, int64_t n, int64_t m,
             return;
         }
     }
-    auto emit = [&](uint32_t pos, uint32_t key) { runs[lo + pos] = key; };
-    typename SS::Smem &sm = *reinterpret_cast<typename SS::Smem *>(smem_raw);
-    if (threadIdx.x == 0) sm.stalled = 0;
-    __syncthreads();
-    bool done = SS::run(smem_raw, keys + lo, len, 0u, 0xffffffffu, emit, st, PhiOf<DT>());
-    __syncthreads();
-    if (sm.stalled) {  // the staged load's wait ran out: wait for the copy once more, give the block back
-        SS::wait_staged(sm, kSpinLimit);
-        done = false;
-    }
-    if (!done && threadIdx.x == 0) retry[k] = 1u;
+    uint32_t kmin, kmax;
+    CS::bounds(smem_raw, keys + lo, (int)len, PhiOf<DT>(), kmin, kmax);
+    if (!CS::run(smem_raw, keys + lo, (int)len, kmin, kmax, runs + lo, g, G, PhiOf<DT>(), [](uint32_t v) { return v; }) &&
+        threadIdx.x == 0)
+        retry[k] = 1u;
 }
 
 // Tags of the sampled keys of a block sorted by run_sample_count_kernel: the
@@ -1334,27 +1329,25 @@ template <int DT, int CL> static cudaError_t launch_run_sample_keys(const Ctx &c
     return cudaGetLastError();
 }
 
-// the kept blocks are sorted by the counting sort: keys without payloads
-// (it moves keys only), whole 16-byte groups of keys in every block and in
-// the input (its bulk copies read nothing past n)
+// the kept blocks are sorted by the counting sort: keys without payloads (it
+// moves keys only)
 bool counting_block_sort(const Ctx &c) {
     const Plan &p = c.pl;
-    return p.keep_runs && !p.pairs && p.key_bytes == 4 && run_keys_cluster(p) != 0 && p.m % 4 == 0 &&
-           p.n % 4 == 0 && ((uintptr_t)c.keys_in & 15) == 0;
+    return p.keep_runs && !p.pairs && p.key_bytes == 4 && run_keys_cluster(p) != 0;
 }
 
-template <int DT, int CL> static cudaError_t launch_run_sample_count(const Ctx &c) {
-    using SS = BucketKeys32<CL>;
-    const size_t smem = SS::smem_bytes();
-    auto kern = run_sample_count_kernel<DT, CL>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int DT, int SIZE> static cudaError_t launch_run_sample_count(const Ctx &c) {
+    using CS = typename CountShape<SIZE>::template Sort<uint32_t>;
+    auto kern = run_sample_count_kernel<DT, SIZE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS::smem_bytes());
     if (e != cudaSuccess) return e;
     const Plan &p = c.pl;
     e = cudaMemsetAsync(c.ly.run_retry, 0, (size_t)p.R * 4, c.stream);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)(p.R * CL), 512, smem, c.stream>>>((const uint32_t *)c.keys_in, p.n, p.m, p.M, p.s, p.x,
-                                                        (uint32_t *)c.ly.sphi[0], c.ly.stag[0], c.ly.run_retry,
-                                                        (uint32_t *)c.ly.runs, c.ly.status);
+    const int G = count_sort_ctas<SIZE>(p.R, p.m);
+    kern<<<(unsigned)(p.R * G), CountShape<SIZE>::T, CS::smem_bytes(), c.stream>>>(
+        (const uint32_t *)c.keys_in, p.n, p.m, p.M, p.s, p.x, (uint32_t *)c.ly.sphi[0], c.ly.stag[0], c.ly.run_retry,
+        (uint32_t *)c.ly.runs, G);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int bits = tag_slot_bits(p);
@@ -1389,11 +1382,10 @@ template <int DT> static cudaError_t launch_sample_t(const Ctx &c) {
     if constexpr (sizeof(K) == 4) {
         cudaError_t e = cudaSuccess;
         if (counting_block_sort(c)) {
-            switch (run_keys_cluster(p)) {
-            case 1: e = launch_run_sample_count<DT, 1>(c); break;
-            case 2: e = launch_run_sample_count<DT, 2>(c); break;
-            case 4: e = launch_run_sample_count<DT, 4>(c); break;
-            default: e = launch_run_sample_count<DT, 8>(c); break;
+            switch (count_sort_size(p.m, 4)) {
+            case kCountSmall: e = launch_run_sample_count<DT, kCountSmall>(c); break;
+            case kCountMedium: e = launch_run_sample_count<DT, kCountMedium>(c); break;
+            default: e = launch_run_sample_count<DT, kCountLarge>(c); break;
             }
             only = c.ly.run_retry;
         } else {
