@@ -3,8 +3,9 @@
 #include <cmath>
 #include <cstring>
 
-#include "kernels.cuh"
+#include "many.cuh"
 #include "mlp.cuh"
+#include "small.cuh"
 
 namespace bsps {
 
@@ -86,6 +87,7 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     }
     if (pl.sample_size >= ((int64_t)1 << 31) || pl.p > 65535) return BSPS_ERR_TOO_LARGE;
 
+    pl.lut_bits = kLutBits;
     // sub-buckets: the smallest refinement whose expected size fits one
     // cluster's shared memory with head room for the sampling imbalance
     const int64_t cap_cta = cta_capacity(pl.key_bytes, pairs);
@@ -149,9 +151,12 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     pl.cap = (pl.cap + 3) & ~int64_t(3);  // 16-byte aligned regions
     if (!pl.merge && (double)pl.P * pl.cap >= 4.0e9) return BSPS_ERR_TOO_LARGE;
     pl.tiles = (n + kRouteTile - 1) / kRouteTile;
-    pl.lsd_tiles = (pl.sample_size + kLsdTile - 1) / kLsdTile;
-    pl.lsd_npos = 4 + pl.key_bytes;
     if (route_smem_bytes(pl) > 227 * 1024) return BSPS_ERR_TOO_LARGE;
+    // a finer radix index where the routing kernel has room for it and the
+    // sample buffer that holds it (make_layout) is large enough
+    if (!pairs && !pl.keep_runs && route_keys_fine_index(pl) &&
+        pl.sample_size * pl.key_bytes >= ((1 << kLutBitsFine) + 2) * 2)
+        pl.lut_bits = kLutBitsFine;
 
     // workspace size
     int64_t o = 0;
@@ -160,9 +165,7 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     const int64_t S = std::max<int64_t>(pl.sample_size, 1);
     take(S * pl.key_bytes); take(S * pl.key_bytes);
     take(S * 4); take(S * 4);
-    take(std::max<int64_t>(pl.lsd_tiles, 1) * 256 * 4);
-    take(16 * 256 * 4);
-    take(64 * 4);
+    take((int64_t)sample_scratch_bytes(pl));
     take(pl.P * pl.key_bytes);
     take(pl.P * 4);
     take((kLutCells + 2) * 2);
@@ -210,12 +213,11 @@ static Layout make_layout(const Plan &pl, void *ws) {
     l.sphi[1] = take(S * pl.key_bytes);
     l.stag[0] = (uint32_t *)take(S * 4);
     l.stag[1] = (uint32_t *)take(S * 4);
-    l.lsd_counts = (uint32_t *)take(std::max<int64_t>(pl.lsd_tiles, 1) * 256 * 4);
-    l.lsd_hist = (uint32_t *)take(16 * 256 * 4);
-    l.lsd_table = (int32_t *)take(64 * 4);
+    l.pivots = take((int64_t)sample_scratch_bytes(pl));
     l.vphi = take(pl.P * pl.key_bytes);
     l.vtag = (uint32_t *)take(pl.P * 4);
     l.lut = (uint16_t *)take((kLutCells + 2) * 2);
+    if (pl.lut_bits > kLutBits) l.lut = (uint16_t *)l.sphi[1 - sample_final(pl)];  // free once the splitters are chosen
     l.lutp = take(64);
     const bool look_back = pl.pairs && !pl.keep_runs;
     l.state = (uint32_t *)take(look_back ? std::max<int64_t>(pl.tiles, 1) * pl.P * 4 : 0);
@@ -270,17 +272,14 @@ static void to_public(const Plan &p, bsps_plan *out) {
     out->bucket_cluster = p.bucket_cl; out->route_tiles = p.tiles; out->workspace_bytes = p.ws_bytes;
 }
 
-// Kernels one call launches (the sample sort launches all its pass slots;
-// slots whose byte position is constant return at once).
+// Kernels one call launches.
 static int kernels_per_call(const Ctx &c) {
     const Plan &pl = c.pl;
     int k = 1;                                   // sample (random draw or block sort)
     if (run_keys_cluster(pl)) k += 2;            // keys-only and few-values block samplers before the stable one
     if (counting_block_sort(c)) k += 1;          // the counting sort's tags
-    if (pl.sampling == BSPS_RANDOM && pl.sample_size == 0) k = 0;
-    k += 2 + (pl.lsd_tiles > 0 ? 3 * pl.lsd_npos : 0);  // histogram, pass table, passes
-    if (msd_sample_sort(pl)) k += 4;                 // MSD histogram, plan, scatter, bin sorts
-    k += 2;                                      // splitters, radix index
+    k += sample_sort_kernels(pl);
+    k += 1;                                      // splitters and radix index
     if (pl.merge) return k + 3;                  // partition, bucket offsets, merge
     k += 2;                                      // routing (partition and segment copy: one more), bucket offsets
     if (pl.seg_route) k += 1;
@@ -304,10 +303,10 @@ static int debug_kernels(const Ctx &c) {
         if ((call) != cudaSuccess) return BSPS_ERR_CUDA;  \
     } while (0)
 
-static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uint32_t *vals_out, int64_t n,
-               int32_t dtype, const bsps_params *prm, int64_t *bucket_sizes, const bsps_debug *dbg, void *ws,
-               size_t ws_bytes, void *stream) {
-    Ctx c;
+// The plan and the argument checks of one call; c is filled up to its layout.
+static int prepare_call(Ctx &c, const void *keys_in, const uint32_t *vals_in, void *keys_out, uint32_t *vals_out, int64_t n,
+                        int32_t dtype, const bsps_params *prm, int64_t *bucket_sizes, const bsps_debug *dbg, void *ws,
+                        size_t ws_bytes, void *stream) {
     std::memset(&c, 0, sizeof(c));
     const int pairs = vals_in != nullptr;
     int rc = make_plan(n, dtype, prm, pairs, c.pl);
@@ -326,53 +325,105 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
     c.bucket_sizes = bucket_sizes;
     if (dbg) c.dbg = *dbg;
     c.stream = (cudaStream_t)stream;
-    BSPS_CUDA(cudaMemsetAsync(c.ly.status, 0, sizeof(DevStatus), c.stream));
+    return BSPS_OK;
+}
+
+int prepare_keys_call(Ctx &c, const void *keys_in, void *keys_out, int64_t n, int32_t dtype, const bsps_params *prm,
+                      int64_t *bucket_sizes, void *ws, size_t ws_bytes, void *stream) {
+    return prepare_call(c, keys_in, nullptr, keys_out, nullptr, n, dtype, prm, bucket_sizes, nullptr, ws, ws_bytes, stream);
+}
+
+// Random sampling, keys only, n >= 1: the whole path, for one call or for all
+// the calls of a batch (mark(i): phase boundary i).
+template <typename Mark> static int run_keys(Exec &x, Mark mark) {
+    BSPS_CUDA(mark(0));
+    BSPS_CUDA(launch_sample_random(x));
+    BSPS_CUDA(mark(1));
+    BSPS_CUDA(launch_sample_sort(x));
+    BSPS_CUDA(mark(2));
+    BSPS_CUDA(launch_splitters(x));
+    BSPS_CUDA(launch_mlp_train(x));
+    BSPS_CUDA(mark(3));
+    BSPS_CUDA(launch_route_keys(x));
+    BSPS_CUDA(launch_bucket_finish(x));
+    BSPS_CUDA(mark(4));
+    BSPS_CUDA(launch_bucket_keys(x));
+    BSPS_CUDA(mark(5));
+    return BSPS_OK;
+}
+int run_keys_calls(Exec &x) {
+    return run_keys(x, [](int) { return cudaSuccess; });
+}
+
+static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uint32_t *vals_out, int64_t n,
+               int32_t dtype, const bsps_params *prm, int64_t *bucket_sizes, const bsps_debug *dbg, void *ws,
+               size_t ws_bytes, void *stream) {
+    Ctx c;
+    const int rc = prepare_call(c, keys_in, vals_in, keys_out, vals_out, n, dtype, prm, bucket_sizes, dbg, ws, ws_bytes, stream);
+    if (rc) return rc;
+    if (!dbg && small_call(c.pl)) {
+        BSPS_CUDA(launch_small_call(c));
+        return BSPS_OK;
+    }
     if (n == 0) {
+        BSPS_CUDA(cudaMemsetAsync(c.ly.status, 0, sizeof(DevStatus), c.stream));
         if (bucket_sizes) BSPS_CUDA(cudaMemsetAsync(bucket_sizes, 0, sizeof(int64_t) * c.pl.p, c.stream));
         if (dbg && dbg->pad_sizes) BSPS_CUDA(cudaMemsetAsync(dbg->pad_sizes, 0, sizeof(int64_t) * c.pl.p, c.stream));
         return BSPS_OK;
     }
     void *const *ev = dbg ? dbg->phase_events : nullptr;
     auto mark = [&](int i) { return ev ? cudaEventRecord((cudaEvent_t)ev[i], c.stream) : cudaSuccess; };
-    if (c.pl.pairs && !c.pl.keep_runs)
-        BSPS_CUDA(cudaMemsetAsync(c.ly.state, 0, (size_t)c.pl.tiles * c.pl.P * 4, c.stream));
-    BSPS_CUDA(cudaMemsetAsync(c.ly.cursor, 0, (size_t)c.pl.P * 4, c.stream));
-    if (!c.pl.pairs) BSPS_CUDA(cudaMemsetAsync(c.ly.retry_flag, 0, (size_t)c.pl.P * 4, c.stream));
-    BSPS_CUDA(mark(0));
-    BSPS_CUDA(launch_sample(c));
-    if (c.pl.keep_runs) {  // every block's own sample records, for the partition (the sample sort reuses the buffer)
-        BSPS_CUDA(cudaMemcpyAsync(c.ly.rs_phi, c.ly.sphi[0], (size_t)c.pl.sample_size * 4, cudaMemcpyDeviceToDevice,
-                                  c.stream));
-        BSPS_CUDA(cudaMemcpyAsync(c.ly.rs_tag, c.ly.stag[0], (size_t)c.pl.sample_size * 4, cudaMemcpyDeviceToDevice,
-                                  c.stream));
-    }
-    BSPS_CUDA(mark(1));
-    BSPS_CUDA(launch_sample_sort(c));
-    BSPS_CUDA(mark(2));
-    BSPS_CUDA(launch_splitters(c));
-    if (c.pl.classify == BSPS_LEARNED) BSPS_CUDA(launch_mlp_train(c));
-    BSPS_CUDA(mark(3));
-    if (c.pl.keep_runs) {
-        BSPS_CUDA(launch_merge_partition(c));
-        BSPS_CUDA(launch_bucket_finish(c));
-        if (c.pl.merge) {
-            BSPS_CUDA(mark(4));
-            BSPS_CUDA(launch_merge_buckets(c));
-        } else {
-            BSPS_CUDA(launch_segment_copy(c));
-            BSPS_CUDA(mark(4));
-            BSPS_CUDA(launch_bucket_sort(c));
-        }
-        if (dbg && dbg->partition)  // the rows of the p - 1 splitters among the sub-bucket splitters' rows
-            BSPS_CUDA(cudaMemcpy2DAsync(dbg->partition, (size_t)c.pl.R * 4, c.ly.part, (size_t)(c.pl.B * c.pl.R * 4),
-                                        (size_t)c.pl.R * 4, (size_t)(c.pl.p + 1), cudaMemcpyDeviceToDevice,
-                                        c.stream));
+    Exec x = {&c, 1, c.stream};
+    if (c.pl.sampling == BSPS_RANDOM && !c.pl.pairs) {
+        const int rk = run_keys(x, mark);
+        if (rk) return rk;
     } else {
-        BSPS_CUDA(launch_route(c));
-        BSPS_CUDA(mark(4));
-        BSPS_CUDA(launch_bucket_sort(c));
+        const bool random = c.pl.sampling == BSPS_RANDOM;
+        if (!random) {
+            BSPS_CUDA(cudaMemsetAsync(c.ly.status, 0, sizeof(DevStatus), c.stream));
+            BSPS_CUDA(cudaMemsetAsync(c.ly.cursor, 0, (size_t)c.pl.P * 4, c.stream));
+            if (!c.pl.pairs) BSPS_CUDA(cudaMemsetAsync(c.ly.retry_flag, 0, (size_t)c.pl.P * 4, c.stream));
+        }
+        if (c.pl.pairs && !c.pl.keep_runs)
+            BSPS_CUDA(cudaMemsetAsync(c.ly.state, 0, (size_t)c.pl.tiles * c.pl.P * 4, c.stream));
+        BSPS_CUDA(mark(0));
+        BSPS_CUDA(random ? launch_sample_random(x) : launch_sample(c));
+        if (c.pl.keep_runs) {  // every block's own sample records, for the partition (the sample sort reuses the buffer)
+            BSPS_CUDA(cudaMemcpyAsync(c.ly.rs_phi, c.ly.sphi[0], (size_t)c.pl.sample_size * 4, cudaMemcpyDeviceToDevice,
+                                      c.stream));
+            BSPS_CUDA(cudaMemcpyAsync(c.ly.rs_tag, c.ly.stag[0], (size_t)c.pl.sample_size * 4, cudaMemcpyDeviceToDevice,
+                                      c.stream));
+        }
+        BSPS_CUDA(mark(1));
+        BSPS_CUDA(launch_sample_sort(x));
+        BSPS_CUDA(mark(2));
+        BSPS_CUDA(launch_splitters(x));
+        BSPS_CUDA(launch_mlp_train(x));
+        BSPS_CUDA(mark(3));
+        auto bucket_sort = [&] { return c.pl.pairs ? launch_bucket_pairs(x) : launch_bucket_keys(x); };
+        if (c.pl.keep_runs) {
+            BSPS_CUDA(launch_merge_partition(c));
+            BSPS_CUDA(launch_bucket_finish(x));
+            if (c.pl.merge) {
+                BSPS_CUDA(mark(4));
+                BSPS_CUDA(launch_merge_buckets(c));
+            } else {
+                BSPS_CUDA(launch_segment_copy(c));
+                BSPS_CUDA(mark(4));
+                BSPS_CUDA(bucket_sort());
+            }
+            if (dbg && dbg->partition)  // the rows of the p - 1 splitters among the sub-bucket splitters' rows
+                BSPS_CUDA(cudaMemcpy2DAsync(dbg->partition, (size_t)c.pl.R * 4, c.ly.part, (size_t)(c.pl.B * c.pl.R * 4),
+                                            (size_t)c.pl.R * 4, (size_t)(c.pl.p + 1), cudaMemcpyDeviceToDevice,
+                                            c.stream));
+        } else {
+            BSPS_CUDA(c.pl.pairs ? launch_route(c) : launch_route_keys(x));
+            BSPS_CUDA(launch_bucket_finish(x));
+            BSPS_CUDA(mark(4));
+            BSPS_CUDA(bucket_sort());
+        }
+        BSPS_CUDA(mark(5));
     }
-    BSPS_CUDA(mark(5));
     if (dbg) BSPS_CUDA(launch_debug(c));
     if (dbg && dbg->launches) *dbg->launches = kernels_per_call(c) + debug_kernels(c);
     return BSPS_OK;

@@ -2,166 +2,30 @@
 // (no counterpart in the paper; each instance is the paper's sort, Fig. 2 /
 // Fig. 3, with its own parameters).
 //
-// Small instances run the whole method on chip, one CTA of 1024 threads per
-// instance, in one persistent launch: the random sample (Fig. 3 step 4, the
-// same counter-based draws as the single-instance path), the sample sort
-// (Fig. 1 step 5), the splitters of rank i*s (Fig. 2 step 6), classification
-// with the tag-free tie-break (Fig. 2 step 9), the bucket histogram and its
-// prefix (Fig. 1 step 9), routing into buckets (Fig. 1 step 11) and the final
-// sort of the buckets (Fig. 2 step 12), all in shared memory.  The buckets are
-// contiguous, ordered value ranges after routing, so one bitonic network over
-// the routed array sorts every bucket in place.  Larger instances run the
-// single-instance pipeline on several streams; the whole call is recorded
-// into one CUDA graph that later calls with the same arguments relaunch.
+// Small instances run the whole method on chip, one CTA per instance
+// (small.cu), in one launch per shape.  The larger ones, with random sampling,
+// run the single-call kernels together: every step of the path is one launch
+// for all of them (many.cuh), in waves that reuse one workspace.  With regular sampling they run the single-call pipeline on several
+// streams, recorded into one CUDA graph that later calls with the same
+// arguments relaunch.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <vector>
 
-#include "kernels.cuh"
+#include "many.cuh"
+#include "small.cuh"
 
 namespace bsps {
 
-constexpr int kSmallThreads = 1024;
 constexpr int kSmallMax = BSPS_BATCH_SMALL_MAX;    // keys of an on-chip instance
 constexpr int kSampleMax = BSPS_BATCH_SAMPLE_MAX;  // sample records of an on-chip instance
-constexpr int kSmallBucketsMax = 256;              // buckets of an on-chip instance
 constexpr int kLanesMax = 16;
+constexpr size_t kWaveBytes = (size_t)32 << 20;      // workspace of a wave of larger instances, per lane of the table
+constexpr size_t kTableBytes = 6144;                // argument tables of one larger instance, at most
 
-struct SmallJob {
-    int64_t off;    // first key of the instance
-    int64_t bbase;  // first bucket-size entry
-    uint64_t seed;
-    int32_t n, p, s, S;  // keys, buckets, samples per bucket, sample records (s*p - 1)
-};
-
-// Ascending bitonic network over a[0..n2), n2 a power of two, whole CTA.
-template <typename V> __device__ void bitonic_sort(V *a, int n2) {
-    for (int k = 2; k <= n2; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < (n2 >> 1); t += blockDim.x) {
-                const int i = 2 * t - (t & (j - 1));  // bit j of i is clear
-                const int l = i + j;
-                const bool up = (i & k) == 0;
-                const V x = a[i], y = a[l];
-                if ((x > y) == up) {
-                    a[i] = y;
-                    a[l] = x;
-                }
-            }
-            __syncthreads();
-        }
-}
-
-__host__ __device__ inline int pow2_ceil(int v) {
-    int r = 1;
-    while (r < v) r <<= 1;
-    return r;
-}
-
-// Shared memory of the on-chip kernel.
-struct SmallSmem {
-    uint64_t rec[kSampleMax];        // sample records (phi << 32 | tag)
-    uint32_t phi[kSmallMax];         // the instance's keys
-    uint32_t stage[kSmallMax];       // the keys routed into buckets
-    uint32_t hist[kSmallBucketsMax + 1];
-    uint32_t tmp[40];
-};
-
-template <int DT>
-__global__ void __launch_bounds__(kSmallThreads, 1)
-batch_small_kernel(const typename KeyTraits<DT>::T *__restrict__ keys_in, typename KeyTraits<DT>::T *keys_out,
-                   const SmallJob *jobs, int32_t njobs, int64_t *bucket_sizes) {
-    static_assert(sizeof(typename KeyTraits<DT>::T) == 4, "on-chip instances hold 32-bit keys");
-    constexpr int T = kSmallThreads, IT = kSmallMax / kSmallThreads;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmallSmem &sm = *reinterpret_cast<SmallSmem *>(smem_raw);
-    const int tid = threadIdx.x;
-
-    for (int32_t jb = blockIdx.x; jb < njobs; jb += gridDim.x) {
-        const SmallJob J = jobs[jb];
-        const int n = J.n, p = J.p;
-        if (n == 0) {
-            if (bucket_sizes)
-                for (int b = tid; b < p; b += T) bucket_sizes[J.bbase + b] = 0;
-            continue;
-        }
-        const typename KeyTraits<DT>::T *src = keys_in + J.off;
-        for (int e = tid; e < n; e += T) sm.phi[e] = KeyTraits<DT>::phi(src[e]);
-        __syncthreads();
-        // ---- random sample of s*p - 1 records (Fig. 3 step 4) and its sort ----
-        const int S = J.S;
-        if (p > 1 && S > 0) {
-            const int S2 = pow2_ceil(S);
-            for (int blk = tid; blk * 4 < S2; blk += T) {
-                uint64_t c[4] = {(uint64_t)blk, 0, 0, 0};
-                if (blk * 4 < S) philox4x64_10(c, J.seed, 0);
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const int j = blk * 4 + w;
-                    if (j < S) {
-                        const uint32_t g = (uint32_t)__umul64hi(c[w], (uint64_t)n);
-                        sm.rec[j] = (uint64_t)sm.phi[g] << 32 | g;
-                    } else if (j < S2) {
-                        sm.rec[j] = ~0ull;
-                    }
-                }
-            }
-            __syncthreads();
-            bitonic_sort(sm.rec, S2);
-        }
-        // ---- classify (splitter i is the record of rank i*s), histogram ----
-        for (int b = tid; b <= p; b += T) sm.hist[b] = 0;
-        __syncthreads();
-        uint32_t br[IT];  // bucket << 16 | rank inside the bucket
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = i * T + tid;
-            if (e < n) {
-                const uint64_t key = (uint64_t)sm.phi[e] << 32 | (uint32_t)e;
-                uint32_t lo = 0, hi = (uint32_t)p - 1;  // #{splitters <= key} in [lo, hi]
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1;
-                    if (sm.rec[(int64_t)mid * J.s - 1] <= key) lo = mid;
-                    else hi = mid - 1;
-                }
-                br[i] = lo << 16 | atomicAdd(&sm.hist[lo], 1u);
-            }
-        }
-        __syncthreads();
-        if (tid < 32) {  // bucket sizes and the buckets' starts
-            uint32_t carry = 0;
-            for (int b0 = 0; b0 < p; b0 += 32) {
-                const int b = b0 + tid;
-                const uint32_t c = b < p ? sm.hist[b] : 0u;
-                if (bucket_sizes && b < p) bucket_sizes[J.bbase + b] = c;
-                uint32_t tot;
-                const uint32_t ex = warp_excl_scan(c, &tot);
-                if (b < p) sm.hist[b] = carry + ex;
-                carry += tot;
-            }
-        }
-        __syncthreads();
-        // ---- route into the buckets (Fig. 1 step 11) ----
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = i * T + tid;
-            if (e < n) sm.stage[sm.hist[br[i] >> 16] + (br[i] & 0xffffu)] = sm.phi[e];
-        }
-        const int n2 = pow2_ceil(n);
-        for (int e = n + tid; e < n2; e += T) sm.stage[e] = 0xffffffffu;
-        __syncthreads();
-        // ---- final sort of the buckets (Fig. 2 step 12) ----
-        bitonic_sort(sm.stage, n2);
-        typename KeyTraits<DT>::T *dst = keys_out + J.off;
-        for (int e = tid; e < n; e += T) dst[e] = KeyTraits<DT>::inv(sm.stage[e]);
-        __syncthreads();
-    }
-}
-
-// Folds one instance's device status into the batch's.
-__global__ void merge_status_kernel(const DevStatus *from, DevStatus *into) {
-    if (threadIdx.x != 0) return;
+// Folds instances' device statuses into the batch's, one thread each.
+__device__ void fold_status(const DevStatus *from, DevStatus *into) {
     if (from->error) set_error(into, from->error);
     if (from->overflow) atomicExch(&into->overflow, 1);
     atomicAdd(&into->timeouts, from->timeouts);
@@ -170,6 +34,13 @@ __global__ void merge_status_kernel(const DevStatus *from, DevStatus *into) {
     atomicMax(&into->max_vbucket, from->max_vbucket);
     atomicAdd(&into->mispredicted, from->mispredicted);
     atomicAdd(&into->correction_steps, from->correction_steps);
+}
+__global__ void merge_status_kernel(const DevStatus *from, DevStatus *into) {
+    if (threadIdx.x == 0) fold_status(from, into);
+}
+__global__ void merge_statuses_kernel(const DevStatus *const *from, int count, DevStatus *into) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) fold_status(from[i], into);
 }
 
 // ---------------------------------------------------------------------------
@@ -200,8 +71,14 @@ struct BatchPlan {
     std::vector<Instance> inst;
     std::vector<SmallJob> jobs;
     std::vector<int64_t> bbase;
+    int first[4] = {0, 0, 0, 0};  // the jobs of each on-chip shape (small.cuh), in `jobs`
     size_t lane_ws = 0, jobs_bytes = 0, total = 0;
     int lanes = 1;
+    // random sampling: the larger instances by wave, their workspaces' offsets
+    // in the wave's and the workspace of the largest wave
+    std::vector<std::vector<int32_t>> waves;
+    std::vector<size_t> ws_at, ws_of;
+    size_t wave_ws = 0, tables_bytes = 0;
 };
 
 static int make_batch_plan(const int64_t *h_off, int32_t num, int32_t dtype, const bsps_params *prm,
@@ -216,6 +93,11 @@ static int make_batch_plan(const int64_t *h_off, int32_t num, int32_t dtype, con
     bp.jobs.clear();
     bp.lanes = t->lanes;
     size_t lane_ws = 0;
+    const bool grouped = prm->sampling == BSPS_RANDOM;
+    bp.ws_at.assign(num, 0);
+    bp.ws_of.assign(num, 0);
+    size_t largest = 0, sum = 0;
+    std::vector<int32_t> larger;
     for (int32_t i = 0; i < num; ++i) {
         const int64_t n = h_off[i + 1] - h_off[i];
         if (n < 0) return BSPS_ERR_INVALID_ARG;
@@ -234,10 +116,10 @@ static int make_batch_plan(const int64_t *h_off, int32_t num, int32_t dtype, con
         I.s = (int)pl.s;
         I.S = (int)pl.sample_size;
         I.small = c <= t->small_max_log2 && n <= kSmallMax && dtype != BSPS_F64 &&
-                  I.prm.sampling == BSPS_RANDOM && I.prm.classify == BSPS_TREE && I.prm.p <= kSmallBucketsMax &&
+                  I.prm.sampling == BSPS_RANDOM && I.prm.classify == BSPS_TREE && I.prm.p <= kSmallBuckets &&
                   pl.sample_size <= kSampleMax;
         if (I.small) {
-            SmallJob J;
+            SmallJob J = {};
             J.off = I.off;
             J.bbase = bp.bbase[i];
             J.seed = I.prm.seed;
@@ -250,13 +132,41 @@ static int make_batch_plan(const int64_t *h_off, int32_t num, int32_t dtype, con
             size_t w = 0;
             const int rc2 = bsps_workspace_size(n, dtype, &I.prm, 0, &w);
             if (rc2) return rc2;
-            lane_ws = std::max(lane_ws, w);
+            if (!grouped) {
+                lane_ws = std::max(lane_ws, w);
+            } else if (n > 0) {
+                bp.ws_of[i] = (w + 255) & ~size_t(255);
+                largest = std::max(largest, bp.ws_of[i]);
+                sum += bp.ws_of[i];
+                larger.push_back(i);
+            }
         }
     }
+    // waves of the larger instances: as many as a workspace for `lanes` of the
+    // largest holds, or for all of them up to kWaveBytes a lane
+    bp.wave_ws = std::max(std::min(sum, kWaveBytes * t->lanes), largest * t->lanes);
+    size_t used = 0;
+    for (const int32_t i : larger) {
+        if (bp.waves.empty() || used + bp.ws_of[i] > bp.wave_ws) {
+            bp.waves.emplace_back();
+            used = 0;
+        }
+        bp.waves.back().push_back(i);
+        bp.ws_at[i] = used;
+        used += bp.ws_of[i];
+    }
+    // by shape, and inside a shape the largest first
+    std::stable_sort(bp.jobs.begin(), bp.jobs.end(), [](const SmallJob &a, const SmallJob &b) {
+        const int x = small_size(a.n, a.S), y = small_size(b.n, b.S);
+        return x != y ? x < y : a.n > b.n;
+    });
+    for (const SmallJob &J : bp.jobs)
+        for (int size = small_size(J.n, J.S) + 1; size <= 3; ++size) ++bp.first[size];
     auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
     bp.lane_ws = up(lane_ws);
     bp.jobs_bytes = up(std::max<size_t>(1, bp.jobs.size()) * sizeof(SmallJob));
-    bp.total = up(sizeof(DevStatus)) + bp.jobs_bytes + (bp.lane_ws ? bp.lane_ws * bp.lanes : 0);
+    bp.tables_bytes = up(larger.size() * kTableBytes);
+    bp.total = up(sizeof(DevStatus)) + bp.jobs_bytes + bp.tables_bytes + bp.wave_ws + (bp.lane_ws ? bp.lane_ws * bp.lanes : 0);
     return BSPS_OK;
 }
 
@@ -293,31 +203,6 @@ static int lanes_for_device(LaneSet *&L) {
     return BSPS_OK;
 }
 
-template <int DT> static cudaError_t launch_small_t(const void *in, void *out, const SmallJob *jobs, int32_t njobs,
-                                                    int64_t *bsz, cudaStream_t st) {
-    using K = typename KeyTraits<DT>::T;
-    auto kern = batch_small_kernel<DT>;
-    const int smem = (int)sizeof(SmallSmem);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = std::max(1, std::min<int>(njobs, sms));
-    kern<<<grid, kSmallThreads, smem, st>>>((const K *)in, (K *)out, jobs, njobs, bsz);
-    return cudaGetLastError();
-}
-
-static cudaError_t launch_small(int32_t dtype, const void *in, void *out, const SmallJob *jobs, int32_t njobs,
-                                int64_t *bsz, cudaStream_t st) {
-    switch (dtype) {
-    case BSPS_U32: return launch_small_t<BSPS_U32>(in, out, jobs, njobs, bsz, st);
-    case BSPS_I32: return launch_small_t<BSPS_I32>(in, out, jobs, njobs, bsz, st);
-    case BSPS_F32: return launch_small_t<BSPS_F32>(in, out, jobs, njobs, bsz, st);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
 // Everything the call queues, on `stream` and the lanes forked from it.
 static int enqueue_batch(const BatchPlan &bp, const void *in, void *out, int32_t dtype, int64_t *bsz,
                          unsigned char *ws, cudaStream_t stream, LaneSet *L) {
@@ -327,12 +212,15 @@ static int enqueue_batch(const BatchPlan &bp, const void *in, void *out, int32_t
     } while (0)
     DevStatus *bst = (DevStatus *)ws;
     const SmallJob *djobs = (const SmallJob *)(ws + ((sizeof(DevStatus) + 255) & ~size_t(255)));
-    unsigned char *lane_ws = ws + ((sizeof(DevStatus) + 255) & ~size_t(255)) + bp.jobs_bytes;
+    unsigned char *lane_ws = ws + ((sizeof(DevStatus) + 255) & ~size_t(255)) + bp.jobs_bytes + bp.tables_bytes + bp.wave_ws;
     BSPS_CK(cudaMemsetAsync(bst, 0, sizeof(DevStatus), stream));
     const int nl = bp.lane_ws ? bp.lanes : 0;
     BSPS_CK(cudaEventRecord(L->fork, stream));
     for (int l = 0; l < nl; ++l) BSPS_CK(cudaStreamWaitEvent(L->s[l], L->fork, 0));
-    if (!bp.jobs.empty()) BSPS_CK(launch_small(dtype, in, out, djobs, (int32_t)bp.jobs.size(), bsz, stream));
+    for (int size = 2; size >= 0; --size) {  // the largest first
+        const int first = bp.first[size], count = bp.first[size + 1] - first;
+        if (count > 0) BSPS_CK(launch_small_jobs(dtype, size, in, out, djobs + first, count, bsz, stream));
+    }
     int l = 0;
     for (size_t i = 0; i < bp.inst.size(); ++i) {
         const Instance &I = bp.inst[i];
@@ -350,6 +238,63 @@ static int enqueue_batch(const BatchPlan &bp, const void *in, void *out, int32_t
         BSPS_CK(cudaEventRecord(L->join[q], L->s[q]));
         BSPS_CK(cudaStreamWaitEvent(stream, L->join[q], 0));
     }
+    return BSPS_OK;
+#undef BSPS_CK
+}
+
+// The on-chip instances in one launch per shape and, wave by wave, the larger
+// ones in one launch per step (random sampling).  The argument tables are
+// gathered first and uploaded in one copy (from pageable memory: the copy has
+// read it when cudaMemcpyAsync returns); nothing is kept between calls.
+static int run_grouped(const BatchPlan &bp, const void *in, void *out, int32_t dtype, int64_t *bsz, unsigned char *ws,
+                       cudaStream_t stream) {
+#define BSPS_CK(call)                                    \
+    do {                                                 \
+        if ((call) != cudaSuccess) return BSPS_ERR_CUDA; \
+    } while (0)
+    DevStatus *bst = (DevStatus *)ws;
+    const size_t at_jobs = (sizeof(DevStatus) + 255) & ~size_t(255);
+    const SmallJob *djobs = (const SmallJob *)(ws + at_jobs);
+    unsigned char *tables_at = ws + at_jobs + bp.jobs_bytes, *wave_ws = tables_at + bp.tables_bytes;
+    const size_t kb = dtype == BSPS_F64 ? 8 : 4;
+    std::vector<unsigned char> tables;
+    std::vector<std::function<cudaError_t()>> later;
+    for (const auto &wave : bp.waves) {
+        std::vector<Ctx> calls(wave.size());
+        std::vector<const DevStatus *> statuses;
+        for (size_t k = 0; k < wave.size(); ++k) {
+            const int32_t i = wave[k];
+            const Instance &I = bp.inst[i];
+            const int rc = prepare_keys_call(calls[k], (const unsigned char *)in + I.off * kb, (unsigned char *)out + I.off * kb,
+                                             I.n, dtype, &I.prm, bsz ? bsz + bp.bbase[i] : nullptr, wave_ws + bp.ws_at[i],
+                                             bp.ws_of[i], stream);
+            if (rc) return rc;
+            statuses.push_back(calls[k].ly.status);
+        }
+        Exec x = {calls.data(), (int)calls.size(), stream, true, &tables, tables_at, &later};
+        const int rc = run_keys_calls(x);
+        if (rc) return rc;
+        const size_t at = x.put(statuses);
+        const int count = (int)statuses.size();
+        later.push_back([=]() -> cudaError_t {
+            merge_statuses_kernel<<<(count + 127) / 128, 128, 0, stream>>>((const DevStatus *const *)(tables_at + at), count, bst);
+            return cudaGetLastError();
+        });
+    }
+    if (tables.size() > bp.tables_bytes) return BSPS_ERR_WORKSPACE_TOO_SMALL;
+    BSPS_CK(cudaMemsetAsync(bst, 0, sizeof(DevStatus), stream));
+    if (!bp.jobs.empty())
+        BSPS_CK(cudaMemcpyAsync(ws + at_jobs, bp.jobs.data(), bp.jobs.size() * sizeof(SmallJob), cudaMemcpyHostToDevice, stream));
+    if (!tables.empty())
+        BSPS_CK(cudaMemcpyAsync(tables_at, tables.data(), tables.size(), cudaMemcpyHostToDevice, stream));
+    for (int size = 2; size >= 0; --size) {  // the largest first
+        const int first = bp.first[size], count = bp.first[size + 1] - first;
+        if (count > 0) BSPS_CK(launch_small_jobs(dtype, size, in, out, djobs + first, count, bsz, stream));
+    }
+    for (const auto &f : later) BSPS_CK(f());
+    for (size_t i = 0; i < bp.inst.size(); ++i)  // empty instances that are not on chip
+        if (bp.inst[i].n == 0 && !bp.inst[i].small && bsz)
+            BSPS_CK(cudaMemsetAsync(bsz + bp.bbase[i], 0, sizeof(int64_t) * bp.inst[i].prm.p, stream));
     return BSPS_OK;
 #undef BSPS_CK
 }
@@ -411,6 +356,7 @@ int bsps_sort_batched(const void *d_keys_in, void *d_keys_out, const int64_t *h_
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return BSPS_ERR_CUDA;
     if (cs != cudaStreamCaptureStatusNone) return BSPS_ERR_CAPTURE;
+    if (prm->sampling == BSPS_RANDOM) return run_grouped(bp, d_keys_in, d_keys_out, dtype, d_bucket_sizes, ws, st);
     std::lock_guard<std::mutex> lock(g_mu);
     LaneSet *L = nullptr;
     if ((rc = lanes_for_device(L))) return rc;

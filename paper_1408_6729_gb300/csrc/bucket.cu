@@ -8,7 +8,7 @@
 //      stable cluster sort of segsort.cuh over a list;
 //   3. sub-buckets larger than a cluster's shared memory: an out-of-core
 //      radix sort in global memory.
-#include "kernels.cuh"
+#include "many.cuh"
 #include "segsort.cuh"
 #include "countsort.cuh"
 
@@ -32,11 +32,23 @@ template <typename K> struct BucketArgs {
     const int32_t *only_count;
     int64_t slow_above;       // keys a cluster of the stable sort holds
     int one_value_done;       // sub-buckets of one key value are already in the output
+    int G;                    // tier 1: CTAs per sub-bucket
+    K *reg_keys_rw;           // tier 3 sorts between the regions and the output
+    uint32_t *reg_vals_rw;
 };
 
-template <int DT, bool PAIRS, int CL, int ITEMS>
+// The listed and the out-of-core tier work through every call of a batch.
+template <bool MANY, typename A, typename F> __device__ __forceinline__ void each_call(const Many<A> &m, F f) {
+    if constexpr (MANY) {
+        for (int i = 0; i < m.count; ++i) f(m.all[i]);
+    } else {
+        f(m.one);
+    }
+}
+
+template <int DT, bool PAIRS, int CL, int ITEMS, bool MANY>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(1024, 1)
-bucket_sort_kernel(const BucketArgs<typename KeyTraits<DT>::T> a) {
+bucket_sort_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
     using K = typename KeyTraits<DT>::T;
     using SS = SegSort<K, PAIRS, CL, ITEMS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -44,11 +56,11 @@ bucket_sort_kernel(const BucketArgs<typename KeyTraits<DT>::T> a) {
     K *buf = reinterpret_cast<K *>(smem_raw + ((sizeof(typename SS::Smem) + 15) & ~size_t(15)));
     uint32_t *slots = reinterpret_cast<uint32_t *>(buf + SS::CAP);
 
-    // every sub-bucket (one per cluster), or the listed ones (clusters loop)
-    const int64_t nitems = a.only ? *a.only_count : a.P;
-    const int64_t clusters = gridDim.x / CL;
-    for (int64_t it = blockIdx.x / CL; it < nitems; it += (a.only ? clusters : nitems)) {
-        const int64_t v = a.only ? a.only[it] : it;
+    // the listed sub-buckets
+    each_call<MANY>(many, [&](const BucketArgs<K> &a) {
+    const int64_t nitems = *a.only_count, clusters = gridDim.x / CL;
+    for (int64_t it = blockIdx.x / CL; it < nitems; it += clusters) {
+        const int64_t v = a.only[it];
         const int64_t cnt = imin64(a.vsize[v], a.cap);
         if (cnt == 0) continue;
         const uint64_t off = a.voff[v];
@@ -66,9 +78,9 @@ bucket_sort_kernel(const BucketArgs<typename KeyTraits<DT>::T> a) {
             a.slow_list[atomicAdd(&a.st->slow_count, 1)] = (uint32_t)v;
         }
         // the next sub-bucket reuses every CTA's shared memory
-        if (a.only) cg::this_cluster().sync();
-        else __syncthreads();
+        cg::this_cluster().sync();
     }
+    });
 }
 
 // With payloads, before the cluster sort: a sub-bucket between two splitters
@@ -102,20 +114,28 @@ __global__ void __launch_bounds__(kCopyThreads) bucket_copy_kernel(const BucketA
 }
 
 // Tier 1 (keys only): G CTAs per sub-bucket, the streamed counting sort of
-// countsort.cuh; its bounds are the two splitters around it (the smallest and
-// largest key for the end buckets).
-template <int DT, int SIZE>
+// countsort.cuh; its bounds are the two splitters around it (for the end
+// buckets its smallest or largest key).
+template <int DT, int SIZE, bool MANY>
 __global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
-bucket_count_kernel(const BucketArgs<typename KeyTraits<DT>::T> a, int G) {
+bucket_count_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
     using K = typename KeyTraits<DT>::T;
     using CS = typename CountShape<SIZE>::template Sort<K>;
+    const Pick<MANY, BucketArgs<K>> pk(many);
+    const BucketArgs<K> &a = pk.a;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int64_t v = blockIdx.x / G;
-    const int g = (int)(blockIdx.x % G);
+    const int G = a.G;
+    const int64_t v = pk.block / G;
+    const int g = (int)(pk.block % G);
     const int64_t cnt = imin64(a.vsize[v], a.cap);
     if (cnt == 0) return;
-    const K lo = v > 0 ? a.vphi[v - 1] : (K)~a.st->ext_min_inv;
-    const K hi = v < a.P - 1 ? a.vphi[v] : (K)a.st->ext_max;
+    auto same = [](K k) { return k; };
+    auto inv = [](K k) { return KeyTraits<DT>::inv(k); };
+    const KeySource<K, CountShape<SIZE>::T, decltype(same)> src{a.reg_keys + v * a.cap, same};
+    K lo, hi;
+    if (v == 0 || v == a.P - 1) CS::bounds(smem_raw, src, (int)cnt, lo, hi);  // no splitter on one side
+    if (v > 0) lo = a.vphi[v - 1];
+    if (v < a.P - 1) hi = a.vphi[v];
     K *out_k = a.out_keys + a.voff[v];
     bool done = true;
     if (lo == hi) {  // one key value: nothing to read
@@ -124,8 +144,7 @@ bucket_count_kernel(const BucketArgs<typename KeyTraits<DT>::T> a, int G) {
 #pragma unroll 4
         for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) out_k[e] = x;
     } else {
-        done = CS::run(smem_raw, a.reg_keys + v * a.cap, (int)cnt, lo, hi, out_k, g, G, [](K k) { return k; },
-                       [](K k) { return KeyTraits<DT>::inv(k); });
+        done = CS::run(smem_raw, src, (int)cnt, lo, hi, KeySink<K, decltype(inv)>{out_k, inv}, g, G);
         // larger than a cluster of the stable sort holds: sorted out of core, part by part
         if (done && cnt > a.slow_above && g == 0 && threadIdx.x == 0) atomicAdd(&a.st->slow_buckets, 1);
     }
@@ -137,23 +156,22 @@ bucket_count_kernel(const BucketArgs<typename KeyTraits<DT>::T> a, int G) {
 // Out-of-core path: one CTA sorts one oversized sub-bucket by LSD passes
 // between its region and its output range, chunk by chunk, stably.
 // ---------------------------------------------------------------------------
-template <int DT, bool PAIRS>
-__global__ void __launch_bounds__(kSlowThreads) bucket_slow_kernel(BucketArgs<typename KeyTraits<DT>::T> a,
-                                                                  typename KeyTraits<DT>::T *reg_keys_rw,
-                                                                  uint32_t *reg_vals_rw) {
+template <int DT, bool PAIRS, bool MANY>
+__global__ void __launch_bounds__(kSlowThreads) bucket_slow_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
     using K = typename KeyTraits<DT>::T;
     using Rank = BlockRank<kSlowThreads, kSlowItems, 8>;
     constexpr int CH = kSlowThreads * kSlowItems;
     __shared__ typename Rank::Smem rsm;
     __shared__ uint32_t hist[256], run[256], tmp[40];
     __shared__ K red[2];
+    each_call<MANY>(many, [&](const BucketArgs<K> &a) {
     const int nslow = a.st->slow_count;
     for (int idx = blockIdx.x; idx < nslow; idx += gridDim.x) {
         const int64_t v = a.slow_list[idx];
         const int64_t cnt = imin64(a.vsize[v], a.cap);
         const uint64_t off = a.voff[v];
-        K *bufk[2] = {reg_keys_rw + v * a.cap, reinterpret_cast<K *>(a.out_keys) + off};
-        uint32_t *bufv[2] = {PAIRS ? reg_vals_rw + v * a.cap : nullptr, PAIRS ? a.out_vals + off : nullptr};
+        K *bufk[2] = {a.reg_keys_rw + v * a.cap, reinterpret_cast<K *>(a.out_keys) + off};
+        uint32_t *bufv[2] = {PAIRS ? a.reg_vals_rw + v * a.cap : nullptr, PAIRS ? a.out_vals + off : nullptr};
         // key range
         K mn = all_ones<K>(), mx = 0;
         for (int64_t e = threadIdx.x; e < cnt; e += kSlowThreads) {
@@ -226,41 +244,19 @@ __global__ void __launch_bounds__(kSlowThreads) bucket_slow_kernel(BucketArgs<ty
         }
         __syncthreads();
     }
+    });
 }
 
-template <int DT, bool PAIRS, int CL, int ITEMS>
-static cudaError_t launch_cluster(const Ctx &c, const BucketArgs<typename KeyTraits<DT>::T> &a, bool listed) {
+static int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
+
+template <int DT> static void bucket_args(const Ctx &c, BucketArgs<typename KeyTraits<DT>::T> &a) {
     using K = typename KeyTraits<DT>::T;
-    using SS = SegSort<K, PAIRS, CL, ITEMS>;
-    const size_t smem = SS::smem_bytes();
-    auto kern = bucket_sort_kernel<DT, PAIRS, CL, ITEMS>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int64_t clusters = c.pl.P;
-    if (listed) {  // as many clusters as run at once (one CTA per SM), at least 16
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        clusters = imin64(c.pl.P, imax64(16, sms / CL));
-    }
-    kern<<<(unsigned)(clusters * CL), 1024, smem, c.stream>>>(a);
-    return cudaGetLastError();
-}
-
-template <int DT, int SIZE>
-static cudaError_t launch_keys(const Ctx &c, const BucketArgs<typename KeyTraits<DT>::T> &a) {
-    using CS = typename CountShape<SIZE>::template Sort<typename KeyTraits<DT>::T>;
-    auto kern = bucket_count_kernel<DT, SIZE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS::smem_bytes());
-    if (e != cudaSuccess) return e;
-    const int G = count_sort_ctas<SIZE>(c.pl.P, c.pl.n / c.pl.P);
-    kern<<<(unsigned)(c.pl.P * G), CountShape<SIZE>::T, CS::smem_bytes(), c.stream>>>(a, G);
-    return cudaGetLastError();
-}
-
-template <int DT, bool PAIRS> static cudaError_t launch_bucket_t(const Ctx &c) {
-    using K = typename KeyTraits<DT>::T;
-    BucketArgs<K> a;
+    a = {};
     a.reg_keys = (const K *)c.ly.reg_keys;
     a.reg_vals = c.ly.reg_vals;
     a.vsize = c.ly.vsize;
@@ -274,55 +270,108 @@ template <int DT, bool PAIRS> static cudaError_t launch_bucket_t(const Ctx &c) {
     a.P = c.pl.P;
     a.retry_flag = c.ly.retry_flag;
     a.retry_list = c.ly.retry_list;
-    a.only = nullptr;
-    a.only_count = nullptr;
+    a.only = c.ly.retry_list;
+    a.only_count = &c.ly.status->retry_count;
     a.slow_above = (int64_t)8 * 1024 * (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32);
     a.one_value_done = c.pl.seg_route;
-    constexpr int IT = PAIRS ? (sizeof(K) == 8 ? kPairItems64 : kPairItems32)
-                             : (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32);
-    cudaError_t e = cudaSuccess;
-    if constexpr (!PAIRS) {
-        switch (count_sort_size(c.pl.n / c.pl.P, sizeof(K))) {
-        case kCountSmall: e = launch_keys<DT, kCountSmall>(c, a); break;
-        case kCountMedium: e = launch_keys<DT, kCountMedium>(c, a); break;
-        default: e = launch_keys<DT, kCountLarge>(c, a); break;
-        }
-        if (e != cudaSuccess) return e;
-        // what tier 1 gave back: the stable cluster sort over the list
-        a.only = c.ly.retry_list;
-        a.only_count = &c.ly.status->retry_count;
-        e = launch_cluster<DT, false, 8, IT>(c, a, true);
-    } else {
-        // one-value sub-buckets are copied; the cluster sort takes the list of the others
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        bucket_copy_kernel<DT, PAIRS><<<(unsigned)imin64(c.pl.P, 4 * (int64_t)sms), kCopyThreads, 0, c.stream>>>(
-            a, c.ly.retry_list, &c.ly.status->retry_count);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        a.only = c.ly.retry_list;
-        a.only_count = &c.ly.status->retry_count;
-        switch (c.pl.bucket_cl) {
-        case 1: e = launch_cluster<DT, PAIRS, 1, IT>(c, a, true); break;
-        case 2: e = launch_cluster<DT, PAIRS, 2, IT>(c, a, true); break;
-        case 4: e = launch_cluster<DT, PAIRS, 4, IT>(c, a, true); break;
-        case 8: e = launch_cluster<DT, PAIRS, 8, IT>(c, a, true); break;
-        default: return cudaErrorInvalidValue;
-        }
-    }
-    if (e != cudaSuccess) return e;
-    bucket_slow_kernel<DT, PAIRS><<<64, kSlowThreads, 0, c.stream>>>(a, (K *)c.ly.reg_keys, c.ly.reg_vals);
-    return cudaGetLastError();
+    a.reg_keys_rw = (K *)c.ly.reg_keys;
+    a.reg_vals_rw = c.ly.reg_vals;
 }
 
-cudaError_t launch_bucket_sort(const Ctx &c) {
-    const bool pr = c.pl.pairs != 0;
-    switch (c.pl.dtype) {
-    case BSPS_U32: return pr ? launch_bucket_t<BSPS_U32, true>(c) : launch_bucket_t<BSPS_U32, false>(c);
-    case BSPS_I32: return pr ? launch_bucket_t<BSPS_I32, true>(c) : launch_bucket_t<BSPS_I32, false>(c);
-    case BSPS_F32: return pr ? launch_bucket_t<BSPS_F32, true>(c) : launch_bucket_t<BSPS_F32, false>(c);
-    default: return pr ? launch_bucket_t<BSPS_F64, true>(c) : launch_bucket_t<BSPS_F64, false>(c);
+// The cluster sort over the listed sub-buckets and the out-of-core sort: as
+// many clusters as run at once (one CTA per SM), at least 16, for all calls.
+// (Their kernels read a batch's arguments from the table, so the grid is given
+// whole, by the first call.)
+template <typename A, typename K1, typename KN>
+static cudaError_t launch_listed(Exec &x, K1 single, KN all, unsigned grid, unsigned threads, size_t smem,
+                                 void (*fill)(const Ctx &, A &)) {
+    bool first = true;
+    return launch_calls<A>(x, single, all, threads, smem, [&](const Ctx &c, A &a) {
+        fill(c, a);
+        const unsigned g = first ? grid : 0u;
+        first = false;
+        return x.many ? (g ? g : kNoBlocks) : g;
+    });
+}
+
+template <int DT, bool PAIRS, int CL, int ITEMS> static cudaError_t launch_cluster(Exec &x) {
+    using K = typename KeyTraits<DT>::T;
+    using SS = SegSort<K, PAIRS, CL, ITEMS>;
+    const int64_t clusters = imax64(16, sm_count() / CL);
+    const int64_t most = x.many ? clusters : imin64(x.calls[0].pl.P, clusters);
+    return launch_listed<BucketArgs<K>>(x, bucket_sort_kernel<DT, PAIRS, CL, ITEMS, false>,
+                                        bucket_sort_kernel<DT, PAIRS, CL, ITEMS, !PAIRS>, (unsigned)(most * CL), 1024,
+                                        SS::smem_bytes(), bucket_args<DT>);
+}
+
+template <int DT, bool PAIRS> static cudaError_t launch_slow(Exec &x) {
+    return launch_listed<BucketArgs<typename KeyTraits<DT>::T>>(x, bucket_slow_kernel<DT, PAIRS, false>,
+                                                                bucket_slow_kernel<DT, PAIRS, !PAIRS>, 64, kSlowThreads, 0,
+                                                                bucket_args<DT>);
+}
+
+template <int DT, int SIZE> static cudaError_t launch_count(Exec &x) {
+    using K = typename KeyTraits<DT>::T;
+    using CS = typename CountShape<SIZE>::template Sort<K>;
+    int64_t all = 0;
+    for (int i = 0; i < x.count; ++i) all += x.calls[i].pl.P;
+    return launch_calls<BucketArgs<K>>(x, bucket_count_kernel<DT, SIZE, false>, bucket_count_kernel<DT, SIZE, true>,
+                                       CountShape<SIZE>::T, CS::smem_bytes(), [=](const Ctx &c, BucketArgs<K> &a) {
+        const int64_t mean = c.pl.n / c.pl.P;
+        if (count_sort_size(mean, sizeof(K)) != SIZE) return 0u;
+        bucket_args<DT>(c, a);
+        a.G = count_sort_ctas<SIZE>(all, mean);
+        return (uint32_t)(c.pl.P * a.G);
+    });
+}
+
+template <int DT> static cudaError_t launch_bucket_keys_t(Exec &x) {
+    using K = typename KeyTraits<DT>::T;
+    cudaError_t e = launch_count<DT, kCountSmall>(x);
+    if (e == cudaSuccess) e = launch_count<DT, kCountMedium>(x);
+    if (e == cudaSuccess) e = launch_count<DT, kCountLarge>(x);
+    // what tier 1 gave back
+    if (e == cudaSuccess) e = launch_cluster<DT, false, 8, (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32)>(x);
+    if (e == cudaSuccess) e = launch_slow<DT, false>(x);
+    return e;
+}
+
+cudaError_t launch_bucket_keys(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_bucket_keys_t<BSPS_U32>(x);
+    case BSPS_I32: return launch_bucket_keys_t<BSPS_I32>(x);
+    case BSPS_F32: return launch_bucket_keys_t<BSPS_F32>(x);
+    default: return launch_bucket_keys_t<BSPS_F64>(x);
+    }
+}
+
+template <int DT> static cudaError_t launch_bucket_pairs_t(Exec &x) {
+    using K = typename KeyTraits<DT>::T;
+    const Ctx &c = x.calls[0];
+    BucketArgs<K> a;
+    bucket_args<DT>(c, a);
+    // one-value sub-buckets are copied; the cluster sort takes the list of the others
+    bucket_copy_kernel<DT, true><<<(unsigned)imin64(c.pl.P, 4 * (int64_t)sm_count()), kCopyThreads, 0, c.stream>>>(
+        a, c.ly.retry_list, &c.ly.status->retry_count);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    constexpr int IT = sizeof(K) == 8 ? kPairItems64 : kPairItems32;
+    switch (c.pl.bucket_cl) {
+    case 1: e = launch_cluster<DT, true, 1, IT>(x); break;
+    case 2: e = launch_cluster<DT, true, 2, IT>(x); break;
+    case 4: e = launch_cluster<DT, true, 4, IT>(x); break;
+    case 8: e = launch_cluster<DT, true, 8, IT>(x); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return e != cudaSuccess ? e : launch_slow<DT, true>(x);
+}
+
+cudaError_t launch_bucket_pairs(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_bucket_pairs_t<BSPS_U32>(x);
+    case BSPS_I32: return launch_bucket_pairs_t<BSPS_I32>(x);
+    case BSPS_F32: return launch_bucket_pairs_t<BSPS_F32>(x);
+    default: return launch_bucket_pairs_t<BSPS_F64>(x);
     }
 }
 

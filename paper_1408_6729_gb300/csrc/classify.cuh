@@ -31,4 +31,19 @@ __device__ __forceinline__ uint32_t classify_key(K phi, uint32_t tag, const LutP
     return lo;
 }
 
+// Entry c of the radix index: the number of splitters whose phi lies below
+// cell c (at(i): phi of splitter i).
+template <typename K, typename At>
+__device__ __forceinline__ uint32_t lut_cell(uint32_t c, const LutParams<K> &lp, At at) {
+    if ((K)c > (lp.span >> lp.shift)) return lp.nsplit;
+    const K thr = lp.base + ((K)c << lp.shift);
+    uint32_t lo = 0, hi = lp.nsplit;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (at(mid) < thr) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
 } // namespace bsps

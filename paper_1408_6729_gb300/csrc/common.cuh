@@ -66,8 +66,6 @@ struct DevStatus {
     int32_t retry_count;        // sub-buckets for the stable cluster sort (keys only: given back)
     int32_t slow_count;         // entries of the out-of-core list
     uint32_t pad_[4];
-    unsigned long long ext_min_inv;  // ~(smallest phi of bucket 0); 0 = none seen
-    unsigned long long ext_max;      // largest phi of the last bucket
 };
 
 __device__ __forceinline__ void set_error(DevStatus *st, int code) {

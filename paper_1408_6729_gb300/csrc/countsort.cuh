@@ -19,7 +19,7 @@
 //      more) and writes the middle 224 with 16-byte stores; every bin touching
 //      those lies inside the 256.  Longer bins (skewed or repeated keys) are
 //      listed by the scan and sorted in the stage first: not at all when all
-//      their keys are equal, else by a bitonic network.
+//      their keys are equal, else by a warp or, above kWarpBin keys, by the CTA.
 // Per key that is two shared-memory atomics and one shared store, and no
 // exchange between CTAs.
 //
@@ -42,36 +42,183 @@
 
 namespace bsps {
 
-template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
-    using S = typename std::conditional<sizeof(K) == 8, uint32_t, uint16_t>::type;  // word of a narrow stage
-    static constexpr int UB = sizeof(K) == 8 ? 31 : 15;  // bits of a unit
-    static constexpr int W = T / 32;
-    static constexpr int V = 16 / (int)sizeof(K);    // keys per 16-byte access
-    static constexpr int kSegBins = 256;             // bins per scan step of a warp
-    static constexpr int kSegs = NBMAX / kSegBins;
-    static constexpr int kWin = 256, kEdge = 16, kStep = kWin - 2 * kEdge;
-    static constexpr int kPer = kWin / 32;           // keys of a window per lane
-    static constexpr int kLongMax = NBMAX / 16;      // listed long bins
-    static constexpr int kWarpBin = 1024;            // long bins up to this size are sorted by one warp
-    static constexpr int kPartsMax = 32;
-    static constexpr int kUnits = 256;               // units of a narrow stage
-    static constexpr uint32_t kUseWide = STAGE / sizeof(K) - 8, kUseNarrow = STAGE / sizeof(S) - 8;
-    static_assert(NBMAX % 512 == 0 && kSegs <= 128 && NBMAX <= 65536, "the segments are scanned by one warp, four to a lane");
-    static_assert(kUseWide < 65528 && STAGE % 16 == 0, "16-bit positions inside a part");
+// A wide record: 64-bit phi and 32-bit tag in one comparable word.
+using u128 = unsigned __int128;
 
-    struct Smem {
-        uint32_t seg[kSegs + 1];              // first position of every segment of 256 bins
-        uint32_t pseg[kPartsMax + 1];         // first segment of every part
-        uint32_t unit[kUnits + 2];            // first position of every unit (narrow stage)
-        uint32_t longs[kLongMax];             // bin | length << 16
-        uint32_t nlong, nparts, bad, half;
+template <typename K> __device__ __forceinline__ K shfl_up_one(K v) {
+    if constexpr (sizeof(K) == 16) {
+        const uint64_t a = __shfl_up_sync(0xffffffffu, (uint64_t)(v >> 64), 1), b = __shfl_up_sync(0xffffffffu, (uint64_t)v, 1);
+        return (u128)a << 64 | b;
+    } else {
+        return __shfl_up_sync(0xffffffffu, v, 1);
+    }
+}
+template <typename K> __device__ __forceinline__ K shfl_down_one(K v) {
+    if constexpr (sizeof(K) == 16) {
+        const uint64_t a = __shfl_down_sync(0xffffffffu, (uint64_t)(v >> 64), 1), b = __shfl_down_sync(0xffffffffu, (uint64_t)v, 1);
+        return (u128)a << 64 | b;
+    } else {
+        return __shfl_down_sync(0xffffffffu, v, 1);
+    }
+}
+template <typename K> __device__ __forceinline__ K shfl_xor_any(K v, int o) {
+    if constexpr (sizeof(K) == 16) {
+        const uint64_t a = __shfl_xor_sync(0xffffffffu, (uint64_t)(v >> 64), o), b = __shfl_xor_sync(0xffffffffu, (uint64_t)v, o);
+        return (u128)a << 64 | b;
+    } else {
+        return __shfl_xor_sync(0xffffffffu, v, o);
+    }
+}
+template <typename K> __device__ __forceinline__ int word_bits(K v) {
+    if constexpr (sizeof(K) == 16) return (v >> 64) ? 64 + bit_length<uint64_t>((uint64_t)(v >> 64)) : bit_length<uint64_t>((uint64_t)v);
+    else return bit_length<K>(v);
+}
+
+// Ascending bitonic network over a[0..len) by `size` threads, this one being
+// `rank`; every comparator puts the larger key higher, so positions past len
+// act as keys above all others and are never touched.
+template <typename E, typename Sync>
+__device__ void bitonic(E *a, int len, int rank, int size, Sync sync) {
+    int n2 = 1;
+    while (n2 < len) n2 <<= 1;
+    auto step = [&](int i, int l) {
+        if (l < len) {
+            const E x = a[i], y = a[l];
+            if (x > y) {
+                a[i] = y;
+                a[l] = x;
+            }
+        }
     };
-    static constexpr size_t kHead = (sizeof(Smem) + 15) & ~size_t(15);
-    static constexpr size_t smem_bytes() { return kHead + (size_t)NBMAX * 2 + STAGE; }
+    for (int h = 1; h < n2; h <<= 1) {  // runs of h sorted: merge pairs of them
+        for (int t = rank; t < (n2 >> 1); t += size) {
+            const int b = (t & ~(h - 1)) * 2, o = t & (h - 1);
+            step(b + o, b + 2 * h - 1 - o);
+        }
+        sync();
+        for (int j = h >> 1; j > 0; j >>= 1) {
+            for (int t = rank; t < (n2 >> 1); t += size) {
+                const int i = 2 * t - (t & (j - 1));
+                step(i, i + j);
+            }
+            sync();
+        }
+    }
+}
 
-    // f(key) for every key of the segment; xf maps a loaded word to the key
-    template <typename Xf, typename F>
-    __device__ static void for_each(const K *__restrict__ src, int n, Xf xf, F f) {
+// One warp's sort of a[0..len): nothing when all keys are equal, in registers
+// up to 32 of them.
+template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t len) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (len <= 32) {
+        E x = lane < len ? a[lane] : all_ones<E>();
+#pragma unroll
+        for (int h = 1; h < 32; h <<= 1) {
+            if ((uint32_t)h >= len) break;
+#pragma unroll
+            for (int j = h; j > 0; j >>= 1) {
+                const E y = shfl_xor_any(x, j == h ? 2 * h - 1 : j);  // a merge's first step pairs mirrored lanes
+                x = (lane & j) == 0 ? (y < x ? y : x) : (y > x ? y : x);
+            }
+        }
+        if (lane < len) a[lane] = x;
+        return;
+    }
+    bool differ = false;
+    const E first = a[0];
+    for (uint32_t e = lane; e < len; e += 32) differ |= a[e] != first;
+    if (__any_sync(0xffffffffu, differ)) bitonic(a, (int)len, (int)lane, 32, [] { __syncwarp(); });
+}
+
+// A whole CTA's sort of a[0..n) in shared memory that no distribution slows
+// down: M keys, one drawn from each of M stretches, are put in order one to a
+// thread (shuffles up to 32 apart), every key finds its bin among them, and a
+// warp finishes each bin.
+template <typename E, int T> struct BlockSort {
+    static constexpr int M = T < 512 ? T : 512, ITEMS = T == 1024 ? 8 : 16, kMost = T * ITEMS;
+    struct Smem {
+        E piv[M];
+        uint32_t cnt[M + 4];
+        uint32_t tmp[40];
+    };
+    // the M keys at sm.piv (threads < M hold one each) in ascending order
+    __device__ static void sort_pivots(E *piv, E x) {
+        const int t = threadIdx.x;
+        for (int h = 1; h < M; h <<= 1) {
+            for (int j = h; j > 0; j >>= 1) {
+                // the first step of a merge pairs mirrored positions
+                const int o = j == h ? 2 * h - 1 : j;
+                E y;
+                if (o < 32) {
+                    y = shfl_xor_any(x, o);
+                } else {
+                    if (t < M) piv[t] = x;
+                    __syncthreads();
+                    y = t < M ? piv[t ^ o] : x;
+                    __syncthreads();
+                }
+                const bool low = (t & (j == h ? h : j)) == 0;
+                x = low ? (y < x ? y : x) : (y > x ? y : x);
+            }
+        }
+        if (t < M) piv[t] = x;
+        __syncthreads();
+    }
+
+    __device__ __noinline__ static void run(Smem &sm, E *a, int n) {
+        const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+        if (n <= M) {
+            sort_pivots(sm.piv, t < n ? a[t] : all_ones<E>());
+            if (t < n) a[t] = sm.piv[t];
+            __syncthreads();
+            return;
+        }
+        if (n > kMost) {
+            bitonic(a, n, t, T, [] { __syncthreads(); });
+            return;
+        }
+        const uint32_t stretch = (uint32_t)n / M;
+        E x = all_ones<E>();
+        if (t < M) x = a[(uint32_t)t * stretch + __umulhi((uint32_t)t * 0x9e3779b1u, stretch)];
+        for (int i = t; i < M + 4; i += T) sm.cnt[i] = 0;
+        sort_pivots(sm.piv, x);
+        E k[ITEMS];
+        uint32_t br[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int e = i * T + t;
+            if (e < n) {
+                k[i] = a[e];
+                uint32_t b = 0;  // pivots 0 .. M - 2 at or below the key
+#pragma unroll
+                for (int w = M / 2; w > 0; w >>= 1)
+                    if (!(k[i] < sm.piv[b + w - 1])) b += w;
+                br[i] = b << 16 | atomicAdd(&sm.cnt[b], 1u);
+            }
+        }
+        __syncthreads();
+        const uint32_t total = block_excl_scan_smem<T>(sm.cnt, M, sm.tmp);
+        if (t == 0) sm.cnt[M] = total;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (i * T + t < n) a[sm.cnt[br[i] >> 16] + (br[i] & 0xffffu)] = k[i];
+        __syncthreads();
+        for (int b = warp; b < M; b += T / 32) {
+            const uint32_t at = sm.cnt[b], len = sm.cnt[b + 1] - at;
+            if (len >= 2) warp_sort(a + at, len);
+        }
+        __syncthreads();
+    }
+};
+
+// Where a segment's keys come from: each(n, f) calls f(key) for all n of them,
+// shared out over the T threads of a CTA.
+template <typename K, int T, typename Xf> struct KeySource {
+    const K *__restrict__ src;
+    Xf xf;  // a loaded word to the key sorted
+    template <typename F> __device__ void each(int n, F f) const {
+        constexpr int V = 16 / (int)sizeof(K);
         const int tid = threadIdx.x;
         if (((uintptr_t)src & 15) == 0) {
             const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
@@ -106,38 +253,113 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             for (; e < n; e += T) f(xf(src[e]));
         }
     }
+};
 
-    // Ascending bitonic network over a[0..len) by `size` threads, this one
-    // being `rank`; every comparator puts the larger key higher, so positions
-    // past len act as keys above all others and are never touched.
-    template <typename E, typename Sync>
-    __device__ static void bitonic(E *a, int len, int rank, int size, Sync sync) {
-        int n2 = 1;
-        while (n2 < len) n2 <<= 1;
-        auto step = [&](int i, int l) {
-            if (l < len) {
-                const E x = a[i], y = a[l];
-                if (x > y) {
-                    a[i] = y;
-                    a[l] = x;
-                }
+// Records (phi, tag) of two arrays as single words, every stride-th of them.
+template <typename P, int T> struct RecordSource {
+    using K = typename std::conditional<sizeof(P) == 8, u128, uint64_t>::type;
+    const P *__restrict__ phi;
+    const uint32_t *__restrict__ tag;
+    int64_t stride;
+    template <typename F> __device__ void each(int n, F f) const {
+        int e = threadIdx.x;
+        for (; e + 3 * T < n; e += 4 * T) {
+            P a[4];
+            uint32_t b[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                a[j] = phi[(e + j * T) * stride];
+                b[j] = tag[(e + j * T) * stride];
             }
-        };
-        for (int h = 1; h < n2; h <<= 1) {  // runs of h sorted: merge pairs of them
-            for (int t = rank; t < (n2 >> 1); t += size) {
-                const int b = (t & ~(h - 1)) * 2, o = t & (h - 1);
-                step(b + o, b + 2 * h - 1 - o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) f((K)a[j] << 32 | b[j]);
+        }
+        for (; e < n; e += T) f((K)phi[e * stride] << 32 | tag[e * stride]);
+    }
+};
+
+// Where the sorted keys go: pad(p) is position p's offset from 16-byte
+// alignment, eight() stores the keys of eight positions from an aligned one.
+template <typename K, typename Inv> struct KeySink {
+    K *out;
+    Inv inv;  // a sorted key to the word stored
+    static constexpr int V = 16 / (int)sizeof(K);
+    __device__ int pad(uint32_t p) const { return (int)(((uintptr_t)(out + p) / sizeof(K)) & (V - 1)); }
+    __device__ void one(int64_t p, K k) const { out[p] = inv(k); }
+    template <typename Key> __device__ void eight(int64_t p, Key key) const {
+#pragma unroll
+        for (int j = 0; j < 8 / V; ++j) {
+            uint4 w;
+            if constexpr (sizeof(K) == 4) {
+                w = make_uint4(inv(key(j * 4)), inv(key(j * 4 + 1)), inv(key(j * 4 + 2)), inv(key(j * 4 + 3)));
+            } else {
+                const uint64_t a = inv(key(j * 2)), b = inv(key(j * 2 + 1));
+                w = make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
             }
-            sync();
-            for (int j = h >> 1; j > 0; j >>= 1) {
-                for (int t = rank; t < (n2 >> 1); t += size) {
-                    const int i = 2 * t - (t & (j - 1));
-                    step(i, i + j);
-                }
-                sync();
-            }
+            *reinterpret_cast<uint4 *>(out + p + j * V) = w;
         }
     }
+};
+
+// Records back into two arrays (16-byte aligned).
+template <typename P> struct RecordSink {
+    using K = typename std::conditional<sizeof(P) == 8, u128, uint64_t>::type;
+    P *phi;
+    uint32_t *tag;
+    int64_t at;  // array index of position 0
+    __device__ int pad(uint32_t p) const { return (int)((at + p) & 3); }
+    __device__ void one(int64_t p, K k) const {
+        phi[at + p] = (P)(k >> 32);
+        tag[at + p] = (uint32_t)k;
+    }
+    template <typename Key> __device__ void eight(int64_t p, Key key) const {
+#pragma unroll
+        for (int j = 0; j < 8; j += 4) {
+            const K a = key(j), b = key(j + 1), c = key(j + 2), d = key(j + 3);
+            if constexpr (sizeof(P) == 4) {
+                *reinterpret_cast<uint4 *>(phi + at + p + j) =
+                    make_uint4((uint32_t)(a >> 32), (uint32_t)(b >> 32), (uint32_t)(c >> 32), (uint32_t)(d >> 32));
+            } else {
+                phi[at + p + j] = (P)(a >> 32);
+                phi[at + p + j + 1] = (P)(b >> 32);
+                phi[at + p + j + 2] = (P)(c >> 32);
+                phi[at + p + j + 3] = (P)(d >> 32);
+            }
+            *reinterpret_cast<uint4 *>(tag + at + p + j) = make_uint4((uint32_t)a, (uint32_t)b, (uint32_t)c, (uint32_t)d);
+        }
+    }
+};
+
+template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
+    using S = typename std::conditional<sizeof(K) >= 8, uint32_t, uint16_t>::type;  // word of a narrow stage
+    static constexpr int UB = sizeof(K) >= 8 ? 31 : 15;  // bits of a unit
+    static constexpr int W = T / 32;
+    static constexpr int V = 16 / (int)sizeof(K);    // keys per 16-byte access
+    static constexpr int kSegBins = 256;             // bins per scan step of a warp
+    static constexpr int kSegs = NBMAX / kSegBins;
+    static constexpr int kWin = 256, kEdge = 16, kStep = kWin - 2 * kEdge;
+    static constexpr int kPer = kWin / 32;           // keys of a window per lane
+    static constexpr int kLongMax = NBMAX / 16;      // listed long bins
+    static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp
+    static constexpr int kPartsMax = 32;
+    static constexpr int kUnits = 256;               // units of a narrow stage
+    static constexpr uint32_t kUseWide = STAGE / sizeof(K) - 8, kUseNarrow = STAGE / sizeof(S) - 8;
+    static_assert(NBMAX % 512 == 0 && kSegs <= 128 && NBMAX <= 65536, "the segments are scanned by one warp, four to a lane");
+    static_assert(kUseWide < 65528 && STAGE % 16 == 0, "16-bit positions inside a part");
+
+    struct Smem {
+        uint32_t seg[kSegs + 1];              // first position of every segment of 256 bins
+        uint32_t pseg[kPartsMax + 1];         // first segment of every part
+        uint32_t unit[kUnits + 2];            // first position of every unit (narrow stage)
+        uint32_t longs[kLongMax];             // bin | length << 16
+        uint32_t nlong, nparts, bad, half;
+        alignas(16) unsigned char sort[sizeof(typename BlockSort<K, T>::Smem)];  // of a long bin by the whole CTA
+    };
+    static constexpr size_t kHead = (sizeof(Smem) + 15) & ~size_t(15);
+    static constexpr size_t smem_bytes() { return kHead + (size_t)NBMAX * 2 + STAGE; }
+    // the bins' words (NBMAX of 16 bits): free for the sink's use while the
+    // only part of a segment is written
+    __device__ static uint32_t *bins(unsigned char *smem) { return reinterpret_cast<uint32_t *>(smem + kHead); }
 
     // The long bins inside bins [b0, b0 + bn), each unsorted in the len slots
     // that end at its cursor.
@@ -149,10 +371,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
             if (b - b0 >= bn || len > (uint32_t)kWarpBin) continue;
             E *a = stage + (end_of(b) - len);
-            bool differ = false;
-            const E first = a[0];
-            for (uint32_t e = lane; e < len; e += 32) differ |= a[e] != first;
-            if (__any_sync(0xffffffffu, differ)) bitonic(a, (int)len, lane, 32, [] { __syncwarp(); });
+            warp_sort(a, len);
         }
         for (uint32_t i = 0; i < nl; ++i) {
             const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
@@ -161,7 +380,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             bool differ = false;
             const E first = a[0];
             for (uint32_t e = tid; e < len; e += T) differ |= a[e] != first;
-            if (__syncthreads_or(differ)) bitonic(a, (int)len, tid, T, [] { __syncthreads(); });
+            if (__syncthreads_or(differ)) BlockSort<E, T>::run(*reinterpret_cast<typename BlockSort<E, T>::Smem *>(sm.sort), a, (int)len);
         }
     }
 
@@ -186,8 +405,8 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         E nx[4], pv[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            nx[j] = __shfl_down_sync(0xffffffffu, x[j], 1);
-            pv[j] = __shfl_up_sync(0xffffffffu, x[4 + j], 1);
+            nx[j] = shfl_down_one(x[j]);
+            pv[j] = shfl_up_one(x[4 + j]);
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -200,12 +419,12 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             bool bad = false;
 #pragma unroll
             for (int j = 0; j + 1 < kPer; ++j) bad |= x[j + 1] < x[j];
-            const E nxt = __shfl_down_sync(0xffffffffu, x[0], 1);
+            const E nxt = shfl_down_one(x[0]);
             bad |= lane < 31 && nxt < x[kPer - 1];
             if (!__any_sync(0xffffffffu, bad)) break;
 #pragma unroll
             for (int j = 0; j + 1 < kPer; j += 2) order(x[j], x[j + 1]);
-            const E up = __shfl_up_sync(0xffffffffu, x[kPer - 1], 1), dn = __shfl_down_sync(0xffffffffu, x[0], 1);
+            const E up = shfl_up_one(x[kPer - 1]), dn = shfl_down_one(x[0]);
 #pragma unroll
             for (int j = 1; j + 1 < kPer; j += 2) order(x[j], x[j + 1]);
             if (lane > 0) x[0] = up > x[0] ? up : x[0];
@@ -213,34 +432,24 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         }
     }
 
-    // Writes a lane's keys key(j) to ob[at + j]; at the ends of a part only
-    // those inside [pad, end).
-    template <typename Key>
-    __device__ static void put(K *ob, int at, bool inner, int pad, int end, Key key) {
+    // Writes a lane's keys key(j) of slots at + j, position p0 being slot pad; at
+    // the ends of a part only those inside [pad, end).
+    template <typename Sink, typename Key>
+    __device__ static void put(const Sink &sink, uint32_t p0, int at, bool inner, int pad, int end, Key key) {
+        const int64_t p = (int64_t)p0 + at - pad;
+        if (inner) {
+            sink.eight(p, key);
+        } else {
 #pragma unroll
-        for (int j = 0; j < kPer / V; ++j) {
-            const int o = at + j * V;
-            if (inner) {
-                uint4 w;
-                if constexpr (sizeof(K) == 4) {
-                    w = make_uint4(key(j * 4), key(j * 4 + 1), key(j * 4 + 2), key(j * 4 + 3));
-                } else {
-                    const uint64_t a = key(j * 2), b = key(j * 2 + 1);
-                    w = make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
-                }
-                *reinterpret_cast<uint4 *>(ob + o) = w;
-            } else {
-#pragma unroll
-                for (int e = 0; e < V; ++e)
-                    if (o + e >= pad && o + e < end) ob[o + e] = key(j * V + e);
-            }
+            for (int j = 0; j < kPer; ++j)
+                if (at + j >= pad && at + j < end) sink.one(p + j, key(j));
         }
     }
 
-    // A part of np keys at stage[pad..): its windows, written to out[0..np)
-    // (out + j and stage[pad + j] have the same 16-byte alignment).
-    template <typename Inv>
-    __device__ static void emit_wide(const K *stage, int pad, int np, K *out, Inv inv) {
+    // A part of np keys at stage[pad..): its windows, written to positions p0 on
+    // (position p0 + j and slot pad + j have the same 16-byte alignment).
+    template <typename Sink>
+    __device__ static void emit_wide(const K *stage, int pad, int np, uint32_t p0, const Sink &sink) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, end = pad + np;
         for (int w0 = warp * kStep; w0 < end; w0 += W * kStep) {
             const int at = w0 - kEdge + lane * kPer;
@@ -252,6 +461,8 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     const uint4 w = *reinterpret_cast<const uint4 *>(stage + at + j * V);
                     if constexpr (sizeof(K) == 4) {
                         x[j * 4] = w.x; x[j * 4 + 1] = w.y; x[j * 4 + 2] = w.z; x[j * 4 + 3] = w.w;
+                    } else if constexpr (sizeof(K) == 16) {
+                        x[j] = (u128)((uint64_t)w.w << 32 | w.z) << 64 | ((uint64_t)w.y << 32 | w.x);
                     } else {
                         x[j * 2] = (uint64_t)w.y << 32 | w.x;
                         x[j * 2 + 1] = (uint64_t)w.w << 32 | w.z;
@@ -264,14 +475,14 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             }
             sort_window(x);
             if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
-                put(out - pad, at, inner, pad, end, [&](int j) { return inv(x[j]); });
+                put(sink, p0, at, inner, pad, end, [&](int j) { return x[j]; });
         }
     }
 
-    // The same from a narrow stage, whose first slot (pad) is position p0.
-    template <typename Inv>
+    // The same from a narrow stage.
+    template <typename Sink>
     __device__ static void emit_narrow(const Smem &sm, const S *stage, int pad, int np, uint32_t p0, uint32_t nunits, K lo,
-                                       K *out, Inv inv) {
+                                       const Sink &sink) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, end = pad + np;
         for (int w0 = warp * kStep; w0 < end; w0 += W * kStep) {
             const int at = w0 - kEdge + lane * kPer;
@@ -310,7 +521,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 sort_window(s);
                 const K base = lo + ((K)u0 << UB);
                 if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
-                    put(out - pad, at, inner, pad, end, [&](int j) { return inv(base + s[j]); });
+                    put(sink, p0, at, inner, pad, end, [&](int j) { return base + s[j]; });
             } else {
                 K x[kPer];
 #pragma unroll
@@ -325,24 +536,24 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 }
                 sort_window(x);
                 if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
-                    put(out - pad, at, inner, pad, end, [&](int j) { return inv(x[j]); });
+                    put(sink, p0, at, inner, pad, end, [&](int j) { return x[j]; });
             }
         }
     }
 
     // Smallest and largest key of the segment (n >= 1), for every thread.
-    template <typename Xf>
-    __device__ static void bounds(unsigned char *smem, const K *__restrict__ src, int n, Xf xf, K &lo, K &hi) {
+    template <typename Source>
+    __device__ static void bounds(unsigned char *smem, const Source &src, int n, K &lo, K &hi) {
         K *red = reinterpret_cast<K *>(smem);
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         K mn = all_ones<K>(), mx = K(0);
-        for_each(src, n, xf, [&](K k) {
+        src.each(n, [&](K k) {
             mn = k < mn ? k : mn;
             mx = k > mx ? k : mx;
         });
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const K a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+            const K a = shfl_xor_any(mn, o), b = shfl_xor_any(mx, o);
             mn = a < mn ? a : mn;
             mx = b > mx ? b : mx;
         }
@@ -360,12 +571,11 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         __syncthreads();
     }
 
-    // Sorts the n keys at src into out[0..n), as CTA g of G.  Returns false
+    // Sorts the n keys of src into positions [0, n) of sink, as CTA g of G.  Returns false
     // (in every CTA of the segment alike, with nothing written) when a run of
     // 256 bins holds more keys than a part or there are too many long bins.
-    template <typename Xf, typename Inv>
-    __device__ static bool run(unsigned char *smem, const K *__restrict__ src, int n, K lo, K hi, K *out, int g, int G,
-                               Xf xf, Inv inv) {
+    template <typename Source, typename Sink>
+    __device__ static bool run(unsigned char *smem, const Source &src, int n, K lo, K hi, const Sink &sink, int g, int G) {
         Smem &sm = *reinterpret_cast<Smem *>(smem);
         uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + kHead);
         unsigned char *stage = smem + kHead + (size_t)NBMAX * 2;
@@ -374,13 +584,13 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         int nbl = 9;
         while ((1 << nbl) < NBMAX && (1 << nbl) < n) ++nbl;
         const K range = hi - lo;
-        const int bits = bit_length<K>(range);
+        const int bits = word_bits<K>(range);
         const int shift = bits > nbl ? bits - nbl : 0;
         const uint32_t nb = 1u << nbl, nseg = nb / kSegBins, hseg = nseg / 2, wmask = nb / 2 - 1;
         // a narrow stage where a wide one would need more parts (or, of 64-bit
         // keys, wherever it can be: its windows sort half words)
         const K nu = (range >> UB) + 1;
-        const bool narrow = (sizeof(K) == 8 || (uint32_t)n > kUseWide) && shift + 3 <= UB && nu <= (K)kUnits &&
+        const bool narrow = sizeof(K) <= 8 && (sizeof(K) == 8 || (uint32_t)n > kUseWide) && shift + 3 <= UB && nu <= (K)kUnits &&
                             (nu <= 2 || (uint64_t)nu * kWin <= (uint64_t)n);
         const uint32_t nunits = (uint32_t)nu;
         for (uint32_t q = tid; q < nb / 8; q += T) reinterpret_cast<uint4 *>(cnt)[q] = make_uint4(0u, 0u, 0u, 0u);
@@ -391,7 +601,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         __syncthreads();
         // keys outside [lo, hi] (a region that overflowed, which is reported) stay in bounds
         auto bin_of = [&](K v) { return min((uint32_t)(v >> shift), nb - 1u); };
-        for_each(src, n, xf, [&](K k) {
+        src.each(n, [&](K k) {
             const uint32_t b = bin_of(k - lo);
             atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u);
         });
@@ -509,7 +719,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     sm.unit[bin0 >> (UB - shift)] = p;
                 // relative to the part's start (or the middle) and the stage's pad
                 const uint32_t pstart = sm.seg[sm.pseg[ps]];
-                p += (uint32_t)(((uintptr_t)(out + pstart) / sizeof(K)) & (V - 1)) - pstart - (hi_half ? half : 0u);
+                p += (uint32_t)sink.pad(pstart) - pstart - (hi_half ? half : 0u);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     out_w[j] |= p << (16 * hi_half);
@@ -546,19 +756,19 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             const uint32_t b0 = s0 * kSegBins, bn = (s1 - s0) * kSegBins;
             if (nparts == 1) {
                 if (narrow) {
-                    for_each(src, n, xf, [&](K k) {
+                    src.each(n, [&](K k) {
                         const K v = k - lo;
                         const uint32_t b = bin_of(v);
                         reinterpret_cast<S *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = (S)v;
                     });
                 } else {
-                    for_each(src, n, xf, [&](K k) {
+                    src.each(n, [&](K k) {
                         const uint32_t b = bin_of(k - lo);
                         reinterpret_cast<K *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = k;
                     });
                 }
             } else {
-                for_each(src, n, xf, [&](K k) {
+                src.each(n, [&](K k) {
                     const K v = k - lo;
                     const uint32_t b = bin_of(v);
                     if (b - b0 < bn) place(b, v, k);
@@ -566,20 +776,20 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             }
             __syncthreads();
             auto end_of = [&](uint32_t b) { return slot_of(b, cnt[b & wmask]); };
-            K *o = out + p0;
-            const int pad = (int)(((uintptr_t)o / sizeof(K)) & (V - 1));
-            if (narrow) {
+            const int pad = sink.pad(p0);
+            if constexpr (sizeof(K) <= 8) if (narrow) {
                 if (sm.nlong) {
                     sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, end_of);
                     __syncthreads();
                 }
-                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, nunits, lo, o, inv);
-            } else {
+                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, nunits, lo, sink);
+            }
+            if (!narrow) {
                 if (sm.nlong) {
                     sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, end_of);
                     __syncthreads();
                 }
-                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, o, inv);
+                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, p0, sink);
             }
             __syncthreads();  // the next part reuses the stage
         }
@@ -588,15 +798,15 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
 };
 
 // The shapes it runs in: one CTA of 1024 threads per SM, two of 512, or five
-// of 256 (228 KB of shared memory per SM, 1 KB of it reserved per CTA).
-enum { kCountSmall = 0, kCountMedium = 1, kCountLarge = 2 };
+// of 256 (228 KB of shared memory per SM, 1 KB of it reserved per CTA); for the
+// 128-bit words of wide records two of 256 with twice the registers.
+enum { kCountSmall = 0, kCountMedium = 1, kCountLarge = 2, kCountRecord = 3 };
 template <int SIZE> struct CountShape {
     static constexpr int T = SIZE == kCountLarge ? 1024 : SIZE == kCountMedium ? 512 : 256;
-    static constexpr int kPerSm = SIZE == kCountLarge ? 1 : SIZE == kCountMedium ? 2 : 5;
-    static constexpr int kBins = SIZE == kCountLarge ? 32768 : SIZE == kCountMedium ? 16384 : 4096;
-    static constexpr int kStageBytes = SIZE == kCountLarge ? 155648 : SIZE == kCountMedium ? 75776 : 32768;
+    static constexpr int kPerSm = SIZE == kCountLarge ? 1 : SIZE == kCountSmall ? 5 : 2;
+    static constexpr int kBins = SIZE == kCountLarge ? 32768 : SIZE == kCountMedium ? 16384 : SIZE == kCountRecord ? 8192 : 4096;
+    static constexpr int kStageBytes = SIZE == kCountLarge ? 149504 : SIZE == kCountMedium ? 69632 : SIZE == kCountRecord ? 81920 : 30720;
     template <typename K> using Sort = CountSort<K, T, kBins, kStageBytes>;
-    static_assert(kPerSm * (Sort<uint32_t>::smem_bytes() + 1024) <= 228 * 1024, "resident CTAs");
     static_assert(kPerSm * (Sort<uint64_t>::smem_bytes() + 1024) <= 228 * 1024, "resident CTAs");
 };
 

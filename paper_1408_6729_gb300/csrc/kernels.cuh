@@ -11,6 +11,7 @@ struct MlpNorm;
 // Number of cells of the radix index placed in front of the splitter tree.
 constexpr int kLutBits = 14;
 constexpr int kLutCells = 1 << kLutBits;
+constexpr int kLutBitsFine = kLutBits + 1;  // keys without payloads, where it fits
 
 // Routing geometry (Fig. 1 steps 9-11).
 constexpr int kRouteThreads = 1024;
@@ -18,11 +19,6 @@ constexpr int kRouteTile = 65536;                           // keys per look-bac
 template <typename K> constexpr int route_items() { return sizeof(K) == 8 ? 4 : 8; }
 template <typename K> constexpr int route_chunk() { return kRouteThreads * route_items<K>(); }
 constexpr size_t kRouteSmemBudget = 220 * 1024;
-
-// Sample-sort geometry (Fig. 1 step 5).
-constexpr int kLsdThreads = 512;
-constexpr int kLsdItems = 16;
-constexpr int kLsdTile = kLsdThreads * kLsdItems;
 
 // Bucket / block sort geometry (Fig. 1 step 3, Fig. 2 step 12): 1024-thread
 // CTAs, keys per thread of the on-chip segment sort.
@@ -46,7 +42,7 @@ template <typename K> struct LutParams {
     uint32_t nsplit; // number of splitters (vbuckets - 1)
 };
 
-template <typename K> struct LsdBuffers {
+template <typename K> struct RecordBuffers {
     K *phi[2];
     uint32_t *tag[2];
 };
@@ -66,8 +62,7 @@ struct Plan {
     int run_cl;        // cluster size of the block sort (regular sampling)
     int bucket_cl;     // cluster size of the sub-bucket sort
     int64_t tiles;     // routing tiles
-    int64_t lsd_tiles; // sample-sort tiles
-    int lsd_npos;      // radix digit positions of a sample record
+    int lut_bits;      // cells of the radix index: 2^lut_bits
     int key_bytes;
     size_t ws_bytes;
 };
@@ -77,12 +72,10 @@ struct Layout {
     DevStatus *status;
     void *sphi[2];          // sample record phi (ping-pong), key width
     uint32_t *stag[2];      // sample record tag (ping-pong)
-    uint32_t *lsd_counts;   // lsd_tiles * 256
-    uint32_t *lsd_hist;     // lsd_npos * 256
-    int32_t *lsd_table;     // pass table of the sample sort
+    void *pivots;           // scratch of the sample sort
     void *vphi;             // P-1 sub-bucket splitters, phi
     uint32_t *vtag;         // P-1 sub-bucket splitters, tag
-    uint16_t *lut;          // kLutCells + 1 (sub-bucket counts fit 16 bits)
+    uint16_t *lut;          // 2^lut_bits + 1 entries (sub-bucket counts fit 16 bits)
     void *lutp;             // LutParams<K>
     uint32_t *state;        // tiles * P lookback words
     uint16_t *ids;          // tiles * kRouteTile sub-bucket ids (routing scratch)
@@ -128,25 +121,21 @@ struct Ctx {
 // pad at local index j of virtual processor k; phi of a pad is all ones.
 // (pad, phi, k*M+j) order == (phi', tag') order with these encodings.
 
-// launchers (each returns cudaSuccess or the launch error)
-cudaError_t launch_sample(const Ctx &c);          // Fig. 1 steps 3-4 / Fig. 3 step 4
-cudaError_t launch_sample_sort(const Ctx &c);     // Fig. 1 step 5
-cudaError_t launch_splitters(const Ctx &c);       // Fig. 1 steps 6-7
-cudaError_t launch_route(const Ctx &c);           // Fig. 1 steps 9-11
-cudaError_t launch_bucket_finish(const Ctx &c);   // sizes in cursor -> offsets, bucket sizes, statistics
-cudaError_t launch_bucket_sort(const Ctx &c);     // Fig. 2 step 12
+// launchers (each returns cudaSuccess or the launch error); those that serve
+// a single call and a batch's calls alike are in many.cuh
+cudaError_t launch_sample(const Ctx &c);          // Fig. 1 steps 3-4
+cudaError_t launch_route(const Ctx &c);           // Fig. 1 steps 9-11, with payloads
 cudaError_t launch_debug(const Ctx &c);           // optional diagnostics
-cudaError_t launch_mlp_train(const Ctx &c);       // learned classifier: training set, spline start, training,
-                                                  // evaluation tables and the index over its output
 int mlp_train_kernels();                          // kernels launch_mlp_train queues
 size_t mlp_opt_bytes();
 
 // Byte counts of dynamic shared memory (host side).
 size_t route_smem_bytes(const Plan &pl);
-bool msd_sample_sort(const Plan &p);                // MSD sample sort is launched (32-bit keys, large samples)
+size_t sample_scratch_bytes(const Plan &p);         // Layout::pivots
+int sample_final(const Plan &p);                    // the buffer the sorted sample ends in
+int sample_sort_kernels(const Plan &p);
 int run_keys_cluster(const Plan &p);               // keys-only block sort for regular sampling (0: not used)
 bool counting_block_sort(const Ctx &c);            // kept blocks sorted by the counting sort (and tags recovered)
-cudaError_t launch_route_keys(const Ctx &c);      // keys without payloads, one pass
 // merge final step (Fig. 1 steps 9-12)
 cudaError_t launch_merge_partition(const Ctx &c); // c[k][v] and the sub-bucket sizes (into cursor)
 cudaError_t launch_segment_copy(const Ctx &c);    // the route as segment copies into the regions
@@ -156,6 +145,7 @@ int64_t merge_capacity(int cl);                   // keys a cluster of cl CTAs m
 int64_t merge_runs_max();                         // largest R
 constexpr int64_t kSegRouteRunsMax = 16384;       // largest R of the segment-copy route (shared memory)
 size_t route_keys_smem_bytes(const Plan &pl);
+bool route_keys_fine_index(const Plan &pl);           // ... and a radix index of 2^kLutBitsFine cells
 bool route_keys_splitters_in_smem(const Plan &pl);  // keys-only routing holds the splitters on chip
 
 } // namespace bsps

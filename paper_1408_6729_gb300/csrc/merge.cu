@@ -43,17 +43,14 @@ __device__ __forceinline__ uint32_t key_of_phi32(int dtype, uint32_t v) {
 // blocks first), and S_i's own block has c = (j+1)*x - 1, the splitter's own
 // sorted position.  A pad splitter follows every key.  Without duplicate
 // handling the comparisons use the key value alone.  Rows 0 and p hold 0 and
-// the block's key count (and the blocks' first and last keys give the
-// smallest and largest key, the outer bounds of the first and last bucket).  The bucket sizes come out as differences of row
-// sums: size_i = sum_k c[k][i+1] - sum_k c[k][i].  The splitters may be the
+// the block's key count.  The bucket sizes come out as differences of row sums: size_i = sum_k c[k][i+1] - sum_k c[k][i].  The splitters may be the
 // sub-bucket splitters (any sample records): p below is their number plus one.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kPartWarps * 32)
 merge_partition_kernel(const uint32_t *__restrict__ runs, const uint32_t *__restrict__ rs_phi,
                        const uint32_t *__restrict__ rs_tag, const uint32_t *__restrict__ vphi,
                        const uint32_t *__restrict__ vtag, int64_t n, int64_t p, int64_t R, int64_t m, int64_t s,
-                       int64_t x, int dup_off, uint32_t *__restrict__ part, uint32_t *__restrict__ cursor,
-                       DevStatus *st) {
+                       int64_t x, int dup_off, uint32_t *__restrict__ part, uint32_t *__restrict__ cursor) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t k = (int64_t)blockIdx.x * 32 + lane;
     const bool live = k < R;
@@ -71,19 +68,6 @@ merge_partition_kernel(const uint32_t *__restrict__ runs, const uint32_t *__rest
         }
         const uint32_t tot = warp_sum((uint32_t)len);
         if (lane == 0) atomicAdd(&cursor[p - 1], tot);
-        // the smallest and the largest key (bounds of the first and last
-        // bucket for the bucket sort): the blocks' first and last keys
-        uint32_t mn = 0xffffffffu, mx = 0u;
-        if (len > 0) {
-            mn = runs[lo];
-            mx = runs[lo + len - 1];
-        }
-        mn = __reduce_min_sync(0xffffffffu, mn);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (lane == 0 && tot) {
-            atomicMax(&st->ext_min_inv, ~(unsigned long long)mn);
-            atomicMax(&st->ext_max, (unsigned long long)mx);
-        }
     }
     const int64_t rows = p - 1;
     const int64_t nw = (int64_t)gridDim.y * kPartWarps;
@@ -507,7 +491,7 @@ cudaError_t launch_merge_partition(const Ctx &c) {
     dim3 grid((unsigned)((p.R + 31) / 32), (unsigned)gy);
     merge_partition_kernel<<<grid, kPartWarps * 32, 0, c.stream>>>(
         (const uint32_t *)c.ly.runs, c.ly.rs_phi, c.ly.rs_tag, (const uint32_t *)c.ly.vphi, c.ly.vtag, p.n,
-        p.P, p.R, p.m, p.s, p.x, p.dup_off, c.ly.part, c.ly.cursor, c.ly.status);
+        p.P, p.R, p.m, p.s, p.x, p.dup_off, c.ly.part, c.ly.cursor);
     return cudaGetLastError();
 }
 

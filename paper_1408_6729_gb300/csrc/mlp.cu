@@ -6,6 +6,7 @@
 // trained network, and the index over the splitters' outputs.
 #include <algorithm>
 
+#include "many.cuh"
 #include "mlp.cuh"
 
 namespace bsps {
@@ -124,16 +125,30 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_grad_kernel(const float *para
 
 // One training step's partial gradients: as mlp_grad_kernel, with the point
 // count read from the device (CTAs past it contribute zeros).
-__global__ void __launch_bounds__(kMlpThreads) mlp_step_grad_kernel(const float *params, const float *x,
-                                                                    const float *y, const int64_t *npts,
-                                                                    float *part) {
+struct MlpOpt;
+struct MlpPieceScratch;
+struct MlpStepArgs {
+    float *params;
+    const float *x, *y;
+    const int64_t *npts;
+    float *part;  // G partial gradients and losses
+    MlpOpt *opt;
+    float *loss_first, *loss_last;
+    int32_t G, step, last, pad_;
+};
+template <bool MANY>
+__global__ void __launch_bounds__(kMlpThreads) mlp_step_grad_kernel(const Many<MlpStepArgs> many) {
+    const Pick<MANY, MlpStepArgs> pk(many);
+    const float *params = pk.a.params, *x = pk.a.x, *y = pk.a.y;
+    const int64_t *npts = pk.a.npts;
+    float *part = pk.a.part;
     __shared__ float w[kParams + 3];
     __shared__ float scratch[kMlpScratchFloats];
     for (int k = threadIdx.x; k < kParams; k += kMlpThreads) w[k] = params[k];
     __syncthreads();
     const int64_t m = *npts;
-    const int64_t p0 = (int64_t)blockIdx.x * kMlpThreads;
-    float *pp = part + (int64_t)blockIdx.x * (kParams + 1);
+    const int64_t p0 = (int64_t)pk.block * kMlpThreads;
+    float *pp = part + (int64_t)pk.block * (kParams + 1);
     if (p0 >= m) {
         for (int k = threadIdx.x; k <= kParams; k += kMlpThreads) pp[k] = 0.0f;
         return;
@@ -156,9 +171,14 @@ static size_t mlp_scratch_offset() { return (sizeof(MlpOpt) + 15) & ~size_t(15);
 // or drops them (it shrinks); then, unless `last`, sets the parameters to the
 // next trial, best - eta * grad(best).  After the last evaluation the best
 // parameters are written back.
-__global__ void __launch_bounds__(1024) mlp_descent_kernel(float *params, const float *part, int G,
-                                                           const int64_t *npts, MlpOpt *opt, int step, int last,
-                                                           float *loss_first, float *loss_last) {
+template <bool MANY> __global__ void __launch_bounds__(1024) mlp_descent_kernel(const Many<MlpStepArgs> many) {
+    const Pick<MANY, MlpStepArgs> pk(many);
+    float *params = pk.a.params;
+    const float *part = pk.a.part;
+    const int64_t *npts = pk.a.npts;
+    MlpOpt *opt = pk.a.opt;
+    const int G = pk.a.G, step = pk.a.step, last = pk.a.last;
+    float *loss_first = pk.a.loss_first, *loss_last = pk.a.loss_last;
     __shared__ float s_loss, s_red[32];
     __shared__ int s_keep;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -228,9 +248,17 @@ struct MlpPieceScratch {
     MlpPieceSet set[2];  // the trained parameters, the fallback
 };
 
-__global__ void __launch_bounds__(32) mlp_pieces_kernel(const float *params_in, const float *fallback,
-                                                        MlpPieceScratch *scr) {
-    const int which = blockIdx.x / (kH + 1), k = blockIdx.x % (kH + 1), lane = threadIdx.x;
+struct MlpTableArgs {
+    const float *params, *fallback;
+    const MlpNorm *norm;
+    MlpTables *tables;
+    MlpPieceScratch *scr;
+};
+template <bool MANY> __global__ void __launch_bounds__(32) mlp_pieces_kernel(const Many<MlpTableArgs> many) {
+    const Pick<MANY, MlpTableArgs> pk(many);
+    const float *params_in = pk.a.params, *fallback = pk.a.fallback;
+    MlpPieceScratch *scr = pk.a.scr;
+    const int which = pk.block / (kH + 1), k = pk.block % (kH + 1), lane = threadIdx.x;
     const float *params = which == 0 ? params_in : fallback;
     if (!params) return;
     MlpPieceSet &S = scr->set[which];
@@ -317,8 +345,12 @@ __global__ void __launch_bounds__(32) mlp_pieces_kernel(const float *params_in, 
 }
 
 constexpr int kTablesThreads = 1024;
-__global__ void __launch_bounds__(kTablesThreads) mlp_tables_kernel(const MlpPieceScratch *scr, int has_fallback,
-                                                                    const MlpNorm *norm, MlpTables *T) {
+template <bool MANY> __global__ void __launch_bounds__(kTablesThreads) mlp_tables_kernel(const Many<MlpTableArgs> many) {
+    const Pick<MANY, MlpTableArgs> pk(many);
+    const MlpPieceScratch *scr = pk.a.scr;
+    const bool has_fallback = pk.a.fallback != nullptr;
+    const MlpNorm *norm = pk.a.norm;
+    MlpTables *T = pk.a.tables;
     __shared__ float s_x[kMlpPiecesAll], s_y[kMlpPiecesAll], s_s[kMlpPiecesAll];
     __shared__ int s_n[kH + 1], s_off[kH + 2];
     __shared__ double knots[kH];
@@ -392,26 +424,42 @@ __global__ void __launch_bounds__(kTablesThreads) mlp_tables_kernel(const MlpPie
     for (int q = np - 1 + t; q < kMlpCutsPad; q += kTablesThreads) T->cut[q] = __int_as_float(0x7f800000);
 }
 
-// both kernels of the evaluation form
-static cudaError_t launch_tables(const float *params, const float *fallback, const MlpNorm *norm, MlpTables *T,
-                                 MlpPieceScratch *scr, cudaStream_t st) {
-    mlp_pieces_kernel<<<2 * (kH + 1), 32, 0, st>>>(params, fallback, scr);
-    mlp_tables_kernel<<<1, kTablesThreads, 0, st>>>(scr, fallback != nullptr, norm, T);
-    return cudaGetLastError();
+// both kernels of the evaluation form; args(ctx, a) returns whether the call takes them
+template <typename Args> static cudaError_t launch_tables(Exec &x, Args args) {
+    cudaError_t e = launch_calls<MlpTableArgs>(x, mlp_pieces_kernel<false>, mlp_pieces_kernel<true>, 32, 0,
+                                               [=](const Ctx &c, MlpTableArgs &a) { return args(c, a) ? 2u * (kH + 1) : 0u; });
+    if (e != cudaSuccess) return e;
+    return launch_calls<MlpTableArgs>(x, mlp_tables_kernel<false>, mlp_tables_kernel<true>, kTablesThreads, 0,
+                                      [=](const Ctx &c, MlpTableArgs &a) { return args(c, a) ? 1u : 0u; });
 }
 
+struct MlpIndexArgs {
+    const MlpTables *tables;
+    const void *vphi;
+    int64_t nsplit;
+    float *ys;
+    uint16_t *ylut;
+};
+
 // The network's output for every splitter (S_{j+1} at index j).
-template <int DT>
-__global__ void mlp_ysplit_kernel(const MlpTables *T, const typename KeyTraits<DT>::T *vphi, int64_t nsplit,
-                                  float *ys) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+template <int DT, bool MANY> __global__ void __launch_bounds__(256) mlp_ysplit_kernel(const Many<MlpIndexArgs> many) {
+    const Pick<MANY, MlpIndexArgs> pk(many);
+    const MlpTables *T = pk.a.tables;
+    const auto *vphi = reinterpret_cast<const typename KeyTraits<DT>::T *>(pk.a.vphi);
+    const int64_t nsplit = pk.a.nsplit;
+    float *ys = pk.a.ys;
+    const int64_t j = (int64_t)pk.block * blockDim.x + threadIdx.x;
     if (j < nsplit) ys[j] = mlp_eval(*T, mlp_input<DT>(KeyTraits<DT>::inv(vphi[j]), T->norm));
 }
 
 // The index over the network's output: ylut[c] = number of splitters whose
 // output cell (after a running maximum over the splitters, so that the
 // counts grow with c) is below c, for c = 0 .. kYCells.
-__global__ void __launch_bounds__(1024) mlp_ylut_kernel(float *ys, int64_t nsplit, uint16_t *ylut) {
+template <bool MANY> __global__ void __launch_bounds__(1024) mlp_ylut_kernel(const Many<MlpIndexArgs> many) {
+    const Pick<MANY, MlpIndexArgs> pk(many);
+    float *ys = pk.a.ys;
+    const int64_t nsplit = pk.a.nsplit;
+    uint16_t *ylut = pk.a.ylut;
     __shared__ float tmp[32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     // running maximum, in place: 1024 threads over consecutive slices
@@ -486,13 +534,23 @@ __global__ void mlp_grad_reduce_kernel(const float *part, int G, int64_t m, floa
 // weights are the slope changes at the knots, each unit rescaled so that its
 // three weights are equal in size.  Training then refines it.
 // ---------------------------------------------------------------------------
-template <int DT>
-__global__ void mlp_prepare_kernel(LsdBuffers<typename KeyTraits<DT>::T> b, const int32_t *table, int npos, int64_t S,
-                                   int64_t n, MlpNorm *norm, float *x, float *y, int64_t *npts_out) {
+struct MlpPrepareArgs {
+    const void *phi;  // the sorted sample
+    const uint32_t *tag;
+    int64_t S, n;
+    MlpNorm *norm;
+    float *x, *y, *params;
+    int64_t *npts;
+};
+template <int DT, bool MANY> __global__ void __launch_bounds__(256) mlp_prepare_kernel(const Many<MlpPrepareArgs> many) {
     using K = typename KeyTraits<DT>::T;
-    const int fin = table[1 + 3 * npos];
-    const K *sphi_sorted = b.phi[fin];
-    const uint32_t *stag_sorted = b.tag[fin];
+    const Pick<MANY, MlpPrepareArgs> pk(many);
+    const K *sphi_sorted = reinterpret_cast<const K *>(pk.a.phi);
+    const uint32_t *stag_sorted = pk.a.tag;
+    const int64_t S = pk.a.S, n = pk.a.n;
+    MlpNorm *norm = pk.a.norm;
+    float *x = pk.a.x, *y = pk.a.y;
+    int64_t *npts_out = pk.a.npts;
     __shared__ int64_t s_real;
     if (threadIdx.x == 0) {
         int64_t lo = 0, hi = S;  // first pad record (tag >= n)
@@ -526,7 +584,11 @@ __global__ void mlp_prepare_kernel(LsdBuffers<typename KeyTraits<DT>::T> b, cons
     }
 }
 
-__global__ void mlp_init_kernel(const float *x, const float *y, const int64_t *npts, float *params) {
+template <bool MANY> __global__ void __launch_bounds__(256) mlp_init_kernel(const Many<MlpPrepareArgs> many) {
+    const Pick<MANY, MlpPrepareArgs> pk(many);
+    const float *x = pk.a.x, *y = pk.a.y;
+    const int64_t *npts = pk.a.npts;
+    float *params = pk.a.params;
     const int t = threadIdx.x;  // blockDim >= kH
     const int64_t M = *npts;
     __shared__ float kx[kH + 1], ky[kH + 1];
@@ -569,59 +631,71 @@ __global__ void mlp_init_kernel(const float *x, const float *y, const int64_t *n
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <int DT> static cudaError_t launch_mlp_train_t(const Ctx &c) {
-    using K = typename KeyTraits<DT>::T;
-    const Plan &p = c.pl;
-    const int npos = 4 + (int)sizeof(K);
-    LsdBuffers<K> b;
-    b.phi[0] = (K *)c.ly.sphi[0];
-    b.phi[1] = (K *)c.ly.sphi[1];
-    b.tag[0] = c.ly.stag[0];
-    b.tag[1] = c.ly.stag[1];
-    mlp_prepare_kernel<DT><<<1, 256, 0, c.stream>>>(b, c.ly.lsd_table, npos, p.sample_size, p.n, c.ly.mlp_norm,
-                                                    c.ly.mlp_x, c.ly.mlp_y, c.ly.mlp_npts);
-    mlp_init_kernel<<<1, 256, 0, c.stream>>>(c.ly.mlp_x, c.ly.mlp_y, c.ly.mlp_npts, c.ly.mlp_params);
+template <int DT> static cudaError_t launch_mlp_train_t(Exec &x) {
+    auto learned = [](const Ctx &c) { return c.pl.classify == BSPS_LEARNED; };
+    auto prepare = [=](const Ctx &c, MlpPrepareArgs &a) {
+        if (!learned(c)) return 0u;
+        const int fin = sample_final(c.pl);
+        a = {c.ly.sphi[fin], c.ly.stag[fin], c.pl.sample_size, c.pl.n, c.ly.mlp_norm, c.ly.mlp_x, c.ly.mlp_y,
+             c.ly.mlp_params, c.ly.mlp_npts};
+        return 1u;
+    };
+    cudaError_t e = launch_calls<MlpPrepareArgs>(x, mlp_prepare_kernel<DT, false>, mlp_prepare_kernel<DT, true>, 256, 0, prepare);
+    if (e == cudaSuccess)
+        e = launch_calls<MlpPrepareArgs>(x, mlp_init_kernel<false>, mlp_init_kernel<true>, 256, 0, prepare);
     // full-batch gradient descent on every parameter: the partial gradients
     // of the current parameters, then the step (kMlpSteps trials after the
     // start's evaluation)
-    const int64_t max_pts = std::min<int64_t>(p.sample_size, kMlpTrainPoints);
-    const int G = (int)std::max<int64_t>(1, (max_pts + kMlpThreads - 1) / kMlpThreads);
-    MlpOpt *opt = reinterpret_cast<MlpOpt *>(c.ly.mlp_opt);
-    for (int step = 0; step <= kMlpSteps; ++step) {
-        mlp_step_grad_kernel<<<G, kMlpThreads, 0, c.stream>>>(c.ly.mlp_params, c.ly.mlp_x, c.ly.mlp_y,
-                                                              c.ly.mlp_npts, c.ly.mlp_part);
-        mlp_descent_kernel<<<1, 1024, 0, c.stream>>>(c.ly.mlp_params, c.ly.mlp_part, G, c.ly.mlp_npts, opt, step,
-                                                  step == kMlpSteps, c.dbg.mlp_loss ? c.dbg.mlp_loss : nullptr,
-                                                  c.dbg.mlp_loss ? c.dbg.mlp_loss + 1 : nullptr);
+    for (int step = 0; step <= kMlpSteps && e == cudaSuccess; ++step) {
+        auto args = [=](const Ctx &c, MlpStepArgs &a) {
+            const int64_t max_pts = std::min<int64_t>(c.pl.sample_size, kMlpTrainPoints);
+            const int G = (int)std::max<int64_t>(1, (max_pts + kMlpThreads - 1) / kMlpThreads);
+            float *loss = c.dbg.mlp_loss;
+            a = {c.ly.mlp_params, c.ly.mlp_x, c.ly.mlp_y, c.ly.mlp_npts, c.ly.mlp_part, reinterpret_cast<MlpOpt *>(c.ly.mlp_opt),
+                 loss, loss ? loss + 1 : nullptr, G, step, step == kMlpSteps, 0};
+            return learned(c);
+        };
+        e = launch_calls<MlpStepArgs>(x, mlp_step_grad_kernel<false>, mlp_step_grad_kernel<true>, kMlpThreads, 0,
+                                      [=](const Ctx &c, MlpStepArgs &a) { return args(c, a) ? (uint32_t)a.G : 0u; });
+        if (e == cudaSuccess)
+            e = launch_calls<MlpStepArgs>(x, mlp_descent_kernel<false>, mlp_descent_kernel<true>, 1024, 0,
+                                          [=](const Ctx &c, MlpStepArgs &a) { return args(c, a) ? 1u : 0u; });
     }
     // the trained network in its evaluation form, and the index over the
     // splitters' outputs
-    cudaError_t e0 = launch_tables(c.ly.mlp_params, opt->start, c.ly.mlp_norm, c.ly.mlp_tables,
-                                   reinterpret_cast<MlpPieceScratch *>(reinterpret_cast<unsigned char *>(c.ly.mlp_opt) +
-                                                                       mlp_scratch_offset()),
-                                   c.stream);
-    if (e0 != cudaSuccess) return e0;
-    const int64_t nsplit = p.P - 1;
-    if (nsplit > 0)
-        mlp_ysplit_kernel<DT><<<(unsigned)((nsplit + 255) / 256), 256, 0, c.stream>>>(
-            c.ly.mlp_tables, (const K *)c.ly.vphi, nsplit, c.ly.mlp_ysplit);
-    mlp_ylut_kernel<<<1, 1024, 0, c.stream>>>(c.ly.mlp_ysplit, nsplit, c.ly.ylut);
-    cudaError_t e = cudaGetLastError();
-    if (c.dbg.mlp_params)
-        e = cudaMemcpyAsync(c.dbg.mlp_params, c.ly.mlp_params, sizeof(float) * kParams, cudaMemcpyDeviceToDevice,
-                            c.stream);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_tables(x, [=](const Ctx &c, MlpTableArgs &a) {
+            a = {c.ly.mlp_params, reinterpret_cast<MlpOpt *>(c.ly.mlp_opt)->start, c.ly.mlp_norm, c.ly.mlp_tables,
+                 reinterpret_cast<MlpPieceScratch *>(reinterpret_cast<unsigned char *>(c.ly.mlp_opt) + mlp_scratch_offset())};
+            return learned(c);
+        });
+    auto index = [=](const Ctx &c, MlpIndexArgs &a) {
+        a = {c.ly.mlp_tables, c.ly.vphi, c.pl.P - 1, c.ly.mlp_ysplit, c.ly.ylut};
+        return learned(c);
+    };
+    if (e == cudaSuccess)
+        e = launch_calls<MlpIndexArgs>(x, mlp_ysplit_kernel<DT, false>, mlp_ysplit_kernel<DT, true>, 256, 0,
+                                       [=](const Ctx &c, MlpIndexArgs &a) {
+            return index(c, a) ? (uint32_t)((a.nsplit + 255) / 256) : 0u;
+        });
+    if (e == cudaSuccess)
+        e = launch_calls<MlpIndexArgs>(x, mlp_ylut_kernel<false>, mlp_ylut_kernel<true>, 1024, 0,
+                                       [=](const Ctx &c, MlpIndexArgs &a) { return index(c, a) ? 1u : 0u; });
+    if (e == cudaSuccess && !x.many && x.calls[0].dbg.mlp_params)
+        e = cudaMemcpyAsync(x.calls[0].dbg.mlp_params, x.calls[0].ly.mlp_params, sizeof(float) * kParams,
+                            cudaMemcpyDeviceToDevice, x.stream);
+    return e;
 }
 
 int mlp_train_kernels() { return 2 + 2 * (kMlpSteps + 1) + 4; }
 size_t mlp_opt_bytes() { return mlp_scratch_offset() + sizeof(MlpPieceScratch); }
 
-cudaError_t launch_mlp_train(const Ctx &c) {
-    switch (c.pl.dtype) {
-    case BSPS_U32: return launch_mlp_train_t<BSPS_U32>(c);
-    case BSPS_I32: return launch_mlp_train_t<BSPS_I32>(c);
-    case BSPS_F32: return launch_mlp_train_t<BSPS_F32>(c);
-    default: return launch_mlp_train_t<BSPS_F64>(c);
+cudaError_t launch_mlp_train(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_mlp_train_t<BSPS_U32>(x);
+    case BSPS_I32: return launch_mlp_train_t<BSPS_I32>(x);
+    case BSPS_F32: return launch_mlp_train_t<BSPS_F32>(x);
+    default: return launch_mlp_train_t<BSPS_F64>(x);
     }
 }
 
@@ -658,9 +732,12 @@ extern "C" int bsps_mlp_predict(const float *d_params, const float *d_x, int64_t
         return BSPS_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t s = (cudaStream_t)stream;
     MlpTables *T = (MlpTables *)d_ws;
-    if (launch_tables(d_params, nullptr, nullptr, T,
-                      reinterpret_cast<MlpPieceScratch *>(reinterpret_cast<unsigned char *>(d_ws) + toff),
-                      s) != cudaSuccess)
+    const Ctx none = {};
+    Exec x = {&none, 1, s};
+    if (launch_tables(x, [=](const Ctx &, MlpTableArgs &a) {
+            a = {d_params, nullptr, nullptr, T, reinterpret_cast<MlpPieceScratch *>(reinterpret_cast<unsigned char *>(d_ws) + toff)};
+            return true;
+        }) != cudaSuccess)
         return BSPS_ERR_CUDA;
     if (m > 0) mlp_predict_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(T, d_x, m, d_y);
     return cudaGetLastError() == cudaSuccess ? BSPS_OK : BSPS_ERR_CUDA;

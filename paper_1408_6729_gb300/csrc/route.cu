@@ -13,6 +13,7 @@
 // Inside every region keys keep their input order (Fig. 1 step 11), which
 // makes the final per-bucket sort stable.
 #include "classify.cuh"
+#include "many.cuh"
 #include "mlp.cuh"
 #include "radix.cuh"
 
@@ -349,9 +350,24 @@ __global__ void __launch_bounds__(kRouteThreads, 1) route_kernel(const RouteArgs
 // Sizes and offsets of the sub-buckets (inclusive prefix of the last tile),
 // bucket sizes for the caller and the balance statistics (Lemma 5.1).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-bucket_finish_kernel(const uint32_t *cursor, uint32_t P, int64_t B, int64_t cap, uint32_t *vsize, uint64_t *voff,
-                     int64_t *bucket_sizes, DevStatus *st) {
+struct FinishArgs {
+    const uint32_t *cursor;
+    uint32_t P, pad_;
+    int64_t B, cap;
+    uint32_t *vsize;
+    uint64_t *voff;
+    int64_t *bucket_sizes;
+    DevStatus *st;
+};
+template <bool MANY> __global__ void __launch_bounds__(1024) bucket_finish_kernel(const Many<FinishArgs> many) {
+    const Pick<MANY, FinishArgs> pk(many);
+    const uint32_t *cursor = pk.a.cursor;
+    const uint32_t P = pk.a.P;
+    const int64_t B = pk.a.B, cap = pk.a.cap;
+    uint32_t *vsize = pk.a.vsize;
+    uint64_t *voff = pk.a.voff;
+    int64_t *bucket_sizes = pk.a.bucket_sizes;
+    DevStatus *st = pk.a.st;
     __shared__ uint32_t tmp[40];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t per = ((int64_t)P + 1023) / 1024;
@@ -446,18 +462,16 @@ static cudaError_t launch_route_pairs(const Ctx &c) {
     }
 }
 
-cudaError_t launch_route(const Ctx &c) {
-    cudaError_t e = c.pl.pairs ? launch_route_pairs(c) : launch_route_keys(c);
-    if (e != cudaSuccess) return e;
-    return launch_bucket_finish(c);
-}
+cudaError_t launch_route(const Ctx &c) { return launch_route_pairs(c); }
 
 // sub-bucket sizes (in cursor) -> sizes, output offsets, bucket sizes, maxima
-cudaError_t launch_bucket_finish(const Ctx &c) {
-    const Plan &p = c.pl;
-    bucket_finish_kernel<<<1, 1024, 0, c.stream>>>(c.ly.cursor, (uint32_t)p.P, p.B, p.cap, c.ly.vsize, c.ly.voff,
-                                                   c.bucket_sizes, c.ly.status);
-    return cudaGetLastError();
+cudaError_t launch_bucket_finish(Exec &x) {
+    return launch_calls<FinishArgs>(x, bucket_finish_kernel<false>, bucket_finish_kernel<true>, 1024, 0,
+                                    [](const Ctx &c, FinishArgs &a) {
+        const Plan &p = c.pl;
+        a = {c.ly.cursor, (uint32_t)p.P, 0u, p.B, p.cap, c.ly.vsize, c.ly.voff, c.bucket_sizes, c.ly.status};
+        return 1u;
+    });
 }
 
 size_t route_smem_bytes(const Plan &pl) {

@@ -3,14 +3,32 @@
 //
 // Without payloads the order of keys inside a bucket is free (equal keys
 // cannot be told apart), so the per-bucket prefix of Fig. 1 step 9 need not
-// follow input order: every chunk of kRkChunk keys reserves its run in each
-// bucket region with one atomic on that bucket's cursor.  A chunk is loaded
-// into registers with 16-byte loads, each key is classified once (Fig. 2
-// step 9) and ranked inside the chunk with a shared-memory atomic, the chunk
-// is grouped by bucket in shared memory, and every bucket's run is written
+// follow input order: every chunk of keys reserves its run in each bucket
+// region with one atomic on that bucket's cursor.  A chunk is loaded into
+// registers with 16-byte loads, each key is classified once (Fig. 2 step 9)
+// and ranked inside the chunk with a shared-memory atomic, the chunk is
+// grouped by bucket in shared memory, and every bucket's run is written
 // contiguously into its region.  One CTA of 1024 threads per SM; chunks of
 // 16K keys keep the reservations to about one per four keys.
+//
+// The kernel is bound by the shared-memory pipe (a random access costs a warp
+// about 3.5 wavefronts) and by latency between barriers:
+//  - Each step runs over all of a thread's keys before the next, so the loads
+//    of one step overlap.
+//  - The radix index says of a key's cell whether splitters share it: none (7
+//    of 8 cells at 2^15 cells and 4096 splitters), and the cell names the
+//    bucket; one or two, and as many comparisons decide; more, or a key equal
+//    to a splitter, and the thread's keys search.
+//  - The grouped chunk keeps no bucket numbers.  A bit marks where each
+//    bucket's run starts, so a slot's run is a bit count away, and the runs are
+//    reserved and written by their ordinal among the chunk's non-empty buckets.
+//  - The counters are double-buffered: one chunk is written while the next is
+//    classified, with no barrier between the two.
+#include <algorithm>
+#include <type_traits>
+
 #include "classify.cuh"
+#include "many.cuh"
 #include "mlp.cuh"
 
 namespace bsps {
@@ -45,81 +63,135 @@ template <typename K> struct RouteKeysArgs {
     DevStatus *st;
     const MlpTables *mlp_tables;  // learned classifier (nullable): the network's evaluation form
     const uint16_t *ylut;         // ... and the index over its output
+    int lut_bits;                 // cells of `lut`
     uint32_t tag_floor;           // a key's tag is max(position, tag_floor): n - 1 drops the tie-break
 };
 
 // Shared memory: the radix index (with the learned classifier: the index over
 // the network's output, in the same slot, and the network's tables), the
-// splitters' phi (global memory, L1-cached, when they do not fit), per-bucket
-// counts and write offsets, and the chunk grouped by bucket.
+// splitters' phi (global memory, L1-cached, when they do not fit), two sets of
+// per-bucket counts, the non-empty buckets of a chunk with their starts and
+// region offsets, the run marks, and the chunk grouped by bucket.
 template <typename K, bool LEARNED> struct RouteKeysLayout {
-    size_t mlp, lut, sphi, cnt, dlt, stage_k, stage_b, total;
-    bool sphi_in_smem;
-    __host__ __device__ RouteKeysLayout(uint32_t P) {
+    // Buckets a call may have: the bound bsps_get_plan documents (counters,
+    // offsets, the index and a chunk with 16-bit bucket numbers in 227 KB; the
+    // layout below needs less).  `fits` says whether the splitters fit, too.
+    static size_t limit_bytes(uint32_t P, bool &fits) {
+        size_t total = 0;
         for (int pass = 0; pass < 2; ++pass) {
-            sphi_in_smem = pass == 0;
-            size_t o = 64;  // LutParams
-            mlp = o;     o += LEARNED ? sizeof(MlpTables) : 0;
-            o = (o + 15) & ~size_t(15);
-            lut = o;     o += sizeof(uint16_t) * (kLutCells + 2);
-            o = (o + 15) & ~size_t(15);
-            sphi = o;    o += sphi_in_smem ? sizeof(K) * (P > 1 ? P - 1 : 1) : 0;
-            o = (o + 15) & ~size_t(15);
-            cnt = o;     o += sizeof(uint32_t) * (P + 4);
-            o = (o + 15) & ~size_t(15);
-            dlt = o;     o += sizeof(uint32_t) * (P + 4);
-            o = (o + 15) & ~size_t(15);
-            stage_k = o; o += sizeof(K) * rk_chunk<K, LEARNED>();
-            stage_b = o; o += sizeof(uint16_t) * rk_chunk<K, LEARNED>();
-            o += 128;    // scan scratch
-            total = o;
+            fits = pass == 0;
+            total = 64;
+            auto take = [&](size_t bytes) { total = (total + bytes + 15) & ~size_t(15); };
+            take(LEARNED ? sizeof(MlpTables) : 0);
+            take(sizeof(uint16_t) * (kLutCells + 2));
+            take(fits ? sizeof(K) * (P > 1 ? P - 1 : 1) : 0);
+            take(sizeof(uint32_t) * (P + 4));
+            take(sizeof(uint32_t) * (P + 4));
+            total += (sizeof(K) + 2) * rk_chunk<K, LEARNED>() + 128;
             if (total <= kRkSmemBudget) break;
+        }
+        return total;
+    }
+    size_t mlp, lut, sphi, cnt, dlt, heads, ord, stage, total;
+    bool sphi_in_smem, two_counts;
+    __host__ __device__ RouteKeysLayout(uint32_t P, int lut_bits) {
+        constexpr int CH = rk_chunk<K, LEARNED>();
+        for (int pass = 0; pass < 4; ++pass) {  // what many buckets leave no room for goes
+            sphi_in_smem = pass < 2;
+            two_counts = pass % 2 == 0;
+            size_t o = 64;  // LutParams
+            auto take = [&](size_t bytes) {
+                const size_t at = o;
+                o = (o + bytes + 15) & ~size_t(15);
+                return at;
+            };
+            mlp = take(LEARNED ? sizeof(MlpTables) : 0);
+            lut = take(sizeof(uint16_t) * ((1 << lut_bits) + 2));
+            sphi = take(sphi_in_smem ? sizeof(K) * P : 0);
+            cnt = take(sizeof(uint32_t) * (two_counts ? 2 : 1) * P);
+            dlt = take(sizeof(uint32_t) * P);
+            heads = take(CH / 8);
+            ord = take(CH / 32 * 2);
+            stage = take(sizeof(K) * CH);
+            total = o + 128;  // scan scratch
+            if (total <= kRkSmemBudget - 512) break;  // (a batch's arguments are kept there, too)
         }
     }
 };
 static_assert(sizeof(LutParams<uint64_t>) <= 64, "radix index parameters fit their slot");
 
-template <int DT, bool LEARNED>
-__global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const RouteKeysArgs<typename KeyTraits<DT>::T> a) {
+// A shared-memory word where `take` holds, else all ones: the lanes that do not
+// take it cost the access no bank.
+__device__ __forceinline__ uint32_t ld_shared_if(const uint32_t *p, bool take) {
+    uint32_t v;
+    asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; mov.u32 %0, 0xffffffff; @q ld.shared.u32 %0, [%1]; }"
+        : "=r"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"((uint32_t)take));
+    return v;
+}
+__device__ __forceinline__ uint64_t ld_shared_if(const uint64_t *p, bool take) {
+    uint64_t v;
+    asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; mov.u64 %0, 0xffffffffffffffff; @q ld.shared.u64 %0, [%1]; }"
+        : "=l"(v) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"((uint32_t)take));
+    return v;
+}
+
+template <int DT, bool LEARNED, bool MANY>
+__global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<RouteKeysArgs<typename KeyTraits<DT>::T>> many) {
     using K = typename KeyTraits<DT>::T;
+    const Pick<MANY, RouteKeysArgs<K>> pk(many);
+    const RouteKeysArgs<K> &a = pk.a;
     constexpr int T = kRkThreads, IT = rk_items<K, LEARNED>(), CH = rk_chunk<K, LEARNED>(), V = 16 / (int)sizeof(K);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const RouteKeysLayout<K, LEARNED> L(a.P);
+    const RouteKeysLayout<K, LEARNED> L(a.P, a.lut_bits);
     LutParams<K> &lps = *reinterpret_cast<LutParams<K> *>(smem_raw);
     MlpTables *mt = reinterpret_cast<MlpTables *>(smem_raw + L.mlp);
     uint16_t *lut = reinterpret_cast<uint16_t *>(smem_raw + L.lut);
     K *sphi_s = reinterpret_cast<K *>(smem_raw + L.sphi);
     const K *sphi = L.sphi_in_smem ? sphi_s : a.vphi;
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(smem_raw + L.cnt);
-    uint32_t *dlt = reinterpret_cast<uint32_t *>(smem_raw + L.dlt);
-    K *stage_k = reinterpret_cast<K *>(smem_raw + L.stage_k);
-    uint16_t *stage_b = reinterpret_cast<uint16_t *>(smem_raw + L.stage_b);
+    uint32_t *cnt_a = reinterpret_cast<uint32_t *>(smem_raw + L.cnt), *cnt = cnt_a;  // this chunk's counts, then starts
+    uint32_t *dlt = reinterpret_cast<uint32_t *>(smem_raw + L.dlt);            // run -> bucket | keys << 16, then region slot - chunk slot
+    uint32_t *heads = reinterpret_cast<uint32_t *>(smem_raw + L.heads);        // bit s: a run starts at slot s
+    uint16_t *ord = reinterpret_cast<uint16_t *>(smem_raw + L.ord);            // run holding slot 32 w
+    K *stage = reinterpret_cast<K *>(smem_raw + L.stage);
     uint32_t *tmp = reinterpret_cast<uint32_t *>(smem_raw + L.total - 128);
+    __shared__ uint32_t overflowed, nruns_s;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t P = a.P;
     static_assert(kYCells == kLutCells, "the learned index takes the radix index's slot");
+    const int cells = 1 << a.lut_bits;
+    // index entry: splitters below the cell, and whether one or more share it
+    constexpr uint32_t kDropped = 0xffffffffu;
+    constexpr uint32_t kOne = 0x4000u, kMore = 0x8000u, kBelow = 0x3fffu;
     const uint16_t *lut_src = LEARNED ? a.ylut : a.lut;
-    for (int i = tid; i <= kLutCells; i += T) lut[i] = lut_src[i];
-    if (L.sphi_in_smem)
-        for (uint32_t i = tid; i + 1 < P; i += T) sphi_s[i] = a.vphi[i];
-    for (uint32_t b = tid; b < P; b += T) cnt[b] = 0;
+    for (int i = tid; i <= cells; i += T) {
+        const uint32_t v = lut_src[i];
+        const uint32_t in = !LEARNED && i < cells ? lut_src[i + 1] - v : 0u;
+        lut[i] = (uint16_t)(v | (in == 0 ? 0u : in == 1 ? kOne : kMore));
+    }
+    if (L.sphi_in_smem)  // (entry P - 1 is all ones)
+        for (uint32_t i = tid; i < P; i += T) sphi_s[i] = a.vphi[i];
+    for (uint32_t b = tid; b < (L.two_counts ? 2 * P : P); b += T) cnt[b] = 0;
     if constexpr (LEARNED) {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(a.mlp_tables);
         uint32_t *dst = reinterpret_cast<uint32_t *>(mt);
         for (int q = tid; q < (int)(sizeof(MlpTables) / 4); q += T) dst[q] = src[q];
     }
-    if (tid == 0) lps = *a.lutp;
+    if (tid == 0) {
+        lps = *a.lutp;
+        overflowed = 0;
+    }
     __syncthreads();
     const LutParams<K> lp = lps;
     const bool vec = ((uintptr_t)a.keys & 15) == 0;
-    // buckets [b_lo, b_hi) are this thread's in the scan and the reservation
+    // buckets [b_lo, b_hi) are this thread's in the scan
     const uint32_t per = (P + T - 1) / T;
     const uint32_t b_lo = min(P, tid * per), b_hi = min(P, b_lo + per);
-    K kmin = all_ones<K>(), kmax = K(0);
+    const uint32_t cap = (uint32_t)a.cap;
     uint32_t n_mis = 0, n_steps = 0;
 
-    // chunk keys into registers (key i of a thread is chunk key lidx(i))
+    // chunk keys into registers (key i of a thread is chunk key at(i))
+    auto at = [&](int i) { return ((i / V) * T + tid) * V + i % V; };
     K kk[IT];
     auto load_chunk = [&](int64_t ch) {
         const int64_t e0 = ch * CH;
@@ -141,44 +213,97 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const RouteKe
             }
         }
     };
-    if ((int64_t)blockIdx.x < a.chunks) load_chunk(blockIdx.x);
+    if ((int64_t)pk.block < a.chunks) load_chunk(pk.block);
 
-    for (int64_t ch = blockIdx.x; ch < a.chunks; ch += gridDim.x) {
+    for (int64_t ch = pk.block; ch < a.chunks; ch += pk.blocks) {
         const int64_t e0 = ch * CH;
         const int nh = (int)imin64(CH, a.n - e0);
-        // ---- classify (Fig. 2 step 9) and rank inside the chunk ----
-        uint32_t br[IT];  // bucket << 16 | rank inside the chunk (bucket P: no key)
-        bool agg = true;  // warp-uniform: merge the atomics of lanes sharing lane 0's bucket
+        // ---- classify (Fig. 2 step 9): bucket of every key, P for none ----
+        uint32_t br[IT];
+        auto classify = [&](auto full) {  // full: a whole chunk
+            auto mine = [&](int i) { return decltype(full)::value || at(i) < nh; };
+            if constexpr (LEARNED) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int q = ((i / V) * T + tid) * V + i % V;
-            const bool ok = q < nh;
-            const K raw = kk[i], ph = KeyTraits<DT>::phi(raw);
-            kk[i] = ph;
-            uint32_t b = P;
-            if (ok) {
-                const uint32_t g = max((uint32_t)(e0 + q), a.tag_floor);  // tag: input position
-                if constexpr (LEARNED) {
-                    uint32_t steps;
-                    bool mis;
-                    b = classify_learned<DT>(raw, g, *mt, lut, P - 1, sphi, a.vtag, steps, mis);
-                    n_mis += mis;
-                    n_steps += steps;
-                } else {
-                    b = classify_key(ph, g, lp, lut, sphi, a.vtag);
+                for (int i = 0; i < IT; ++i) {
+                    const K raw = kk[i];
+                    kk[i] = KeyTraits<DT>::phi(raw);
+                    br[i] = P;
+                    if (mine(i)) {
+                        uint32_t steps;
+                        bool mis;
+                        br[i] = classify_learned<DT>(raw, max((uint32_t)(e0 + at(i)), a.tag_floor), *mt, lut, P - 1, sphi,
+                                                     a.vtag, steps, mis);
+                        n_mis += mis;
+                        n_steps += steps;
+                    }
                 }
-                kmin = ph < kmin ? ph : kmin;
-                kmax = ph > kmax ? ph : kmax;
+            } else {
+                const K base = lp.base, span = lp.span;
+#pragma unroll
+                for (int i = 0; i < IT; ++i) {
+                    kk[i] = KeyTraits<DT>::phi(kk[i]);
+                    const K d = (kk[i] > base ? kk[i] : base) - base;
+                    br[i] = lut[(uint32_t)((d < span ? d : span) >> lp.shift)];
+                }
+                // the cell's first splitter and, where more than one share it, the
+                // second; a third, or a key equal to a splitter: search
+                bool search = false;
+                auto decide = [&](auto splitter) {
+#pragma unroll
+                    for (int i = 0; i < IT; ++i) {
+                        const uint32_t e = br[i], j = e & kBelow;
+                        const K s1 = splitter(j, e >= kOne), s2 = splitter(j + 1, e >= kMore);
+                        search |= s1 == kk[i] | s2 <= kk[i];
+                        br[i] = mine(i) ? j + (s1 < kk[i] ? 1u : 0u) : P;
+                    }
+                };
+                if (L.sphi_in_smem) decide([&](uint32_t j, bool take) { return ld_shared_if(sphi_s + j, take); });
+                else decide([&](uint32_t j, bool take) { return take ? a.vphi[j] : all_ones<K>(); });
+                if (__any_sync(0xffffffffu, search)) {
+                    if (search) {  // this thread's keys again, exactly
+#pragma unroll 1
+                        for (int i = 0; i < IT; ++i) {
+                            K k = kk[0];
+#pragma unroll
+                            for (int q = 1; q < IT; ++q) k = q == i ? kk[q] : k;
+                            const uint32_t g = (uint32_t)e0 + ((i / V) * T + tid) * V + i % V;
+                            uint32_t lo = 0, hi = P - 1;
+                            if (k < base) hi = 0;
+                            else if (k - base > span) lo = P - 1;
+                            else {
+                                const uint32_t c = (uint32_t)((k - base) >> lp.shift);
+                                lo = lut[c] & kBelow;
+                                hi = lut[c + 1] & kBelow;
+                            }
+                            while (lo < hi) {
+                                const uint32_t mid = (lo + hi) >> 1;
+                                const K s = sphi[mid];
+                                bool le = s < k;
+                                if (s == k) le = a.vtag[mid] <= max(g, a.tag_floor);  // tags are read on ties only
+                                lo = le ? mid + 1 : lo;
+                                hi = le ? hi : mid;
+                            }
+#pragma unroll
+                            for (int q = 0; q < IT; ++q)
+                                if (q == i && mine(q)) br[q] = lo;
+                        }
+                    }
+                }
             }
-            // keys of lane 0's bucket are ranked with one atomic (runs of equal
-            // buckets are common in skewed inputs); the warp keeps doing so in
-            // this chunk only if its first two items had such runs
-            uint32_t r = 0;
-            if (i < 2 || agg) {
-                const uint32_t b0 = __shfl_sync(0xffffffffu, b, 0);
+        };
+        if (nh == CH) classify(std::true_type());
+        else classify(std::false_type());
+        // ---- rank inside the chunk: bucket << 16 | rank ----
+        // where a warp's first keys share lane 0's bucket (runs of one bucket
+        // are common in skewed inputs) its lanes' atomics are merged
+        const uint32_t first = __shfl_sync(0xffffffffu, br[0], 0);
+        if (__popc(__ballot_sync(0xffffffffu, br[0] == first)) > 4) {
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                const uint32_t b = br[i], b0 = __shfl_sync(0xffffffffu, b, 0);
+                const bool ok = b < P;
                 const uint32_t same = __ballot_sync(0xffffffffu, ok && b == b0);
-                if (i == 0) agg = __popc(same) > 1;
-                if (i == 1) agg |= __popc(same) > 1;
+                uint32_t r = 0;
                 if (ok) {
                     if (b != b0) {
                         r = atomicAdd(&cnt[b], 1u);
@@ -189,102 +314,115 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const RouteKe
                         r = __shfl_sync(same, r0, leader) + __popc(same & lanemask_lt());
                     }
                 }
-            } else if (ok) {
-                r = atomicAdd(&cnt[b], 1u);
+                br[i] = b << 16 | r;
             }
-            br[i] = b << 16 | r;
+        } else if (nh == CH) {
+#pragma unroll
+            for (int i = 0; i < IT; ++i) br[i] = br[i] << 16 | atomicAdd(&cnt[br[i]], 1u);
+        } else {
+#pragma unroll
+            for (int i = 0; i < IT; ++i) br[i] = br[i] << 16 | (br[i] < P ? atomicAdd(&cnt[br[i]], 1u) : 0u);
         }
         __syncthreads();
-        // ---- where each bucket starts inside the chunk ----
-        uint32_t local = 0;
-        for (uint32_t b = b_lo; b < b_hi; ++b) local += cnt[b];
+        // ---- where each bucket starts inside the chunk, and its run's ordinal ----
+        for (int w = tid; w < CH / 32; w += T) heads[w] = 0;
+        uint32_t local = 0;  // keys | non-empty buckets << 16
+        for (uint32_t b = b_lo; b < b_hi; ++b) {
+            const uint32_t c = cnt[b];
+            local += c + (c ? 0x10000u : 0u);
+        }
         uint32_t wtot;
         const uint32_t wex = warp_excl_scan(local, &wtot);
         if (lane == 31) tmp[warp] = wtot;
         __syncthreads();
-        if (warp == 0) {
-            const uint32_t y = lane < T / 32 ? tmp[lane] : 0u;
-            uint32_t t;
-            const uint32_t ye = warp_excl_scan(y, &t);
-            if (lane < T / 32) tmp[lane] = ye;
+        uint32_t run = wex;
+        {
+            uint32_t all;
+            const uint32_t ye = warp_excl_scan(tmp[lane], &all);  // T / 32 = 32 warps
+            run += __shfl_sync(0xffffffffu, ye, warp);
+            if (tid == 0) nruns_s = all >> 16;
+        }
+        for (uint32_t b = b_lo; b < b_hi; ++b) {
+            const uint32_t c = cnt[b];
+            if (c) {
+                const uint32_t s0 = run & 0xffffu, o = run >> 16, w0 = (s0 + 31) >> 5, w1 = (s0 + c + 31) >> 5;
+                cnt[b] = s0;
+                dlt[o] = b | c << 16;
+                atomicOr(&heads[s0 >> 5], 1u << (s0 & 31u));
+                for (uint32_t w = w0; w < w1; ++w) ord[w] = (uint16_t)o;
+                run += c + 0x10000u;
+            }
         }
         __syncthreads();
-        uint32_t run = tmp[warp] + wex;
-        // the first kEarly of my buckets reserve their runs now, so that the
-        // atomics' round trip overlaps the grouping below
+        const uint32_t nruns = nruns_s;
+        // the first kEarly of my runs are reserved now, so that the atomics'
+        // round trip overlaps the grouping below
         uint32_t at_e[kEarly];
 #pragma unroll
         for (int j = 0; j < kEarly; ++j) {
-            const uint32_t b = b_lo + j;
+            const uint32_t o = j * T + tid;
             at_e[j] = 0;
-            if (b < b_hi) {
-                const uint32_t c = cnt[b];
-                cnt[b] = run;  // start of the bucket inside the chunk
-                dlt[b] = c;
-                run += c;
-                if (c) at_e[j] = atomicAdd(&a.cursor[b], c);
-            }
+            if (o < nruns) at_e[j] = atomicAdd(&a.cursor[dlt[o] & 0xffffu], dlt[o] >> 16);
         }
-        for (uint32_t b = b_lo + kEarly; b < b_hi; ++b) {
-            const uint32_t c = cnt[b];
-            cnt[b] = run;
-            dlt[b] = c;
-            run += c;
-        }
-        __syncthreads();
         // ---- group the chunk by bucket ----
+        if (nh == CH) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const uint32_t b = br[i] >> 16;
-            if (b < P) {
-                const uint32_t pos = cnt[b] + (br[i] & 0xffffu);
-                stage_k[pos] = kk[i];
-                stage_b[pos] = (uint16_t)b;
-            }
+            for (int i = 0; i < IT; ++i) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = kk[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < IT; ++i)
+                if (br[i] >> 16 < P) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = kk[i];
         }
         // the next chunk's keys load while this one is reserved and written
-        if (ch + gridDim.x < a.chunks) load_chunk(ch + gridDim.x);
+        if (ch + pk.blocks < a.chunks) load_chunk(ch + pk.blocks);
         // ---- reserve each bucket's run: one atomic per bucket and chunk ----
-        auto reserved = [&](uint32_t b, uint32_t c, uint32_t at) {
-            if ((uint64_t)at + c > (uint64_t)a.cap) {
+        auto reserved = [&](uint32_t o, uint32_t got) {
+            const uint32_t b = dlt[o] & 0xffffu, c = dlt[o] >> 16;
+            const bool fits = got + c <= cap;  // (fewer than 2^31 keys)
+            if (!fits) {
+                overflowed = 1;
                 atomicExch(&a.st->overflow, 1);
                 set_error(a.st, BSPS_ERR_BUCKET_OVERFLOW);
             }
-            dlt[b] = at - cnt[b];  // region slot of chunk position s: dlt[b] + s
+            dlt[o] = fits ? b * cap + got - cnt[b] : kDropped;  // region slot of chunk slot s: dlt[o] + s
         };
 #pragma unroll
         for (int j = 0; j < kEarly; ++j)
-            if (b_lo + j < b_hi) reserved(b_lo + j, dlt[b_lo + j], at_e[j]);
-        for (uint32_t g0 = b_lo + kEarly; g0 < b_hi; g0 += 8) {
-            uint32_t c8[8], at[8];  // eight reservations in flight at a time
+            if (j * T + tid < nruns) reserved(j * T + tid, at_e[j]);
+        for (uint32_t g0 = kEarly * T + tid; g0 < nruns; g0 += 8 * T) {
+            uint32_t got[8];  // eight reservations in flight at a time
 #pragma unroll
-            for (int j = 0; j < 8; ++j) c8[j] = g0 + j < b_hi ? dlt[g0 + j] : 0u;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) at[j] = c8[j] ? atomicAdd(&a.cursor[g0 + j], c8[j]) : 0u;
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t o = g0 + j * T;
+                got[j] = o < nruns ? atomicAdd(&a.cursor[dlt[o] & 0xffffu], dlt[o] >> 16) : 0u;
+            }
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (g0 + j < b_hi) reserved(g0 + j, c8[j], at[j]);
+                if (g0 + j * T < nruns) reserved(g0 + j * T, got[j]);
         }
         __syncthreads();
         // ---- every bucket's run, contiguously into its region ----
-        for (int s = tid; s < nh; s += T) {
-            const uint32_t b = stage_b[s];
-            const uint32_t idx = dlt[b] + (uint32_t)s;
-            if (idx < a.cap) a.reg_keys[(int64_t)b * a.cap + idx] = stage_k[s];
+        auto run_of = [&](uint32_t s) {  // (a warp's slots are one word of the marks)
+            return ord[s >> 5] + (uint32_t)__popc(heads[s >> 5] & (0xfffffffeu & (0xffffffffu >> (31 - (s & 31u)))));
+        };
+        if (overflowed) {  // a run that passes its region's end is not written (the overflow is reported)
+            for (int s = tid; s < nh; s += T) {
+                const uint32_t d = dlt[run_of(s)];
+                if (d != kDropped) a.reg_keys[d + (uint32_t)s] = stage[s];
+            }
+        } else if (nh == CH) {
+#pragma unroll 8
+            for (int i = 0; i < IT; ++i) {
+                const uint32_t s = i * T + tid;
+                a.reg_keys[dlt[run_of(s)] + s] = stage[s];
+            }
+        } else {
+            for (int s = tid; s < nh; s += T) a.reg_keys[dlt[run_of(s)] + (uint32_t)s] = stage[s];
         }
-        for (uint32_t b = b_lo; b < b_hi; ++b) cnt[b] = 0;
-        __syncthreads();
-    }
-    // smallest and largest key: outer bounds of the first and last sub-bucket
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const K x = __shfl_xor_sync(0xffffffffu, kmin, o), y = __shfl_xor_sync(0xffffffffu, kmax, o);
-        kmin = x < kmin ? x : kmin;
-        kmax = y > kmax ? y : kmax;
-    }
-    if (lane == 0 && kmin <= kmax) {
-        atomicMax(&a.st->ext_min_inv, ~(unsigned long long)kmin);
-        atomicMax(&a.st->ext_max, (unsigned long long)kmax);
+        // this chunk's counts are free again; the next chunk counts in the others
+        for (uint32_t b = tid; b < P; b += T) cnt[b] = 0;
+        if (L.two_counts) cnt = cnt == cnt_a ? cnt_a + P : cnt_a;
+        else __syncthreads();
     }
     if constexpr (LEARNED) {
         const uint32_t m = __reduce_add_sync(0xffffffffu, n_mis), stp = __reduce_add_sync(0xffffffffu, n_steps);
@@ -295,64 +433,91 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const RouteKe
     }
 }
 
-template <int DT, bool LEARNED> static cudaError_t launch_t(const Ctx &c) {
+template <int DT, bool LEARNED> static cudaError_t launch_t(Exec &x) {
     using K = typename KeyTraits<DT>::T;
-    const Plan &p = c.pl;
-    RouteKeysArgs<K> a;
-    a.keys = (const K *)c.keys_in;
-    a.n = p.n;
-    a.lutp = (const LutParams<K> *)c.ly.lutp;
-    a.lut = c.ly.lut;
-    a.vphi = (const K *)c.ly.vphi;
-    a.vtag = c.ly.vtag;
-    a.P = (uint32_t)p.P;
-    a.chunks = (p.n + rk_chunk<K, LEARNED>() - 1) / rk_chunk<K, LEARNED>();
-    a.cursor = c.ly.cursor;
-    a.reg_keys = (K *)c.ly.reg_keys;
-    a.cap = p.cap;
-    a.st = c.ly.status;
-    a.mlp_tables = c.ly.mlp_tables;
-    a.ylut = c.ly.ylut;
-    a.tag_floor = c.pl.dup_off ? (uint32_t)(c.pl.n - 1) : 0u;
-    if (a.chunks == 0) return cudaSuccess;
-    const size_t smem = RouteKeysLayout<K, LEARNED>((uint32_t)p.P).total;
-    auto kern = route_keys_kernel<DT, LEARNED>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, occ = 0;
+    auto takes = [](const Ctx &c) { return (c.pl.classify == BSPS_LEARNED) == LEARNED; };
+    size_t smem = 0;
+    int64_t all = 0;  // chunks of every call
+    for (int i = 0; i < x.count; ++i)
+        if (takes(x.calls[i])) {
+            const Plan &p = x.calls[i].pl;
+            smem = std::max(smem, RouteKeysLayout<K, LEARNED>((uint32_t)p.P, LEARNED ? kLutBits : p.lut_bits).total);
+            all += (p.n + rk_chunk<K, LEARNED>() - 1) / rk_chunk<K, LEARNED>();
+        }
+    if (smem == 0) return cudaSuccess;
+    if (smem > kRkSmemBudget - 512) return cudaErrorInvalidValue;
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kRkThreads, smem);
-    const int64_t grid = imin64(a.chunks, (int64_t)max(occ, 1) * sms);
-    kern<<<(unsigned)grid, kRkThreads, smem, c.stream>>>(a);
-    return cudaGetLastError();
+    sms = std::max(sms, 1);
+    return launch_calls<RouteKeysArgs<K>>(x, route_keys_kernel<DT, LEARNED, false>, route_keys_kernel<DT, LEARNED, true>,
+                                          kRkThreads, smem, [=](const Ctx &c, RouteKeysArgs<K> &a) {
+        if (!takes(c)) return 0u;
+        const Plan &p = c.pl;
+        a.keys = (const K *)c.keys_in;
+        a.n = p.n;
+        a.lutp = (const LutParams<K> *)c.ly.lutp;
+        a.lut = c.ly.lut;
+        a.vphi = (const K *)c.ly.vphi;
+        a.vtag = c.ly.vtag;
+        a.P = (uint32_t)p.P;
+        a.chunks = (p.n + rk_chunk<K, LEARNED>() - 1) / rk_chunk<K, LEARNED>();
+        a.cursor = c.ly.cursor;
+        a.reg_keys = (K *)c.ly.reg_keys;
+        a.cap = p.cap;
+        a.st = c.ly.status;
+        a.mlp_tables = c.ly.mlp_tables;
+        a.ylut = c.ly.ylut;
+        a.lut_bits = LEARNED ? kLutBits : p.lut_bits;
+        a.tag_floor = p.dup_off ? (uint32_t)(p.n - 1) : 0u;
+        // one CTA per SM; of a batch's CTAs (each loads the index first) every
+        // call gets its share of two waves
+        const int64_t share = all <= 2 * sms ? a.chunks : imax64(1, 2 * sms * a.chunks / all);
+        return (uint32_t)imin64(a.chunks, c.pl.n == 0 ? 0 : imin64(sms, share));
+    });
 }
 
-template <int DT> static cudaError_t launch_d(const Ctx &c) {
-    return c.pl.classify == BSPS_LEARNED ? launch_t<DT, true>(c) : launch_t<DT, false>(c);
+template <int DT> static cudaError_t launch_d(Exec &x) {
+    const cudaError_t e = launch_t<DT, false>(x);
+    return e != cudaSuccess ? e : launch_t<DT, true>(x);
 }
 
-cudaError_t launch_route_keys(const Ctx &c) {
-    switch (c.pl.dtype) {
-    case BSPS_U32: return launch_d<BSPS_U32>(c);
-    case BSPS_I32: return launch_d<BSPS_I32>(c);
-    case BSPS_F32: return launch_d<BSPS_F32>(c);
-    default: return launch_d<BSPS_F64>(c);
+cudaError_t launch_route_keys(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_d<BSPS_U32>(x);
+    case BSPS_I32: return launch_d<BSPS_I32>(x);
+    case BSPS_F32: return launch_d<BSPS_F32>(x);
+    default: return launch_d<BSPS_F64>(x);
     }
 }
 
-size_t route_keys_smem_bytes(const Plan &pl) {
+static size_t limit_bytes(const Plan &pl, bool &fits) {
     const uint32_t P = (uint32_t)pl.P;
     const bool l = pl.classify == BSPS_LEARNED;
-    if (pl.key_bytes == 8) return l ? RouteKeysLayout<uint64_t, true>(P).total : RouteKeysLayout<uint64_t, false>(P).total;
-    return l ? RouteKeysLayout<uint32_t, true>(P).total : RouteKeysLayout<uint32_t, false>(P).total;
+    if (pl.key_bytes == 8) return l ? RouteKeysLayout<uint64_t, true>::limit_bytes(P, fits) : RouteKeysLayout<uint64_t, false>::limit_bytes(P, fits);
+    return l ? RouteKeysLayout<uint32_t, true>::limit_bytes(P, fits) : RouteKeysLayout<uint32_t, false>::limit_bytes(P, fits);
+}
+
+size_t route_keys_smem_bytes(const Plan &pl) {
+    bool fits;
+    return limit_bytes(pl, fits);
 }
 
 bool route_keys_splitters_in_smem(const Plan &pl) {
+    bool fits;
+    limit_bytes(pl, fits);
+    return fits;
+}
+
+bool route_keys_fine_index(const Plan &pl) {
+    if (pl.classify == BSPS_LEARNED) return false;
     const uint32_t P = (uint32_t)pl.P;
-    const bool l = pl.classify == BSPS_LEARNED;
-    if (pl.key_bytes == 8) return l ? RouteKeysLayout<uint64_t, true>(P).sphi_in_smem : RouteKeysLayout<uint64_t, false>(P).sphi_in_smem;
-    return l ? RouteKeysLayout<uint32_t, true>(P).sphi_in_smem : RouteKeysLayout<uint32_t, false>(P).sphi_in_smem;
+    if (pl.key_bytes == 8) {
+        const RouteKeysLayout<uint64_t, false> l(P, kLutBitsFine);
+        return l.sphi_in_smem && l.two_counts;
+    }
+    const RouteKeysLayout<uint32_t, false> l(P, kLutBitsFine);
+    return l.sphi_in_smem && l.two_counts;
 }
 
 } // namespace bsps

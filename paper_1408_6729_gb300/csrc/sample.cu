@@ -1,6 +1,9 @@
 // sample.cu -- oversampling, sample sort, splitter selection (Fig. 1 steps
 // 3-7, Fig. 3 steps 3-9) and the optional diagnostics.
+#include <algorithm>
+
 #include "classify.cuh"
+#include "many.cuh"
 #include "mlp.cuh"
 #include "segsort.cuh"
 #include "segsort_keys.cuh"
@@ -12,22 +15,37 @@ namespace bsps {
 // Random oversampling (Fig. 3 step 4): s*p-1 positions drawn i.i.d. from the
 // Philox4x64-10 stream; the record of draw j is (phi(key[g_j]), g_j).
 // ---------------------------------------------------------------------------
-template <int DT>
-__global__ void sample_random_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, int64_t n,
-                                     int64_t S, uint64_t seed, typename KeyTraits<DT>::T *sphi,
-                                     uint32_t *stag) {
-    const int64_t blk = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+template <typename K> struct SampleArgs {
+    const K *keys;
+    int64_t n, S;
+    uint64_t seed;
+    K *sphi;
+    uint32_t *stag;
+    DevStatus *st;          // cleared here, before anything of the call uses them
+    uint32_t *cursor, *retry_flag;
+    int64_t P;
+};
+template <int DT, bool MANY>
+__global__ void __launch_bounds__(256) sample_random_kernel(const Many<SampleArgs<typename KeyTraits<DT>::T>> many) {
+    const Pick<MANY, SampleArgs<typename KeyTraits<DT>::T>> pk(many);
+    const auto &a = pk.a;
+    const int64_t blk = (int64_t)pk.block * blockDim.x + threadIdx.x;
+    if (blk == 0) *a.st = DevStatus{};
+    for (int64_t v = blk; v < a.P; v += (int64_t)pk.blocks * blockDim.x) {
+        a.cursor[v] = 0;
+        a.retry_flag[v] = 0;
+    }
     const int64_t j0 = blk * 4;
-    if (j0 >= S) return;
+    if (j0 >= a.S) return;
     uint64_t c[4] = {(uint64_t)blk, 0, 0, 0};
-    philox4x64_10(c, seed, 0);
+    philox4x64_10(c, a.seed, 0);
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
         const int64_t j = j0 + w;
-        if (j < S) {
-            const uint64_t g = __umul64hi(c[w], (uint64_t)n);
-            sphi[j] = KeyTraits<DT>::phi(keys[g]);
-            stag[j] = (uint32_t)g;
+        if (j < a.S) {
+            const uint64_t g = __umul64hi(c[w], (uint64_t)a.n);
+            a.sphi[j] = KeyTraits<DT>::phi(a.keys[g]);
+            a.stag[j] = (uint32_t)g;
         }
     }
 }
@@ -215,8 +233,10 @@ run_sample_count_kernel(const uint32_t *__restrict__ keys, int64_t n, int64_t m,
         }
     }
     uint32_t kmin, kmax;
-    CS::bounds(smem_raw, keys + lo, (int)len, PhiOf<DT>(), kmin, kmax);
-    if (!CS::run(smem_raw, keys + lo, (int)len, kmin, kmax, runs + lo, g, G, PhiOf<DT>(), [](uint32_t v) { return v; }) &&
+    const KeySource<uint32_t, CountShape<SIZE>::T, PhiOf<DT>> src{keys + lo, PhiOf<DT>()};
+    CS::bounds(smem_raw, src, (int)len, kmin, kmax);
+    auto same = [](uint32_t v) { return v; };
+    if (!CS::run(smem_raw, src, (int)len, kmin, kmax, KeySink<uint32_t, decltype(same)>{runs + lo, same}, g, G) &&
         threadIdx.x == 0)
         retry[k] = 1u;
 }
@@ -406,10 +426,6 @@ run_sample_tags_kernel(const uint32_t *__restrict__ keys, const uint32_t *__rest
     }
 }
 
-// ---------------------------------------------------------------------------
-// Sample sort (Fig. 1 step 5): LSD radix sort of the records (phi, tag) by the
-// bytes of tag, then of phi.  Byte positions on which every record agrees are
-// skipped; the pass table is built on the device.
 // ---------------------------------------------------------------------------
 // Blocks of few distinct keys (regular sampling, 32-bit keys): a block's
 // sorted order by (phi, tag) is its distinct values in order, each repeated in
@@ -646,502 +662,390 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
     if (tid == 0) retry[k] = 0;  // done
 }
 
-template <typename K>
-__device__ __forceinline__ uint32_t record_digit(K phi, uint32_t tag, int q) {
-    return q < 4 ? (tag >> (8 * q)) & 255u : (uint32_t)(phi >> (8 * (q - 4))) & 255u;
-}
-
-template <typename K>
-__global__ void lsd_hist_kernel(const K *__restrict__ phi, const uint32_t *__restrict__ tag, int64_t S,
-                                uint32_t *hist) {
-    constexpr int NPOS = 4 + (int)sizeof(K);
-    __shared__ uint32_t h[NPOS][256];
-    for (int i = threadIdx.x; i < NPOS * 256; i += blockDim.x) (&h[0][0])[i] = 0;
-    __syncthreads();
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < S;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const K f = phi[r];
-        const uint32_t t = tag[r];
-#pragma unroll
-        for (int q = 0; q < NPOS; ++q) atomicAdd(&h[q][record_digit(f, t, q)], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < NPOS * 256; i += blockDim.x) {
-        const uint32_t v = (&h[0][0])[i];
-        if (v) atomicAdd(&hist[i], v);
-    }
-    if constexpr (sizeof(K) == 4) {  // value range of the sample, for the MSD sort
-        uint32_t mn_inv = 0, mx = 0;
-        for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < S;
-             r += (int64_t)gridDim.x * blockDim.x) {
-            const uint32_t f = (uint32_t)phi[r];
-            mn_inv = max(mn_inv, ~f);
-            mx = max(mx, f);
-        }
-        mn_inv = __reduce_max_sync(0xffffffffu, mn_inv);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&hist[NPOS * 256], mn_inv);
-            atomicMax(&hist[NPOS * 256 + 1], mx);
-        }
-    }
-}
-
-// table[0] = passes; then (position, src, dst) per pass; table[1+3*NPOS] = final buffer
-template <typename K>
-__global__ void lsd_plan_kernel(const uint32_t *hist, int64_t S, int32_t *table, int phi_only) {
-    constexpr int NPOS = 4 + (int)sizeof(K);
-    __shared__ int trivial[NPOS];
-    if (threadIdx.x < NPOS) trivial[threadIdx.x] = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < NPOS * 256; i += blockDim.x)
-        if ((int64_t)hist[i] == S) trivial[i / 256] = 1;  // every record has this byte
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    int np = 0, cur = 0;
-    for (int q = phi_only ? 4 : 0; q < NPOS; ++q) {
-        if (trivial[q]) continue;
-        table[1 + 3 * np] = q;
-        table[2 + 3 * np] = cur;
-        table[3 + 3 * np] = 1 - cur;
-        cur = 1 - cur;
-        ++np;
-    }
-    table[0] = np;
-    table[1 + 3 * NPOS] = cur;
-}
-
-template <typename K>
-__global__ void __launch_bounds__(kLsdThreads)
-lsd_upsweep_kernel(const LsdBuffers<K> b, int64_t S, int pass, const int32_t *table, uint32_t *counts,
-                   int64_t tiles) {
-    if (pass >= table[0]) return;
-    const int q = table[1 + 3 * pass], src = table[2 + 3 * pass];
-    __shared__ uint32_t h[256];
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-        __syncthreads();
-        const int64_t t0 = tile * kLsdTile;
-        for (int i = threadIdx.x; i < kLsdTile; i += kLsdThreads) {
-            const int64_t r = t0 + i;
-            if (r < S) atomicAdd(&h[record_digit(b.phi[src][r], b.tag[src][r], q)], 1u);
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < 256; d += blockDim.x) counts[(int64_t)d * tiles + tile] = h[d];
-        __syncthreads();
-    }
-}
-
-// Exclusive scan of the per-tile counts of one digit (CTA d scans digit d)
-// plus the number of records with a smaller digit.
-__global__ void __launch_bounds__(256) lsd_scan_kernel(uint32_t *counts, int64_t tiles, int pass,
-                                                       const int32_t *table, const uint32_t *hist) {
-    if (pass >= table[0]) return;
-    __shared__ uint32_t tmp[40];
-    __shared__ uint32_t dbase;
-    const int q = table[1 + 3 * pass];
-    const int d = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t below = tid < d ? hist[q * 256 + tid] : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
-    if (lane == 0) tmp[warp] = below;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t t = 0;
-        for (int w = 0; w < 8; ++w) t += tmp[w];
-        dbase = t;
-    }
-    __syncthreads();
-    uint32_t *c = counts + (int64_t)d * tiles;
-    const int64_t per = (tiles + 255) / 256;
-    const int64_t lo = tid * per, hi = imin64(tiles, lo + per);
-    uint32_t local = 0;
-    for (int64_t i = lo; i < hi; ++i) local += c[i];
-    uint32_t wt;
-    const uint32_t we = warp_excl_scan(local, &wt);
-    __syncthreads();
-    if (lane == 31) tmp[warp] = wt;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t t;
-        const uint32_t e = warp_excl_scan(lane < 8 ? tmp[lane] : 0u, &t);
-        if (lane < 8) tmp[lane] = e;
-    }
-    __syncthreads();
-    uint32_t run = dbase + tmp[warp] + we;
-    for (int64_t i = lo; i < hi; ++i) {
-        const uint32_t v = c[i];
-        c[i] = run;
-        run += v;
-    }
-}
-
-// Scatter of one pass: the tile is ranked stably per digit, grouped by digit
-// in shared memory, and each digit's run is written contiguously.
-template <typename K> constexpr size_t lsd_downsweep_smem() {
-    return sizeof(typename BlockRank<kLsdThreads, kLsdItems, 8>::Smem) + 256 * 4 * 2 + 40 * 4 +
-           (size_t)kLsdTile * (sizeof(K) + 4);
-}
-
-template <typename K>
-__global__ void __launch_bounds__(kLsdThreads)
-lsd_downsweep_kernel(LsdBuffers<K> b, int64_t S, int pass, const int32_t *table,
-                     const uint32_t *counts, int64_t tiles) {
-    if (pass >= table[0]) return;
-    const int q = table[1 + 3 * pass], src = table[2 + 3 * pass], dst = table[3 + 3 * pass];
-    using Rank = BlockRank<kLsdThreads, kLsdItems, 8>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    typename Rank::Smem &sm = *reinterpret_cast<typename Rank::Smem *>(smem_raw);
-    uint32_t *base = reinterpret_cast<uint32_t *>(smem_raw + sizeof(typename Rank::Smem));
-    uint32_t *start = base + 256;
-    uint32_t *tmp = start + 256;
-    K *st_f = reinterpret_cast<K *>(tmp + 40);
-    st_f = reinterpret_cast<K *>((reinterpret_cast<uintptr_t>(st_f) + 15) & ~uintptr_t(15));
-    uint32_t *st_t = reinterpret_cast<uint32_t *>(st_f + kLsdTile);
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int64_t t0 = tile * kLsdTile;
-        const int n_here = (int)imin64(kLsdTile, S - t0);
-        K f[kLsdItems];
-        uint32_t t[kLsdItems], d[kLsdItems], rk[kLsdItems];
-#pragma unroll
-        for (int i = 0; i < kLsdItems; ++i) {
-            const int64_t r = t0 + striped_slot<kLsdThreads, kLsdItems>(i);
-            if (r < S) {
-                f[i] = b.phi[src][r];
-                t[i] = b.tag[src][r];
-                d[i] = record_digit(f[i], t[i], q);
-            } else {
-                d[i] = 255;  // after every real record of digit 255 (higher slots)
-            }
-        }
-        Rank::rank(sm, d, rk);
-        for (int dd = threadIdx.x; dd < 256; dd += kLsdThreads) {
-            base[dd] = counts[(int64_t)dd * tiles + tile];
-            start[dd] = sm.digit_tot[dd];
-        }
-        __syncthreads();
-        digit_excl_scan<kLsdThreads, 256>(start, tmp);
-#pragma unroll
-        for (int i = 0; i < kLsdItems; ++i) {
-            const int64_t r = t0 + striped_slot<kLsdThreads, kLsdItems>(i);
-            if (r < S) {
-                const uint32_t s = start[d[i]] + rk[i];
-                st_f[s] = f[i];
-                st_t[s] = t[i];
-            }
-        }
-        __syncthreads();
-        // staged slot s holds a record of digit dg; its place is base[dg] + s - start[dg]
-        for (int s = threadIdx.x; s < n_here; s += kLsdThreads) {
-            const uint32_t dg = record_digit(st_f[s], st_t[s], q);
-            const uint32_t pos = base[dg] + (uint32_t)s - start[dg];
-            b.phi[dst][pos] = st_f[s];
-            b.tag[dst][pos] = st_t[s];
-        }
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------------------
-// MSD sample sort for 32-bit keys: records are put into 2^BITS bins (4096 up
-// to 8M records, 8192 above) by the top BITS bits of phi - min(phi) in one staged pass, and every bin is sorted in
-// shared memory by (phi, tag).  Used when no bin holds more than kMsdBinMax
-// records; otherwise the LSD passes above run.  Both give the same (unique)
-// sorted sample.
-//
-// Table slots: [kMsdFlag] = 1 when this path is taken, [kMsdShift] = bin
-// shift, [kMsdMin] = min(phi).  Scratch in the LSD tile counts: bin counts
-// [0, B), bin starts [B, 2B+1), bin cursors [2B+4, 3B+4), B = 2^BITS.
+// Sample sort (Fig. 1 step 5): the records (phi, tag) in order.  A sample of at
+// most kOneSample records is sorted by one CTA.  A larger one is itself sample
+// sorted, which no distribution of the keys unbalances: one CTA sorts
+// candidates, one drawn from each of equal stretches of the sample (a plain
+// stride would meet the same rank of every block of a regular sample), every
+// few of them is a pivot (and where several pivots share a key value, so are
+// that value's first and last possible record: a bin then holds no part of it
+// beside other values, whose tags and phi would spread it unevenly), the
+// records are counted and scattered into the
+// pivots' bins, and every bin is sorted on chip by the counting sort of
+// countsort.cuh over words phi << 32 | tag.  Four
+// launches for any sample (an LSD radix sort over the record's bytes, which
+// this replaces, took 24 to 36 of them).
 // ---------------------------------------------------------------------------
-constexpr int kMsdBinMax = 4096;  // records one CTA sorts in shared memory
-constexpr int kMsdFlag = 40, kMsdShift = 41, kMsdMin = 42;
-constexpr int64_t kMsdWideSample = 8 << 20;  // samples above this use 8192 bins
-template <int BITS> struct Msd {
-    static constexpr int kBins = 1 << BITS, kStart = kBins, kCursor = 2 * kBins + 4;
+constexpr int64_t kOneSample = 8192;
+constexpr int kPivotBinsMax = 4096;
+constexpr int kPivotCells = 4096;  // cells of the index over the pivots
+constexpr int kPivotThreads = 512;
+constexpr int kOneThreads = 1024;
+
+// Bins of a sample of S records (a power of two; half of them between chosen
+// pivots, about 512 to 1024 records each up to 2^21 records, half for the ends
+// of repeated values), and the candidates the pivots are chosen from.
+static int pivot_bins(int64_t S) {
+    int b = 64;
+    while (b < kPivotBinsMax / 2 && (int64_t)b * 1024 < S) b *= 2;
+    return 2 * b;
+}
+static int pivot_candidates(int bins) { return std::min(bins * 2, (int)kOneSample / 2); }
+
+// The sample sort's scratch (Layout::pivots): bin counts, starts, cursors and
+// a ticket, the pivots, their index.
+template <typename P> struct PivotScratch {
+    uint32_t *count, *start, *cursor, *ticket;
+    P *phi;
+    uint32_t *tag;
+    LutParams<P> *lutp;
+    uint16_t *lut;
+    __host__ __device__ static size_t bytes(int bins) {
+        return (size_t)bins * 4 * 4 + 64 + (size_t)bins * sizeof(P) + 64 + (kPivotCells + 2) * 2;
+    }
+    PivotScratch() = default;
+    __host__ __device__ PivotScratch(void *at, int bins) {
+        unsigned char *b = (unsigned char *)at;
+        phi = (P *)b;                 b += (size_t)bins * sizeof(P);
+        lutp = (LutParams<P> *)b;     b += 64;
+        count = (uint32_t *)b;        b += (size_t)bins * 4;
+        cursor = (uint32_t *)b;       b += (size_t)bins * 4;
+        ticket = (uint32_t *)b;       b += 16;
+        start = (uint32_t *)b;        b += (size_t)(bins + 4) * 4;
+        tag = (uint32_t *)b;          b += (size_t)bins * 4;
+        lut = (uint16_t *)b;
+    }
 };
-constexpr int64_t kMsdMinSample = 1 << 19;  // smaller samples: the LSD passes
 
-__device__ __forceinline__ uint32_t msd_bin(uint32_t f, uint32_t mn, int shift) {
-    return (f - mn) >> shift;  // < Msd<BITS>::kBins by the choice of shift
+size_t sample_scratch_bytes(const Plan &p) {
+    if (p.sample_size <= kOneSample) return 1;
+    const int bins = pivot_bins(p.sample_size);
+    return p.key_bytes == 8 ? PivotScratch<uint64_t>::bytes(bins) : PivotScratch<uint32_t>::bytes(bins);
+}
+int sample_sort_kernels(const Plan &p) { return p.sample_size == 0 ? 0 : p.sample_size <= kOneSample ? 1 : 4; }
+int sample_final(const Plan &p) { return p.sample_size <= kOneSample ? 1 : 0; }
+
+template <typename P> using OneSort = BlockSort<typename RecordSink<P>::K, kOneThreads>;
+template <typename P> static size_t one_smem(int n) {
+    return ((sizeof(typename OneSort<P>::Smem) + 15) & ~size_t(15)) + (size_t)n * sizeof(typename RecordSink<P>::K);
+}
+static_assert(OneSort<uint32_t>::kMost >= kOneSample && OneSort<uint64_t>::kMost >= kOneSample, "records one CTA sorts");
+
+template <typename P> struct SortArgs {
+    RecordBuffers<P> b;
+    int64_t S;
+    int cand, bins;
+    PivotScratch<P> sc;
+};
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kOneThreads, 1) sample_one_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    P *out_phi = pk.a.b.phi[1];
+    uint32_t *out_tag = pk.a.b.tag[1];
+    const int S = (int)pk.a.S;
+    using K = typename RecordSink<P>::K;
+    using Smem = typename OneSort<P>::Smem;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    K *a = reinterpret_cast<K *>(smem_raw + ((sizeof(Smem) + 15) & ~size_t(15)));
+    for (int i = threadIdx.x; i < S; i += kOneThreads) a[i] = (K)phi[i] << 32 | tag[i];
+    __syncthreads();
+    OneSort<P>::run(*reinterpret_cast<Smem *>(smem_raw), a, S);
+    for (int i = threadIdx.x; i < S; i += kOneThreads) {
+        out_phi[i] = (P)(a[i] >> 32);
+        out_tag[i] = (uint32_t)a[i];
+    }
 }
 
-template <int BITS>
-__global__ void __launch_bounds__(256) msd_hist_kernel(const uint32_t *__restrict__ phi, int64_t S,
-                                                       const uint32_t *lsd_hist, int npos, uint32_t *counts) {
-    __shared__ uint32_t h[Msd<BITS>::kBins];
-    for (int i = threadIdx.x; i < Msd<BITS>::kBins; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    const uint32_t mn = ~lsd_hist[npos * 256], mx = lsd_hist[npos * 256 + 1];
-    const int bl = bit_length<uint32_t>(mx - mn);
-    const int shift = bl > BITS ? bl - BITS : 0;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < S; r += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&h[msd_bin(phi[r], mn, shift)], 1u);
-    __syncthreads();
-    for (int i = threadIdx.x; i < Msd<BITS>::kBins; i += blockDim.x)
-        if (h[i]) atomicAdd(&counts[i], h[i]);
-}
-
-// Bin starts; the MSD path is taken when every bin fits one CTA.
-template <int BITS>
-__global__ void __launch_bounds__(1024) msd_plan_kernel(uint32_t *counts, const uint32_t *lsd_hist, int npos,
-                                                        int32_t *table) {
-    __shared__ uint32_t tmp[40];
-    __shared__ int big;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) big = 0;
-    __syncthreads();
-    constexpr int PER = Msd<BITS>::kBins / 1024;
-    uint32_t v[PER], local = 0;
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kOneThreads, 1) sample_pivots_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    const int64_t S = pk.a.S;
+    const int cand = pk.a.cand, bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    using K = typename RecordSink<P>::K;
+    using Smem = typename OneSort<P>::Smem;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    K *a = reinterpret_cast<K *>(smem_raw + ((sizeof(Smem) + 15) & ~size_t(15)));
+    P *piv_phi = reinterpret_cast<P *>(a + cand);  // bins entries
+    const uint32_t stretch = (uint32_t)(S / cand);
+    for (int i = threadIdx.x; i < bins; i += kOneThreads) sc.count[i] = 0;
+    if (threadIdx.x == 0) *sc.ticket = 0;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        v[q] = counts[tid * PER + q];
-        local += v[q];
-        if (v[q] > (uint32_t)kMsdBinMax) big = 1;
-    }
-    uint32_t wt;
-    const uint32_t we = warp_excl_scan(local, &wt);
-    if (lane == 31) tmp[warp] = wt;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t t;
-        const uint32_t e = warp_excl_scan(tmp[lane], &t);
-        tmp[lane] = e;
-    }
-    __syncthreads();
-    uint32_t run = tmp[warp] + we;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        counts[Msd<BITS>::kStart + tid * PER + q] = run;
-        counts[Msd<BITS>::kCursor + tid * PER + q] = 0;
-        run += v[q];
-    }
-    if (tid == 1023) counts[Msd<BITS>::kStart + Msd<BITS>::kBins] = run;
-    if (tid == 0) {
-        const uint32_t mn = ~lsd_hist[npos * 256], mx = lsd_hist[npos * 256 + 1];
-        const int bl = bit_length<uint32_t>(mx - mn);
-        const bool take = !big;
-        table[kMsdFlag] = take ? 1 : 0;
-        table[kMsdShift] = bl > BITS ? bl - BITS : 0;
-        table[kMsdMin] = (int32_t)mn;
-        if (take) {
-            table[0] = 0;              // no LSD passes
-            table[1 + 3 * npos] = 1;   // the sorted sample ends in buffer 1
+    for (int j = 0; j < (int)(kOneSample / kOneThreads); ++j) {
+        const int i = j * kOneThreads + threadIdx.x;
+        if (i < cand) {
+            // a place in stretch i: the top bits of a multiplicative hash
+            const int64_t r = (int64_t)i * stretch + __umulhi((uint32_t)i * 0x9e3779b1u, stretch);
+            a[i] = (K)phi[r] << 32 | tag[r];
         }
     }
+    __syncthreads();
+    OneSort<P>::run(*reinterpret_cast<Smem *>(smem_raw), a, cand);
+    // chosen pivot i: candidate of 1-indexed rank (i + 1) * step.  A value that
+    // two neighbouring pivots share gets two more, before its first and past
+    // its last record.
+    const int chosen = bins / 2 - 1, step = cand / (bins / 2);
+    auto phi_of = [&](int i) { return (P)(a[(i + 1) * step - 1] >> 32); };
+    __shared__ uint32_t tmp[40];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int PER = kPivotBinsMax / 2 / kOneThreads;
+    uint32_t extra[PER], loc = 0;  // 1: before, 2: after
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x * PER + j;
+        extra[j] = 0;
+        if (i < chosen) {
+            const bool as_prev = i > 0 && phi_of(i - 1) == phi_of(i), as_next = i + 1 < chosen && phi_of(i + 1) == phi_of(i);
+            if (as_next && !as_prev) extra[j] = 1;
+            if (as_prev && !as_next && phi_of(i) != all_ones<P>()) extra[j] = 2;
+            loc += 1 + (extra[j] != 0);
+        }
+    }
+    uint32_t tot;
+    const uint32_t ex = warp_excl_scan(loc, &tot);
+    if (lane == 31) tmp[warp] = tot;
+    __syncthreads();
+    uint32_t at = ex, all = 0;
+    for (int w = 0; w < kOneThreads / 32; ++w) {
+        at += w < warp ? tmp[w] : 0u;
+        all += tmp[w];
+    }
+    for (int i = (int)all + threadIdx.x; i < bins; i += kOneThreads) {  // the rest: past every record
+        piv_phi[i] = all_ones<P>();
+        sc.phi[i] = all_ones<P>();
+        sc.tag[i] = 0xffffffffu;
+    }
+    auto put = [&](P f, uint32_t t) {
+        piv_phi[at] = f;
+        sc.phi[at] = f;
+        sc.tag[at] = t;
+        ++at;
+    };
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x * PER + j;
+        if (i < chosen) {
+            if (extra[j] == 1) put(phi_of(i), 0u);
+            put(phi_of(i), (uint32_t)a[(i + 1) * step - 1]);
+            if (extra[j] == 2) put(phi_of(i) + 1, 0u);
+        }
+    }
+    __syncthreads();
+    // the index over the pivots, as over the splitters
+    LutParams<P> lp;
+    lp.base = piv_phi[0];
+    lp.span = piv_phi[all - 1] - lp.base;  // (all >= 31 pivots)
+    const int bl = bit_length<P>(lp.span);
+    lp.shift = bl > 12 ? (uint32_t)(bl - 12) : 0u;
+    lp.nsplit = all;
+    static_assert(kPivotCells == 1 << 12, "cells of the index");
+    if (threadIdx.x == 0) *sc.lutp = lp;
+    for (int c = threadIdx.x; c <= kPivotCells; c += kOneThreads)
+        sc.lut[c] = (uint16_t)lut_cell((uint32_t)c, lp, [&](uint32_t i) { return piv_phi[i]; });
+}
+
+// Records of a CTA's tiles per bin; the last CTA to finish turns the totals
+// into the bins' starts.
+template <typename P> constexpr size_t pivot_smem(int bins) {
+    return 64 + (size_t)bins * (sizeof(P) + 4) + (kPivotCells + 8) * 2;  // (tags, read on ties, stay in global memory)
+}
+template <typename P> struct PivotSmem {
+    LutParams<P> *lp;
+    P *phi;
+    uint32_t *cnt;
+    uint16_t *lut;
+    __device__ PivotSmem(unsigned char *b, int bins) {
+        lp = (LutParams<P> *)b;   b += 64;
+        phi = (P *)b;             b += (size_t)bins * sizeof(P);
+        cnt = (uint32_t *)b;      b += (size_t)bins * 4;
+        lut = (uint16_t *)b;
+    }
+    __device__ void load(const PivotScratch<P> &sc, int bins) {
+        for (int i = threadIdx.x; i < bins; i += kPivotThreads) {
+            phi[i] = sc.phi[i];
+            cnt[i] = 0;
+        }
+        for (int i = threadIdx.x; i <= kPivotCells; i += kPivotThreads) lut[i] = sc.lut[i];
+        if (threadIdx.x == 0) *lp = *sc.lutp;
+        __syncthreads();
+    }
+};
+
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kPivotThreads) sample_hist_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    const int64_t S = pk.a.S;
+    const int bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PivotSmem<P> sm(smem_raw, bins);
+    __shared__ uint32_t tmp[40];
+    __shared__ bool last;
+    sm.load(sc, bins);
+    const LutParams<P> lp = *sm.lp;
+    const int64_t step = (int64_t)pk.blocks * kPivotThreads;
+    for (int64_t r = (int64_t)pk.block * kPivotThreads + threadIdx.x; r < S; r += 4 * step) {
+        P f[4];
+        uint32_t t[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r + j * step < S) {
+                f[j] = phi[r + j * step];
+                t[j] = tag[r + j * step];
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r + j * step < S) atomicAdd(&sm.cnt[classify_key(f[j], t[j], lp, sm.lut, sm.phi, sc.tag)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads)
+        if (sm.cnt[i]) atomicAdd(&sc.count[i], sm.cnt[i]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(sc.ticket, 1u) == pk.blocks - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads) {
+        sm.cnt[i] = ld_volatile(&sc.count[i]);
+        sc.cursor[i] = 0;
+    }
+    __syncthreads();
+    const uint32_t tot = block_excl_scan_smem<kPivotThreads>(sm.cnt, bins, tmp);
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads) sc.start[i] = sm.cnt[i];
+    if (threadIdx.x == 0) sc.start[bins] = tot;
 }
 
 // Records of a tile, grouped by bin in shared memory, each bin's run written
-// contiguously at its bin start plus a reserved offset.
-constexpr int kMsdThreads = 512, kMsdItems = 16, kMsdTile = kMsdThreads * kMsdItems;
-template <int BITS>
-__global__ void __launch_bounds__(kMsdThreads) msd_scatter_kernel(LsdBuffers<uint32_t> b, int64_t S,
-                                                                  const int32_t *table, uint32_t *counts) {
-    if (table[kMsdFlag] == 0) return;
+// contiguously at its bin's start plus a reserved offset.
+template <typename P, int ITEMS> constexpr size_t pivot_scatter_smem(int bins) {
+    return pivot_smem<P>(bins) + (size_t)bins * 4 + (size_t)kPivotThreads * ITEMS * (sizeof(P) + 4 + 2) + 64;
+}
+template <typename P, int ITEMS, bool MANY>
+__global__ void __launch_bounds__(kPivotThreads) sample_scatter_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const RecordBuffers<P> &b = pk.a.b;
+    const int64_t S = pk.a.S;
+    const int bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    constexpr int TILE = kPivotThreads * ITEMS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(smem_raw);      // Msd<BITS>::kBins + 4
-    uint32_t *dlt = cnt + Msd<BITS>::kBins + 4;                           // Msd<BITS>::kBins
-    uint32_t *st_f = dlt + Msd<BITS>::kBins;                              // kMsdTile
-    uint32_t *st_t = st_f + kMsdTile;                             // kMsdTile
-    uint16_t *st_b = reinterpret_cast<uint16_t *>(st_t + kMsdTile);  // kMsdTile
+    PivotSmem<P> sm(smem_raw, bins);
+    unsigned char *at8 = smem_raw + ((pivot_smem<P>(bins) + 15) & ~size_t(15));
+    P *st_f = (P *)at8;
+    uint32_t *st_t = (uint32_t *)(st_f + TILE), *dlt = st_t + TILE;
+    uint16_t *st_b = (uint16_t *)(dlt + bins);
     __shared__ uint32_t tmp[40];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int shift = table[kMsdShift];
-    const uint32_t mn = (uint32_t)table[kMsdMin];
-    const int64_t t0 = (int64_t)blockIdx.x * kMsdTile;
-    const int nh = (int)imin64(kMsdTile, S - t0);
-    for (int i = tid; i < Msd<BITS>::kBins; i += kMsdThreads) cnt[i] = 0;
-    __syncthreads();
-    uint32_t f[kMsdItems], t[kMsdItems], br[kMsdItems];
+    sm.load(sc, bins);
+    const LutParams<P> lp = *sm.lp;
+    const int tid = threadIdx.x;
+    for (int64_t t0 = (int64_t)pk.block * TILE; t0 < S; t0 += (int64_t)pk.blocks * TILE) {
+        const int nh = (int)imin64(TILE, S - t0);
+        P f[ITEMS];
+        uint32_t t[ITEMS], br[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kMsdItems; ++i) {
-        const int s = i * kMsdThreads + tid;
-        if (s < nh) {
-            f[i] = b.phi[0][t0 + s];
-            t[i] = b.tag[0][t0 + s];
-            const uint32_t bin = msd_bin(f[i], mn, shift);
-            br[i] = bin << 16 | atomicAdd(&cnt[bin], 1u);
+        for (int i = 0; i < ITEMS; ++i) {
+            const int s = i * kPivotThreads + tid;
+            if (s < nh) {
+                f[i] = b.phi[0][t0 + s];
+                t[i] = b.tag[0][t0 + s];
+            }
         }
-    }
-    __syncthreads();
-    // starts of the bins inside the tile (8 bins per thread) and reservations
-    constexpr int PER = Msd<BITS>::kBins / kMsdThreads;
-    uint32_t c[PER], local = 0;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        c[q] = cnt[tid * PER + q];
-        local += c[q];
-    }
-    uint32_t wt;
-    const uint32_t we = warp_excl_scan(local, &wt);
-    if (lane == 31) tmp[warp] = wt;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t tt;
-        const uint32_t e = warp_excl_scan(lane < kMsdThreads / 32 ? tmp[lane] : 0u, &tt);
-        if (lane < kMsdThreads / 32) tmp[lane] = e;
-    }
-    __syncthreads();
-    uint32_t run = tmp[warp] + we;
-    uint32_t at[PER];
-#pragma unroll
-    for (int q = 0; q < PER; ++q) at[q] = c[q] ? atomicAdd(&counts[Msd<BITS>::kCursor + tid * PER + q], c[q]) : 0u;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int bin = tid * PER + q;
-        cnt[bin] = run;
-        dlt[bin] = counts[Msd<BITS>::kStart + bin] + at[q] - run;  // output slot of tile position s: dlt + s
-        run += c[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kMsdItems; ++i) {
-        const int s = i * kMsdThreads + tid;
-        if (s < nh) {
-            const uint32_t bin = br[i] >> 16, pos = cnt[bin] + (br[i] & 0xffffu);
-            st_f[pos] = f[i];
-            st_t[pos] = t[i];
-            st_b[pos] = (uint16_t)bin;
+        for (int i = 0; i < ITEMS; ++i)
+            if (i * kPivotThreads + tid < nh) {
+                const uint32_t bin = classify_key(f[i], t[i], lp, sm.lut, sm.phi, sc.tag);
+                br[i] = bin << 16 | atomicAdd(&sm.cnt[bin], 1u);
+            }
+        __syncthreads();
+        for (int i = tid; i < bins; i += kPivotThreads) {
+            const uint32_t c = sm.cnt[i];
+            dlt[i] = c ? sc.start[i] + atomicAdd(&sc.cursor[i], c) : 0u;
         }
-    }
-    __syncthreads();
-    for (int s = tid; s < nh; s += kMsdThreads) {
-        const uint32_t o = dlt[st_b[s]] + (uint32_t)s;
-        b.phi[1][o] = st_f[s];
-        b.tag[1][o] = st_t[s];
+        __syncthreads();
+        block_excl_scan_smem<kPivotThreads>(sm.cnt, bins, tmp);
+        for (int i = tid; i < bins; i += kPivotThreads) dlt[i] -= sm.cnt[i];  // output slot of tile position s: dlt + s
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (i * kPivotThreads + tid < nh) {
+                const uint32_t bin = br[i] >> 16, pos = sm.cnt[bin] + (br[i] & 0xffffu);
+                st_f[pos] = f[i];
+                st_t[pos] = t[i];
+                st_b[pos] = (uint16_t)bin;
+            }
+        __syncthreads();
+        for (int s = tid; s < nh; s += kPivotThreads) {
+            const uint32_t o = dlt[st_b[s]] + (uint32_t)s;
+            b.phi[1][o] = st_f[s];
+            b.tag[1][o] = st_t[s];
+        }
+        for (int i = tid; i < bins; i += kPivotThreads) sm.cnt[i] = 0;
+        __syncthreads();
     }
 }
-template <int BITS>
-constexpr size_t msd_scatter_smem() { return (size_t)(2 * Msd<BITS>::kBins + 4 + 2 * kMsdTile) * 4 + (size_t)kMsdTile * 2; }
 
-// One bin per CTA, (phi, tag) as one 64-bit key: a counting pass on the top
-// 11 bits of the bin's range, then each key's place inside its count bin by
-// comparison; a bin whose count bins are too long is sorted by a bitonic
-// network instead.  (Sampling with replacement can repeat a record: equal
-// keys are ordered by their slot.)
-constexpr int kMsdLocalThreads = 512, kMsdLocalItems = kMsdBinMax / kMsdLocalThreads;
-constexpr int kMsdCountBits = 11, kMsdCountBins = 1 << kMsdCountBits;
-template <int BITS>
-__global__ void __launch_bounds__(kMsdLocalThreads) msd_local_kernel(LsdBuffers<uint32_t> b, const int32_t *table,
-                                                                      const uint32_t *counts) {
-    if (table[kMsdFlag] == 0) return;
-    __shared__ uint64_t a[kMsdBinMax];
-    __shared__ uint32_t ch[kMsdCountBins + 4];
-    __shared__ uint32_t tmp[40];
-    constexpr int T = kMsdLocalThreads, IT = kMsdLocalItems;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t lo = counts[Msd<BITS>::kStart + blockIdx.x], hi = counts[Msd<BITS>::kStart + blockIdx.x + 1];
-    const int n = (int)(hi - lo);
-    if (n <= 1) return;
-    // keys of this bin lie in [klo, khi]
-    const int shift = table[kMsdShift];
-    const uint32_t mn = (uint32_t)table[kMsdMin];
-    const uint64_t flo = (uint64_t)mn + ((uint64_t)blockIdx.x << shift);
-    const uint64_t klo = flo << 32, span = (((uint64_t)1 << shift) << 32) - 1;
-    const int bits = bit_length<uint64_t>(span);
-    const int sh = bits > kMsdCountBits ? bits - kMsdCountBits : 0;
-    uint64_t k[IT];
-    uint32_t r[IT];
-    for (int i = tid; i < kMsdCountBins; i += T) ch[i] = 0;
+// One bin per CTA, from buffer 1 into its place in buffer 0.  A bin that the
+// counting sort gives back (a run of its bins above the stage: the pivots keep
+// bins near their mean, so this is out of reach in practice) is put in order
+// where it lies by a bitonic network.
+template <typename P, int SIZE, bool MANY>
+__global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
+sample_bins_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const RecordBuffers<P> &b = pk.a.b;
+    const PivotScratch<P> &sc = pk.a.sc;
+    using K = typename RecordSink<P>::K;
+    using CS = typename CountShape<SIZE>::template Sort<K>;
+    constexpr int T = CountShape<SIZE>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t at = sc.start[pk.block];
+    const int n = (int)(sc.start[pk.block + 1] - at);
+    if (n == 0) return;
+    P *f = b.phi[1] + at;
+    uint32_t *t = b.tag[1] + at;
+    const RecordSource<P, T> src{f, t, 1};
+    K lo, hi;
+    CS::bounds(smem_raw, src, n, lo, hi);
+    if (CS::run(smem_raw, src, n, lo, hi, RecordSink<P>{b.phi[0], b.tag[0], (int64_t)at}, 0, 1)) return;
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        const int e = i * T + tid;
-        if (e < n) {
-            k[i] = (uint64_t)b.phi[1][lo + e] << 32 | b.tag[1][lo + e];
-            const uint64_t d = (k[i] - klo) >> sh;
-            r[i] = atomicAdd(&ch[d < kMsdCountBins ? (uint32_t)d : kMsdCountBins - 1], 1u);
-        }
-    }
-    __syncthreads();
-    // exclusive scan of the count bins (8 per thread), longest bin
-    constexpr int PER = kMsdCountBins / T;
-    uint32_t v[PER], loc = 0, mx = 0;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        v[q] = ch[tid * PER + q];
-        loc += v[q];
-        mx = max(mx, v[q]);
-    }
-    uint32_t wt;
-    const uint32_t we = warp_excl_scan(loc, &wt);
-    if (lane == 31) tmp[warp] = wt;
-    const bool too_long = __syncthreads_or(mx > 64);
-    if (!too_long) {
-        if (warp == 0) {
-            uint32_t t;
-            const uint32_t e = warp_excl_scan(lane < T / 32 ? tmp[lane] : 0u, &t);
-            if (lane < T / 32) tmp[lane] = e;
-        }
-        __syncthreads();
-        uint32_t run = tmp[warp] + we;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            ch[tid * PER + q] = run;
-            run += v[q];
-        }
-        if (tid == 0) ch[kMsdCountBins] = (uint32_t)n;
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = i * T + tid;
-            if (e < n) {
-                const uint64_t d = (k[i] - klo) >> sh;
-                r[i] += ch[d < kMsdCountBins ? (uint32_t)d : kMsdCountBins - 1];
-                a[r[i]] = k[i];
+    int n2 = 1;
+    while (n2 < n) n2 <<= 1;
+    auto step = [&](int i, int l) {
+        if (l < n) {
+            const P x = f[i], y = f[l];
+            const uint32_t u = t[i], v = t[l];
+            if (x > y || (x == y && u > v)) {
+                f[i] = y;
+                f[l] = x;
+                t[i] = v;
+                t[l] = u;
             }
         }
-        __syncthreads();
-        // keys sharing a count bin: place = bin start + smaller keys in the bin
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = i * T + tid;
-            if (e < n) {
-                const uint64_t d = (k[i] - klo) >> sh;
-                const uint32_t cb = d < kMsdCountBins ? (uint32_t)d : kMsdCountBins - 1;
-                const uint32_t b0 = ch[cb], b1 = ch[cb + 1], self = r[i];
-                if (b1 - b0 > 1) {
-                    uint32_t pos = b0;
-                    for (uint32_t y = b0; y < b1; ++y) {
-                        const uint64_t x = a[y];
-                        pos += (x < k[i]) | ((x == k[i]) & (y < self));
-                    }
-                    r[i] = pos;
-                }
-            }
+    };
+    for (int h = 1; h < n2; h <<= 1) {
+        for (int q = threadIdx.x; q < n2 / 2; q += T) {
+            const int c = (q & ~(h - 1)) * 2, o = q & (h - 1);
+            step(c + o, c + 2 * h - 1 - o);
         }
         __syncthreads();
-#pragma unroll
-        for (int i = 0; i < IT; ++i)
-            if (i * T + tid < n) a[r[i]] = k[i];
-        __syncthreads();
-    } else {
-        int n2 = 1;
-        while (n2 < n) n2 <<= 1;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = i * T + tid;
-            if (e < n) a[e] = k[i];
-        }
-        for (int e = n + tid; e < n2; e += T) a[e] = ~0ull;
-        __syncthreads();
-        for (int kk = 2; kk <= n2; kk <<= 1)
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                for (int t = tid; t < (n2 >> 1); t += T) {
-                    const int i = 2 * t - (t & (j - 1));
-                    const int l = i + j;
-                    const bool up = (i & kk) == 0;
-                    const uint64_t x = a[i], y = a[l];
-                    if ((x > y) == up) {
-                        a[i] = y;
-                        a[l] = x;
-                    }
-                }
-                __syncthreads();
+        for (int j = h >> 1; j > 0; j >>= 1) {
+            for (int q = threadIdx.x; q < n2 / 2; q += T) {
+                const int i = 2 * q - (q & (j - 1));
+                step(i, i + j);
             }
+            __syncthreads();
+        }
     }
-    for (int i = tid; i < n; i += T) {
-        b.phi[1][lo + i] = (uint32_t)(a[i] >> 32);
-        b.tag[1][lo + i] = (uint32_t)a[i];
+    for (int i = threadIdx.x; i < n; i += T) {
+        b.phi[0][at + i] = f[i];
+        b.tag[0][at + i] = t[i];
     }
 }
 
@@ -1152,52 +1056,47 @@ __global__ void __launch_bounds__(kMsdLocalThreads) msd_local_kernel(LsdBuffers<
 // j = i*B these are the paper's splitters, so the buckets are unchanged.
 // "Broadcast" (Fig. 1 step 7) is the copy into every CTA's shared memory.
 // ---------------------------------------------------------------------------
-template <typename K>
-__global__ void splitter_kernel(LsdBuffers<K> b, const int32_t *table, int npos, int64_t P, int64_t Q,
-                                int64_t B, K *vphi, uint32_t *vtag, LutParams<K> *lutp) {
-    const int fin = table[1 + 3 * npos];
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x + 1;
-    if (j < P) {
-        const int64_t r = (j * Q) / B;  // 1-indexed rank
-        vphi[j - 1] = b.phi[fin][r - 1];
-        vtag[j - 1] = b.tag[fin][r - 1];
+template <typename K> struct SplitterArgs {
+    const K *phi;
+    const uint32_t *tag;
+    int64_t P, Q, B;
+    K *vphi;
+    uint32_t *vtag;
+    LutParams<K> *lutp;
+    uint16_t *lut;
+    int lut_bits, pad_;
+};
+template <typename K, bool MANY>
+__global__ void __launch_bounds__(256) splitter_kernel(const Many<SplitterArgs<K>> many) {
+    const Pick<MANY, SplitterArgs<K>> pk(many);
+    const K *phi = pk.a.phi;
+    const uint32_t *tag = pk.a.tag;
+    const int64_t P = pk.a.P, Q = pk.a.Q, B = pk.a.B;
+    K *vphi = pk.a.vphi;
+    uint32_t *vtag = pk.a.vtag;
+    LutParams<K> *lutp = pk.a.lutp;
+    uint16_t *lut = pk.a.lut;
+    const int lut_bits = pk.a.lut_bits;
+    auto rank = [&](int64_t j) { return (j * Q) / B - 1; };  // sorted index of splitter j, 1 <= j < P
+    LutParams<K> lp;
+    lp.base = P > 1 ? phi[rank(1)] : K(0);
+    lp.span = P > 1 ? phi[rank(P - 1)] - lp.base : K(0);
+    const int bl = bit_length<K>(lp.span);
+    lp.shift = bl > lut_bits ? (uint32_t)(bl - lut_bits) : 0u;
+    lp.nsplit = (uint32_t)(P - 1);
+    const int64_t t = (int64_t)pk.block * blockDim.x + threadIdx.x;
+    if (t == 0) *lutp = lp;
+    if (t < P - 1) {
+        const int64_t r = rank(t + 1);
+        vphi[t] = phi[r];
+        vtag[t] = tag[r];
+    } else if (t == P - 1) {  // above every key, for comparisons without a bounds check
+        vphi[t] = all_ones<K>();
+        vtag[t] = 0xffffffffu;
     }
-    if (j == 1 || (P == 1 && blockIdx.x == 0 && threadIdx.x == 0)) {
-        LutParams<K> lp;
-        if (P > 1) {
-            const K lo = b.phi[fin][(1 * Q) / B - 1];
-            const K hi = b.phi[fin][((P - 1) * Q) / B - 1];
-            lp.base = lo;
-            lp.span = hi - lo;
-            const int bl = bit_length<K>(lp.span);
-            lp.shift = bl > kLutBits ? (uint32_t)(bl - kLutBits) : 0u;
-        } else {
-            lp.base = 0;
-            lp.span = 0;
-            lp.shift = 0;
-        }
-        lp.nsplit = (uint32_t)(P - 1);
-        *lutp = lp;
-    }
-}
-
-template <typename K>
-__global__ void lut_kernel(const K *vphi, const LutParams<K> *lutp, uint16_t *lut) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c > kLutCells) return;
-    const LutParams<K> lp = *lutp;
-    uint32_t lo = 0, hi = lp.nsplit;
-    if ((K)c > (lp.span >> lp.shift)) {
-        lo = lp.nsplit;
-    } else {
-        const K thr = lp.base + ((K)c << lp.shift);
-        while (lo < hi) {  // number of splitters with phi < thr
-            const uint32_t mid = (lo + hi) >> 1;
-            if (vphi[mid] < thr) lo = mid + 1;
-            else hi = mid;
-        }
-    }
-    lut[c] = (uint16_t)lo;
+    // the radix index, from the sorted sample itself
+    if (t <= (1 << lut_bits))
+        lut[t] = (uint16_t)lut_cell((uint32_t)t, lp, [&](uint32_t i) { return phi[rank((int64_t)i + 1)]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -1221,9 +1120,8 @@ __device__ __forceinline__ bsps_record to_record(K phi, uint32_t tag, int64_t n,
 }
 
 template <typename K>
-__global__ void sample_records_kernel(LsdBuffers<K> b, const int32_t *table, int npos, int64_t S,
+__global__ void sample_records_kernel(RecordBuffers<K> b, int fin, int64_t S,
                                       int64_t n, int64_t m, int64_t M, bool regular, bsps_record *out) {
-    const int fin = table[1 + 3 * npos];
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < S) out[i] = to_record(b.phi[fin][i], b.tag[fin][i], n, m, M, regular);
 }
@@ -1288,9 +1186,9 @@ __global__ void pad_sizes_kernel(int64_t n, int64_t R, int64_t m, int64_t M, int
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-template <int DT> static LsdBuffers<typename KeyTraits<DT>::T> lsd_buffers(const Ctx &c) {
+template <int DT> static RecordBuffers<typename KeyTraits<DT>::T> record_buffers(const Ctx &c) {
     using K = typename KeyTraits<DT>::T;
-    LsdBuffers<K> b;
+    RecordBuffers<K> b;
     b.phi[0] = (K *)c.ly.sphi[0];
     b.phi[1] = (K *)c.ly.sphi[1];
     b.tag[0] = c.ly.stag[0];
@@ -1371,13 +1269,6 @@ int run_keys_cluster(const Plan &p) {
 template <int DT> static cudaError_t launch_sample_t(const Ctx &c) {
     using K = typename KeyTraits<DT>::T;
     const Plan &p = c.pl;
-    if (p.sampling == BSPS_RANDOM) {
-        if (p.sample_size == 0) return cudaSuccess;
-        const int64_t blocks4 = (p.sample_size + 3) / 4;
-        sample_random_kernel<DT><<<(unsigned)((blocks4 + 255) / 256), 256, 0, c.stream>>>(
-            (const K *)c.keys_in, p.n, p.sample_size, p.seed, (K *)c.ly.sphi[0], c.ly.stag[0]);
-        return cudaGetLastError();
-    }
     const uint32_t *only = nullptr;
     if constexpr (sizeof(K) == 4) {
         cudaError_t e = cudaSuccess;
@@ -1419,6 +1310,26 @@ template <int DT> static cudaError_t launch_sample_t(const Ctx &c) {
     }
 }
 
+template <int DT> static cudaError_t launch_sample_random_t(Exec &x) {
+    using K = typename KeyTraits<DT>::T;
+    return launch_calls<SampleArgs<K>>(x, sample_random_kernel<DT, false>, sample_random_kernel<DT, true>, 256, 0,
+                                       [](const Ctx &c, SampleArgs<K> &a) {
+        const Plan &p = c.pl;
+        a = {(const K *)c.keys_in, p.n, p.sample_size, p.seed, (K *)c.ly.sphi[0], c.ly.stag[0], c.ly.status, c.ly.cursor,
+             c.ly.retry_flag, p.P};
+        return (uint32_t)imax64(1, (p.sample_size + 1023) / 1024);
+    });
+}
+
+cudaError_t launch_sample_random(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_sample_random_t<BSPS_U32>(x);
+    case BSPS_I32: return launch_sample_random_t<BSPS_I32>(x);
+    case BSPS_F32: return launch_sample_random_t<BSPS_F32>(x);
+    default: return launch_sample_random_t<BSPS_F64>(x);
+    }
+}
+
 cudaError_t launch_sample(const Ctx &c) {
     switch (c.pl.dtype) {
     case BSPS_U32: return launch_sample_t<BSPS_U32>(c);
@@ -1428,103 +1339,135 @@ cudaError_t launch_sample(const Ctx &c) {
     }
 }
 
-template <int BITS> static cudaError_t launch_msd(const Ctx &c, LsdBuffers<uint32_t> b, int hist_blocks) {
-    const Plan &p = c.pl;
-    constexpr int NPOS = 8;
-    uint32_t *cnt = c.ly.lsd_counts;
-    cudaError_t e = cudaMemsetAsync(cnt, 0, Msd<BITS>::kBins * sizeof(uint32_t), c.stream);
-    if (e != cudaSuccess) return e;
-    msd_hist_kernel<BITS><<<max(hist_blocks, 1), 256, 0, c.stream>>>(b.phi[0], p.sample_size, c.ly.lsd_hist, NPOS,
-                                                                    cnt);
-    msd_plan_kernel<BITS><<<1, 1024, 0, c.stream>>>(cnt, c.ly.lsd_hist, NPOS, c.ly.lsd_table);
-    e = cudaFuncSetAttribute(msd_scatter_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)msd_scatter_smem<BITS>());
-    if (e != cudaSuccess) return e;
-    const unsigned mt = (unsigned)((p.sample_size + kMsdTile - 1) / kMsdTile);
-    msd_scatter_kernel<BITS><<<mt, kMsdThreads, msd_scatter_smem<BITS>(), c.stream>>>(b, p.sample_size,
-                                                                                        c.ly.lsd_table, cnt);
-    msd_local_kernel<BITS><<<Msd<BITS>::kBins, kMsdLocalThreads, 0, c.stream>>>(b, c.ly.lsd_table, cnt);
-    return cudaGetLastError();
-}
-
-template <typename K> static cudaError_t launch_sample_sort_t(const Ctx &c, LsdBuffers<K> b) {
-    const Plan &p = c.pl;
-    constexpr int NPOS = 4 + (int)sizeof(K);
-    cudaError_t e = cudaMemsetAsync(c.ly.lsd_hist, 0, (NPOS * 256 + 2) * sizeof(uint32_t), c.stream);
-    if (e != cudaSuccess) return e;
-    const int hist_blocks = (int)imin64(1024, (p.sample_size + 1023) / 1024);
-    lsd_hist_kernel<K><<<max(hist_blocks, 1), 256, 0, c.stream>>>(b.phi[0], b.tag[0], p.sample_size,
-                                                                  c.ly.lsd_hist);
-    // A regular sample without pads is R runs, each sorted by (phi, tag), in
-    // block order; every tag of a block is below every tag of the next, so a
-    // stable sort by phi alone leaves equal phi in tag order: the tag bytes
-    // need no passes.  (A pad's tag exceeds every key's, so pads break this.)
-    const int phi_only = p.sampling == BSPS_REGULAR && p.n == p.R * p.M;
-    lsd_plan_kernel<K><<<1, 256, 0, c.stream>>>(c.ly.lsd_hist, p.sample_size, c.ly.lsd_table, phi_only);
-    if constexpr (sizeof(K) == 4) {
-        if (msd_sample_sort(p)) {
-            e = p.sample_size > kMsdWideSample ? launch_msd<13>(c, b, hist_blocks) : launch_msd<12>(c, b, hist_blocks);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    const unsigned tiles = (unsigned)p.lsd_tiles;
-    const size_t dsm = lsd_downsweep_smem<K>() + 16;
+static int sm_count() {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned lsd_grid = (unsigned)std::min<int64_t>(p.lsd_tiles, 2 * (int64_t)std::max(sms, 1));
-    e = cudaFuncSetAttribute(lsd_downsweep_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm);
-    if (e != cudaSuccess) return e;
-    for (int pass = 0; pass < NPOS && tiles > 0; ++pass) {
-        lsd_upsweep_kernel<K><<<lsd_grid, kLsdThreads, 0, c.stream>>>(b, p.sample_size, pass, c.ly.lsd_table,
-                                                                     c.ly.lsd_counts, p.lsd_tiles);
-        lsd_scan_kernel<<<256, 256, 0, c.stream>>>(c.ly.lsd_counts, p.lsd_tiles, pass, c.ly.lsd_table,
-                                                   c.ly.lsd_hist);
-        lsd_downsweep_kernel<K><<<lsd_grid, kLsdThreads, dsm, c.stream>>>(b, p.sample_size, pass,
-                                                                         c.ly.lsd_table, c.ly.lsd_counts,
-                                                                         p.lsd_tiles);
+    return std::max(sms, 1);
+}
+
+template <typename K> static RecordBuffers<K> buffers_of(const Ctx &c) {
+    RecordBuffers<K> b;
+    b.phi[0] = (K *)c.ly.sphi[0];
+    b.phi[1] = (K *)c.ly.sphi[1];
+    b.tag[0] = c.ly.stag[0];
+    b.tag[1] = c.ly.stag[1];
+    return b;
+}
+
+template <typename K> static void sort_args(const Ctx &c, SortArgs<K> &a) {
+    a.b = buffers_of<K>(c);
+    a.S = c.pl.sample_size;
+    a.bins = pivot_bins(a.S);
+    a.cand = pivot_candidates(a.bins);
+    a.sc = PivotScratch<K>(c.ly.pivots, a.bins);
+}
+
+// The shape that sorts a bin (its mean is 2 S / bins records, twice that fits
+// the stage), and the tiles of the scatter: 2K records until there are enough
+// of 4K to fill the GPU.
+static int bins_shape(int64_t S, int key_bytes) {
+    if (key_bytes == 8) return kCountRecord;
+    const int64_t half = S / pivot_bins(S);
+    return half <= 700 ? kCountSmall : half <= 2000 ? kCountMedium : kCountLarge;
+}
+static int scatter_items(int64_t S) { return S < (1 << 20) ? 4 : 8; }
+
+template <typename K, int SIZE> static cudaError_t launch_sample_bins(Exec &x) {
+    using CS = typename CountShape<SIZE>::template Sort<typename RecordSink<K>::K>;
+    return launch_calls<SortArgs<K>>(x, sample_bins_kernel<K, SIZE, false>, sample_bins_kernel<K, SIZE, true>,
+                                     CountShape<SIZE>::T, CS::smem_bytes(), [](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample || bins_shape(c.pl.sample_size, sizeof(K)) != SIZE) return 0u;
+        sort_args(c, a);
+        return (uint32_t)a.bins;
+    });
+}
+
+template <typename K, int ITEMS> static cudaError_t launch_sample_scatter(Exec &x, int bins) {
+    const int64_t wave = 2 * sm_count();
+    return launch_calls<SortArgs<K>>(x, sample_scatter_kernel<K, ITEMS, false>, sample_scatter_kernel<K, ITEMS, true>,
+                                     kPivotThreads, pivot_scatter_smem<K, ITEMS>(bins), [=](const Ctx &c, SortArgs<K> &a) {
+        const int64_t S = c.pl.sample_size, tile = (int64_t)kPivotThreads * ITEMS;
+        if (S <= kOneSample || scatter_items(S) != ITEMS) return 0u;
+        sort_args(c, a);
+        return (uint32_t)imin64((S + tile - 1) / tile, wave);
+    });
+}
+
+template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
+    // shared memory: for the largest sample among the calls
+    int64_t one = 0, most = 0;
+    for (int i = 0; i < x.count; ++i) {
+        const int64_t S = x.calls[i].pl.sample_size;
+        if (S <= kOneSample) one = imax64(one, S);
+        else most = imax64(most, S);
     }
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (one > 0)
+        e = launch_calls<SortArgs<K>>(x, sample_one_kernel<K, false>, sample_one_kernel<K, true>, kOneThreads,
+                                      one_smem<K>((int)one), [](const Ctx &c, SortArgs<K> &a) {
+            if (c.pl.sample_size == 0 || c.pl.sample_size > kOneSample) return 0u;
+            a.b = buffers_of<K>(c);
+            a.S = c.pl.sample_size;
+            return 1u;
+        });
+    if (e != cudaSuccess || most == 0) return e;
+    const int bins = pivot_bins(most);
+    e = launch_calls<SortArgs<K>>(x, sample_pivots_kernel<K, false>, sample_pivots_kernel<K, true>, kOneThreads,
+                                  one_smem<K>(pivot_candidates(bins)) + (size_t)bins * sizeof(K),
+                                  [](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample) return 0u;
+        sort_args(c, a);
+        return 1u;
+    });
+    if (e != cudaSuccess) return e;
+    const int64_t wave = 2 * sm_count();
+    e = launch_calls<SortArgs<K>>(x, sample_hist_kernel<K, false>, sample_hist_kernel<K, true>, kPivotThreads,
+                                  pivot_smem<K>(bins), [=](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample) return 0u;
+        sort_args(c, a);
+        return (uint32_t)imin64(wave, (a.S + 4 * kPivotThreads - 1) / (4 * kPivotThreads));
+    });
+    if (e == cudaSuccess) e = launch_sample_scatter<K, 4>(x, bins);
+    if (e == cudaSuccess) e = launch_sample_scatter<K, 8>(x, bins);
+    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(K) == 8) {
+        return launch_sample_bins<K, kCountRecord>(x);
+    } else {
+        e = launch_sample_bins<K, kCountSmall>(x);
+        if (e == cudaSuccess) e = launch_sample_bins<K, kCountMedium>(x);
+        if (e == cudaSuccess) e = launch_sample_bins<K, kCountLarge>(x);
+        return e;
+    }
 }
 
-bool msd_sample_sort(const Plan &p) {
-    // large samples of 32-bit keys; the tile counts double as the MSD scratch
-    const int64_t need = p.sample_size > kMsdWideSample ? Msd<13>::kCursor + Msd<13>::kBins
-                                                        : Msd<12>::kCursor + Msd<12>::kBins;
-    return p.key_bytes == 4 && p.sample_size >= kMsdMinSample && std::max<int64_t>(p.lsd_tiles, 1) * 256 >= need;
+cudaError_t launch_sample_sort(Exec &x) {
+    return x.calls[0].pl.key_bytes == 8 ? launch_sample_sort_t<uint64_t>(x) : launch_sample_sort_t<uint32_t>(x);
 }
 
-cudaError_t launch_sample_sort(const Ctx &c) {
-    if (c.pl.key_bytes == 8) return launch_sample_sort_t<uint64_t>(c, lsd_buffers<BSPS_F64>(c));
-    return launch_sample_sort_t<uint32_t>(c, lsd_buffers<BSPS_U32>(c));
+template <typename K> static cudaError_t launch_splitters_t(Exec &x) {
+    return launch_calls<SplitterArgs<K>>(x, splitter_kernel<K, false>, splitter_kernel<K, true>, 256, 0,
+                                         [](const Ctx &c, SplitterArgs<K> &a) {
+        const Plan &p = c.pl;
+        const RecordBuffers<K> b = buffers_of<K>(c);
+        const int fin = sample_final(p);
+        a = {b.phi[fin], b.tag[fin], p.P, p.Q, p.B, (K *)c.ly.vphi, c.ly.vtag, (LutParams<K> *)c.ly.lutp, c.ly.lut, p.lut_bits, 0};
+        return (uint32_t)((imax64(p.P, (1 << p.lut_bits) + 1) + 255) / 256);
+    });
 }
 
-template <typename K> static cudaError_t launch_splitters_t(const Ctx &c, LsdBuffers<K> b) {
-    const Plan &p = c.pl;
-    const int npos = 4 + (int)sizeof(K);
-    const int64_t nthreads = imax64(p.P - 1, 1);
-    splitter_kernel<K><<<(unsigned)((nthreads + 255) / 256), 256, 0, c.stream>>>(
-        b, c.ly.lsd_table, npos, p.P, p.Q, p.B, (K *)c.ly.vphi, c.ly.vtag, (LutParams<K> *)c.ly.lutp);
-    lut_kernel<K><<<(kLutCells + 1 + 255) / 256, 256, 0, c.stream>>>((const K *)c.ly.vphi,
-                                                                     (const LutParams<K> *)c.ly.lutp,
-                                                                     c.ly.lut);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_splitters(const Ctx &c) {
-    if (c.pl.key_bytes == 8) return launch_splitters_t<uint64_t>(c, lsd_buffers<BSPS_F64>(c));
-    return launch_splitters_t<uint32_t>(c, lsd_buffers<BSPS_U32>(c));
+cudaError_t launch_splitters(Exec &x) {
+    return x.calls[0].pl.key_bytes == 8 ? launch_splitters_t<uint64_t>(x) : launch_splitters_t<uint32_t>(x);
 }
 
 template <int DT> static cudaError_t launch_debug_t(const Ctx &c) {
     using K = typename KeyTraits<DT>::T;
     const Plan &p = c.pl;
     const bool regular = p.sampling == BSPS_REGULAR;
-    LsdBuffers<K> b = lsd_buffers<DT>(c);
-    const int npos = 4 + (int)sizeof(K);
+    RecordBuffers<K> b = record_buffers<DT>(c);
     if (c.dbg.sample && p.sample_size > 0)
         sample_records_kernel<K><<<(unsigned)((p.sample_size + 255) / 256), 256, 0, c.stream>>>(
-            b, c.ly.lsd_table, npos, p.sample_size, p.n, p.m, p.M, regular, c.dbg.sample);
+            b, sample_final(p), p.sample_size, p.n, p.m, p.M, regular, c.dbg.sample);
     if (c.dbg.splitters && p.p > 1)
         splitter_records_kernel<K><<<(unsigned)((p.p + 255) / 256), 256, 0, c.stream>>>(
             (const K *)c.ly.vphi, c.ly.vtag, p.p, p.B, p.n, p.m, p.M, regular, c.dbg.splitters);

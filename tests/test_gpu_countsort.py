@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 
-from .gpu_util import assert_same, run_gpu
+from .gpu_util import assert_same, code_of, lib, run_gpu, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -21,9 +21,9 @@ def check(keys, p, s=0):
     same(run_gpu(keys, p, s, 0, oracle.RANDOM, 5, refine=1, debug=False), ref)
 
 
-# around a shape's stage (8192, 18944 and 38912 keys of 4 bytes, half of 8), one part more, 16-byte remainders
+# around a shape's stage (7680, 17408 and 37376 keys of 4 bytes, half of 8), one part more, 16-byte remainders
 @pytest.mark.parametrize("dt", [np.int32, np.float64])
-@pytest.mark.parametrize("n", [1, 2, 255, 1023, 4088, 4097, 8184, 8193, 9464, 9473, 18936, 18945, 38904, 38913, 77_817, 120_003])
+@pytest.mark.parametrize("n", [1, 2, 255, 1023, 3832, 3841, 7672, 7681, 8696, 8705, 17400, 17409, 37368, 37377, 74_745, 120_003])
 def test_one_bucket(n, dt):
     rng = np.random.default_rng(n)
     keys = rng.integers(-2**31, 2**31, n).astype(np.int32) if dt == np.int32 else rng.normal(0, 1, n)
@@ -32,7 +32,7 @@ def test_one_bucket(n, dt):
 
 # half-word stages: few units of 2^15 (2^31) values, one and two parts, most keys in one half of the bins,
 # windows over more than two units
-@pytest.mark.parametrize("n", [38_905, 65_001, 65_540, 77_816, 77_821, 150_000])
+@pytest.mark.parametrize("n", [37_369, 65_001, 65_540, 74_744, 74_749, 150_000])
 @pytest.mark.parametrize("span_log2", [16, 18, 21, 23])
 @pytest.mark.parametrize("shape", ["even", "low", "high", "gaps"])
 def test_half_word_stage(n, span_log2, shape):
@@ -91,3 +91,62 @@ def test_floats_around_zero(n):
     keys[::50], keys[1::50], keys[2::60], keys[3::60] = 0.0, -0.0, np.inf, -np.inf
     keys[4::70], keys[5::90] = np.nan, -np.float32(np.nan)
     check(keys, 2)
+
+
+# the sample sort (Fig. 1 step 5): around the one-CTA size, one and more records per bin of the larger form, tiles
+# of both sizes, keys that repeat (ties by tag) and skewed doubles; every record is compared
+@pytest.mark.parametrize("n, p, s", [(300, 3, 2), (9000, 1, 8193), (9000, 1, 8194), (20_000, 2, 4500), (60_000, 64, 1100), (50_000, 16, 70_000)])
+@pytest.mark.parametrize("kind", ["uniform", "few_values", "skewed_doubles"])
+def test_sample_sort(n, p, s, kind):
+    rng = np.random.default_rng(n)
+    if kind == "skewed_doubles":
+        keys = rng.choice([-700.0, 3.0, 512.5], n, p=[0.1, 0.2, 0.7]) + rng.normal(0, 1, n) * rng.choice([1e-9, 0.01, 50.0], n)
+    else:
+        keys = rng.integers(0, 5 if kind == "few_values" else 2**31, n).astype(np.int32)
+    ref = oracle.sort(keys, p, s, 0, oracle.RANDOM, seed=3, want_sample=True)
+    assert_same(run_gpu(keys, p, s, 0, oracle.RANDOM, 3), ref)
+
+
+def plain_call(keys, vals, p, s, **kw):
+    """bsps_sort_keys or bsps_sort_pairs (run_gpu goes through bsps_sort_debug)."""
+    import torch
+    bsps, n, code = lib(), len(keys), code_of(keys)
+    prm = bsps.make_params(p, s=s, sampling=bsps.BSPS_RANDOM, seed=9, **kw)
+    ws = torch.empty(bsps.bsps_workspace_size(n, code, prm, vals is not None), dtype=torch.uint8, device="cuda:0")
+    kin, sizes = to_dev(keys), torch.full((p,), -1, dtype=torch.int64, device="cuda:0")
+    out = torch.empty_like(kin)
+    if vals is None:
+        assert bsps.bsps_sort_keys(kin, out, n, code, prm, sizes, ws) == 0
+    else:
+        vin = to_dev(vals)
+        vout = torch.empty_like(vin)
+        assert bsps.bsps_sort_pairs(kin, vin, out, vout, n, code, prm, sizes, ws) == 0
+    st = bsps.bsps_read_stats(ws)
+    return (out.cpu().numpy().view(keys.dtype), None if vals is None else vout.cpu().numpy().view(np.uint32),
+            sizes.cpu().numpy(), st)
+
+
+# single calls of up to 2^14 keys run on chip in one launch (no diagnostics asked for): the shapes' ends, several
+# bucket counts and sample sizes, equal keys, payloads, and the status block, against the multi-kernel path's oracle
+@pytest.mark.parametrize("dt", [np.uint32, np.int32, np.float32])
+@pytest.mark.parametrize("n", [1, 2, 31, 600, 4095, 4096, 4097, 8192, 8193, 16_383, 16_384, 16_385])
+@pytest.mark.parametrize("p, s", [(1, 0), (3, 0), (16, 0), (256, 20), (5, 1)])
+def test_small_calls(n, p, s, dt):
+    rng = np.random.default_rng(n + p)
+    for few in (False, True):
+        keys = (rng.integers(0, 7, n) if few else rng.integers(0, 2**32, n)).astype(np.uint32).view(dt)
+        if dt == np.float32:
+            keys = rng.integers(0, 7, n).astype(np.float32) if few else rng.normal(0, 1, n).astype(np.float32)
+        vals = rng.integers(0, 2**32, n).astype(np.uint32)
+        for v in (None, vals):
+            ref = oracle.sort(keys, p, s, 0, oracle.RANDOM, seed=9, vals=v, want_sample=False)
+            out, vout, sizes, st = plain_call(keys, v, p, s)
+            assert out.tobytes() == ref.keys.tobytes() and np.array_equal(sizes, ref.bucket_sizes)
+            assert v is None or np.array_equal(vout, ref.vals)
+            assert (st.status, st.slow_buckets, st.max_bucket) == (0, 0, ref.bucket_sizes.max())
+
+
+def test_small_call_reports_overflow():
+    keys = np.random.default_rng(1).integers(0, 2**31, 10_000).astype(np.int32)
+    st = plain_call(keys, None, 8, 4, capacity_pct=50)[3]
+    assert (st.status, st.overflow) == (-4, 1)
