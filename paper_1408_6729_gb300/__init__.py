@@ -253,7 +253,12 @@ def bsps_mlp_predict(params, x, m, y, workspace, stream=None) -> int:
 
 
 def _offsets(offsets):
-    """Host int64 offsets (a sequence or numpy array) as a ctypes array."""
+    """Host int64 offsets as an argument: a contiguous numpy int64 array where it
+    lies, any other sequence as a ctypes array."""
+    flags = getattr(offsets, "flags", None)
+    if flags is not None and getattr(offsets, "ndim", 0) == 1 and offsets.dtype == "int64" and flags.c_contiguous \
+            and flags.aligned and offsets.dtype.isnative and len(offsets):
+        return offsets.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), len(offsets) - 1
     vals = [int(v) for v in offsets]
     return (ctypes.c_int64 * max(1, len(vals)))(*vals), len(vals) - 1
 
