@@ -12,7 +12,9 @@
 namespace bsps {
 
 constexpr int kMlpThreads = 128;       // one training point per thread per step
-constexpr int kMlpMaxPoints = kMlpPointsMax;
+constexpr int kMlpRow = kH + 4;        // floats of a point's row in shared memory
+constexpr int kMlpParamsPad = (kParams + 3) / 4 * 4;
+static_assert(kMlpThreads == 4 * kH, "the sums' split over the threads");
 // Full-batch gradient descent on all 1153 parameters from the (balanced)
 // spline start, with backtracking: each step goes from the best parameters
 // so far along their negative gradient; a step that lowers the loss is kept
@@ -28,31 +30,38 @@ constexpr int kMlpTrainPoints = 4096;  // training points drawn from the sorted 
 // Writes the 1153 partial sums to `part` and returns the partial loss sum.
 __device__ float mlp_cta_grad(const float *w, const float *__restrict__ x, const float *__restrict__ y, int64_t p0,
                               int np, int64_t m, float *part, float *scratch) {
-    // scratch: h1[kMlpThreads][33], dz2[kMlpThreads][33], dz1[kMlpThreads][33], h2[..][33], xs, dy
+    // scratch: h1, dz2, dz1, h2 [kMlpThreads][kMlpRow], x, dy, losses.  Rows of
+    // 36 floats: 16-byte accesses by consecutive threads meet distinct banks.
     float *sh1 = scratch;
-    float *sdz2 = sh1 + kMlpThreads * 33;
-    float *sdz1 = sdz2 + kMlpThreads * 33;
-    float *sh2 = sdz1 + kMlpThreads * 33;
-    float *sx = sh2 + kMlpThreads * 33;
+    float *sdz2 = sh1 + kMlpThreads * kMlpRow;
+    float *sdz1 = sdz2 + kMlpThreads * kMlpRow;
+    float *sh2 = sdz1 + kMlpThreads * kMlpRow;
+    float *sx = sh2 + kMlpThreads * kMlpRow;
     float *sdy = sx + kMlpThreads;
     float *sloss = sdy + kMlpThreads;
     const int t = threadIdx.x;
     float lossp = 0.0f;
     if (t < np) {
         const float xi = x[p0 + t];
-        float z1[kH], h1[kH], z2[kH];
+        float h1[kH];
 #pragma unroll
-        for (int j = 0; j < kH; ++j) {
-            z1[j] = fmaf(w[kW1 + j], xi, w[kB1 + j]);
-            h1[j] = fmaxf(z1[j], 0.0f);
-        }
+        for (int j = 0; j < kH; ++j) h1[j] = fmaxf(fmaf(w[kW1 + j], xi, w[kB1 + j]), 0.0f);
+#pragma unroll
+        for (int j = 0; j < kH; j += 4)
+            *reinterpret_cast<float4 *>(sh1 + t * kMlpRow + j) = make_float4(h1[j], h1[j + 1], h1[j + 2], h1[j + 3]);
         float out = w[kB3];
-        for (int i = 0; i < kH; ++i) {
-            float z = w[kB2 + i];
+#pragma unroll 1
+        for (int i = 0; i < kH; i += 4) {  // four units of layer 2 at a time
+            float z[4];
 #pragma unroll
-            for (int j = 0; j < kH; ++j) z = fmaf(w[kW2 + i * kH + j], h1[j], z);
-            z2[i] = z;
-            out = fmaf(w[kW3 + i], fmaxf(z, 0.0f), out);
+            for (int q = 0; q < 4; ++q) {
+                z[q] = w[kB2 + i + q];
+#pragma unroll
+                for (int j = 0; j < kH; ++j) z[q] = fmaf(w[kW2 + (i + q) * kH + j], h1[j], z[q]);
+                z[q] = fmaxf(z[q], 0.0f);
+                out = fmaf(w[kW3 + i + q], z[q], out);
+            }
+            *reinterpret_cast<float4 *>(sh2 + t * kMlpRow + i) = make_float4(z[0], z[1], z[2], z[3]);
         }
         const float r = out - y[p0 + t];
         lossp = r * r;
@@ -60,40 +69,74 @@ __device__ float mlp_cta_grad(const float *w, const float *__restrict__ x, const
         float dz1[kH];
 #pragma unroll
         for (int j = 0; j < kH; ++j) dz1[j] = 0.0f;
-        for (int i = 0; i < kH; ++i) {
-            const float d2 = z2[i] > 0.0f ? dy * w[kW3 + i] : 0.0f;
-            sdz2[t * 33 + i] = d2;
-            sh2[t * 33 + i] = fmaxf(z2[i], 0.0f);
+#pragma unroll 1
+        for (int i = 0; i < kH; i += 4) {
+            const float4 h2 = *reinterpret_cast<const float4 *>(sh2 + t * kMlpRow + i);
+            const float on[4] = {h2.x, h2.y, h2.z, h2.w};
+            float d2[4];
 #pragma unroll
-            for (int j = 0; j < kH; ++j) dz1[j] = fmaf(d2, w[kW2 + i * kH + j], dz1[j]);
+            for (int q = 0; q < 4; ++q) {
+                d2[q] = on[q] > 0.0f ? dy * w[kW3 + i + q] : 0.0f;
+#pragma unroll
+                for (int j = 0; j < kH; ++j) dz1[j] = fmaf(d2[q], w[kW2 + (i + q) * kH + j], dz1[j]);
+            }
+            *reinterpret_cast<float4 *>(sdz2 + t * kMlpRow + i) = make_float4(d2[0], d2[1], d2[2], d2[3]);
         }
 #pragma unroll
-        for (int j = 0; j < kH; ++j) {
-            sh1[t * 33 + j] = h1[j];
-            sdz1[t * 33 + j] = z1[j] > 0.0f ? dz1[j] : 0.0f;
-        }
+        for (int j = 0; j < kH; ++j) dz1[j] = fmaf(w[kW1 + j], xi, w[kB1 + j]) > 0.0f ? dz1[j] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kH; j += 4)
+            *reinterpret_cast<float4 *>(sdz1 + t * kMlpRow + j) = make_float4(dz1[j], dz1[j + 1], dz1[j + 2], dz1[j + 3]);
         sx[t] = xi;
         sdy[t] = dy;
     }
     __syncthreads();
-    // sums over the CTA's points, one or more parameters per thread
-    for (int k = t; k < kParams; k += kMlpThreads) {
-        float g = 0.0f;
-        if (k < kB1) {                     // W1[j] = sum dz1[j] * x
-            for (int p = 0; p < np; ++p) g = fmaf(sdz1[p * 33 + k], sx[p], g);
-        } else if (k < kW2) {              // b1[j] = sum dz1[j]
-            for (int p = 0; p < np; ++p) g += sdz1[p * 33 + (k - kB1)];
-        } else if (k < kB2) {              // W2[i][j] = sum dz2[i] * h1[j]
-            const int i = (k - kW2) / kH, j = (k - kW2) % kH;
-            for (int p = 0; p < np; ++p) g = fmaf(sdz2[p * 33 + i], sh1[p * 33 + j], g);
-        } else if (k < kW3) {              // b2[i] = sum dz2[i]
-            for (int p = 0; p < np; ++p) g += sdz2[p * 33 + (k - kB2)];
-        } else if (k < kB3) {              // w3[i] = sum dy * h2[i]
-            for (int p = 0; p < np; ++p) g = fmaf(sdy[p], sh2[p * 33 + (k - kW3)], g);
-        } else {                           // b3 = sum dy
-            for (int p = 0; p < np; ++p) g += sdy[p];
+    // sums over the CTA's points, each parameter's in the points' order.  W2:
+    // a thread takes a tile of 2 x 4, two loads a point for eight sums.
+    {
+        const int i = (t >> 3) * 2, j = (t & 7) * 4;
+        float g[2][4] = {};
+#pragma unroll 4
+        for (int p = 0; p < np; ++p) {  // W2[i][j] = sum dz2[i] * h1[j]
+            const float2 d = *reinterpret_cast<const float2 *>(sdz2 + p * kMlpRow + i);
+            const float4 h = *reinterpret_cast<const float4 *>(sh1 + p * kMlpRow + j);
+            g[0][0] = fmaf(d.x, h.x, g[0][0]); g[0][1] = fmaf(d.x, h.y, g[0][1]);
+            g[0][2] = fmaf(d.x, h.z, g[0][2]); g[0][3] = fmaf(d.x, h.w, g[0][3]);
+            g[1][0] = fmaf(d.y, h.x, g[1][0]); g[1][1] = fmaf(d.y, h.y, g[1][1]);
+            g[1][2] = fmaf(d.y, h.z, g[1][2]); g[1][3] = fmaf(d.y, h.w, g[1][3]);
         }
-        part[k] = g;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            part[kW2 + i * kH + j + q] = g[0][q];
+            part[kW2 + (i + 1) * kH + j + q] = g[1][q];
+        }
+    }
+    {   // the vectors, one entry a thread: W1[k], b1[k], b2[k], w3[k]
+        const int k = t & 31, which = t >> 5;
+        float g = 0.0f;
+        if (which == 0) {
+#pragma unroll 8
+            for (int p = 0; p < np; ++p) g = fmaf(sdz1[p * kMlpRow + k], sx[p], g);
+            part[kW1 + k] = g;
+        } else if (which == 1) {
+#pragma unroll 8
+            for (int p = 0; p < np; ++p) g += sdz1[p * kMlpRow + k];
+            part[kB1 + k] = g;
+        } else if (which == 2) {
+#pragma unroll 8
+            for (int p = 0; p < np; ++p) g += sdz2[p * kMlpRow + k];
+            part[kB2 + k] = g;
+        } else {
+#pragma unroll 8
+            for (int p = 0; p < np; ++p) g = fmaf(sdy[p], sh2[p * kMlpRow + k], g);
+            part[kW3 + k] = g;
+        }
+        if (t == 0) {
+            g = 0.0f;
+#pragma unroll 8
+            for (int p = 0; p < np; ++p) g += sdy[p];
+            part[kB3] = g;
+        }
     }
     // partial loss
     float l = lossp;
@@ -107,13 +150,14 @@ __device__ float mlp_cta_grad(const float *w, const float *__restrict__ x, const
     return tot;
 }
 
-constexpr int kMlpScratchFloats = 4 * kMlpThreads * 33 + 2 * kMlpThreads + 8;
+constexpr int kMlpScratchFloats = 4 * kMlpThreads * kMlpRow + 2 * kMlpThreads + 8;
+constexpr size_t kMlpSmem = (kMlpScratchFloats + kMlpParamsPad) * sizeof(float);
 
 // Loss and gradient only (for the gradient check against the CPU oracle).
 __global__ void __launch_bounds__(kMlpThreads) mlp_grad_kernel(const float *params, const float *x, const float *y,
                                                                int64_t m, float *part) {
-    __shared__ float w[kParams + 3];
-    __shared__ float scratch[kMlpScratchFloats];
+    extern __shared__ __align__(16) float mlp_smem[];
+    float *w = mlp_smem, *scratch = mlp_smem + kMlpParamsPad;
     for (int k = threadIdx.x; k < kParams; k += kMlpThreads) w[k] = params[k];
     __syncthreads();
     const int64_t p0 = (int64_t)blockIdx.x * kMlpThreads;
@@ -123,9 +167,15 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_grad_kernel(const float *para
     if (threadIdx.x == 0) pp[kParams] = lp;
 }
 
-// One training step's partial gradients: as mlp_grad_kernel, with the point
-// count read from the device (CTAs past it contribute zeros).
-struct MlpOpt;
+// Descent state: the best parameters, their loss and gradient, the step size.
+struct MlpOpt {
+    float best[kParams], grad[kParams], start[kParams];
+    float best_loss, eta;
+    unsigned ticket;  // CTAs of the current step that have finished
+};
+// the descent state, then (16-byte aligned) the scratch of the evaluation form
+static size_t mlp_scratch_offset() { return (sizeof(MlpOpt) + 15) & ~size_t(15); }
+
 struct MlpPieceScratch;
 struct MlpStepArgs {
     float *params;
@@ -134,73 +184,93 @@ struct MlpStepArgs {
     float *part;  // G partial gradients and losses
     MlpOpt *opt;
     float *loss_first, *loss_last;
-    int32_t G, step, last, pad_;
+    int32_t step, last;
 };
-template <bool MANY>
-__global__ void __launch_bounds__(kMlpThreads) mlp_step_grad_kernel(const Many<MlpStepArgs> many) {
+
+// One training step.  Every CTA writes the partial gradient of its points at
+// the current parameters (CTAs past the point count, zeros).  The last CTA to
+// finish sums them and their losses; keeps the parameters as the best if their
+// loss is the lowest so far (the step size grows) or drops them (it shrinks);
+// then, unless `last`, sets them to the next trial, best - eta * grad(best).
+// After the last evaluation the best parameters are written back.
+template <bool MANY> __global__ void __launch_bounds__(kMlpThreads) mlp_step_kernel(const Many<MlpStepArgs> many) {
     const Pick<MANY, MlpStepArgs> pk(many);
-    const float *params = pk.a.params, *x = pk.a.x, *y = pk.a.y;
-    const int64_t *npts = pk.a.npts;
-    float *part = pk.a.part;
-    __shared__ float w[kParams + 3];
-    __shared__ float scratch[kMlpScratchFloats];
-    for (int k = threadIdx.x; k < kParams; k += kMlpThreads) w[k] = params[k];
+    const MlpStepArgs &A = pk.a;
+    extern __shared__ __align__(16) float mlp_smem[];
+    float *w = mlp_smem, *scratch = mlp_smem + kMlpParamsPad;
+    __shared__ float s_loss, s_red[kMlpThreads / 32];
+    __shared__ int s_flag;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, G = (int)pk.blocks;
+    float *params = A.params;
+    const float *part = A.part;
+    MlpOpt *opt = A.opt;
+    const int64_t m = *A.npts;
+    for (int k = t; k < kParams; k += kMlpThreads) w[k] = params[k];
     __syncthreads();
-    const int64_t m = *npts;
-    const int64_t p0 = (int64_t)pk.block * kMlpThreads;
-    float *pp = part + (int64_t)pk.block * (kParams + 1);
-    if (p0 >= m) {
-        for (int k = threadIdx.x; k <= kParams; k += kMlpThreads) pp[k] = 0.0f;
-        return;
+    {
+        const int64_t p0 = (int64_t)pk.block * kMlpThreads;
+        float *pp = A.part + (int64_t)pk.block * (kParams + 1);
+        if (p0 >= m) {
+            for (int k = t; k <= kParams; k += kMlpThreads) pp[k] = 0.0f;
+        } else {
+            const float lp = mlp_cta_grad(w, A.x, A.y, p0, (int)imin64(kMlpThreads, m - p0), m, pp, scratch);
+            if (t == 0) pp[kParams] = lp;
+        }
     }
-    const int np = (int)imin64(kMlpThreads, m - p0);
-    const float lp = mlp_cta_grad(w, x, y, p0, np, m, pp, scratch);
-    if (threadIdx.x == 0) pp[kParams] = lp;
-}
-
-// Descent state: the best parameters, their loss and gradient, the step size.
-struct MlpOpt {
-    float best[kParams], grad[kParams], start[kParams];
-    float best_loss, eta;
-};
-// the descent state, then (16-byte aligned) the scratch of the evaluation form
-static size_t mlp_scratch_offset() { return (sizeof(MlpOpt) + 15) & ~size_t(15); }
-
-// Sums the G partial gradients and losses of the current parameters; keeps
-// them as the best if their loss is the lowest so far (the step size grows)
-// or drops them (it shrinks); then, unless `last`, sets the parameters to the
-// next trial, best - eta * grad(best).  After the last evaluation the best
-// parameters are written back.
-template <bool MANY> __global__ void __launch_bounds__(1024) mlp_descent_kernel(const Many<MlpStepArgs> many) {
-    const Pick<MANY, MlpStepArgs> pk(many);
-    float *params = pk.a.params;
-    const float *part = pk.a.part;
-    const int64_t *npts = pk.a.npts;
-    MlpOpt *opt = pk.a.opt;
-    const int G = pk.a.G, step = pk.a.step, last = pk.a.last;
-    float *loss_first = pk.a.loss_first, *loss_last = pk.a.loss_last;
-    __shared__ float s_loss, s_red[32];
-    __shared__ int s_keep;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t m = *npts;
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_flag = atomicAdd(&opt->ticket, 1u) == (unsigned)G - 1;
+    __syncthreads();
+    if (!s_flag) return;
+    __threadfence();
+    if (t == 0) opt->ticket = 0;
     if (m == 0) return;
-    if (t == 0) {
+    // the losses in the CTAs' order
+    if (warp == 0) {
         float l = 0.0f;
-        for (int c = 0; c < G; ++c) l += part[(int64_t)c * (kParams + 1) + kParams];
-        s_loss = l / (float)m;
-        s_keep = step == 0 || s_loss < opt->best_loss;
+        for (int c0 = 0; c0 < G; c0 += 32) {
+            const float v = c0 + lane < G ? __ldcg(part + (int64_t)(c0 + lane) * (kParams + 1) + kParams) : 0.0f;
+            for (int c = 0; c < 32 && c0 + c < G; ++c) l += __shfl_sync(0xffffffffu, v, c);
+        }
+        if (lane == 0) {
+            s_loss = l / (float)m;
+            s_flag = A.step == 0 || s_loss < opt->best_loss;
+        }
     }
     __syncthreads();
-    const bool keep = s_keep;
+    const bool keep = s_flag;
     float g2 = 0.0f;
-    for (int k = t; k < kParams; k += 1024) {
-        if (step == 0) opt->start[k] = params[k];
-        if (keep) {
-            float g = 0.0f;
-            for (int c = 0; c < G; ++c) g += part[(int64_t)c * (kParams + 1) + k];
-            opt->best[k] = params[k];
-            opt->grad[k] = g;
-            g2 = fmaf(g, g, g2);
+    if (A.step == 0)
+        for (int k = t; k < kParams; k += kMlpThreads) opt->start[k] = w[k];
+    if (keep) {
+        // three parameters of a thread at a time, sixteen partial sums of each
+        // in flight, added in the CTAs' order
+        constexpr int KB = 3;
+        for (int k0 = t; k0 < kParams; k0 += KB * kMlpThreads) {
+            float g[KB] = {};
+            for (int c0 = 0; c0 < G; c0 += 16) {
+                float v[KB][16];
+#pragma unroll
+                for (int q = 0; q < KB; ++q)
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        v[q][c] = c0 + c < G && k0 + q * kMlpThreads < kParams
+                                      ? __ldcg(part + (int64_t)(c0 + c) * (kParams + 1) + k0 + q * kMlpThreads) : 0.0f;
+#pragma unroll
+                for (int q = 0; q < KB; ++q)
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        if (c0 + c < G) g[q] += v[q][c];
+            }
+#pragma unroll
+            for (int q = 0; q < KB; ++q) {
+                const int k = k0 + q * kMlpThreads;
+                if (k < kParams) {
+                    opt->best[k] = w[k];
+                    opt->grad[k] = g[q];
+                    g2 = fmaf(g[q], g[q], g2);
+                }
+            }
         }
     }
     // |grad|^2 for the first step size
@@ -209,21 +279,21 @@ template <bool MANY> __global__ void __launch_bounds__(1024) mlp_descent_kernel(
     if (lane == 0) s_red[warp] = g2;
     __syncthreads();
     if (t == 0) {
-        if (step == 0) {
+        if (A.step == 0) {
             float tot = 0.0f;
-            for (int w = 0; w < 32; ++w) tot += s_red[w];
+            for (int q = 0; q < kMlpThreads / 32; ++q) tot += s_red[q];
             opt->eta = tot > 0.0f ? kMlpFirst * s_loss / tot : 0.0f;
-            if (loss_first) *loss_first = s_loss;
+            if (A.loss_first) *A.loss_first = s_loss;
         } else {
             opt->eta *= keep ? kMlpGrow : kMlpShrink;
         }
         if (keep) opt->best_loss = s_loss;
-        if (last && loss_last) *loss_last = opt->best_loss;
+        if (A.last && A.loss_last) *A.loss_last = opt->best_loss;
     }
     __syncthreads();
     const float eta = opt->eta;
-    for (int k = t; k < kParams; k += 1024)
-        params[k] = last ? opt->best[k] : opt->best[k] - eta * opt->grad[k];
+    for (int k = t; k < kParams; k += kMlpThreads)
+        params[k] = A.last ? opt->best[k] : opt->best[k] - eta * opt->grad[k];
 }
 
 // The piecewise-linear form of the network `params` (see MlpTables), in
@@ -266,21 +336,25 @@ template <bool MANY> __global__ void __launch_bounds__(32) mlp_pieces_kernel(con
     __shared__ double cutd[kH + 1];
     __shared__ int nk;
     const double INF = __longlong_as_double(0x7ff0000000000000ll);
-    if (lane == 0) {
-        int c = 0;
+    {
+        // the knots in order (equal ones by unit): each lane counts those before its own
+        const double w = params[kW1 + lane];
+        const double v = w != 0.0 ? -(double)params[kB1 + lane] / w : 0.0;
+        const uint32_t real = __ballot_sync(0xffffffffu, w != 0.0);
+        int rank = 0;
+#pragma unroll
         for (int j = 0; j < kH; ++j) {
-            const double w = params[kW1 + j];
-            if (w != 0.0) {  // insertion into the sorted list
-                const double v = -(double)params[kB1 + j] / w;
-                int q = c++;
-                while (q > 0 && knots[q - 1] > v) { knots[q] = knots[q - 1]; --q; }
-                knots[q] = v;
-            }
+            const double vj = __shfl_sync(0xffffffffu, v, j);
+            // (NaN, which no training gives, after every number)
+            rank += (real >> j & 1u) && (vj < v || (vj == v && j < lane) || (v != v && (vj == vj || j < lane)));
         }
-        nk = c;
-        if (k == 0) {
-            S.nk = c;
-            for (int j = 0; j < c; ++j) S.knots[j] = knots[j];
+        if (w != 0.0) {
+            knots[rank] = v;
+            if (k == 0) S.knots[rank] = v;
+        }
+        if (lane == 0) {
+            nk = __popc(real);
+            if (k == 0) S.nk = __popc(real);
         }
     }
     __syncwarp();
@@ -541,6 +615,7 @@ struct MlpPrepareArgs {
     MlpNorm *norm;
     float *x, *y, *params;
     int64_t *npts;
+    MlpOpt *opt;
 };
 template <int DT, bool MANY> __global__ void __launch_bounds__(256) mlp_prepare_kernel(const Many<MlpPrepareArgs> many) {
     using K = typename KeyTraits<DT>::T;
@@ -553,6 +628,7 @@ template <int DT, bool MANY> __global__ void __launch_bounds__(256) mlp_prepare_
     int64_t *npts_out = pk.a.npts;
     __shared__ int64_t s_real;
     if (threadIdx.x == 0) {
+        pk.a.opt->ticket = 0;
         int64_t lo = 0, hi = S;  // first pad record (tag >= n)
         while (lo < hi) {
             const int64_t mid = (lo + hi) / 2;
@@ -637,7 +713,7 @@ template <int DT> static cudaError_t launch_mlp_train_t(Exec &x) {
         if (!learned(c)) return 0u;
         const int fin = sample_final(c.pl);
         a = {c.ly.sphi[fin], c.ly.stag[fin], c.pl.sample_size, c.pl.n, c.ly.mlp_norm, c.ly.mlp_x, c.ly.mlp_y,
-             c.ly.mlp_params, c.ly.mlp_npts};
+             c.ly.mlp_params, c.ly.mlp_npts, reinterpret_cast<MlpOpt *>(c.ly.mlp_opt)};
         return 1u;
     };
     cudaError_t e = launch_calls<MlpPrepareArgs>(x, mlp_prepare_kernel<DT, false>, mlp_prepare_kernel<DT, true>, 256, 0, prepare);
@@ -647,19 +723,15 @@ template <int DT> static cudaError_t launch_mlp_train_t(Exec &x) {
     // of the current parameters, then the step (kMlpSteps trials after the
     // start's evaluation)
     for (int step = 0; step <= kMlpSteps && e == cudaSuccess; ++step) {
-        auto args = [=](const Ctx &c, MlpStepArgs &a) {
-            const int64_t max_pts = std::min<int64_t>(c.pl.sample_size, kMlpTrainPoints);
-            const int G = (int)std::max<int64_t>(1, (max_pts + kMlpThreads - 1) / kMlpThreads);
+        e = launch_calls<MlpStepArgs>(x, mlp_step_kernel<false>, mlp_step_kernel<true>, kMlpThreads, kMlpSmem,
+                                      [=](const Ctx &c, MlpStepArgs &a) {
+            if (!learned(c)) return 0u;
             float *loss = c.dbg.mlp_loss;
             a = {c.ly.mlp_params, c.ly.mlp_x, c.ly.mlp_y, c.ly.mlp_npts, c.ly.mlp_part, reinterpret_cast<MlpOpt *>(c.ly.mlp_opt),
-                 loss, loss ? loss + 1 : nullptr, G, step, step == kMlpSteps, 0};
-            return learned(c);
-        };
-        e = launch_calls<MlpStepArgs>(x, mlp_step_grad_kernel<false>, mlp_step_grad_kernel<true>, kMlpThreads, 0,
-                                      [=](const Ctx &c, MlpStepArgs &a) { return args(c, a) ? (uint32_t)a.G : 0u; });
-        if (e == cudaSuccess)
-            e = launch_calls<MlpStepArgs>(x, mlp_descent_kernel<false>, mlp_descent_kernel<true>, 1024, 0,
-                                          [=](const Ctx &c, MlpStepArgs &a) { return args(c, a) ? 1u : 0u; });
+                 loss, loss ? loss + 1 : nullptr, step, step == kMlpSteps};
+            const int64_t points = std::min<int64_t>(c.pl.sample_size, kMlpTrainPoints);
+            return (uint32_t)std::max<int64_t>(1, (points + kMlpThreads - 1) / kMlpThreads);
+        });
     }
     // the trained network in its evaluation form, and the index over the
     // splitters' outputs
@@ -687,7 +759,7 @@ template <int DT> static cudaError_t launch_mlp_train_t(Exec &x) {
     return e;
 }
 
-int mlp_train_kernels() { return 2 + 2 * (kMlpSteps + 1) + 4; }
+int mlp_train_kernels() { return 2 + (kMlpSteps + 1) + 4; }
 size_t mlp_opt_bytes() { return mlp_scratch_offset() + sizeof(MlpPieceScratch); }
 
 cudaError_t launch_mlp_train(Exec &x) {
@@ -719,7 +791,8 @@ extern "C" int bsps_mlp_loss_grad(const float *d_params, const float *d_x, const
     if (!d_ws || ws_bytes < need) return BSPS_ERR_WORKSPACE_TOO_SMALL;
     const int G = (int)((m + kMlpThreads - 1) / kMlpThreads);
     cudaStream_t s = (cudaStream_t)stream;
-    mlp_grad_kernel<<<G, kMlpThreads, 0, s>>>(d_params, d_x, d_y, m, (float *)d_ws);
+    if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem) != cudaSuccess) return BSPS_ERR_CUDA;
+    mlp_grad_kernel<<<G, kMlpThreads, kMlpSmem, s>>>(d_params, d_x, d_y, m, (float *)d_ws);
     mlp_grad_reduce_kernel<<<(kParams + 1 + 255) / 256, 256, 0, s>>>((const float *)d_ws, G, m, d_grad, d_loss);
     return cudaGetLastError() == cudaSuccess ? BSPS_OK : BSPS_ERR_CUDA;
 }

@@ -23,7 +23,9 @@ constexpr int kParams = kB3 + 1;  // 1153
 constexpr int kMlpPointsMax = 16384;    // training points taken from the sample
 constexpr int kMlpGridMax = 128;        // CTAs of the training launch (128 points each)
 
-// x = (value(key) - lo) * scale, value() the key's numeric value
+// x = (value(key) - lo) * scale, value() the key's numeric value.  (The
+// product is rounded here: were it fused into a later subtraction in one place
+// and not in another, a key and a splitter of equal value could differ.)
 struct MlpNorm {
     double lo;
     float scale;
@@ -31,10 +33,10 @@ struct MlpNorm {
 };
 
 template <int DT> __device__ __forceinline__ float mlp_input(typename KeyTraits<DT>::T bits, const MlpNorm &nm) {
-    if constexpr (DT == BSPS_U32) return ((float)bits - nm.lo_f) * nm.scale;
-    else if constexpr (DT == BSPS_I32) return ((float)(int32_t)bits - nm.lo_f) * nm.scale;
-    else if constexpr (DT == BSPS_F32) return (__uint_as_float(bits) - nm.lo_f) * nm.scale;
-    else return (float)(__longlong_as_double((long long)bits) - nm.lo) * nm.scale;
+    if constexpr (DT == BSPS_U32) return __fmul_rn((float)bits - nm.lo_f, nm.scale);
+    else if constexpr (DT == BSPS_I32) return __fmul_rn((float)(int32_t)bits - nm.lo_f, nm.scale);
+    else if constexpr (DT == BSPS_F32) return __fmul_rn(__uint_as_float(bits) - nm.lo_f, nm.scale);
+    else return __fmul_rn((float)(__longlong_as_double((long long)bits) - nm.lo), nm.scale);
 }
 
 template <int DT> __host__ __device__ __forceinline__ double key_value(typename KeyTraits<DT>::T bits) {
@@ -82,17 +84,22 @@ struct MlpTables {
     MlpNorm norm;
 };
 
-__device__ __forceinline__ float mlp_eval(const MlpTables &T, float x) {
-    // p = number of cut points <= x (a fixed-depth search)
-    int p = 0;
-    for (int st = T.npad >> 1; st >= 1; st >>= 1) p += T.cut[p + st - 1] <= x ? st : 0;
+// the network's output at x, which lies in piece p
+__device__ __forceinline__ float mlp_piece(const MlpTables &T, int p, float x) {
     const float4 pc = T.piece[p];
-    float y = fmaf(pc.z, x - pc.x, pc.y);
+    float y = fmaf(pc.z, __fsub_rn(x, pc.x), pc.y);
     if (T.monotone) {  // clamped to the piece's end values
         y = fminf(y, pc.w);
         if (p > 0) y = fmaxf(y, pc.y);  // piece 0 extends to -inf; its anchor is its right end
     }
     return y;
+}
+
+__device__ __forceinline__ float mlp_eval(const MlpTables &T, float x) {
+    // p = number of cut points <= x (a fixed-depth search)
+    int p = 0;
+    for (int st = T.npad >> 1; st >= 1; st >>= 1) p += T.cut[p + st - 1] <= x ? st : 0;
+    return mlp_piece(T, p, x);
 }
 
 // Cell of the index over the network's output y (an estimate of the key's
