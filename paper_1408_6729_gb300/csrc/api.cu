@@ -106,16 +106,18 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     // the routing kernel keeps two words per sub-bucket in shared memory:
     // refine less (larger sub-buckets go to the slower sort tiers) if needed,
     // and also while its splitters would have to stay in global memory, as
-    // long as the expected sub-bucket stays within 2.5 clusters' capacity
+    // long as the expected sub-bucket stays within 2.5 clusters' capacity (4 of
+    // 8-byte keys: routing reads splitters of a skewed key's cell again and
+    // again, and the bucket sort takes a larger sub-bucket in more parts)
     while (prm->refine == 0 && pl.B > 1 && route_smem_bytes(pl) > 227 * 1024) {
         pl.B /= 2;
         pl.P = pl.p * pl.B;
     }
-    while (prm->refine == 0 && pl.B > 1 && !pl.pairs && pl.key_bytes == 4 && !route_keys_splitters_in_smem(pl)) {
+    while (prm->refine == 0 && pl.B > 1 && !pl.pairs && !route_keys_splitters_in_smem(pl)) {
         Plan half = pl;
         half.B /= 2;
         half.P = half.p * half.B;
-        if ((double)n / half.P * headroom(half.B) > 2.5 * 8.0 * cap_cta) break;
+        if ((double)n / half.P * headroom(half.B) > (pl.key_bytes == 8 ? 4.0 : 2.5) * 8.0 * cap_cta) break;
         pl = half;
     }
     B = pl.B;
@@ -157,6 +159,8 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     if (!pairs && !pl.keep_runs && route_keys_fine_index(pl) &&
         pl.sample_size * pl.key_bytes >= ((1 << kLutBitsFine) + 2) * 2)
         pl.lut_bits = kLutBitsFine;
+
+    pl.pair_words = pairs && pl.key_bytes == 4 && !pl.keep_runs && pl.P <= kPairWordsMax;
 
     // workspace size
     int64_t o = 0;
@@ -382,9 +386,11 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
         if (!random) {
             BSPS_CUDA(cudaMemsetAsync(c.ly.status, 0, sizeof(DevStatus), c.stream));
             BSPS_CUDA(cudaMemsetAsync(c.ly.cursor, 0, (size_t)c.pl.P * 4, c.stream));
-            if (!c.pl.pairs) BSPS_CUDA(cudaMemsetAsync(c.ly.retry_flag, 0, (size_t)c.pl.P * 4, c.stream));
+            if (!c.pl.pairs || c.pl.pair_words) BSPS_CUDA(cudaMemsetAsync(c.ly.retry_flag, 0, (size_t)c.pl.P * 4, c.stream));
         }
-        if (c.pl.pairs && !c.pl.keep_runs)
+        // (the test hook of the bounded waits stalls a tile of the look-back routing)
+        const bool words = c.pl.pair_words && c.dbg.stall_tile == 0;
+        if (c.pl.pairs && !c.pl.keep_runs && !words)
             BSPS_CUDA(cudaMemsetAsync(c.ly.state, 0, (size_t)c.pl.tiles * c.pl.P * 4, c.stream));
         BSPS_CUDA(mark(0));
         BSPS_CUDA(random ? launch_sample_random(x) : launch_sample(c));
@@ -417,10 +423,10 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
                                             (size_t)c.pl.R * 4, (size_t)(c.pl.p + 1), cudaMemcpyDeviceToDevice,
                                             c.stream));
         } else {
-            BSPS_CUDA(c.pl.pairs ? launch_route(c) : launch_route_keys(x));
+            BSPS_CUDA(words ? launch_route_words(x) : c.pl.pairs ? launch_route(c) : launch_route_keys(x));
             BSPS_CUDA(launch_bucket_finish(x));
             BSPS_CUDA(mark(4));
-            BSPS_CUDA(bucket_sort());
+            BSPS_CUDA(words ? launch_pair_words(x) : bucket_sort());
         }
         BSPS_CUDA(mark(5));
     }

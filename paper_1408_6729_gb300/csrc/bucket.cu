@@ -56,7 +56,12 @@ bucket_sort_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
     K *buf = reinterpret_cast<K *>(smem_raw + ((sizeof(typename SS::Smem) + 15) & ~size_t(15)));
     uint32_t *slots = reinterpret_cast<uint32_t *>(buf + SS::CAP);
 
-    // the listed sub-buckets
+    // the listed sub-buckets (of a batch's calls: rarely any)
+    if constexpr (MANY) {
+        bool any = false;
+        for (int i = threadIdx.x; i < many.count; i += blockDim.x) any |= *many.all[i].only_count != 0;
+        if (!__syncthreads_or(any)) return;  // (every CTA of the grid alike)
+    }
     each_call<MANY>(many, [&](const BucketArgs<K> &a) {
     const int64_t nitems = *a.only_count, clusters = gridDim.x / CL;
     for (int64_t it = blockIdx.x / CL; it < nitems; it += clusters) {
@@ -164,6 +169,11 @@ __global__ void __launch_bounds__(kSlowThreads) bucket_slow_kernel(const Many<Bu
     __shared__ typename Rank::Smem rsm;
     __shared__ uint32_t hist[256], run[256], tmp[40];
     __shared__ K red[2];
+    if constexpr (MANY) {
+        bool any = false;
+        for (int i = threadIdx.x; i < many.count; i += blockDim.x) any |= many.all[i].st->slow_count != 0;
+        if (!__syncthreads_or(any)) return;
+    }
     each_call<MANY>(many, [&](const BucketArgs<K> &a) {
     const int nslow = a.st->slow_count;
     for (int idx = blockIdx.x; idx < nslow; idx += gridDim.x) {

@@ -53,6 +53,7 @@ struct Plan {
     int dup_off;       // keys compared by value alone (no tie-break by position)
     int merge;         // final step: merge of the sorted blocks' segments (Fig. 1 step 12)
     int seg_route;     // route by the sorted blocks' partition and segment copies (Fig. 1 steps 9-11)
+    int pair_words;    // pairs are routed and sorted as words phi << 32 | position
     int keep_runs;     // the block sorts keep the sorted blocks (merge or seg_route)
     uint64_t seed;
     int64_t B;         // refine: sub-buckets per bucket
@@ -143,6 +144,7 @@ cudaError_t launch_merge_buckets(const Ctx &c);   // gather + stable merge per b
 int merge_cluster(const Plan &pl);                // CTAs per bucket for a bound pl.cap (0: too large)
 int64_t merge_capacity(int cl);                   // keys a cluster of cl CTAs merges
 int64_t merge_runs_max();                         // largest R
+constexpr int64_t kPairWordsMax = 8192;           // largest P of pairs as words (index, splitters and a chunk on chip)
 constexpr int64_t kSegRouteRunsMax = 16384;       // largest R of the segment-copy route (shared memory)
 size_t route_keys_smem_bytes(const Plan &pl);
 bool route_keys_fine_index(const Plan &pl);           // ... and a radix index of 2^kLutBitsFine cells

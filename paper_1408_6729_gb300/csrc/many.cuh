@@ -129,6 +129,8 @@ cudaError_t launch_mlp_train(Exec &x);
 cudaError_t launch_route_keys(Exec &x);
 cudaError_t launch_bucket_finish(Exec &x);
 cudaError_t launch_bucket_keys(Exec &x);
+cudaError_t launch_route_words(Exec &x);     // single calls of 4-byte keys with payloads, as words
+cudaError_t launch_pair_words(Exec &x);      // ... and their final step (pairs.cu)
 cudaError_t launch_bucket_pairs(Exec &x);    // single calls
 
 // api.cu: a call's plan, checks and layout, and the path above for calls that

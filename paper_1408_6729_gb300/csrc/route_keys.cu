@@ -1,8 +1,9 @@
 // route_keys.cu -- classification and the routing permutation for keys
-// without payloads (Fig. 1 steps 9-11; Fig. 2 steps 9-11), in one pass.
+// without payloads (Fig. 1 steps 9-11; Fig. 2 steps 9-11), in one pass, and for
+// 4-byte keys with payloads as words phi << 32 | input position.
 //
 // Without payloads the order of keys inside a bucket is free (equal keys
-// cannot be told apart), so the per-bucket prefix of Fig. 1 step 9 need not
+// cannot be told apart; the words of pairs carry their order with them), so the per-bucket prefix of Fig. 1 step 9 need not
 // follow input order: every chunk of keys reserves its run in each bucket
 // region with one atomic on that bucket's cursor.  A chunk is loaded into
 // registers with 16-byte loads, each key is classified once (Fig. 2 step 9)
@@ -43,10 +44,13 @@ constexpr size_t kRkSmemBudget = 227 * 1024;  // splitters in shared memory up t
 // and a key reads one or two splitters.  The splitter tree reads more (skewed
 // keys crowd a few cells of the radix index) and keeps its splitters on chip
 // with chunks of 8K.
-template <typename K, bool LEARNED = false> constexpr int rk_items() {
-    return sizeof(K) == 8 ? (LEARNED ? 10 : 8) : (LEARNED ? 8 : 16);
+// With payloads (PAIRS) the words that move are twice the keys' size: 8K.
+template <typename K, bool LEARNED = false, bool PAIRS = false> constexpr int rk_items() {
+    return sizeof(K) == 8 ? (LEARNED ? 10 : 8) : (LEARNED || PAIRS ? 8 : 16);
 }
-template <typename K, bool LEARNED = false> constexpr int rk_chunk() { return kRkThreads * rk_items<K, LEARNED>(); }
+template <typename K, bool LEARNED = false, bool PAIRS = false> constexpr int rk_chunk() {
+    return kRkThreads * rk_items<K, LEARNED, PAIRS>();
+}
 
 template <typename K> struct RouteKeysArgs {
     const K *keys;
@@ -58,7 +62,7 @@ template <typename K> struct RouteKeysArgs {
     uint32_t P;
     int64_t chunks;
     uint32_t *cursor;   // keys routed so far per sub-bucket
-    K *reg_keys;
+    void *regions;      // keys, or words phi << 32 | position
     int64_t cap;
     DevStatus *st;
     const MlpTables *mlp_tables;  // learned classifier (nullable): the network's evaluation form
@@ -72,7 +76,7 @@ template <typename K> struct RouteKeysArgs {
 // splitters' phi (global memory, L1-cached, when they do not fit), two sets of
 // per-bucket counts, the non-empty buckets of a chunk with their starts and
 // region offsets, the run marks, and the chunk grouped by bucket.
-template <typename K, bool LEARNED> struct RouteKeysLayout {
+template <typename K, bool LEARNED, bool PAIRS = false> struct RouteKeysLayout {
     // Buckets a call may have: the bound bsps_get_plan documents (counters,
     // offsets, the index and a chunk with 16-bit bucket numbers in 227 KB; the
     // layout below needs less).  `fits` says whether the splitters fit, too.
@@ -95,7 +99,7 @@ template <typename K, bool LEARNED> struct RouteKeysLayout {
     size_t mlp, lut, sphi, cnt, dlt, heads, ord, stage, total;
     bool sphi_in_smem, two_counts;
     __host__ __device__ RouteKeysLayout(uint32_t P, int lut_bits) {
-        constexpr int CH = rk_chunk<K, LEARNED>();
+        constexpr int CH = rk_chunk<K, LEARNED, PAIRS>();
         for (int pass = 0; pass < 4; ++pass) {  // what many buckets leave no room for goes
             sphi_in_smem = pass < 2;
             two_counts = pass % 2 == 0;
@@ -112,7 +116,7 @@ template <typename K, bool LEARNED> struct RouteKeysLayout {
             dlt = take(sizeof(uint32_t) * P);
             heads = take(CH / 8);
             ord = take(CH / 32 * 2);
-            stage = take(sizeof(K) * CH);
+            stage = take((PAIRS ? 8 : sizeof(K)) * CH);
             total = o + 128;  // scan scratch
             if (total <= kRkSmemBudget - 512) break;  // (a batch's arguments are kept there, too)
         }
@@ -135,14 +139,17 @@ __device__ __forceinline__ uint64_t ld_shared_if(const uint64_t *p, bool take) {
     return v;
 }
 
-template <int DT, bool LEARNED, bool MANY>
+template <int DT, bool LEARNED, bool MANY, bool PAIRS = false>
 __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<RouteKeysArgs<typename KeyTraits<DT>::T>> many) {
     using K = typename KeyTraits<DT>::T;
     const Pick<MANY, RouteKeysArgs<K>> pk(many);
     const RouteKeysArgs<K> &a = pk.a;
-    constexpr int T = kRkThreads, IT = rk_items<K, LEARNED>(), CH = rk_chunk<K, LEARNED>(), V = 16 / (int)sizeof(K);
+    constexpr int T = kRkThreads, IT = rk_items<K, LEARNED, PAIRS>(), CH = rk_chunk<K, LEARNED, PAIRS>(),
+                  V = 16 / (int)sizeof(K);
+    using Word = typename std::conditional<PAIRS, uint64_t, K>::type;  // what moves
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const RouteKeysLayout<K, LEARNED> L(a.P, a.lut_bits);
+    const RouteKeysLayout<K, LEARNED, PAIRS> L(a.P, a.lut_bits);
+    Word *regions = reinterpret_cast<Word *>(a.regions);
     LutParams<K> &lps = *reinterpret_cast<LutParams<K> *>(smem_raw);
     MlpTables *mt = reinterpret_cast<MlpTables *>(smem_raw + L.mlp);
     uint16_t *lut = reinterpret_cast<uint16_t *>(smem_raw + L.lut);
@@ -152,7 +159,7 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
     uint32_t *dlt = reinterpret_cast<uint32_t *>(smem_raw + L.dlt);            // run -> bucket | keys << 16, then region slot - chunk slot
     uint32_t *heads = reinterpret_cast<uint32_t *>(smem_raw + L.heads);        // bit s: a run starts at slot s
     uint16_t *ord = reinterpret_cast<uint16_t *>(smem_raw + L.ord);            // run holding slot 32 w
-    K *stage = reinterpret_cast<K *>(smem_raw + L.stage);
+    Word *stage = reinterpret_cast<Word *>(smem_raw + L.stage);
     uint32_t *tmp = reinterpret_cast<uint32_t *>(smem_raw + L.total - 128);
     __shared__ uint32_t overflowed, nruns_s;
 
@@ -223,19 +230,26 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
         auto classify = [&](auto full) {  // full: a whole chunk
             auto mine = [&](int i) { return decltype(full)::value || at(i) < nh; };
             if constexpr (LEARNED) {
-#pragma unroll
+                const MlpTables &M = *mt;
+#pragma unroll 1
                 for (int i = 0; i < IT; ++i) {
-                    const K raw = kk[i];
-                    kk[i] = KeyTraits<DT>::phi(raw);
-                    br[i] = P;
-                    if (mine(i)) {
-                        uint32_t steps;
-                        bool mis;
-                        br[i] = classify_learned<DT>(raw, max((uint32_t)(e0 + at(i)), a.tag_floor), *mt, lut, P - 1, sphi,
-                                                     a.vtag, steps, mis);
-                        n_mis += mis;
-                        n_steps += steps;
-                    }
+                    K raw = kk[0];
+#pragma unroll
+                    for (int q = 1; q < IT; ++q) raw = q == i ? kk[q] : raw;
+                    const int where = ((i / V) * T + tid) * V + i % V;
+                    uint32_t steps = 0, bucket = P;
+                    bool mis = false;
+                    if (where < nh)
+                        bucket = classify_learned<DT>(raw, max((uint32_t)(e0 + where), a.tag_floor), M, lut, P - 1, sphi,
+                                                      a.vtag, steps, mis);
+                    n_mis += mis;
+                    n_steps += steps;
+#pragma unroll
+                    for (int q = 0; q < IT; ++q)
+                        if (q == i) {
+                            kk[q] = KeyTraits<DT>::phi(raw);
+                            br[q] = bucket;
+                        }
                 }
             } else {
                 const K base = lp.base, span = lp.span;
@@ -365,13 +379,17 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
             if (o < nruns) at_e[j] = atomicAdd(&a.cursor[dlt[o] & 0xffffu], dlt[o] >> 16);
         }
         // ---- group the chunk by bucket ----
+        auto word = [&](int i) -> Word {
+            if constexpr (PAIRS) return (uint64_t)kk[i] << 32 | (uint32_t)(e0 + at(i));
+            else return kk[i];
+        };
         if (nh == CH) {
 #pragma unroll
-            for (int i = 0; i < IT; ++i) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = kk[i];
+            for (int i = 0; i < IT; ++i) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = word(i);
         } else {
 #pragma unroll
             for (int i = 0; i < IT; ++i)
-                if (br[i] >> 16 < P) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = kk[i];
+                if (br[i] >> 16 < P) stage[cnt[br[i] >> 16] + (br[i] & 0xffffu)] = word(i);
         }
         // the next chunk's keys load while this one is reserved and written
         if (ch + pk.blocks < a.chunks) load_chunk(ch + pk.blocks);
@@ -408,16 +426,16 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
         if (overflowed) {  // a run that passes its region's end is not written (the overflow is reported)
             for (int s = tid; s < nh; s += T) {
                 const uint32_t d = dlt[run_of(s)];
-                if (d != kDropped) a.reg_keys[d + (uint32_t)s] = stage[s];
+                if (d != kDropped) regions[d + (uint32_t)s] = stage[s];
             }
         } else if (nh == CH) {
 #pragma unroll 8
             for (int i = 0; i < IT; ++i) {
                 const uint32_t s = i * T + tid;
-                a.reg_keys[dlt[run_of(s)] + s] = stage[s];
+                regions[dlt[run_of(s)] + s] = stage[s];
             }
         } else {
-            for (int s = tid; s < nh; s += T) a.reg_keys[dlt[run_of(s)] + (uint32_t)s] = stage[s];
+            for (int s = tid; s < nh; s += T) regions[dlt[run_of(s)] + (uint32_t)s] = stage[s];
         }
         // this chunk's counts are free again; the next chunk counts in the others
         for (uint32_t b = tid; b < P; b += T) cnt[b] = 0;
@@ -433,16 +451,17 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
     }
 }
 
-template <int DT, bool LEARNED> static cudaError_t launch_t(Exec &x) {
+template <int DT, bool LEARNED, bool PAIRS = false> static cudaError_t launch_t(Exec &x) {
     using K = typename KeyTraits<DT>::T;
+    constexpr int64_t CH = rk_chunk<K, LEARNED, PAIRS>();
     auto takes = [](const Ctx &c) { return (c.pl.classify == BSPS_LEARNED) == LEARNED; };
     size_t smem = 0;
     int64_t all = 0;  // chunks of every call
     for (int i = 0; i < x.count; ++i)
         if (takes(x.calls[i])) {
             const Plan &p = x.calls[i].pl;
-            smem = std::max(smem, RouteKeysLayout<K, LEARNED>((uint32_t)p.P, LEARNED ? kLutBits : p.lut_bits).total);
-            all += (p.n + rk_chunk<K, LEARNED>() - 1) / rk_chunk<K, LEARNED>();
+            smem = std::max(smem, RouteKeysLayout<K, LEARNED, PAIRS>((uint32_t)p.P, LEARNED ? kLutBits : p.lut_bits).total);
+            all += (p.n + CH - 1) / CH;
         }
     if (smem == 0) return cudaSuccess;
     if (smem > kRkSmemBudget - 512) return cudaErrorInvalidValue;
@@ -450,8 +469,9 @@ template <int DT, bool LEARNED> static cudaError_t launch_t(Exec &x) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sms = std::max(sms, 1);
-    return launch_calls<RouteKeysArgs<K>>(x, route_keys_kernel<DT, LEARNED, false>, route_keys_kernel<DT, LEARNED, true>,
-                                          kRkThreads, smem, [=](const Ctx &c, RouteKeysArgs<K> &a) {
+    return launch_calls<RouteKeysArgs<K>>(x, route_keys_kernel<DT, LEARNED, false, PAIRS>,
+                                          route_keys_kernel<DT, LEARNED, !PAIRS, PAIRS>, kRkThreads, smem,
+                                          [=](const Ctx &c, RouteKeysArgs<K> &a) {
         if (!takes(c)) return 0u;
         const Plan &p = c.pl;
         a.keys = (const K *)c.keys_in;
@@ -461,9 +481,9 @@ template <int DT, bool LEARNED> static cudaError_t launch_t(Exec &x) {
         a.vphi = (const K *)c.ly.vphi;
         a.vtag = c.ly.vtag;
         a.P = (uint32_t)p.P;
-        a.chunks = (p.n + rk_chunk<K, LEARNED>() - 1) / rk_chunk<K, LEARNED>();
+        a.chunks = (p.n + CH - 1) / CH;
         a.cursor = c.ly.cursor;
-        a.reg_keys = (K *)c.ly.reg_keys;
+        a.regions = c.ly.reg_keys;
         a.cap = p.cap;
         a.st = c.ly.status;
         a.mlp_tables = c.ly.mlp_tables;
@@ -488,6 +508,19 @@ cudaError_t launch_route_keys(Exec &x) {
     case BSPS_I32: return launch_d<BSPS_I32>(x);
     case BSPS_F32: return launch_d<BSPS_F32>(x);
     default: return launch_d<BSPS_F64>(x);
+    }
+}
+
+template <int DT> static cudaError_t launch_pairs_d(Exec &x) {
+    return x.calls[0].pl.classify == BSPS_LEARNED ? launch_t<DT, true, true>(x) : launch_t<DT, false, true>(x);
+}
+
+cudaError_t launch_route_words(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_pairs_d<BSPS_U32>(x);
+    case BSPS_I32: return launch_pairs_d<BSPS_I32>(x);
+    case BSPS_F32: return launch_pairs_d<BSPS_F32>(x);
+    default: return cudaErrorInvalidValue;
     }
 }
 

@@ -150,3 +150,16 @@ def test_small_call_reports_overflow():
     keys = np.random.default_rng(1).integers(0, 2**31, 10_000).astype(np.int32)
     st = plain_call(keys, None, 8, 4, capacity_pct=50)[3]
     assert (st.status, st.overflow) == (-4, 1)
+
+
+# 4-byte keys with payloads as words of key and position: the shapes above through the counting sort, the cluster sort
+# (values too heavy for a part) and the out-of-core sort, payloads of equal keys in input order
+@pytest.mark.parametrize("n, p", [(20_000, 1), (90_000, 1), (90_001, 3), (300_000, 40), (700_000, 1)])
+@pytest.mark.parametrize("name", sorted(SHAPES) + ["uniform"])
+def test_pairs_as_words(name, n, p):
+    rng = np.random.default_rng(n)
+    keys = (rng.integers(-2**31, 2**31, n) if name == "uniform" else SHAPES[name](rng, n)).astype(np.int32)
+    vals = rng.integers(0, 2**32, n).astype(np.uint32)
+    for dt in (np.int32, np.uint32):
+        ref = oracle.sort(keys.view(dt), p, 0, 0, oracle.RANDOM, seed=5, vals=vals, want_sample=False)
+        assert_same(run_gpu(keys.view(dt), p, 0, 0, oracle.RANDOM, 5, vals, refine=1, debug=False), ref)
