@@ -31,6 +31,13 @@
 // put in order and rebuilt from the half words alone.  It is taken when the
 // units are few and long (ranges up to 2^23 values at 65,536 keys).
 //
+// Where 256 bins hold more than half of what the stage takes (keys that crowd
+// in a small part of the range: a narrow component of a mixture, floats around
+// zero, a value with thousands of copies), they are sorted by themselves
+// afterwards, from the keys of the segment that lie in their range, with bins
+// as fine as that needs; a run of one-value bins that is larger than the stage
+// is written from its counts.
+//
 // Several CTAs (G of them) may take one segment: each counts all of it and
 // takes every G-th part.  Every decision is a function of the segment alone,
 // so the CTAs agree without talking to each other.
@@ -166,7 +173,7 @@ template <typename E, int T> struct BlockSort {
     }
 
     __device__ __noinline__ static void run(Smem &sm, E *a, int n) {
-        const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+        const int t = threadIdx.x, warp = t >> 5;
         if (n <= M) {
             sort_pivots(sm.piv, t < n ? a[t] : all_ones<E>());
             if (t < n) a[t] = sm.piv[t];
@@ -343,6 +350,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp
     static constexpr int kPartsMax = 32;
     static constexpr int kUnits = 256;               // units of a narrow stage
+    static constexpr int kTodo = 16;                 // crowded ranges waiting
     static constexpr uint32_t kUseWide = STAGE / sizeof(K) - 8, kUseNarrow = STAGE / sizeof(S) - 8;
     static_assert(NBMAX % 512 == 0 && kSegs <= 128 && NBMAX <= 65536, "the segments are scanned by one warp, four to a lane");
     static_assert(kUseWide < 65528 && STAGE % 16 == 0, "16-bit positions inside a part");
@@ -352,7 +360,9 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         uint32_t pseg[kPartsMax + 1];         // first segment of every part
         uint32_t unit[kUnits + 2];            // first position of every unit (narrow stage)
         uint32_t longs[kLongMax];             // bin | length << 16
-        uint32_t nlong, nparts, bad, half;
+        uint32_t nlong, nparts, bad, half, heavy;  // heavy: bit p, part p is one crowded run of 256 bins
+        uint32_t ntodo, todo_at[kTodo], todo_n[kTodo];
+        alignas(16) K todo_lo[kTodo], todo_hi[kTodo];  // ranges still to sort: bounds, first position, keys
         alignas(16) unsigned char sort[sizeof(typename BlockSort<K, T>::Smem)];  // of a long bin by the whole CTA
     };
     static constexpr size_t kHead = (sizeof(Smem) + 15) & ~size_t(15);
@@ -365,7 +375,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     // that end at its cursor.
     template <typename E, typename End>
     __device__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, End end_of) {
-        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        const int tid = threadIdx.x, warp = tid >> 5;
         const uint32_t nl = sm.nlong;
         for (uint32_t i = warp; i < nl; i += W) {
             const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
@@ -479,10 +489,11 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         }
     }
 
-    // The same from a narrow stage.
+    // The same from a narrow stage (p0: the part's first position in the range,
+    // whose first position is `from` in the sink).
     template <typename Sink>
-    __device__ static void emit_narrow(const Smem &sm, const S *stage, int pad, int np, uint32_t p0, uint32_t nunits, K lo,
-                                       const Sink &sink) {
+    __device__ static void emit_narrow(const Smem &sm, const S *stage, int pad, int np, uint32_t p0, uint32_t from,
+                                       uint32_t nunits, K lo, const Sink &sink) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, end = pad + np;
         for (int w0 = warp * kStep; w0 < end; w0 += W * kStep) {
             const int at = w0 - kEdge + lane * kPer;
@@ -521,7 +532,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 sort_window(s);
                 const K base = lo + ((K)u0 << UB);
                 if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
-                    put(sink, p0, at, inner, pad, end, [&](int j) { return base + s[j]; });
+                    put(sink, from + p0, at, inner, pad, end, [&](int j) { return base + s[j]; });
             } else {
                 K x[kPer];
 #pragma unroll
@@ -536,7 +547,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 }
                 sort_window(x);
                 if (lane >= kEdge / kPer && lane < 32 - kEdge / kPer)
-                    put(sink, p0, at, inner, pad, end, [&](int j) { return x[j]; });
+                    put(sink, from + p0, at, inner, pad, end, [&](int j) { return x[j]; });
             }
         }
     }
@@ -571,18 +582,62 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         __syncthreads();
     }
 
-    // Sorts the n keys of src into positions [0, n) of sink, as CTA g of G.  Returns false
-    // (in every CTA of the segment alike, with nothing written) when a run of
-    // 256 bins holds more keys than a part or there are too many long bins.
+    // Sorts the n keys of src into positions [0, n) of sink, as CTA g of G.
+    // Returns false, in every CTA of the segment alike, when it gives up: more
+    // long bins or crowded ranges than the lists hold, or more parts than there
+    // may be.  What was written by then is rewritten by whoever takes over.
     template <typename Source, typename Sink>
     __device__ static bool run(unsigned char *smem, const Source &src, int n, K lo, K hi, const Sink &sink, int g, int G) {
+        Smem &sm = *reinterpret_cast<Smem *>(smem);
+        if (threadIdx.x == 0) sm.ntodo = 0;
+        if (!run_range(smem, src, n, (uint32_t)n, lo, hi, 0u, sink, g, G)) return false;
+        __syncthreads();
+        return sm.ntodo == 0 || run_crowded(smem, src, n, sink, g, G);
+    }
+
+    // The keys of src in a range.
+    template <typename Source> struct Within {
+        const Source &src;
+        K lo, span;
+        template <typename F> __device__ void each(int n, F f) const {
+            src.each(n, [&](K k) {
+                if (k - lo <= span) f(k);
+            });
+        }
+    };
+    static_assert(2 * W * sizeof(K) <= offsetof(Smem, longs), "bounds() leaves the ranges to sort alone");
+
+    // The crowded ranges, each a small part of the one it came from (so this ends).
+    template <typename Source, typename Sink>
+    __device__ static __noinline__ bool run_crowded(unsigned char *smem, const Source &src, int n, const Sink &sink, int g,
+                                                    int G) {
+        Smem &sm = *reinterpret_cast<Smem *>(smem);
+        for (;;) {
+            __syncthreads();
+            const uint32_t t = sm.ntodo;
+            if (t == 0) return true;
+            const Within<Source> in{src, sm.todo_lo[t - 1], sm.todo_hi[t - 1] - sm.todo_lo[t - 1]};
+            const uint32_t at = sm.todo_at[t - 1], keys = sm.todo_n[t - 1];
+            __syncthreads();
+            if (threadIdx.x == 0) sm.ntodo = t - 1;
+            K lo, hi;  // of the keys themselves: what crowds may be far narrower than its bins
+            bounds(smem, in, n, lo, hi);
+            if (!run_range(smem, in, n, keys, lo, hi, at, sink, g, G)) return false;
+        }
+    }
+
+    // The n keys that src, which reads nsrc, gives, all in [lo, hi], into
+    // positions [base, base + n) of sink.
+    template <typename Source, typename Sink>
+    __device__ static bool run_range(unsigned char *smem, const Source &src, int nsrc, uint32_t n, K lo, K hi, uint32_t base,
+                                     const Sink &sink, int g, int G) {
         Smem &sm = *reinterpret_cast<Smem *>(smem);
         uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + kHead);
         unsigned char *stage = smem + kHead + (size_t)NBMAX * 2;
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         // bins: a power of two about the number of keys
         int nbl = 9;
-        while ((1 << nbl) < NBMAX && (1 << nbl) < n) ++nbl;
+        while ((1 << nbl) < NBMAX && (1u << nbl) < n) ++nbl;
         const K range = hi - lo;
         const int bits = word_bits<K>(range);
         const int shift = bits > nbl ? bits - nbl : 0;
@@ -590,7 +645,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         // a narrow stage where a wide one would need more parts (or, of 64-bit
         // keys, wherever it can be: its windows sort half words)
         const K nu = (range >> UB) + 1;
-        const bool narrow = sizeof(K) <= 8 && (sizeof(K) == 8 || (uint32_t)n > kUseWide) && shift + 3 <= UB && nu <= (K)kUnits &&
+        const bool narrow = sizeof(K) <= 8 && (sizeof(K) == 8 || n > kUseWide) && shift + 3 <= UB && nu <= (K)kUnits &&
                             (nu <= 2 || (uint64_t)nu * kWin <= (uint64_t)n);
         const uint32_t nunits = (uint32_t)nu;
         for (uint32_t q = tid; q < nb / 8; q += T) reinterpret_cast<uint4 *>(cnt)[q] = make_uint4(0u, 0u, 0u, 0u);
@@ -601,7 +656,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         __syncthreads();
         // keys outside [lo, hi] (a region that overflowed, which is reported) stay in bounds
         auto bin_of = [&](K v) { return min((uint32_t)(v >> shift), nb - 1u); };
-        src.each(n, [&](K k) {
+        src.each(nsrc, [&](K k) {
             const uint32_t b = bin_of(k - lo);
             atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u);
         });
@@ -658,18 +713,50 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             // bits shows in the total.)
             const uint32_t use = narrow ? kUseNarrow : kUseWide, mid = sm.seg[hseg];
             uint32_t np = 1, half = mid;
-            bool ok = tot == (uint32_t)n;
-            if ((uint32_t)n > use || G > 1 || mid > 65000u || (uint32_t)n - mid > 65000u) {
-                const uint32_t most = min(use, 65528u);
-                ok = ok && mx < most;
-                np = ok ? ((uint32_t)n + (most - mx) - 1) / (most - mx) : 1u;
-                np = min(max(np, (uint32_t)G), max(np, nseg));
-                ok = ok && np <= (uint32_t)kPartsMax;
+            const uint32_t most = min(use, 65528u);
+            bool ok = tot == n;
+            const bool crowded = n > use && mx > most / 2;
+            if (crowded) {
+                // parts one after the other, a crowded run of bins by itself
                 half = 0;
-            }
-            if (ok) {
-                const uint32_t target = ((uint32_t)n + np - 1) / np;
-                if (lane < (int)np) {  // part `lane` starts at the first segment at or past lane * target
+                if (lane == 0 && ok) {
+                    const uint32_t fits = shift > 0 ? most / 2 : most;
+                    uint32_t from = 0, heavy = 0;
+                    np = 0;
+                    auto part = [&](uint32_t first, bool is_heavy) {
+                        if (np < (uint32_t)kPartsMax) {
+                            sm.pseg[np] = first;
+                            heavy |= (is_heavy ? 1u : 0u) << np;
+                        }
+                        ++np;
+                    };
+                    for (uint32_t s = 0; s < nseg; ++s) {
+                        const uint32_t c = sm.seg[s + 1] - sm.seg[s];
+                        if (c > fits) {
+                            if (s > from) part(from, false);
+                            part(s, true);
+                            from = s + 1;
+                        } else if (sm.seg[s + 1] - sm.seg[from] > most) {
+                            part(from, false);
+                            from = s;
+                        }
+                    }
+                    if (from < nseg) part(from, false);
+                    sm.heavy = heavy;
+                    ok = np <= (uint32_t)kPartsMax;
+                    if (ok) sm.pseg[np] = nseg;
+                }
+                np = __shfl_sync(0xffffffffu, np, 0);
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+            } else {
+                if (n > use || G > 1 || mid > 65000u || n - mid > 65000u) {
+                    np = (n + (most - mx) - 1) / (most - mx);
+                    np = min(max(np, (uint32_t)G), max(np, nseg));
+                    ok = ok && np <= (uint32_t)kPartsMax;
+                    half = 0;
+                }
+                const uint32_t target = (n + np - 1) / np;
+                if (ok && lane < (int)np) {  // part `lane` starts at the first segment at or past lane * target
                     const uint32_t want = lane * target;
                     uint32_t a = 0, b = nseg;
                     while (a < b) {
@@ -680,19 +767,21 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     sm.pseg[lane] = a;
                 }
                 if (lane == 0) {
-                    sm.pseg[np] = nseg;
-                    sm.nparts = np;
-                    sm.half = half;
-                    sm.unit[nunits <= (uint32_t)kUnits ? nunits : 0] = 0xffffffffu;
-                    sm.unit[nunits <= (uint32_t)kUnits ? nunits + 1 : 0] = 0xffffffffu;
+                    if (ok) sm.pseg[np] = nseg;
+                    sm.heavy = 0;
                 }
-            } else if (lane == 0) {
-                sm.bad = 1;
+            }
+            if (lane == 0) {
+                sm.nparts = np;
+                sm.half = half;
+                sm.bad = !ok;
+                sm.unit[nunits <= (uint32_t)kUnits ? nunits : 0] = 0xffffffffu;
+                sm.unit[nunits <= (uint32_t)kUnits ? nunits + 1 : 0] = 0xffffffffu;
             }
         }
         __syncthreads();
         if (sm.bad) return false;
-        const uint32_t nparts = sm.nparts, half = sm.half;
+        const uint32_t nparts = sm.nparts, half = sm.half, heavy = sm.heavy;
         // counts -> each bin's first slot inside its part; units and long bins recorded
         for (uint32_t s = warp; s < hseg; s += W) {
             uint32_t w[8], out_w[8];
@@ -717,9 +806,24 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 const uint32_t bin0 = sg * kSegBins + lane * 8;
                 if (narrow && (bin0 & ((1u << (UB - shift)) - 1u)) == 0u && (bin0 >> (UB - shift)) < nunits)
                     sm.unit[bin0 >> (UB - shift)] = p;
+                if (heavy >> ps & 1u) {
+                    // sorted by itself later; where bins are single values, written here
+                    if (shift == 0)
+                        for (int l = 0; l < 32; ++l) {
+                            uint32_t q = __shfl_sync(0xffffffffu, p, l);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const uint32_t c = __shfl_sync(0xffffffffu, (w[j] >> (16 * hi_half)) & 0xffffu, l);
+                                for (uint32_t e = g * 32 + lane; e < c; e += G * 32)
+                                    sink.one((int64_t)base + q + e, lo + (K)(sg * kSegBins + l * 8 + j));
+                                q += c;
+                            }
+                        }
+                    continue;
+                }
                 // relative to the part's start (or the middle) and the stage's pad
                 const uint32_t pstart = sm.seg[sm.pseg[ps]];
-                p += (uint32_t)sink.pad(pstart) - pstart - (hi_half ? half : 0u);
+                p += (uint32_t)sink.pad(base + pstart) - pstart - (hi_half ? half : 0u);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     out_w[j] |= p << (16 * hi_half);
@@ -752,23 +856,23 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         for (uint32_t part = g; part < nparts; part += G) {
             const uint32_t s0 = sm.pseg[part], s1 = sm.pseg[part + 1];
             const uint32_t p0 = sm.seg[s0], np = sm.seg[s1] - p0;
-            if (np == 0) continue;  // uniform
+            if (np == 0 || (heavy >> part & 1u)) continue;  // uniform
             const uint32_t b0 = s0 * kSegBins, bn = (s1 - s0) * kSegBins;
             if (nparts == 1) {
                 if (narrow) {
-                    src.each(n, [&](K k) {
+                    src.each(nsrc, [&](K k) {
                         const K v = k - lo;
                         const uint32_t b = bin_of(v);
                         reinterpret_cast<S *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = (S)v;
                     });
                 } else {
-                    src.each(n, [&](K k) {
+                    src.each(nsrc, [&](K k) {
                         const uint32_t b = bin_of(k - lo);
                         reinterpret_cast<K *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = k;
                     });
                 }
             } else {
-                src.each(n, [&](K k) {
+                src.each(nsrc, [&](K k) {
                     const K v = k - lo;
                     const uint32_t b = bin_of(v);
                     if (b - b0 < bn) place(b, v, k);
@@ -776,22 +880,37 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             }
             __syncthreads();
             auto end_of = [&](uint32_t b) { return slot_of(b, cnt[b & wmask]); };
-            const int pad = sink.pad(p0);
+            const int pad = sink.pad(base + p0);
             if constexpr (sizeof(K) <= 8) if (narrow) {
                 if (sm.nlong) {
                     sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, end_of);
                     __syncthreads();
                 }
-                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, nunits, lo, sink);
+                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, base, nunits, lo, sink);
             }
             if (!narrow) {
                 if (sm.nlong) {
                     sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, end_of);
                     __syncthreads();
                 }
-                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, p0, sink);
+                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, base + p0, sink);
             }
             __syncthreads();  // the next part reuses the stage
+        }
+        if (heavy && shift > 0) {
+            if (tid == 0)
+                for (uint32_t part = 0; part < nparts; ++part)
+                    if (heavy >> part & 1u) {
+                        const uint32_t s = sm.pseg[part], t = sm.ntodo++;
+                        if (t >= (uint32_t)kTodo) continue;
+                        const K first = (K)(s * kSegBins) << shift, past = ((K)kSegBins << shift) - 1;
+                        sm.todo_lo[t] = lo + first;
+                        sm.todo_hi[t] = range - first < past ? hi : lo + first + past;
+                        sm.todo_at[t] = base + sm.seg[s];
+                        sm.todo_n[t] = sm.seg[s + 1] - sm.seg[s];
+                    }
+            __syncthreads();
+            if (sm.ntodo > (uint32_t)kTodo) return false;
         }
         return true;
     }

@@ -470,7 +470,7 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
     const bool stash = m <= kLowCardStashMax;
     const uint32_t xx = (uint32_t)x;
     const int64_t lo = k * m;
-    const int64_t len = lo < n ? imin64(m, n - lo) : 0;
+    const int64_t len64 = lo < n ? imin64(m, n - lo) : 0;  // < 2^32 (positions are 32 bits wide)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < NS; i += T) slot[i] = 0ull;
     for (int i = tid; i < W * NS; i += T) wcnt[i] = 0;
@@ -488,15 +488,13 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
         return f >> (32 - 9);
     };
     static_assert(NS == 512, "9-bit hash");
-    // slot holding f (inserting it when absent); -1 when the table is full
-    auto find = [&](uint32_t f, bool insert) -> int {
+    // slot holding f, inserted when absent; -1 when the table is full
+    auto find = [&](uint32_t f, uint32_t h) -> int {
         const unsigned long long want = (1ull << 32) | f;
-        uint32_t h = hash(f);
         for (int probe = 0; probe < NS; ++probe, h = (h + 1) & (NS - 1)) {
             unsigned long long cur = slot[h];
             if (cur == want) return (int)h;
             if (cur == 0ull) {
-                if (!insert) return -1;
                 cur = atomicCAS(&slot[h], 0ull, want);
                 if (cur == 0ull) {
                     if (atomicAdd(&ndistinct, 1) >= kLowCardMax) overflow = 1;
@@ -508,35 +506,55 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
         return -1;
     };
     // warp w's segment of the block: [seg0, seg1), whole steps of 32 keys
-    const int64_t seg = ((len + W - 1) / W + 31) / 32 * 32;
-    const int64_t seg0 = imin64(len, warp * seg), seg1 = imin64(len, seg0 + seg);
+    const uint32_t len = (uint32_t)len64, seg = ((len + W - 1) / W + 31) / 32 * 32;
+    const uint32_t seg0 = min(len, warp * seg), seg1 = min(len, seg0 + seg);
     uint32_t *mine = wcnt + warp * NS;
     // keys of kAhead steps of 32 are loaded before the first is used
     constexpr int kAhead = 8;
-    uint32_t fa[kAhead];
-    auto load_ahead = [&](int64_t e0) {
+    const K *blk = keys + lo;
+    // What a key needs in the second pass: its slot, the keys of its value in
+    // lower lanes of its step, whether no higher lane has one.
+    constexpr uint32_t kBelow = 9, kLast = 14;
+    uint32_t word[kAhead];
+    auto look_up = [&](uint32_t e0, bool count) {
+        uint32_t f[kAhead], peers[kAhead];
+        unsigned long long first[kAhead];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            const int64_t e = e0 + u * 32 + lane;
-            fa[u] = e < seg1 ? (uint32_t)KeyTraits<DT>::phi(keys[lo + e]) : 0u;
+            const uint32_t e = e0 + u * 32 + lane;
+            f[u] = e < seg1 ? (uint32_t)KeyTraits<DT>::phi(blk[e]) : 0u;
         }
-    };
-    // pass 1: distinct values, and their keys per segment
-    for (int64_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
-        load_ahead(e0);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            word[u] = hash(f[u]);
+            first[u] = slot[word[u]];
+        }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
             const bool ok = e0 + u * 32 + lane < seg1;
-            const uint32_t act = __ballot_sync(0xffffffffu, ok);
-            if (ok) {
-                const uint32_t f = fa[u];
-                const int h = find(f, true);
-                const uint32_t peers = __match_any_sync(act, f);
-                if (stash) sid16[e0 + u * 32 + lane] = (uint16_t)max(h, 0);
-                if (h < 0) overflow = 1;
-                else if (lane == __ffs(peers) - 1) mine[h] += (uint32_t)__popc(peers);  // this warp's own counts
-            }
+            // (lanes past the end are their own group: the keys' act mask leaves them out)
+            peers[u] = __match_any_sync(0xffffffffu, f[u]) & __ballot_sync(0xffffffffu, ok);
         }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            if (e0 + u * 32 + lane >= seg1) continue;
+            if (first[u] != ((1ull << 32) | f[u])) {
+                const int h = find(f[u], word[u]);
+                if (h < 0) overflow = 1;
+                word[u] = (uint32_t)max(h, 0);
+            }
+            const uint32_t below = (uint32_t)__popc(peers[u] & lanemask_lt()), all = (uint32_t)__popc(peers[u]);
+            if (count && below == 0) atomicAdd(&mine[word[u]], all);
+            word[u] |= below << kBelow | (below + 1 == all ? 1u : 0u) << kLast;
+        }
+    };
+    // pass 1: distinct values, and their keys per segment
+    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
+        look_up(e0, true);
+        if (stash)
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+                if (e0 + u * 32 + lane < seg1) sid16[e0 + u * 32 + lane] = (uint16_t)word[u];
     }
     __syncthreads();
     if (overflow || ndistinct > kLowCardMax) return;  // leave the block to the stable sort
@@ -613,46 +631,46 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
             runs[lo + t] = (K)val_of_rank[r];
         }
     }
-    // pass 2: in position order, sorted rank = start + earlier segments + earlier here
+    // the rank of each value's first key of this segment
+    for (int h = lane; h < NS; h += 32) mine[h] += start[h];
+    __syncwarp();
+    // pass 2: in position order, sorted rank = first rank + earlier here
     const float inv_x = 1.0f / (float)xx;
-    for (int64_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
-        if (!stash) load_ahead(e0);
+    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
+        if (stash) {
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const uint32_t e = e0 + u * 32 + lane;
+                word[u] = e < seg1 ? sid16[e] : 0u;
+            }
+        } else {
+            look_up(e0, false);
+        }
         uint32_t va[kAhead];  // the payloads of the kAhead steps, loaded before the first is stored
         if (runs_val) {
 #pragma unroll
             for (int u = 0; u < kAhead; ++u) {
-                const int64_t e = e0 + u * 32 + lane;
+                const uint32_t e = e0 + u * 32 + lane;
                 va[u] = e < seg1 ? vals_in[lo + e] : 0u;
             }
         }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            const int64_t e = e0 + u * 32 + lane;
+            const uint32_t e = e0 + u * 32 + lane;
             const bool ok = e < seg1;
-            const uint32_t act = __ballot_sync(0xffffffffu, ok);
+            const uint32_t h = word[u] & (NS - 1), r = mine[h] + (word[u] >> kBelow & 31u);
+            __syncwarp();
             if (ok) {
-                int h;
-                uint32_t f;
-                if (stash) {
-                    h = sid16[e];
-                    f = (uint32_t)slot[h];
-                } else {
-                    f = fa[u];
-                    h = max(0, find(f, false));  // present: every key was counted
-                }
-                const uint32_t peers = __match_any_sync(act, (uint32_t)h);
-                const uint32_t g1 = start[h] + mine[h] + (uint32_t)__popc(peers & lanemask_lt()) + 1;  // < 2^32
-                __syncwarp(act);
-                if (lane == __ffs(peers) - 1) mine[h] += (uint32_t)__popc(peers);
-                if (runs_val) runs_val[lo + g1 - 1] = va[u];  // payloads at their ranks
-                // j = g1 / x when x divides g1 (the quotient from a float
+                if (word[u] >> kLast) mine[h] = r + 1;
+                if (runs_val) runs_val[lo + r] = va[u];  // payloads at their ranks
+                // j = (r + 1) / x when x divides it (the quotient from a float
                 // estimate, corrected by one either way)
-                uint32_t j = (uint32_t)((float)g1 * inv_x);
-                int64_t rem = (int64_t)g1 - (int64_t)j * xx;
+                uint32_t j = (uint32_t)((float)(r + 1) * inv_x);
+                int64_t rem = (int64_t)(r + 1) - (int64_t)j * xx;
                 if (rem >= (int64_t)xx) { ++j; rem -= xx; }
                 if (rem < 0) { --j; rem += xx; }
                 if (rem == 0) {
-                    sphi[k * s + (j - 1)] = (K)f;
+                    sphi[k * s + (j - 1)] = (K)(uint32_t)slot[h];
                     stag[k * s + (j - 1)] = (uint32_t)(lo + e);
                 }
             }

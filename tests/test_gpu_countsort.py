@@ -163,3 +163,28 @@ def test_pairs_as_words(name, n, p):
     for dt in (np.int32, np.uint32):
         ref = oracle.sort(keys.view(dt), p, 0, 0, oracle.RANDOM, seed=5, vals=vals, want_sample=False)
         assert_same(run_gpu(keys.view(dt), p, 0, 0, oracle.RANDOM, 5, vals, refine=1, debug=False), ref)
+
+
+# keys that crowd in a small part of a bucket's range, so that 256 bins hold more than half a stage: nested widths,
+# values with thousands of copies (below and past the 16 bits of a bin's count), one and several CTAs a bucket
+CROWDS = {
+    "narrow_component": lambda r, n: np.where(r.random(n) < 0.7, 1e6 + r.normal(0, 1e-3, n), r.normal(0, 1e6, n)),
+    "nested": lambda r, n: r.normal(0, 1, n) * 10.0 ** -r.integers(0, 12, n),
+    "two_heavy_values": lambda r, n: r.choice([3.0, 3.0 + 2.0**-30, 1e5], n, p=[0.45, 0.15, 0.4]) + (r.random(n) < 0.1) * r.normal(0, 1, n),
+    "edge": lambda r, n: np.where(r.random(n) < 0.8, 2.0**30 - 1 - r.integers(0, 50, n), r.integers(0, 2**30, n)).astype(np.float64),
+}
+
+
+@pytest.mark.parametrize("n, p", [(24_000, 1), (60_000, 1), (160_001, 1), (450_000, 2)])
+@pytest.mark.parametrize("name", sorted(CROWDS))
+def test_crowded_ranges(name, n, p):
+    rng = np.random.default_rng(n)
+    keys = CROWDS[name](rng, n)
+    check(keys, p)
+    check(keys.astype(np.float32), p)
+    k32 = keys.astype(np.float32)
+    vals = rng.integers(0, 2**32, n).astype(np.uint32)
+    ref = oracle.sort(k32, p, 0, 0, oracle.RANDOM, seed=9, vals=vals, want_sample=False)
+    got = plain_call(k32, vals, p, 0, refine=1)
+    assert got[0].tobytes() == ref.keys.tobytes() and np.array_equal(got[1], ref.vals)
+    assert np.array_equal(got[2], ref.bucket_sizes)
