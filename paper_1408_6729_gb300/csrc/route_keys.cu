@@ -230,26 +230,19 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
         auto classify = [&](auto full) {  // full: a whole chunk
             auto mine = [&](int i) { return decltype(full)::value || at(i) < nh; };
             if constexpr (LEARNED) {
-                const MlpTables &M = *mt;
-#pragma unroll 1
+#pragma unroll
                 for (int i = 0; i < IT; ++i) {
-                    K raw = kk[0];
-#pragma unroll
-                    for (int q = 1; q < IT; ++q) raw = q == i ? kk[q] : raw;
-                    const int where = ((i / V) * T + tid) * V + i % V;
-                    uint32_t steps = 0, bucket = P;
-                    bool mis = false;
-                    if (where < nh)
-                        bucket = classify_learned<DT>(raw, max((uint32_t)(e0 + where), a.tag_floor), M, lut, P - 1, sphi,
-                                                      a.vtag, steps, mis);
-                    n_mis += mis;
-                    n_steps += steps;
-#pragma unroll
-                    for (int q = 0; q < IT; ++q)
-                        if (q == i) {
-                            kk[q] = KeyTraits<DT>::phi(raw);
-                            br[q] = bucket;
-                        }
+                    const K raw = kk[i];
+                    kk[i] = KeyTraits<DT>::phi(raw);
+                    br[i] = P;
+                    if (mine(i)) {
+                        uint32_t steps;
+                        bool mis;
+                        br[i] = classify_learned<DT>(raw, max((uint32_t)(e0 + at(i)), a.tag_floor), *mt, lut, P - 1, sphi,
+                                                     a.vtag, steps, mis);
+                        n_mis += mis;
+                        n_steps += steps;
+                    }
                 }
             } else {
                 const K base = lp.base, span = lp.span;
