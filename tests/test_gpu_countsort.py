@@ -188,3 +188,12 @@ def test_crowded_ranges(name, n, p):
     got = plain_call(k32, vals, p, 0, refine=1)
     assert got[0].tobytes() == ref.keys.tobytes() and np.array_equal(got[1], ref.vals)
     assert np.array_equal(got[2], ref.bucket_sizes)
+
+
+# a few hundred values: one run of 256 one-value bins as large as a stage or larger, on several CTAs a bucket
+@pytest.mark.parametrize("n", [65_536, 130_000, 400_000])
+@pytest.mark.parametrize("values, p", [(180, 1), (375, 1), (3000, 8)])
+def test_few_values_several_ctas(n, values, p):
+    keys = np.random.default_rng(n).integers(0, values, n)
+    check(keys.astype(np.int32), p)
+    check(keys.astype(np.float64), p)
