@@ -441,25 +441,38 @@ run_sample_tags_kernel(const uint32_t *__restrict__ keys, const uint32_t *__rest
 // runs of equal values in position order and every payload at its key's rank
 // (a stable counting sort).  Blocks with more than kLowCardMax values keep their flag
 // for the stable block sort.
-constexpr int kLowCardThreads = 1024, kLowCardMax = 256, kLowCardSlots = 512;
+//
+// Bound by instructions and shared-memory latency, not bytes.  The table is
+// read two slots at a time and at most a quarter full where counts of 16 bits
+// do (blocks of at most kLowCardStashMax keys), so few keys probe twice; there
+// the first pass also leaves, for each key, its slot and its place among the
+// equal keys of its step (16 bits), and the second neither matches lanes nor
+// reads the table.  2^28 Zipf pairs in blocks of 2^16: 3.45 ms when both passes
+// matched and probed a table half full one slot at a time, 3.29 with the
+// places kept, 2.65 with the pairs of slots.
+constexpr int kLowCardThreads = 1024, kLowCardMax = 256;
 constexpr int kLowCardWarps = kLowCardThreads / 32;
-constexpr size_t kLowCardSmem = sizeof(uint32_t) * kLowCardWarps * kLowCardSlots;  // per-warp counts
-// blocks of at most kLowCardStashMax keys keep every key's slot from the first
-// pass (16 bits each), so the second pass neither reloads nor hashes the keys
 constexpr int64_t kLowCardStashMax = 65536;
-static size_t lowcard_smem(int64_t m) { return kLowCardSmem + (m <= kLowCardStashMax ? 2 * (size_t)m : 0); }
-template <int DT>
+template <bool STASH> struct LowCard {
+    using Count = typename std::conditional<STASH, uint16_t, uint32_t>::type;
+    static constexpr int kBits = STASH ? 10 : 9, NS = 1 << kBits;
+    static constexpr size_t kCounts = sizeof(Count) * kLowCardWarps * NS;
+    static size_t smem(int64_t m) { return kCounts + (STASH ? 2 * (size_t)m : 0); }
+};
+template <int DT, bool STASH>
 __global__ void __launch_bounds__(kLowCardThreads, 1)
 run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, int64_t n, int64_t m, int64_t s,
                           int64_t x, typename KeyTraits<DT>::T *sphi, uint32_t *stag, uint32_t *retry,
                           typename KeyTraits<DT>::T *runs, const uint32_t *__restrict__ vals_in,
                           uint32_t *runs_val) {
     using K = typename KeyTraits<DT>::T;
+    using Count = typename LowCard<STASH>::Count;
     static_assert(sizeof(K) == 4, "32-bit keys");
-    constexpr int T = kLowCardThreads, W = kLowCardWarps, NS = kLowCardSlots;
-    extern __shared__ __align__(16) uint32_t wcnt[];       // [W][NS]: keys per slot in warp w's segment
-    uint16_t *sid16 = reinterpret_cast<uint16_t *>(wcnt + kLowCardWarps * kLowCardSlots);  // slot of each key
-    __shared__ unsigned long long slot[NS];                 // (1 << 32) | phi, 0 = empty
+    constexpr int T = kLowCardThreads, W = kLowCardWarps, NS = LowCard<STASH>::NS;
+    extern __shared__ __align__(16) unsigned char low_smem[];
+    Count *wcnt = reinterpret_cast<Count *>(low_smem);                         // [W][NS]: keys per slot in warp w's segment
+    uint16_t *word16 = reinterpret_cast<uint16_t *>(low_smem + LowCard<STASH>::kCounts);  // per key, for the second pass
+    __shared__ __align__(16) unsigned long long slot[NS];   // (1 << 32) | phi, 0 = empty
     __shared__ uint32_t start[NS];                          // sorted start of the slot's value
     __shared__ uint32_t vals[kLowCardMax], sid[kLowCardMax], rank_of[kLowCardMax], tot_sorted[kLowCardMax];
     __shared__ uint32_t val_of_rank[kLowCardMax];
@@ -467,27 +480,26 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
     __shared__ int ndistinct, overflow;
     const int64_t k = blockIdx.x;
     if (retry[k] == 0) return;  // sorted by the keys-only block sort
-    const bool stash = m <= kLowCardStashMax;
     const uint32_t xx = (uint32_t)x;
     const int64_t lo = k * m;
     const int64_t len64 = lo < n ? imin64(m, n - lo) : 0;  // < 2^32 (positions are 32 bits wide)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < NS; i += T) slot[i] = 0ull;
-    for (int i = tid; i < W * NS; i += T) wcnt[i] = 0;
+    for (int i = tid; i < (int)(LowCard<STASH>::kCounts / 16); i += T)
+        reinterpret_cast<uint4 *>(low_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
         ndistinct = 0;
         overflow = 0;
     }
     __syncthreads();
-    auto hash = [](uint32_t f) {  // murmur3's 32-bit finaliser, top 9 bits
+    auto hash = [](uint32_t f) {  // murmur3's 32-bit finaliser, its top bits: the first of a pair of slots
         f ^= f >> 16;
         f *= 0x85ebca6bu;
         f ^= f >> 13;
         f *= 0xc2b2ae35u;
         f ^= f >> 16;
-        return f >> (32 - 9);
+        return f >> (33 - LowCard<STASH>::kBits) << 1;
     };
-    static_assert(NS == 512, "9-bit hash");
     // slot holding f, inserted when absent; -1 when the table is full
     auto find = [&](uint32_t f, uint32_t h) -> int {
         const unsigned long long want = (1ull << 32) | f;
@@ -508,53 +520,59 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
     // warp w's segment of the block: [seg0, seg1), whole steps of 32 keys
     const uint32_t len = (uint32_t)len64, seg = ((len + W - 1) / W + 31) / 32 * 32;
     const uint32_t seg0 = min(len, warp * seg), seg1 = min(len, seg0 + seg);
-    uint32_t *mine = wcnt + warp * NS;
+    Count *mine = wcnt + warp * NS;
     // keys of kAhead steps of 32 are loaded before the first is used
     constexpr int kAhead = 8;
     const K *blk = keys + lo;
     // What a key needs in the second pass: its slot, the keys of its value in
     // lower lanes of its step, whether no higher lane has one.
-    constexpr uint32_t kBelow = 9, kLast = 14;
+    constexpr uint32_t kBelow = LowCard<STASH>::kBits, kLast = kBelow + 5;
     uint32_t word[kAhead];
-    auto look_up = [&](uint32_t e0, bool count) {
-        uint32_t f[kAhead], peers[kAhead];
-        unsigned long long first[kAhead];
+    auto look_up = [&](uint32_t e0, bool count, auto full) {
+        uint32_t f[kAhead];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
             const uint32_t e = e0 + u * 32 + lane;
-            f[u] = e < seg1 ? (uint32_t)KeyTraits<DT>::phi(blk[e]) : 0u;
+            f[u] = decltype(full)::value || e < seg1 ? (uint32_t)KeyTraits<DT>::phi(blk[e]) : 0u;
         }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            word[u] = hash(f[u]);
-            first[u] = slot[word[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            const bool ok = e0 + u * 32 + lane < seg1;
-            // (lanes past the end are their own group: the keys' act mask leaves them out)
-            peers[u] = __match_any_sync(0xffffffffu, f[u]) & __ballot_sync(0xffffffffu, ok);
-        }
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            if (e0 + u * 32 + lane >= seg1) continue;
-            if (first[u] != ((1ull << 32) | f[u])) {
-                const int h = find(f[u], word[u]);
-                if (h < 0) overflow = 1;
-                word[u] = (uint32_t)max(h, 0);
+            const bool ok = decltype(full)::value || e0 + u * 32 + lane < seg1;
+            uint32_t peers = __match_any_sync(0xffffffffu, f[u]);
+            if (!decltype(full)::value) peers &= __ballot_sync(0xffffffffu, ok);
+            const uint32_t h = hash(f[u]);
+            const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(&slot[h]);
+            const unsigned long long want = (1ull << 32) | f[u];
+            const bool one = e.x == want, two = e.y == want;
+            word[u] = h + (two ? 1u : 0u);
+            if (!(one || two) && ok) {
+                const int at = find(f[u], h);
+                if (at < 0) overflow = 1;
+                word[u] = (uint32_t)max(at, 0);
             }
-            const uint32_t below = (uint32_t)__popc(peers[u] & lanemask_lt()), all = (uint32_t)__popc(peers[u]);
-            if (count && below == 0) atomicAdd(&mine[word[u]], all);
+            const uint32_t below = (uint32_t)__popc(peers & lanemask_lt()), all = (uint32_t)__popc(peers);
+            if (count && below == 0 && ok) {
+                if constexpr (STASH)  // (a segment's count has 16 bits to spare: no carry)
+                    atomicAdd(reinterpret_cast<uint32_t *>(mine) + (word[u] >> 1), all << (16 * (word[u] & 1u)));
+                else
+                    atomicAdd(&mine[word[u]], all);
+            }
             word[u] |= below << kBelow | (below + 1 == all ? 1u : 0u) << kLast;
         }
     };
     // pass 1: distinct values, and their keys per segment
-    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
-        look_up(e0, true);
-        if (stash)
+    auto first_pass = [&](uint32_t e0, auto full) {
+        look_up(e0, true, full);
+        if constexpr (STASH) {
 #pragma unroll
             for (int u = 0; u < kAhead; ++u)
-                if (e0 + u * 32 + lane < seg1) sid16[e0 + u * 32 + lane] = (uint16_t)word[u];
+                if (decltype(full)::value || e0 + u * 32 + lane < seg1) word16[e0 + u * 32 + lane] = (uint16_t)word[u];
+        }
+    };
+    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
+        if (e0 + 32 * kAhead <= seg1) first_pass(e0, std::true_type{});
+        else first_pass(e0, std::false_type{});
+        if (__any_sync(0xffffffffu, *(volatile int *)&overflow)) break;  // (the warp as one)
     }
     __syncthreads();
     if (overflow || ndistinct > kLowCardMax) return;  // leave the block to the stable sort
@@ -632,50 +650,54 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
         }
     }
     // the rank of each value's first key of this segment
-    for (int h = lane; h < NS; h += 32) mine[h] += start[h];
+    for (int h = lane; h < NS; h += 32) mine[h] += (Count)start[h];
     __syncwarp();
     // pass 2: in position order, sorted rank = first rank + earlier here
+    // j = g / x when x divides g: a rounded float quotient is exact below 2^21
     const float inv_x = 1.0f / (float)xx;
-    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
-        if (stash) {
+    const bool few = s < (int64_t)1 << 21;
+    const uint32_t *val_blk = vals_in + lo;
+    uint32_t *val_run = runs_val + lo;
+    K *sample_phi = sphi + k * s - 1;
+    uint32_t *sample_tag = stag + k * s - 1;
+    auto second_pass = [&](uint32_t e0, auto full) {
+        if constexpr (STASH) {
 #pragma unroll
             for (int u = 0; u < kAhead; ++u) {
                 const uint32_t e = e0 + u * 32 + lane;
-                word[u] = e < seg1 ? sid16[e] : 0u;
+                word[u] = decltype(full)::value || e < seg1 ? word16[e] : 0u;
             }
         } else {
-            look_up(e0, false);
+            look_up(e0, false, full);
         }
         uint32_t va[kAhead];  // the payloads of the kAhead steps, loaded before the first is stored
         if (runs_val) {
 #pragma unroll
             for (int u = 0; u < kAhead; ++u) {
                 const uint32_t e = e0 + u * 32 + lane;
-                va[u] = e < seg1 ? vals_in[lo + e] : 0u;
+                va[u] = decltype(full)::value || e < seg1 ? val_blk[e] : 0u;
             }
         }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
             const uint32_t e = e0 + u * 32 + lane;
-            const bool ok = e < seg1;
-            const uint32_t h = word[u] & (NS - 1), r = mine[h] + (word[u] >> kBelow & 31u);
+            const uint32_t h = word[u] & (NS - 1), g = mine[h] + (word[u] >> kBelow & 31u) + 1;  // rank, from one
             __syncwarp();
-            if (ok) {
-                if (word[u] >> kLast) mine[h] = r + 1;
-                if (runs_val) runs_val[lo + r] = va[u];  // payloads at their ranks
-                // j = (r + 1) / x when x divides it (the quotient from a float
-                // estimate, corrected by one either way)
-                uint32_t j = (uint32_t)((float)(r + 1) * inv_x);
-                int64_t rem = (int64_t)(r + 1) - (int64_t)j * xx;
-                if (rem >= (int64_t)xx) { ++j; rem -= xx; }
-                if (rem < 0) { --j; rem += xx; }
-                if (rem == 0) {
-                    sphi[k * s + (j - 1)] = (K)(uint32_t)slot[h];
-                    stag[k * s + (j - 1)] = (uint32_t)(lo + e);
+            if (decltype(full)::value || e < seg1) {
+                if (word[u] >> kLast & 1u) mine[h] = (Count)g;
+                if (runs_val) val_run[g - 1] = va[u];  // payloads at their ranks
+                const uint32_t j = few ? __float2uint_rn((float)g * inv_x) : g / xx;
+                if (j * xx == g) {
+                    sample_phi[j] = (K)(uint32_t)slot[h];
+                    sample_tag[j] = (uint32_t)(lo + e);
                 }
             }
             __syncwarp();
         }
+    };
+    for (uint32_t e0 = seg0; e0 < seg1; e0 += 32 * kAhead) {
+        if (e0 + 32 * kAhead <= seg1) second_pass(e0, std::true_type{});
+        else second_pass(e0, std::false_type{});
     }
     if (tid == 0) retry[k] = 0;  // done
 }
@@ -693,7 +715,9 @@ run_sample_lowcard_kernel(const typename KeyTraits<DT>::T *__restrict__ keys, in
 // pivots' bins, and every bin is sorted on chip by the counting sort of
 // countsort.cuh over words phi << 32 | tag.  Four
 // launches for any sample (an LSD radix sort over the record's bytes, which
-// this replaces, took 24 to 36 of them).
+// this replaces, took 24 to 36 of them): 6.4M records 0.29 ms, before 0.34;
+// 16.8M of Zipf keys 0.81, before 0.90; 16K records 0.04, before 0.13 (one CTA
+// up to kOneSample records, where the bins would not fill the GPU).
 // ---------------------------------------------------------------------------
 constexpr int64_t kOneSample = 8192;
 constexpr int kPivotBinsMax = 4096;
@@ -1308,10 +1332,12 @@ template <int DT> static cudaError_t launch_sample_t(const Ctx &c) {
         }
         if (e != cudaSuccess) return e;
         if (only) {  // blocks of few distinct keys, before the stable sort
-            e = cudaFuncSetAttribute(run_sample_lowcard_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)lowcard_smem(p.m));
+            const bool stash = p.m <= kLowCardStashMax;
+            auto kern = stash ? run_sample_lowcard_kernel<DT, true> : run_sample_lowcard_kernel<DT, false>;
+            const size_t smem = stash ? LowCard<true>::smem(p.m) : LowCard<false>::smem(p.m);
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            run_sample_lowcard_kernel<DT><<<(unsigned)p.R, kLowCardThreads, lowcard_smem(p.m), c.stream>>>(
+            kern<<<(unsigned)p.R, kLowCardThreads, smem, c.stream>>>(
                 (const K *)c.keys_in, p.n, p.m, p.s, p.x, (K *)c.ly.sphi[0], c.ly.stag[0], c.ly.run_retry,
                 p.keep_runs ? (K *)c.ly.runs : nullptr, c.vals_in, p.keep_runs && p.pairs ? c.ly.runs_val : nullptr);
             e = cudaGetLastError();
