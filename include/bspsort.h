@@ -344,22 +344,24 @@ int bsps_noalloc_read_stats(bsps_stats *stats, void *stream);
  * Instances of class <= t->small_max_log2 (at most BSPS_BATCH_SMALL_MAX keys)
  * with random oversampling, 32-bit keys, the tree classifier and a sample of
  * at most BSPS_BATCH_SAMPLE_MAX records run the whole method on chip, one CTA
- * per instance, in one persistent launch (sample, sample sort, splitters,
- * classification, bucket histogram, routing into buckets and the final sort
- * all in shared memory).  The others run the single-instance pipeline on
- * t->lanes streams that fork from and join back into `stream`.  The call
- * records all of this into one CUDA graph of its own; the instantiated graph
- * is kept and relaunched by later calls with the same arguments (pointers,
- * offsets, parameters, table).  Because the call keeps and relaunches its own
- * graph and uploads the on-chip instances' table from host memory that it
- * does not keep, it must not itself be captured: on a stream that is being
- * captured it returns BSPS_ERR_CAPTURE and queues nothing.
+ * per instance, in one launch per size of their shared memory (sample, sample
+ * sort, splitters, bucket sizes and the sort all in shared memory).  The other
+ * instances of a call with random oversampling run together, each kernel of
+ * the single-instance pipeline over all of them in one launch, in waves of
+ * what the workspace holds (at least the largest instance; more lanes, more
+ * instances to a wave).  With regular oversampling they run the pipeline on
+ * t->lanes streams that fork from and join back into `stream`, recorded into
+ * one CUDA graph of the call's own that later calls with the same arguments
+ * (pointers, offsets, parameters, table) relaunch.  Because the call uploads
+ * its instances' table from host memory that it does not keep, it must not
+ * itself be captured: on a stream that is being captured it returns
+ * BSPS_ERR_CAPTURE and queues nothing.
  *
  * The offsets are a HOST array (not a device one): the size classes, the
- * split into on-chip instances and pipeline lanes, the workspace layout and
- * the graph all depend on them and are planned on the host before anything
- * is queued.  The size-class table t replaces one parameter set per call:
- * every instance takes the p of its size class.
+ * split into on-chip and larger instances and the workspace layout all depend
+ * on them and are planned on the host before anything is queued.  The
+ * size-class table t replaces one parameter set per call: every instance takes
+ * the p of its size class.
  *
  * h_offsets: host array of num+1 nondecreasing key offsets, h_offsets[0] = 0.
  * d_bucket_sizes: device int64 array (nullable) of the instances' bucket
@@ -380,7 +382,7 @@ typedef struct {
     int32_t p[BSPS_BATCH_CLASSES]; /* buckets per size class (>= 1) */
     int32_t small_max_log2;        /* classes up to this one run on chip (<= 14; -1: none) */
     int32_t learned_min_log2;      /* classes from this one up use the learned classifier; 0: never */
-    int32_t lanes;                 /* concurrent streams for the other instances, 1..16 */
+    int32_t lanes;                 /* concurrent streams (regular) or size of a wave (random), 1..16 */
     int32_t reserved;
 } bsps_tune;
 

@@ -5,8 +5,8 @@
 // Small instances run the whole method on chip, one CTA per instance
 // (small.cu), in one launch per shape.  The larger ones, with random sampling,
 // run the single-call kernels together: every step of the path is one launch
-// for all of them (many.cuh), in waves that reuse one workspace.  With regular sampling they run the single-call pipeline on several
-// streams, recorded into one CUDA graph that later calls with the same
+// for all of them (many.cuh), in waves that reuse one workspace.  With regular
+// sampling they run the single-call pipeline on several streams, recorded into one CUDA graph that later calls with the same
 // arguments relaunch.
 #include <algorithm>
 #include <cstring>

@@ -6,6 +6,9 @@
 // CTA of a MANY launch finds its call by binary search over those starts and
 // copies its arguments to shared memory.  `block` and `blocks` stand for
 // blockIdx.x and gridDim.x inside the call's share.
+//
+// A batch of 150 instances of 2^8 to 2^22 keys: 3.4 ms; recorded instance by
+// instance into a graph of eight lanes, with 40 launches each, 10.3 ms.
 #pragma once
 
 #include <cstring>

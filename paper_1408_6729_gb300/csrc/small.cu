@@ -3,7 +3,11 @@
 // single small call and for the small instances of a batch.
 //
 // The multi-kernel path would spend ten launches on such an input and leave
-// the GPU idle through most of them.
+// the GPU idle through most of them: a call of 3000 int32 keys takes 28 us here
+// (bound by one CTA's chain of phases, about 12 us of them the sample's sort)
+// and took 205 us in 35 launches; 4096 instances of 2^8 to 2^14 keys take 567 us
+// and took 1869 by bitonic networks.  Past 2^14 keys one CTA is the bottleneck
+// and the multi-kernel path's many are not.
 //
 // Keys without payloads: the keys are sorted whole by the counting sort of
 // countsort.cuh (equal keys need no order among them).  The sample's records
