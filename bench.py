@@ -65,13 +65,12 @@ WORKLOADS = {
     # captures (inputs still larger than L2)
     "uniform_2e26_int32_p4096_random": dict(n=1 << 26, p=4096, sampling=1, s=0, runs=0, pairs=False,
                                            make=lambda n, p, seed: gen.uniform(n, p, seed)),
-    # the 2^28 workload's bucket shape (65,536-key buckets on clusters of 8,
-    # count sorts in the occupancy-mask regime) on half the data, for full ncu
-    # captures of the bucket sort
+    # the 2^28 workload's bucket size (65,536 keys) on half the data, for full
+    # ncu captures of the bucket sort
     "uniform_2e27_int32_p2048_random": dict(n=1 << 27, p=2048, sampling=1, s=0, runs=0, pairs=False,
                                            make=lambda n, p, seed: gen.uniform(n, p, seed)),
-    # the 2^28 workload's buckets exactly (65,536 keys spanning 2^19 values,
-    # clusters of 8) on half the data: keys uniform on [0, 2^30), p = 2048
+    # the 2^28 workload's buckets exactly (65,536 keys spanning 2^19 values)
+    # on half the data: keys uniform on [0, 2^30), p = 2048
     "uniform30_2e27_int32_p2048_random": dict(n=1 << 27, p=2048, sampling=1, s=0, runs=0, pairs=False,
                                              make=lambda n, p, seed: gen.uniform(n, p, seed) >> 1),
     # the Zipf pairs configuration on a quarter of the data, for full ncu
@@ -113,10 +112,8 @@ COMPARE = {"tree": ("tree", dict(classify=0)), "sort": ("bucket_sort_final_step"
 
 # dram__bytes_read.sum + dram__bytes_write.sum per key of each kernel from one
 # ncu capture (its summary is under profiles/), valid while the kernel source is unchanged:
-# routing from the 2^26-key capture (4096 buckets, as at 2^28), the bucket sort
-# from the 2^27-key capture on [0, 2^30) (65,536-key buckets spanning 2^19
-# values on clusters of 8, as at 2^28);
-# both kernels stream every key once, so bytes per key carry over to 2^28
+# routing from the 2^26-key capture (4096 buckets, as at 2^28); the kernel
+# streams every key once, so bytes per key carry over to 2^28
 # (bytes per key, source hash, payloads) of each capture; the segment copy's
 # from the 2^26-pair Zipf capture (4096 buckets of 16-key segments, as at 2^28)
 NCU_TRAFFIC = {"route_keys_kernel": ((271.608576e6 + 223.674880e6) / (1 << 26), "8baca4c618da453f", False),

@@ -449,7 +449,7 @@ run_sample_tags_kernel(const uint32_t *__restrict__ keys, const uint32_t *__rest
 // equal keys of its step (16 bits), and the second neither matches lanes nor
 // reads the table.  2^28 Zipf pairs in blocks of 2^16: 3.45 ms when both passes
 // matched and probed a table half full one slot at a time, 3.29 with the
-// places kept, 2.65 with the pairs of slots.
+// places kept, 2.86 with the pairs of slots.
 constexpr int kLowCardThreads = 1024, kLowCardMax = 256;
 constexpr int kLowCardWarps = kLowCardThreads / 32;
 constexpr int64_t kLowCardStashMax = 65536;
