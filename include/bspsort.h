@@ -30,7 +30,10 @@
  *    errors are detected on the host before anything is launched.  Errors
  *    found on the device (bucket overflow, a bounded wait that expired) are
  *    recorded in the workspace and returned by bsps_read_stats().
- *  - In-place use (input == output) is rejected.  Inputs are never modified.
+ *  - In-place use (input == output) is rejected.  Inputs are never modified,
+ *    unless an output lies on one: a single call (not a batch) whose output
+ *    overlaps an input otherwise -- keys_out on vals_in, say -- reads every
+ *    input before it writes an output, so its results are exact.
  */
 #ifndef BSPSORT_H
 #define BSPSORT_H

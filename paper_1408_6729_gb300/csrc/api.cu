@@ -337,6 +337,23 @@ int prepare_keys_call(Ctx &c, const void *keys_in, void *keys_out, int64_t n, in
     return prepare_call(c, keys_in, nullptr, keys_out, nullptr, n, dtype, prm, bucket_sizes, nullptr, ws, ws_bytes, stream);
 }
 
+// Whether an output lies on an input (in part, or an output on the other
+// input: an input as its own output is refused).  Such a call takes the paths
+// that read every input before they write an output, not the ones that read
+// payloads by position while they write, or keys again after the sort.
+static bool output_on_input(const Ctx &c) {
+    const size_t kb = (size_t)c.pl.n * c.pl.key_bytes, vb = (size_t)c.pl.n * 4;
+    auto meet = [](const void *a, size_t na, const void *b, size_t nb) {
+        const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+        return a && b && x < y + nb && y < x + na;
+    };
+    auto written = [&](const void *in, size_t bytes) {
+        return meet(c.keys_out, kb, in, bytes) || meet(c.vals_out, c.pl.pairs ? vb : 0, in, bytes) ||
+               meet(c.bucket_sizes, (size_t)c.pl.p * 8, in, bytes);
+    };
+    return written(c.keys_in, kb) || (c.pl.pairs && written(c.vals_in, vb));
+}
+
 // Random sampling, keys only, n >= 1: the whole path, for one call or for all
 // the calls of a batch (mark(i): phase boundary i).
 template <typename Mark> static int run_keys(Exec &x, Mark mark) {
@@ -365,7 +382,8 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
     Ctx c;
     const int rc = prepare_call(c, keys_in, vals_in, keys_out, vals_out, n, dtype, prm, bucket_sizes, dbg, ws, ws_bytes, stream);
     if (rc) return rc;
-    if (!dbg && small_call(c.pl)) {
+    const bool on_input = output_on_input(c);
+    if (!dbg && !on_input && small_call(c.pl)) {
         BSPS_CUDA(launch_small_call(c));
         return BSPS_OK;
     }
@@ -389,7 +407,7 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
             if (!c.pl.pairs || c.pl.pair_words) BSPS_CUDA(cudaMemsetAsync(c.ly.retry_flag, 0, (size_t)c.pl.P * 4, c.stream));
         }
         // (the test hook of the bounded waits stalls a tile of the look-back routing)
-        const bool words = c.pl.pair_words && c.dbg.stall_tile == 0;
+        const bool words = c.pl.pair_words && !on_input && c.dbg.stall_tile == 0;
         if (c.pl.pairs && !c.pl.keep_runs && !words)
             BSPS_CUDA(cudaMemsetAsync(c.ly.state, 0, (size_t)c.pl.tiles * c.pl.P * 4, c.stream));
         BSPS_CUDA(mark(0));
