@@ -202,7 +202,7 @@ template <bool MANY> __global__ void __launch_bounds__(kMlpThreads) mlp_step_ker
     extern __shared__ __align__(16) float mlp_smem[];
     float *w = mlp_smem, *scratch = mlp_smem + kMlpParamsPad;
     __shared__ float s_loss, s_red[kMlpThreads / 32];
-    __shared__ int s_flag;
+    __shared__ bool s_last, s_keep;  // (two: a warp may still read the first when the second is written)
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, G = (int)pk.blocks;
     float *params = A.params;
     const float *part = A.part;
@@ -222,9 +222,9 @@ template <bool MANY> __global__ void __launch_bounds__(kMlpThreads) mlp_step_ker
     }
     __threadfence();
     __syncthreads();
-    if (t == 0) s_flag = atomicAdd(&opt->ticket, 1u) == (unsigned)G - 1;
+    if (t == 0) s_last = atomicAdd(&opt->ticket, 1u) == (unsigned)G - 1;
     __syncthreads();
-    if (!s_flag) return;
+    if (!s_last) return;
     __threadfence();
     if (t == 0) opt->ticket = 0;
     if (m == 0) return;
@@ -237,11 +237,11 @@ template <bool MANY> __global__ void __launch_bounds__(kMlpThreads) mlp_step_ker
         }
         if (lane == 0) {
             s_loss = l / (float)m;
-            s_flag = A.step == 0 || s_loss < opt->best_loss;
+            s_keep = A.step == 0 || s_loss < opt->best_loss;
         }
     }
     __syncthreads();
-    const bool keep = s_flag;
+    const bool keep = s_keep;
     float g2 = 0.0f;
     if (A.step == 0)
         for (int k = t; k < kParams; k += kMlpThreads) opt->start[k] = w[k];
