@@ -48,6 +48,20 @@ template <typename K> struct RecordBuffers {
     uint32_t *tag[2];
 };
 
+// Dynamic shared memory of a launch, and the most that any launch of the kernel
+// takes.  A kernel's limit belongs to the device, not to the launch: it is set
+// to the most each time, so that two host threads whose calls differ in size
+// cannot lower it between the other's setting and launch.
+struct DynSmem {
+    size_t bytes, most;
+    DynSmem(size_t b) : bytes(b), most(b) {}
+    DynSmem(size_t b, size_t m) : bytes(b), most(m) {}
+    template <typename K> cudaError_t allow(K kernel) const {
+        if (most <= 48 * 1024) return cudaSuccess;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    }
+};
+
 struct Plan {
     int64_t n, p, R, s, m, M, x, q, sample_size;
     int sampling, dtype, pairs, classify;

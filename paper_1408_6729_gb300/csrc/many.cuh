@@ -81,18 +81,16 @@ constexpr uint32_t kNoBlocks = 0xffffffffu;
 
 // Launches `single` for the one call, or `all` once for every call of a batch.
 // make(ctx, args) fills a call's arguments and returns its blocks (0: the call
-// does not run this kernel); smem is enough for any of them.
+// does not run this kernel); smem.bytes is enough for any of them.
 template <typename A, typename K1, typename KN, typename Make>
-cudaError_t launch_calls(Exec &x, K1 single, KN all, unsigned threads, size_t smem, Make make) {
+cudaError_t launch_calls(Exec &x, K1 single, KN all, unsigned threads, DynSmem smem, Make make) {
     if (!x.many) {
         Many<A> m = {};
         const uint32_t blocks = make(x.calls[0], m.one);
         if (blocks == 0) return cudaSuccess;
-        if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(single, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        single<<<blocks, threads, smem, x.stream>>>(m);
+        const cudaError_t e = smem.allow(single);
+        if (e != cudaSuccess) return e;
+        single<<<blocks, threads, smem.bytes, x.stream>>>(m);
         return cudaGetLastError();
     }
     std::vector<A> args;
@@ -113,11 +111,9 @@ cudaError_t launch_calls(Exec &x, K1 single, KN all, unsigned threads, size_t sm
     const unsigned grid = first.back();
     const cudaStream_t stream = x.stream;
     x.later->push_back([=]() -> cudaError_t {
-        if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        all<<<grid, threads, smem, stream>>>(m);
+        const cudaError_t e = smem.allow(all);
+        if (e != cudaSuccess) return e;
+        all<<<grid, threads, smem.bytes, stream>>>(m);
         return cudaGetLastError();
     });
     return cudaSuccess;

@@ -497,9 +497,10 @@ cudaError_t launch_merge_partition(const Ctx &c) {
 
 cudaError_t launch_segment_copy(const Ctx &c) {
     const Plan &p = c.pl;
-    const size_t smem = (size_t)(2 * p.R + 1) * 4;
+    auto bytes = [](int64_t R) { return (size_t)(2 * R + 1) * 4; };
+    const DynSmem smem(bytes(p.R), bytes(kSegRouteRunsMax));
     auto kern = p.pairs ? segment_copy_kernel<true> : segment_copy_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = smem.allow(kern);
     if (e != cudaSuccess) return e;
     SegCopyArgs a;
     a.runs = (const uint32_t *)c.ly.runs;
@@ -518,7 +519,7 @@ cudaError_t launch_segment_copy(const Ctx &c) {
     a.out_vals = c.vals_out;
     a.dtype = p.dtype;
     a.st = c.ly.status;
-    kern<<<(unsigned)p.P, kSegThreads, smem, c.stream>>>(a);
+    kern<<<(unsigned)p.P, kSegThreads, smem.bytes, c.stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -537,14 +538,14 @@ template <bool PAIRS> static cudaError_t launch_merge_buckets_t(const Ctx &c) {
     a.dtype = p.dtype;
     a.cl = p.bucket_cl;
     a.st = c.ly.status;
-    const size_t smem = merge_smem_bytes<PAIRS>(p.R);
+    const DynSmem smem(merge_smem_bytes<PAIRS>(p.R), merge_smem_bytes<PAIRS>(kMergeRunsMax));
     auto kern = merge_bucket_kernel<PAIRS>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = smem.allow(kern);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.p * p.bucket_cl));
     cfg.blockDim = dim3(kMergeThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = smem.bytes;
     cfg.stream = c.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -436,16 +436,16 @@ template <int DT, bool LEARNED> static cudaError_t launch_route_t(const Ctx &c) 
     a.stall_tile = c.dbg.stall_tile;
     a.spin_limit = c.dbg.wait_polls ? c.dbg.wait_polls : kSpinLimit;
     a.tag_floor = c.pl.dup_off ? (uint32_t)(c.pl.n - 1) : 0u;
-    const size_t smem = RouteSmemLayout<K, LEARNED>((uint32_t)p.P).total;
+    const DynSmem smem(RouteSmemLayout<K, LEARNED>((uint32_t)p.P).total, 227 * 1024);  // (make_plan's bound)
     auto kern = route_kernel<DT, LEARNED>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = smem.allow(kern);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kRouteThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kRouteThreads, smem.bytes);
     const int64_t grid = imin64(p.tiles, (int64_t)max(occ, 1) * sms);
-    kern<<<(unsigned)grid, kRouteThreads, smem, c.stream>>>(a);
+    kern<<<(unsigned)grid, kRouteThreads, smem.bytes, c.stream>>>(a);
     return cudaGetLastError();
 }
 

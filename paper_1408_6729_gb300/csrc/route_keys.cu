@@ -468,7 +468,7 @@ template <int DT, bool LEARNED, bool PAIRS = false> static cudaError_t launch_t(
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sms = std::max(sms, 1);
     return launch_calls<RouteKeysArgs<K>>(x, route_keys_kernel<DT, LEARNED, false, PAIRS>,
-                                          route_keys_kernel<DT, LEARNED, !PAIRS, PAIRS>, kRkThreads, smem,
+                                          route_keys_kernel<DT, LEARNED, !PAIRS, PAIRS>, kRkThreads, DynSmem(smem, kRkSmemBudget - 512),
                                           [=](const Ctx &c, RouteKeysArgs<K> &a) {
         if (!takes(c)) return 0u;
         const Plan &p = c.pl;

@@ -772,6 +772,7 @@ template <typename P> using OneSort = BlockSort<typename RecordSink<P>::K, kOneT
 template <typename P> static size_t one_smem(int n) {
     return ((sizeof(typename OneSort<P>::Smem) + 15) & ~size_t(15)) + (size_t)n * sizeof(typename RecordSink<P>::K);
 }
+template <typename P> static size_t pivots_smem(int bins) { return one_smem<P>(pivot_candidates(bins)) + (size_t)bins * sizeof(P); }
 static_assert(OneSort<uint32_t>::kMost >= kOneSample && OneSort<uint64_t>::kMost >= kOneSample, "records one CTA sorts");
 
 template <typename P> struct SortArgs {
@@ -1334,10 +1335,11 @@ template <int DT> static cudaError_t launch_sample_t(const Ctx &c) {
         if (only) {  // blocks of few distinct keys, before the stable sort
             const bool stash = p.m <= kLowCardStashMax;
             auto kern = stash ? run_sample_lowcard_kernel<DT, true> : run_sample_lowcard_kernel<DT, false>;
-            const size_t smem = stash ? LowCard<true>::smem(p.m) : LowCard<false>::smem(p.m);
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const DynSmem smem = stash ? DynSmem(LowCard<true>::smem(p.m), LowCard<true>::smem(kLowCardStashMax))
+                                       : DynSmem(LowCard<false>::smem(p.m));
+            e = smem.allow(kern);
             if (e != cudaSuccess) return e;
-            kern<<<(unsigned)p.R, kLowCardThreads, smem, c.stream>>>(
+            kern<<<(unsigned)p.R, kLowCardThreads, smem.bytes, c.stream>>>(
                 (const K *)c.keys_in, p.n, p.m, p.s, p.x, (K *)c.ly.sphi[0], c.ly.stag[0], c.ly.run_retry,
                 p.keep_runs ? (K *)c.ly.runs : nullptr, c.vals_in, p.keep_runs && p.pairs ? c.ly.runs_val : nullptr);
             e = cudaGetLastError();
@@ -1429,8 +1431,9 @@ template <typename K, int SIZE> static cudaError_t launch_sample_bins(Exec &x) {
 
 template <typename K, int ITEMS> static cudaError_t launch_sample_scatter(Exec &x, int bins) {
     const int64_t wave = 2 * sm_count();
+    const DynSmem smem(pivot_scatter_smem<K, ITEMS>(bins), pivot_scatter_smem<K, ITEMS>(kPivotBinsMax));
     return launch_calls<SortArgs<K>>(x, sample_scatter_kernel<K, ITEMS, false>, sample_scatter_kernel<K, ITEMS, true>,
-                                     kPivotThreads, pivot_scatter_smem<K, ITEMS>(bins), [=](const Ctx &c, SortArgs<K> &a) {
+                                     kPivotThreads, smem, [=](const Ctx &c, SortArgs<K> &a) {
         const int64_t S = c.pl.sample_size, tile = (int64_t)kPivotThreads * ITEMS;
         if (S <= kOneSample || scatter_items(S) != ITEMS) return 0u;
         sort_args(c, a);
@@ -1449,7 +1452,7 @@ template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
     cudaError_t e = cudaSuccess;
     if (one > 0)
         e = launch_calls<SortArgs<K>>(x, sample_one_kernel<K, false>, sample_one_kernel<K, true>, kOneThreads,
-                                      one_smem<K>((int)one), [](const Ctx &c, SortArgs<K> &a) {
+                                      DynSmem(one_smem<K>((int)one), one_smem<K>((int)kOneSample)), [](const Ctx &c, SortArgs<K> &a) {
             if (c.pl.sample_size == 0 || c.pl.sample_size > kOneSample) return 0u;
             a.b = buffers_of<K>(c);
             a.S = c.pl.sample_size;
@@ -1458,7 +1461,7 @@ template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
     if (e != cudaSuccess || most == 0) return e;
     const int bins = pivot_bins(most);
     e = launch_calls<SortArgs<K>>(x, sample_pivots_kernel<K, false>, sample_pivots_kernel<K, true>, kOneThreads,
-                                  one_smem<K>(pivot_candidates(bins)) + (size_t)bins * sizeof(K),
+                                  DynSmem(pivots_smem<K>(bins), pivots_smem<K>(kPivotBinsMax)),
                                   [](const Ctx &c, SortArgs<K> &a) {
         if (c.pl.sample_size <= kOneSample) return 0u;
         sort_args(c, a);
@@ -1467,7 +1470,7 @@ template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
     if (e != cudaSuccess) return e;
     const int64_t wave = 2 * sm_count();
     e = launch_calls<SortArgs<K>>(x, sample_hist_kernel<K, false>, sample_hist_kernel<K, true>, kPivotThreads,
-                                  pivot_smem<K>(bins), [=](const Ctx &c, SortArgs<K> &a) {
+                                  DynSmem(pivot_smem<K>(bins), pivot_smem<K>(kPivotBinsMax)), [=](const Ctx &c, SortArgs<K> &a) {
         if (c.pl.sample_size <= kOneSample) return 0u;
         sort_args(c, a);
         return (uint32_t)imin64(wave, (a.S + 4 * kPivotThreads - 1) / (4 * kPivotThreads));
