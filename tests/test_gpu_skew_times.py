@@ -1,0 +1,51 @@
+"""Inputs with repeated keys cost a bounded multiple of the same call on distinct keys.  Times are
+CUDA events around a phase of the call, the least of several runs, so that only the kernels count;
+the bounds leave room for what the repeats cost by themselves."""
+import numpy as np
+import pytest
+
+from .gpu_util import code_of, lib, to_dev
+
+pytestmark = pytest.mark.gpu
+
+SAMPLE, SAMPLE_SORT, SPLITTERS, ROUTE, SORT = range(5)
+
+
+def phase_us(keys, p, phases, pairs=False, s=0):
+    """Least time of the given phases (one after the other) over ten runs, and the call's statistics."""
+    import torch
+    bsps, n, code = lib(), len(keys), code_of(keys)
+    prm = bsps.make_params(p, s=s, sampling=bsps.BSPS_RANDOM, seed=9)
+    ws = torch.empty(bsps.bsps_workspace_size(n, code, prm, pairs), dtype=torch.uint8, device="cuda:0")
+    kin, sizes = to_dev(keys), torch.empty(p, dtype=torch.int64, device="cuda:0")
+    out, val = torch.empty_like(kin), torch.arange(n, dtype=torch.int32, device="cuda:0") if pairs else None
+    vout = torch.empty_like(val) if pairs else None
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(6)]
+    for e in ev:
+        e.record()
+    best = float("inf")
+    for _ in range(10):
+        assert bsps.bsps_sort_debug(kin, val, out, vout, n, code, prm, sizes, ws, phase_events=ev) == 0
+        torch.cuda.synchronize()
+        best = min(best, 1e3 * ev[phases[0]].elapsed_time(ev[phases[-1] + 1]))
+    assert out.cpu().numpy().tobytes() == np.sort(keys).tobytes()
+    return best, bsps.bsps_read_stats(ws), ws
+
+
+def uniform(n, seed=1):
+    return np.random.default_rng(seed).integers(0, 2**31, n).astype(np.int32)
+
+
+def copies(n, c, seed=2):
+    """About c copies of every value, the values spread over the range."""
+    v = np.random.default_rng(seed).integers(0, max(1, n // c), n).astype(np.int64)
+    return (v * 2654435761 % 2**31).astype(np.int32)
+
+
+# every key equals splitters, whose tags are then searched: log2 of their number more reads a key
+@pytest.mark.parametrize("pairs", [False, True], ids=["keys", "pairs"])
+def test_routing_few_values(pairs):
+    n, p = 1 << 25, 1024
+    few, base = phase_us(copies(n, n // 100), p, [ROUTE], pairs)[0], phase_us(uniform(n), p, [ROUTE], pairs)[0]
+    print(f"routing: few values {few:.0f} us, uniform {base:.0f} us")
+    assert few <= 2.5 * base, (few, base)
