@@ -18,7 +18,8 @@
 //      across their borders (odd-even transposition rounds where a bin needs
 //      more) and writes the middle 224 with 16-byte stores; every bin touching
 //      those lies inside the 256.  Longer bins (skewed or repeated keys) are
-//      listed by the scan and sorted in the stage first: not at all when all
+//      listed by the scan (or, past the list's room, found again by their
+//      cursors) and sorted in the stage first: not at all when all
 //      their keys are equal, else by a warp or, above kWarpBin keys, by the CTA.
 // Per key that is two shared-memory atomics and one shared store, and no
 // exchange between CTAs.
@@ -127,6 +128,7 @@ template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t l
     const uint32_t lane = threadIdx.x & 31;
     if (len <= 32) {
         E x = lane < len ? a[lane] : all_ones<E>();
+        if (!__any_sync(0xffffffffu, lane < len && x != a[0])) return;
 #pragma unroll
         for (int h = 1; h < 32; h <<= 1) {
             if ((uint32_t)h >= len) break;
@@ -361,6 +363,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     static constexpr int kTodo = 16;                 // crowded ranges waiting
     static constexpr uint32_t kUseWide = STAGE / sizeof(K) - 8, kUseNarrow = STAGE / sizeof(S) - 8;
     static_assert(NBMAX % 512 == 0 && kSegs <= 128 && NBMAX <= 65536, "the segments are scanned by one warp, four to a lane");
+    static_assert(kUseNarrow / (kWarpBin + 1) < kLongMax, "a part's bins for the CTA fit the list");
     static_assert(kUseWide < 65528 && STAGE % 16 == 0, "16-bit positions inside a part");
 
     struct Smem {
@@ -368,7 +371,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         uint32_t pseg[kPartsMax + 1];         // first segment of every part
         uint32_t unit[kUnits + 2];            // first position of every unit (narrow stage)
         uint32_t longs[kLongMax];             // bin | length << 16
-        uint32_t nlong, nparts, bad, half, heavy;  // heavy: bit p, part p is one crowded run of 256 bins
+        uint32_t nlong, nbig, nparts, bad, half, heavy;  // heavy: bit p, part p is one crowded run of 256 bins
         uint32_t ntodo, todo_at[kTodo], todo_n[kTodo];
         alignas(16) K todo_lo[kTodo], todo_hi[kTodo];  // ranges still to sort: bounds, first position, keys
         alignas(16) unsigned char sort[sizeof(typename BlockSort<K, T>::Smem)];  // of a long bin by the whole CTA
@@ -380,16 +383,33 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     __device__ static uint32_t *bins(unsigned char *smem) { return reinterpret_cast<uint32_t *>(smem + kHead); }
 
     // The long bins inside bins [b0, b0 + bn), each unsorted in the len slots
-    // that end at its cursor.
+    // that end at its cursor (the first bin's start at slot pad).
     template <typename E, typename End>
-    __device__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, End end_of) {
-        const int tid = threadIdx.x, warp = tid >> 5;
-        const uint32_t nl = sm.nlong;
-        for (uint32_t i = warp; i < nl; i += W) {
-            const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
-            if (b - b0 >= bn || len > (uint32_t)kWarpBin) continue;
-            E *a = stage + (end_of(b) - len);
-            warp_sort(a, len);
+    __device__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, uint32_t pad, End end_of) {
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        uint32_t nl = sm.nlong;
+        if (nl <= (uint32_t)kLongMax) {
+            for (uint32_t i = warp; i < nl; i += W) {
+                const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
+                if (b - b0 >= bn || len > (uint32_t)kWarpBin) continue;
+                warp_sort(stage + (end_of(b) - len), len);
+            }
+        } else {
+            // more than the list holds (values of a few dozen copies each, say):
+            // every bin is looked at, and the list takes those for the CTA
+            if (tid == 0) sm.nbig = 0;
+            __syncthreads();
+            for (uint32_t c = warp * 32; c < bn; c += T) {
+                const uint32_t b = b0 + c + lane, end = end_of(b), len = end - (c + lane > 0 ? end_of(b - 1) : pad);
+                for (uint32_t m = __ballot_sync(0xffffffffu, len > (uint32_t)kEdge); m; m &= m - 1) {
+                    const int l = __ffs(m) - 1;
+                    const uint32_t n = __shfl_sync(0xffffffffu, len, l), at = __shfl_sync(0xffffffffu, end, l) - n;
+                    if (n <= (uint32_t)kWarpBin) warp_sort(stage + at, n);
+                    else if (lane == 0) sm.longs[atomicAdd(&sm.nbig, 1u)] = (b0 + c + l) | n << 16;
+                }
+            }
+            __syncthreads();
+            nl = sm.nbig;
         }
         for (uint32_t i = 0; i < nl; ++i) {
             const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
@@ -592,8 +612,8 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
 
     // Sorts the n keys of src into positions [0, n) of sink, as CTA g of G.
     // Returns false, in every CTA of the segment alike, when it gives up: more
-    // long bins or crowded ranges than the lists hold, or more parts than there
-    // may be.  What was written by then is rewritten by whoever takes over.
+    // crowded ranges than the list holds, more parts than there may be, or more
+    // than 65,535 keys in a bin.  What was written by then is rewritten by whoever takes over.
     template <typename Source, typename Sink>
     __device__ static bool run(unsigned char *smem, const Source &src, int n, K lo, K hi, const Sink &sink, int g, int G) {
         Smem &sm = *reinterpret_cast<Smem *>(smem);
@@ -853,7 +873,6 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             reinterpret_cast<uint4 *>(cnt)[s * 64 + lane * 2 + 1] = make_uint4(out_w[4], out_w[5], out_w[6], out_w[7]);
         }
         __syncthreads();
-        if (sm.nlong > (uint32_t)kLongMax) return false;
         auto slot_of = [&](uint32_t b, uint32_t word) {
             return b > wmask ? (word >> 16) + half : word & 0xffffu;
         };
@@ -892,14 +911,14 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             const int pad = sink.pad(base + p0);
             if constexpr (sizeof(K) <= 8) if (narrow) {
                 if (sm.nlong) {
-                    sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, end_of);
+                    sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, (uint32_t)pad, end_of);
                     __syncthreads();
                 }
                 emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, base, nunits, lo, sink);
             }
             if (!narrow) {
                 if (sm.nlong) {
-                    sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, end_of);
+                    sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, (uint32_t)pad, end_of);
                     __syncthreads();
                 }
                 emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, base + p0, sink);

@@ -49,3 +49,17 @@ def test_routing_few_values(pairs):
     few, base = phase_us(copies(n, n // 100), p, [ROUTE], pairs)[0], phase_us(uniform(n), p, [ROUTE], pairs)[0]
     print(f"routing: few values {few:.0f} us, uniform {base:.0f} us")
     assert few <= 2.5 * base, (few, base)
+
+
+def given_back(ws):
+    """Sub-buckets the counting sort left to the cluster sort (DevStatus::retry_count of csrc/common.cuh)."""
+    import torch
+    return int(ws[:64].view(torch.int32)[14].item())
+
+
+# values of a few dozen copies fill more bins past the window sort's reach than the scan lists
+@pytest.mark.parametrize("n, p, c", [(1 << 20, 16, 20), (1 << 20, 16, 33), (300_000, 4, 24), (200_000, 1, 40), (16_000, 1, 25), (1 << 22, 256, 18)])
+@pytest.mark.parametrize("dt", [np.int32, np.float64])
+def test_many_long_bins_are_not_given_back(n, p, c, dt):
+    keys = copies(n, c).astype(dt)
+    assert given_back(phase_us(keys, p, [SORT])[2]) == 0
