@@ -1,0 +1,507 @@
+// sample_sort.cu -- the sort of the sample's records (Fig. 1 step 5).
+#include <algorithm>
+
+#include "classify.cuh"
+#include "countsort.cuh"
+#include "many.cuh"
+
+namespace bsps {
+
+// ---------------------------------------------------------------------------
+// Sample sort (Fig. 1 step 5): the records (phi, tag) in order.  A sample of at
+// most kOneSample records is sorted by one CTA.  A larger one is itself sample
+// sorted, which no distribution of the keys unbalances: one CTA sorts
+// candidates, one drawn from each of equal stretches of the sample (a plain
+// stride would meet the same rank of every block of a regular sample), every
+// few of them is a pivot (and where several pivots share a key value, so are
+// that value's first and last possible record: a bin then holds no part of it
+// beside other values, whose tags and phi would spread it unevenly), the
+// records are counted and scattered into the
+// pivots' bins, and every bin is sorted on chip by the counting sort of
+// countsort.cuh over words phi << 32 | tag.  Four
+// launches for any sample (an LSD radix sort over the record's bytes, which
+// this replaces, took 24 to 36 of them): 6.4M records 0.29 ms, before 0.34;
+// 16.8M of Zipf keys 0.81, before 0.90; 16K records 0.04, before 0.13 (one CTA
+// up to kOneSample records, where the bins would not fill the GPU).
+// ---------------------------------------------------------------------------
+constexpr int64_t kOneSample = 8192;
+constexpr int kPivotBinsMax = 4096;
+constexpr int kPivotCells = 4096;  // cells of the index over the pivots
+constexpr int kPivotThreads = 512;
+constexpr int kOneThreads = 1024;
+
+// Bins of a sample of S records (a power of two; half of them between chosen
+// pivots, about 512 to 1024 records each up to 2^21 records, half for the ends
+// of repeated values), and the candidates the pivots are chosen from.
+static int pivot_bins(int64_t S) {
+    int b = 64;
+    while (b < kPivotBinsMax / 2 && (int64_t)b * 1024 < S) b *= 2;
+    return 2 * b;
+}
+static int pivot_candidates(int bins) { return std::min(bins * 2, (int)kOneSample / 2); }
+
+// The sample sort's scratch (Layout::pivots): bin counts, starts, cursors and
+// a ticket, the pivots, their index.
+template <typename P> struct PivotScratch {
+    uint32_t *count, *start, *cursor, *ticket;
+    P *phi;
+    uint32_t *tag;
+    LutParams<P> *lutp;
+    uint16_t *lut;
+    __host__ __device__ static size_t bytes(int bins) {
+        return (size_t)bins * 4 * 4 + 64 + (size_t)bins * sizeof(P) + 64 + (kPivotCells + 2) * 2;
+    }
+    PivotScratch() = default;
+    __host__ __device__ PivotScratch(void *at, int bins) {
+        unsigned char *b = (unsigned char *)at;
+        phi = (P *)b;                 b += (size_t)bins * sizeof(P);
+        lutp = (LutParams<P> *)b;     b += 64;
+        count = (uint32_t *)b;        b += (size_t)bins * 4;
+        cursor = (uint32_t *)b;       b += (size_t)bins * 4;
+        ticket = (uint32_t *)b;       b += 16;
+        start = (uint32_t *)b;        b += (size_t)(bins + 4) * 4;
+        tag = (uint32_t *)b;          b += (size_t)bins * 4;
+        lut = (uint16_t *)b;
+    }
+};
+
+size_t sample_scratch_bytes(const Plan &p) {
+    if (p.sample_size <= kOneSample) return 1;
+    const int bins = pivot_bins(p.sample_size);
+    return p.key_bytes == 8 ? PivotScratch<uint64_t>::bytes(bins) : PivotScratch<uint32_t>::bytes(bins);
+}
+int sample_sort_kernels(const Plan &p) { return p.sample_size == 0 ? 0 : p.sample_size <= kOneSample ? 1 : 4; }
+int sample_final(const Plan &p) { return p.sample_size <= kOneSample ? 1 : 0; }
+
+template <typename P> using OneSort = BlockSort<typename RecordSink<P>::K, kOneThreads>;
+template <typename P> static size_t one_smem(int n) {
+    return ((sizeof(typename OneSort<P>::Smem) + 15) & ~size_t(15)) + (size_t)n * sizeof(typename RecordSink<P>::K);
+}
+template <typename P> static size_t pivots_smem(int bins) { return one_smem<P>(pivot_candidates(bins)) + (size_t)bins * sizeof(P); }
+static_assert(OneSort<uint32_t>::kMost >= kOneSample && OneSort<uint64_t>::kMost >= kOneSample, "records one CTA sorts");
+
+template <typename P> struct SortArgs {
+    RecordBuffers<P> b;
+    int64_t S;
+    int cand, bins;
+    PivotScratch<P> sc;
+};
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kOneThreads, 1) sample_one_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    P *out_phi = pk.a.b.phi[1];
+    uint32_t *out_tag = pk.a.b.tag[1];
+    const int S = (int)pk.a.S;
+    using K = typename RecordSink<P>::K;
+    using Smem = typename OneSort<P>::Smem;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    K *a = reinterpret_cast<K *>(smem_raw + ((sizeof(Smem) + 15) & ~size_t(15)));
+    for (int i = threadIdx.x; i < S; i += kOneThreads) a[i] = (K)phi[i] << 32 | tag[i];
+    __syncthreads();
+    OneSort<P>::run(*reinterpret_cast<Smem *>(smem_raw), a, S);
+    for (int i = threadIdx.x; i < S; i += kOneThreads) {
+        out_phi[i] = (P)(a[i] >> 32);
+        out_tag[i] = (uint32_t)a[i];
+    }
+}
+
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kOneThreads, 1) sample_pivots_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    const int64_t S = pk.a.S;
+    const int cand = pk.a.cand, bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    using K = typename RecordSink<P>::K;
+    using Smem = typename OneSort<P>::Smem;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    K *a = reinterpret_cast<K *>(smem_raw + ((sizeof(Smem) + 15) & ~size_t(15)));
+    P *piv_phi = reinterpret_cast<P *>(a + cand);  // bins entries
+    const uint32_t stretch = (uint32_t)(S / cand);
+    for (int i = threadIdx.x; i < bins; i += kOneThreads) sc.count[i] = 0;
+    if (threadIdx.x == 0) *sc.ticket = 0;
+#pragma unroll
+    for (int j = 0; j < (int)(kOneSample / kOneThreads); ++j) {
+        const int i = j * kOneThreads + threadIdx.x;
+        if (i < cand) {
+            // a place in stretch i: the top bits of a multiplicative hash
+            const int64_t r = (int64_t)i * stretch + __umulhi((uint32_t)i * 0x9e3779b1u, stretch);
+            a[i] = (K)phi[r] << 32 | tag[r];
+        }
+    }
+    __syncthreads();
+    OneSort<P>::run(*reinterpret_cast<Smem *>(smem_raw), a, cand);
+    // chosen pivot i: candidate of 1-indexed rank (i + 1) * step.  A value that
+    // two neighbouring pivots share gets two more, before its first and past
+    // its last record.
+    const int chosen = bins / 2 - 1, step = cand / (bins / 2);
+    auto phi_of = [&](int i) { return (P)(a[(i + 1) * step - 1] >> 32); };
+    __shared__ uint32_t tmp[40];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int PER = kPivotBinsMax / 2 / kOneThreads;
+    uint32_t extra[PER], loc = 0;  // 1: before, 2: after
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x * PER + j;
+        extra[j] = 0;
+        if (i < chosen) {
+            const bool as_prev = i > 0 && phi_of(i - 1) == phi_of(i), as_next = i + 1 < chosen && phi_of(i + 1) == phi_of(i);
+            if (as_next && !as_prev) extra[j] = 1;
+            if (as_prev && !as_next && phi_of(i) != all_ones<P>()) extra[j] = 2;
+            loc += 1 + (extra[j] != 0);
+        }
+    }
+    uint32_t tot;
+    const uint32_t ex = warp_excl_scan(loc, &tot);
+    if (lane == 31) tmp[warp] = tot;
+    __syncthreads();
+    uint32_t at = ex, all = 0;
+    for (int w = 0; w < kOneThreads / 32; ++w) {
+        at += w < warp ? tmp[w] : 0u;
+        all += tmp[w];
+    }
+    for (int i = (int)all + threadIdx.x; i < bins; i += kOneThreads) {  // the rest: past every record
+        piv_phi[i] = all_ones<P>();
+        sc.phi[i] = all_ones<P>();
+        sc.tag[i] = 0xffffffffu;
+    }
+    auto put = [&](P f, uint32_t t) {
+        piv_phi[at] = f;
+        sc.phi[at] = f;
+        sc.tag[at] = t;
+        ++at;
+    };
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int i = threadIdx.x * PER + j;
+        if (i < chosen) {
+            if (extra[j] == 1) put(phi_of(i), 0u);
+            put(phi_of(i), (uint32_t)a[(i + 1) * step - 1]);
+            if (extra[j] == 2) put(phi_of(i) + 1, 0u);
+        }
+    }
+    __syncthreads();
+    // the index over the pivots, as over the splitters
+    LutParams<P> lp;
+    lp.base = piv_phi[0];
+    lp.span = piv_phi[all - 1] - lp.base;  // (all >= 31 pivots)
+    const int bl = bit_length<P>(lp.span);
+    lp.shift = bl > 12 ? (uint32_t)(bl - 12) : 0u;
+    lp.nsplit = all;
+    static_assert(kPivotCells == 1 << 12, "cells of the index");
+    if (threadIdx.x == 0) *sc.lutp = lp;
+    for (int c = threadIdx.x; c <= kPivotCells; c += kOneThreads)
+        sc.lut[c] = (uint16_t)lut_cell((uint32_t)c, lp, [&](uint32_t i) { return piv_phi[i]; });
+}
+
+// Records of a CTA's tiles per bin; the last CTA to finish turns the totals
+// into the bins' starts.
+template <typename P> constexpr size_t pivot_smem(int bins) {
+    return 64 + (size_t)bins * (sizeof(P) + 4) + (kPivotCells + 8) * 2;  // (tags, read on ties, stay in global memory)
+}
+template <typename P> struct PivotSmem {
+    LutParams<P> *lp;
+    P *phi;
+    uint32_t *cnt;
+    uint16_t *lut;
+    __device__ PivotSmem(unsigned char *b, int bins) {
+        lp = (LutParams<P> *)b;   b += 64;
+        phi = (P *)b;             b += (size_t)bins * sizeof(P);
+        cnt = (uint32_t *)b;      b += (size_t)bins * 4;
+        lut = (uint16_t *)b;
+    }
+    __device__ void load(const PivotScratch<P> &sc, int bins) {
+        for (int i = threadIdx.x; i < bins; i += kPivotThreads) {
+            phi[i] = sc.phi[i];
+            cnt[i] = 0;
+        }
+        for (int i = threadIdx.x; i <= kPivotCells; i += kPivotThreads) lut[i] = sc.lut[i];
+        if (threadIdx.x == 0) *lp = *sc.lutp;
+        __syncthreads();
+    }
+};
+
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kPivotThreads) sample_hist_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const P *phi = pk.a.b.phi[0];
+    const uint32_t *tag = pk.a.b.tag[0];
+    const int64_t S = pk.a.S;
+    const int bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PivotSmem<P> sm(smem_raw, bins);
+    __shared__ uint32_t tmp[40];
+    __shared__ bool last;
+    sm.load(sc, bins);
+    const LutParams<P> lp = *sm.lp;
+    const int64_t step = (int64_t)pk.blocks * kPivotThreads;
+    for (int64_t r = (int64_t)pk.block * kPivotThreads + threadIdx.x; r < S; r += 4 * step) {
+        P f[4];
+        uint32_t t[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r + j * step < S) {
+                f[j] = phi[r + j * step];
+                t[j] = tag[r + j * step];
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (r + j * step < S) atomicAdd(&sm.cnt[classify_key(f[j], t[j], lp, sm.lut, sm.phi, sc.tag)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads)
+        if (sm.cnt[i]) atomicAdd(&sc.count[i], sm.cnt[i]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(sc.ticket, 1u) == pk.blocks - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads) {
+        sm.cnt[i] = ld_volatile(&sc.count[i]);
+        sc.cursor[i] = 0;
+    }
+    __syncthreads();
+    const uint32_t tot = block_excl_scan_smem<kPivotThreads>(sm.cnt, bins, tmp);
+    for (int i = threadIdx.x; i < bins; i += kPivotThreads) sc.start[i] = sm.cnt[i];
+    if (threadIdx.x == 0) sc.start[bins] = tot;
+}
+
+// Records of a tile, grouped by bin in shared memory, each bin's run written
+// contiguously at its bin's start plus a reserved offset.
+template <typename P, int ITEMS> constexpr size_t pivot_scatter_smem(int bins) {
+    return pivot_smem<P>(bins) + (size_t)bins * 4 + (size_t)kPivotThreads * ITEMS * (sizeof(P) + 4 + 2) + 64;
+}
+template <typename P, int ITEMS, bool MANY>
+__global__ void __launch_bounds__(kPivotThreads) sample_scatter_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const RecordBuffers<P> &b = pk.a.b;
+    const int64_t S = pk.a.S;
+    const int bins = pk.a.bins;
+    const PivotScratch<P> &sc = pk.a.sc;
+    constexpr int TILE = kPivotThreads * ITEMS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PivotSmem<P> sm(smem_raw, bins);
+    unsigned char *at8 = smem_raw + ((pivot_smem<P>(bins) + 15) & ~size_t(15));
+    P *st_f = (P *)at8;
+    uint32_t *st_t = (uint32_t *)(st_f + TILE), *dlt = st_t + TILE;
+    uint16_t *st_b = (uint16_t *)(dlt + bins);
+    __shared__ uint32_t tmp[40];
+    sm.load(sc, bins);
+    const LutParams<P> lp = *sm.lp;
+    const int tid = threadIdx.x;
+    for (int64_t t0 = (int64_t)pk.block * TILE; t0 < S; t0 += (int64_t)pk.blocks * TILE) {
+        const int nh = (int)imin64(TILE, S - t0);
+        P f[ITEMS];
+        uint32_t t[ITEMS], br[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int s = i * kPivotThreads + tid;
+            if (s < nh) {
+                f[i] = b.phi[0][t0 + s];
+                t[i] = b.tag[0][t0 + s];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (i * kPivotThreads + tid < nh) {
+                const uint32_t bin = classify_key(f[i], t[i], lp, sm.lut, sm.phi, sc.tag);
+                br[i] = bin << 16 | atomicAdd(&sm.cnt[bin], 1u);
+            }
+        __syncthreads();
+        for (int i = tid; i < bins; i += kPivotThreads) {
+            const uint32_t c = sm.cnt[i];
+            dlt[i] = c ? sc.start[i] + atomicAdd(&sc.cursor[i], c) : 0u;
+        }
+        __syncthreads();
+        block_excl_scan_smem<kPivotThreads>(sm.cnt, bins, tmp);
+        for (int i = tid; i < bins; i += kPivotThreads) dlt[i] -= sm.cnt[i];  // output slot of tile position s: dlt + s
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (i * kPivotThreads + tid < nh) {
+                const uint32_t bin = br[i] >> 16, pos = sm.cnt[bin] + (br[i] & 0xffffu);
+                st_f[pos] = f[i];
+                st_t[pos] = t[i];
+                st_b[pos] = (uint16_t)bin;
+            }
+        __syncthreads();
+        for (int s = tid; s < nh; s += kPivotThreads) {
+            const uint32_t o = dlt[st_b[s]] + (uint32_t)s;
+            b.phi[1][o] = st_f[s];
+            b.tag[1][o] = st_t[s];
+        }
+        for (int i = tid; i < bins; i += kPivotThreads) sm.cnt[i] = 0;
+        __syncthreads();
+    }
+}
+
+// One bin per CTA, from buffer 1 into its place in buffer 0.  A bin that the
+// counting sort gives back (a run of its bins above the stage: the pivots keep
+// bins near their mean, so this is out of reach in practice) is put in order
+// where it lies by a bitonic network.
+template <typename P, int SIZE, bool MANY>
+__global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
+sample_bins_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    const RecordBuffers<P> &b = pk.a.b;
+    const PivotScratch<P> &sc = pk.a.sc;
+    using K = typename RecordSink<P>::K;
+    using CS = typename CountShape<SIZE>::template Sort<K>;
+    constexpr int T = CountShape<SIZE>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t at = sc.start[pk.block];
+    const int n = (int)(sc.start[pk.block + 1] - at);
+    if (n == 0) return;
+    P *f = b.phi[1] + at;
+    uint32_t *t = b.tag[1] + at;
+    const RecordSource<P, T> src{f, t, 1};
+    K lo, hi;
+    CS::bounds(smem_raw, src, n, lo, hi);
+    if (CS::run(smem_raw, src, n, lo, hi, RecordSink<P>{b.phi[0], b.tag[0], (int64_t)at}, 0, 1)) return;
+    __syncthreads();
+    int n2 = 1;
+    while (n2 < n) n2 <<= 1;
+    auto step = [&](int i, int l) {
+        if (l < n) {
+            const P x = f[i], y = f[l];
+            const uint32_t u = t[i], v = t[l];
+            if (x > y || (x == y && u > v)) {
+                f[i] = y;
+                f[l] = x;
+                t[i] = v;
+                t[l] = u;
+            }
+        }
+    };
+    for (int h = 1; h < n2; h <<= 1) {
+        for (int q = threadIdx.x; q < n2 / 2; q += T) {
+            const int c = (q & ~(h - 1)) * 2, o = q & (h - 1);
+            step(c + o, c + 2 * h - 1 - o);
+        }
+        __syncthreads();
+        for (int j = h >> 1; j > 0; j >>= 1) {
+            for (int q = threadIdx.x; q < n2 / 2; q += T) {
+                const int i = 2 * q - (q & (j - 1));
+                step(i, i + j);
+            }
+            __syncthreads();
+        }
+    }
+    for (int i = threadIdx.x; i < n; i += T) {
+        b.phi[0][at + i] = f[i];
+        b.tag[0][at + i] = t[i];
+    }
+}
+
+static int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(sms, 1);
+}
+
+template <typename K> static RecordBuffers<K> buffers_of(const Ctx &c) {
+    RecordBuffers<K> b;
+    b.phi[0] = (K *)c.ly.sphi[0];
+    b.phi[1] = (K *)c.ly.sphi[1];
+    b.tag[0] = c.ly.stag[0];
+    b.tag[1] = c.ly.stag[1];
+    return b;
+}
+
+template <typename K> static void sort_args(const Ctx &c, SortArgs<K> &a) {
+    a.b = buffers_of<K>(c);
+    a.S = c.pl.sample_size;
+    a.bins = pivot_bins(a.S);
+    a.cand = pivot_candidates(a.bins);
+    a.sc = PivotScratch<K>(c.ly.pivots, a.bins);
+}
+
+// The shape that sorts a bin (its mean is 2 S / bins records, twice that fits
+// the stage), and the tiles of the scatter: 2K records until there are enough
+// of 4K to fill the GPU.
+static int bins_shape(int64_t S, int key_bytes) {
+    if (key_bytes == 8) return kCountRecord;
+    const int64_t half = S / pivot_bins(S);
+    return half <= 700 ? kCountSmall : half <= 2000 ? kCountMedium : kCountLarge;
+}
+static int scatter_items(int64_t S) { return S < (1 << 20) ? 4 : 8; }
+
+template <typename K, int SIZE> static cudaError_t launch_sample_bins(Exec &x) {
+    using CS = typename CountShape<SIZE>::template Sort<typename RecordSink<K>::K>;
+    return launch_calls<SortArgs<K>>(x, sample_bins_kernel<K, SIZE, false>, sample_bins_kernel<K, SIZE, true>,
+                                     CountShape<SIZE>::T, CS::smem_bytes(), [](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample || bins_shape(c.pl.sample_size, sizeof(K)) != SIZE) return 0u;
+        sort_args(c, a);
+        return (uint32_t)a.bins;
+    });
+}
+
+template <typename K, int ITEMS> static cudaError_t launch_sample_scatter(Exec &x, int bins) {
+    const int64_t wave = 2 * sm_count();
+    const DynSmem smem(pivot_scatter_smem<K, ITEMS>(bins), pivot_scatter_smem<K, ITEMS>(kPivotBinsMax));
+    return launch_calls<SortArgs<K>>(x, sample_scatter_kernel<K, ITEMS, false>, sample_scatter_kernel<K, ITEMS, true>,
+                                     kPivotThreads, smem, [=](const Ctx &c, SortArgs<K> &a) {
+        const int64_t S = c.pl.sample_size, tile = (int64_t)kPivotThreads * ITEMS;
+        if (S <= kOneSample || scatter_items(S) != ITEMS) return 0u;
+        sort_args(c, a);
+        return (uint32_t)imin64((S + tile - 1) / tile, wave);
+    });
+}
+
+template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
+    // shared memory: for the largest sample among the calls
+    int64_t one = 0, most = 0;
+    for (int i = 0; i < x.count; ++i) {
+        const int64_t S = x.calls[i].pl.sample_size;
+        if (S <= kOneSample) one = imax64(one, S);
+        else most = imax64(most, S);
+    }
+    cudaError_t e = cudaSuccess;
+    if (one > 0)
+        e = launch_calls<SortArgs<K>>(x, sample_one_kernel<K, false>, sample_one_kernel<K, true>, kOneThreads,
+                                      DynSmem(one_smem<K>((int)one), one_smem<K>((int)kOneSample)), [](const Ctx &c, SortArgs<K> &a) {
+            if (c.pl.sample_size == 0 || c.pl.sample_size > kOneSample) return 0u;
+            a.b = buffers_of<K>(c);
+            a.S = c.pl.sample_size;
+            return 1u;
+        });
+    if (e != cudaSuccess || most == 0) return e;
+    const int bins = pivot_bins(most);
+    e = launch_calls<SortArgs<K>>(x, sample_pivots_kernel<K, false>, sample_pivots_kernel<K, true>, kOneThreads,
+                                  DynSmem(pivots_smem<K>(bins), pivots_smem<K>(kPivotBinsMax)),
+                                  [](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample) return 0u;
+        sort_args(c, a);
+        return 1u;
+    });
+    if (e != cudaSuccess) return e;
+    const int64_t wave = 2 * sm_count();
+    e = launch_calls<SortArgs<K>>(x, sample_hist_kernel<K, false>, sample_hist_kernel<K, true>, kPivotThreads,
+                                  DynSmem(pivot_smem<K>(bins), pivot_smem<K>(kPivotBinsMax)), [=](const Ctx &c, SortArgs<K> &a) {
+        if (c.pl.sample_size <= kOneSample) return 0u;
+        sort_args(c, a);
+        return (uint32_t)imin64(wave, (a.S + 4 * kPivotThreads - 1) / (4 * kPivotThreads));
+    });
+    if (e == cudaSuccess) e = launch_sample_scatter<K, 4>(x, bins);
+    if (e == cudaSuccess) e = launch_sample_scatter<K, 8>(x, bins);
+    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(K) == 8) {
+        return launch_sample_bins<K, kCountRecord>(x);
+    } else {
+        e = launch_sample_bins<K, kCountSmall>(x);
+        if (e == cudaSuccess) e = launch_sample_bins<K, kCountMedium>(x);
+        if (e == cudaSuccess) e = launch_sample_bins<K, kCountLarge>(x);
+        return e;
+    }
+}
+
+cudaError_t launch_sample_sort(Exec &x) {
+    return x.calls[0].pl.key_bytes == 8 ? launch_sample_sort_t<uint64_t>(x) : launch_sample_sort_t<uint32_t>(x);
+}
+
+} // namespace bsps
