@@ -90,11 +90,12 @@ template <typename K> __device__ __forceinline__ int word_bits(K v) {
     else return bit_length<K>(v);
 }
 
-// Ascending bitonic network over a[0..len) by `size` threads, this one being
-// `rank`; every comparator puts the larger key higher, so positions past len
-// act as keys above all others and are never touched.
+// Ascending bitonic network over a[0..len), whose runs of h0 keys are sorted,
+// by `size` threads, this one being `rank`; every comparator puts the larger
+// key higher, so positions past len act as keys above all others and are never
+// touched.
 template <typename E, typename Sync>
-__device__ void bitonic(E *a, int len, int rank, int size, Sync sync) {
+__device__ void bitonic(E *a, int len, int rank, int size, Sync sync, int h0 = 1) {
     int n2 = 1;
     while (n2 < len) n2 <<= 1;
     auto step = [&](int i, int l) {
@@ -106,7 +107,7 @@ __device__ void bitonic(E *a, int len, int rank, int size, Sync sync) {
             }
         }
     };
-    for (int h = 1; h < n2; h <<= 1) {  // runs of h sorted: merge pairs of them
+    for (int h = h0; h < n2; h <<= 1) {  // runs of h sorted: merge pairs of them
         for (int t = rank; t < (n2 >> 1); t += size) {
             const int b = (t & ~(h - 1)) * 2, o = t & (h - 1);
             step(b + o, b + 2 * h - 1 - o);
@@ -122,29 +123,74 @@ __device__ void bitonic(E *a, int len, int rank, int size, Sync sync) {
     }
 }
 
-// One warp's sort of a[0..len): nothing when all keys are equal, in registers
-// up to 32 of them.
-template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t len) {
+// One warp's sort of a[0..len), len <= 32 * R, in registers: R runs of 32, one
+// key to a lane, then pairs of runs merged (a merge's first step pairs mirrored
+// places).
+template <typename E, int R> __device__ __forceinline__ void warp_sort_regs(E *a, uint32_t len) {
     const uint32_t lane = threadIdx.x & 31;
-    if (len <= 32) {
-        E x = lane < len ? a[lane] : all_ones<E>();
-        if (!__any_sync(0xffffffffu, lane < len && x != a[0])) return;
+    E x[R];
 #pragma unroll
-        for (int h = 1; h < 32; h <<= 1) {
-            if ((uint32_t)h >= len) break;
+    for (int r = 0; r < R; ++r) x[r] = r * 32 + lane < len ? a[r * 32 + lane] : all_ones<E>();
+    auto lanes = [&](E &v, int o, int bit) {  // v against the key o lanes away, the lower lane taking the smaller
+        const E y = shfl_xor_any(v, o);
+        v = (lane & bit) == 0 ? (y < v ? y : v) : (y > v ? y : v);
+    };
 #pragma unroll
-            for (int j = h; j > 0; j >>= 1) {
-                const E y = shfl_xor_any(x, j == h ? 2 * h - 1 : j);  // a merge's first step pairs mirrored lanes
-                x = (lane & j) == 0 ? (y < x ? y : x) : (y > x ? y : x);
+    for (int h = 1; h < 32; h <<= 1) {
+        if (R == 1 && (uint32_t)h >= len) break;
+#pragma unroll
+        for (int j = h; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r) lanes(x[r], j == h ? 2 * h - 1 : j, j);
+    }
+#pragma unroll
+    for (int h = 1; h < R; h <<= 1) {
+#pragma unroll
+        for (int g = 0; g < R; g += 2 * h)
+#pragma unroll
+            for (int q = 0; q < h; ++q) {
+                E &u = x[g + q], &v = x[g + 2 * h - 1 - q];
+                const E uu = shfl_xor_any(u, 31), vv = shfl_xor_any(v, 31);
+                u = vv < u ? vv : u;
+                v = uu > v ? uu : v;
             }
-        }
-        if (lane < len) a[lane] = x;
+#pragma unroll
+        for (int j = h >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((r & j) == 0) {
+                    const E u = x[r], v = x[r + j];
+                    x[r] = u < v ? u : v;
+                    x[r + j] = u < v ? v : u;
+                }
+#pragma unroll
+        for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r) lanes(x[r], j, j);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (r * 32 + lane < len) a[r * 32 + lane] = x[r];
+}
+// ... of more than 32 keys: runs of 256 in registers, those merged where they lie.
+template <typename E> __device__ __noinline__ void warp_sort_more(E *a, uint32_t len) {
+    if (len <= 64) {
+        warp_sort_regs<E, 2>(a, len);
         return;
     }
+    for (uint32_t r = 0; r < len; r += 256) warp_sort_regs<E, 8>(a + r, len - r < 256 ? len - r : 256);
+    __syncwarp();
+    if (len > 256) bitonic(a, (int)len, (int)(threadIdx.x & 31), 32, [] { __syncwarp(); }, 256);
+}
+// One warp's sort of a[0..len): nothing when all keys are equal.
+template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t len) {
+    const uint32_t lane = threadIdx.x & 31;
     bool differ = false;
     const E first = a[0];
     for (uint32_t e = lane; e < len; e += 32) differ |= a[e] != first;
-    if (__any_sync(0xffffffffu, differ)) bitonic(a, (int)len, (int)lane, 32, [] { __syncwarp(); });
+    if (!__any_sync(0xffffffffu, differ)) return;
+    if (len <= 32) warp_sort_regs<E, 1>(a, len);
+    else warp_sort_more(a, len);
 }
 
 // A whole CTA's sort of a[0..n) in shared memory that no distribution slows
@@ -301,6 +347,9 @@ template <typename K, typename Inv> struct KeySink {
     K *out;
     Inv inv;  // a sorted key to the word stored
     static constexpr int V = 16 / (int)sizeof(K);
+    // 8-byte keys are emitted in a function of its own: inlined into the sort
+    // it spills there (2^26 uniform doubles in 4096 sub-buckets 766 us, 738)
+    static constexpr bool kApart = sizeof(K) == 8;
     __device__ int pad(uint32_t p) const { return (int)(((uintptr_t)(out + p) / sizeof(K)) & (V - 1)); }
     __device__ void one(int64_t p, K k) const { out[p] = inv(k); }
     template <typename Key> __device__ void eight(int64_t p, Key key) const {
@@ -324,6 +373,7 @@ template <typename P> struct RecordSink {
     P *phi;
     uint32_t *tag;
     int64_t at;  // array index of position 0
+    static constexpr bool kApart = false;
     __device__ int pad(uint32_t p) const { return (int)((at + p) & 3); }
     __device__ void one(int64_t p, K k) const {
         phi[at + p] = (P)(k >> 32);
@@ -357,7 +407,8 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     static constexpr int kWin = 256, kEdge = 16, kStep = kWin - 2 * kEdge;
     static constexpr int kPer = kWin / 32;           // keys of a window per lane
     static constexpr int kLongMax = NBMAX / 16;      // listed long bins
-    static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp
+    static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp,
+    static constexpr int kWarpMany = 1024;           // up to this where there are many
     static constexpr int kPartsMax = 32;
     static constexpr int kUnits = 256;               // units of a narrow stage
     static constexpr int kTodo = 16;                 // crowded ranges waiting
@@ -382,23 +433,33 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     // only part of a segment is written
     __device__ static uint32_t *bins(unsigned char *smem) { return reinterpret_cast<uint32_t *>(smem + kHead); }
 
+    // The slot that bin b's cursor stands at, given its word.
+    __device__ static uint32_t slot_of(uint32_t b, uint32_t word, uint32_t wmask, uint32_t half) {
+        return b > wmask ? (word >> 16) + half : word & 0xffffu;
+    }
+
     // The long bins inside bins [b0, b0 + bn), each unsorted in the len slots
-    // that end at its cursor (the first bin's start at slot pad).
-    template <typename E, typename End>
-    __device__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, uint32_t pad, End end_of) {
+    // that end at its cursor (the first bin's start at slot pad).  A warp sorts a
+    // bin of up to kWarpBin keys, or up to kWarpMany where there are bins for half
+    // of the warps, and the CTA the others one after the other.
+    template <typename E>
+    __device__ __noinline__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, uint32_t pad,
+                                                   const uint32_t *cnt, uint32_t wmask, uint32_t half) {
+        auto end_of = [=](uint32_t b) { return slot_of(b, cnt[b & wmask], wmask, half); };
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         uint32_t nl = sm.nlong;
+        if (tid == 0) sm.nbig = 0;
+        __syncthreads();
         if (nl <= (uint32_t)kLongMax) {
             for (uint32_t i = warp; i < nl; i += W) {
                 const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
-                if (b - b0 >= bn || len > (uint32_t)kWarpBin) continue;
-                warp_sort(stage + (end_of(b) - len), len);
+                if (b - b0 >= bn) continue;
+                if (len <= (uint32_t)kWarpBin) warp_sort(stage + (end_of(b) - len), len);
+                else if (lane == 0) atomicAdd(&sm.nbig, 1u);
             }
         } else {
             // more than the list holds (values of a few dozen copies each, say):
-            // every bin is looked at, and the list takes those for the CTA
-            if (tid == 0) sm.nbig = 0;
-            __syncthreads();
+            // every bin is looked at, and the list takes the larger ones
             for (uint32_t c = warp * 32; c < bn; c += T) {
                 const uint32_t b = b0 + c + lane, end = end_of(b), len = end - (c + lane > 0 ? end_of(b - 1) : pad);
                 for (uint32_t m = __ballot_sync(0xffffffffu, len > (uint32_t)kEdge); m; m &= m - 1) {
@@ -408,17 +469,30 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     else if (lane == 0) sm.longs[atomicAdd(&sm.nbig, 1u)] = (b0 + c + l) | n << 16;
                 }
             }
-            __syncthreads();
-            nl = sm.nbig;
         }
-        for (uint32_t i = 0; i < nl; ++i) {
-            const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
-            if (b - b0 >= bn || len <= (uint32_t)kWarpBin) continue;  // uniform
-            E *a = stage + (end_of(b) - len);
-            bool differ = false;
-            const E first = a[0];
-            for (uint32_t e = tid; e < len; e += T) differ |= a[e] != first;
-            if (__syncthreads_or(differ)) BlockSort<E, T>::run(*reinterpret_cast<typename BlockSort<E, T>::Smem *>(sm.sort), a, (int)len);
+        __syncthreads();
+        const uint32_t nbig = sm.nbig;
+        if (nbig == 0) return;
+        if (nl > (uint32_t)kLongMax) nl = nbig;
+        uint32_t warps_take = kWarpBin;
+        if (nbig >= (uint32_t)W / 2) {
+            warps_take = kWarpMany;
+            for (uint32_t i = warp; i < nl; i += W) {
+                const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
+                if (b - b0 < bn && len > (uint32_t)kWarpBin && len <= warps_take) warp_sort(stage + (end_of(b) - len), len);
+            }
+        }
+        for (uint32_t i = 0; i < nl; i += 32) {  // (every warp reads the same entries, 32 at a time)
+            const uint32_t mine = i + lane < nl ? sm.longs[i + lane] : 0u;
+            const bool big = (mine & 0xffffu) - b0 < bn && mine >> 16 > warps_take;
+            for (uint32_t m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+                const uint32_t w = __shfl_sync(0xffffffffu, mine, __ffs(m) - 1), len = w >> 16;
+                E *a = stage + (end_of(w & 0xffffu) - len);
+                bool differ = false;
+                const E first = a[0];
+                for (uint32_t e = tid; e < len; e += T) differ |= a[e] != first;
+                if (__syncthreads_or(differ)) BlockSort<E, T>::run(*reinterpret_cast<typename BlockSort<E, T>::Smem *>(sm.sort), a, (int)len);
+            }
         }
     }
 
@@ -578,6 +652,16 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     put(sink, from + p0, at, inner, pad, end, [&](int j) { return x[j]; });
             }
         }
+    }
+
+    template <typename Sink>
+    __device__ static __noinline__ void emit_wide_apart(const K *stage, int pad, int np, uint32_t p0, const Sink &sink) {
+        emit_wide(stage, pad, np, p0, sink);
+    }
+    template <typename Sink>
+    __device__ static __noinline__ void emit_narrow_apart(const Smem &sm, const S *stage, int pad, int np, uint32_t p0, uint32_t from,
+                                                          uint32_t nunits, K lo, const Sink &sink) {
+        emit_narrow(sm, stage, pad, np, p0, from, nunits, lo, sink);
     }
 
     // Smallest and largest key of the segment (n >= 1), for every thread.
@@ -873,11 +957,11 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             reinterpret_cast<uint4 *>(cnt)[s * 64 + lane * 2 + 1] = make_uint4(out_w[4], out_w[5], out_w[6], out_w[7]);
         }
         __syncthreads();
-        auto slot_of = [&](uint32_t b, uint32_t word) {
-            return b > wmask ? (word >> 16) + half : word & 0xffffu;
+        auto next_slot = [&](uint32_t b) {
+            return slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u), wmask, half);
         };
         auto place = [&](uint32_t b, K v, K k) {
-            const uint32_t at = slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u));
+            const uint32_t at = next_slot(b);
             if (narrow) reinterpret_cast<S *>(stage)[at] = (S)v;
             else reinterpret_cast<K *>(stage)[at] = k;
         };
@@ -891,12 +975,12 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     src.each(nsrc, [&](K k) {
                         const K v = k - lo;
                         const uint32_t b = bin_of(v);
-                        reinterpret_cast<S *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = (S)v;
+                        reinterpret_cast<S *>(stage)[next_slot(b)] = (S)v;
                     });
                 } else {
                     src.each(nsrc, [&](K k) {
                         const uint32_t b = bin_of(k - lo);
-                        reinterpret_cast<K *>(stage)[slot_of(b, atomicAdd(&cnt[b & wmask], b > wmask ? 0x10000u : 1u))] = k;
+                        reinterpret_cast<K *>(stage)[next_slot(b)] = k;
                     });
                 }
             } else {
@@ -907,21 +991,21 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                 });
             }
             __syncthreads();
-            auto end_of = [&](uint32_t b) { return slot_of(b, cnt[b & wmask]); };
             const int pad = sink.pad(base + p0);
+            if (sm.nlong) {
+                if (sizeof(K) <= 8 && narrow) sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, (uint32_t)pad, cnt, wmask, half);
+                else sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, (uint32_t)pad, cnt, wmask, half);
+                __syncthreads();
+            }
             if constexpr (sizeof(K) <= 8) if (narrow) {
-                if (sm.nlong) {
-                    sort_long(sm, reinterpret_cast<S *>(stage), b0, bn, (uint32_t)pad, end_of);
-                    __syncthreads();
-                }
-                emit_narrow(sm, reinterpret_cast<const S *>(stage), pad, (int)np, p0, base, nunits, lo, sink);
+                const S *halves = reinterpret_cast<const S *>(stage);
+                if constexpr (Sink::kApart) emit_narrow_apart(sm, halves, pad, (int)np, p0, base, nunits, lo, sink);
+                else emit_narrow(sm, halves, pad, (int)np, p0, base, nunits, lo, sink);
             }
             if (!narrow) {
-                if (sm.nlong) {
-                    sort_long(sm, reinterpret_cast<K *>(stage), b0, bn, (uint32_t)pad, end_of);
-                    __syncthreads();
-                }
-                emit_wide(reinterpret_cast<const K *>(stage), pad, (int)np, base + p0, sink);
+                const K *words = reinterpret_cast<const K *>(stage);
+                if constexpr (Sink::kApart) emit_wide_apart(words, pad, (int)np, base + p0, sink);
+                else emit_wide(words, pad, (int)np, base + p0, sink);
             }
             __syncthreads();  // the next part reuses the stage
         }

@@ -38,6 +38,7 @@ template <int DT> struct PairSink {
     uint32_t *keys, *vals;
     const uint32_t *vals_in;
     uint32_t last;
+    static constexpr bool kApart = false;
     __device__ int pad(uint32_t p) const { return (int)(((uintptr_t)(keys + p) >> 2) & 3); }
     __device__ uint32_t val(uint64_t w) const { return vals_in[min((uint32_t)w, last)]; }
     __device__ void one(int64_t p, uint64_t w) const {

@@ -179,6 +179,7 @@ template <int DT> struct SmallSink {
     uint32_t *vals_out;
     const uint16_t *draws;  // by position
     uint16_t *weight;       // by sorted position
+    static constexpr bool kApart = false;
     __device__ int pad(uint32_t p) const { return (int)(((uintptr_t)(keys + p) >> 2) & 3); }
     __device__ void one(int64_t p, uint64_t k) const {
         const uint32_t at = (uint32_t)k;

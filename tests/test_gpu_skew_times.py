@@ -63,3 +63,12 @@ def given_back(ws):
 def test_many_long_bins_are_not_given_back(n, p, c, dt):
     keys = copies(n, c).astype(dt)
     assert given_back(phase_us(keys, p, [SORT])[2]) == 0
+
+
+# ... and where the list holds them, finding the few that need the whole CTA costs little
+@pytest.mark.parametrize("c", [10, 19])
+def test_many_listed_bins(c):
+    n, p = 1 << 26, 1024
+    some, base = phase_us(copies(n, c), p, [SORT])[0], phase_us(uniform(n), p, [SORT])[0]
+    print(f"bucket sort: {c} copies of every key {some:.0f} us, uniform {base:.0f} us")
+    assert some <= 3 * base, (some, base)
