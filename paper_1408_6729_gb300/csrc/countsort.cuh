@@ -85,6 +85,14 @@ template <typename K> __device__ __forceinline__ K shfl_xor_any(K v, int o) {
         return __shfl_xor_sync(0xffffffffu, v, o);
     }
 }
+template <typename K> __device__ __forceinline__ K shfl_any(K v, int lane) {
+    if constexpr (sizeof(K) == 16) {
+        const uint64_t a = __shfl_sync(0xffffffffu, (uint64_t)(v >> 64), lane), b = __shfl_sync(0xffffffffu, (uint64_t)v, lane);
+        return (u128)a << 64 | b;
+    } else {
+        return __shfl_sync(0xffffffffu, v, lane);
+    }
+}
 template <typename K> __device__ __forceinline__ int word_bits(K v) {
     if constexpr (sizeof(K) == 16) return (v >> 64) ? 64 + bit_length<uint64_t>((uint64_t)(v >> 64)) : bit_length<uint64_t>((uint64_t)v);
     else return bit_length<K>(v);
@@ -193,10 +201,74 @@ template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t l
     else warp_sort_more(a, len);
 }
 
-// A whole CTA's sort of a[0..n) in shared memory that no distribution slows
-// down: M keys, one drawn from each of M stretches, are put in order one to a
-// thread (shuffles up to 32 apart), every key finds its bin among them, and a
-// warp finishes each bin.
+// The key that more than half of 32 spread over a[0..len) are equal to, if three
+// tries find it (every warp that asks finds the same).
+template <typename E> __device__ __forceinline__ bool common_key(const E *a, uint32_t len, E &v) {
+    const E s = a[(threadIdx.x & 31) * len / 32];
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t m = __ballot_sync(0xffffffffu, s == a[(i * 13 + 3) * len / 32]);
+        v = a[(i * 13 + 3) * len / 32];
+        if (__popc(m) > 16) return true;
+    }
+    return false;
+}
+
+// One warp's sort of a[0..len) where at most 32 keys differ from one that most
+// are equal to (a value with many copies, and what shares its bin): they are
+// taken out, put in order, and written to the ends.  False, and nothing
+// changed, elsewhere.
+template <typename E> __device__ __noinline__ bool warp_sort_mostly_one(E *a, uint32_t len) {
+    const uint32_t lane = threadIdx.x & 31;
+    E v, other = all_ones<E>();
+    if (!common_key(a, len, v)) return false;
+    uint32_t n = 0, at = 0;  // lane i < n holds the i-th other key and its place
+    for (uint32_t e0 = 0; e0 < len; e0 += 128) {
+        E x[4];
+        bool d[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t e = e0 + j * 32 + lane;
+            x[j] = e < len ? a[e] : v;
+            d[j] = x[j] != v;
+        }
+        if (!__any_sync(0xffffffffu, d[0] | d[1] | d[2] | d[3])) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            for (uint32_t m = __ballot_sync(0xffffffffu, d[j]); m; m &= m - 1) {
+                const int l = __ffs(m) - 1;
+                const E y = shfl_any(x[j], l);
+                if (n == 32) return false;
+                if (lane == n) {
+                    other = y;
+                    at = e0 + j * 32 + l;
+                }
+                ++n;
+            }
+    }
+    if (lane < n) a[at] = v;
+    __syncwarp();
+#pragma unroll
+    for (int h = 1; h < 32; h <<= 1) {
+        if ((uint32_t)h >= n) break;
+#pragma unroll
+        for (int j = h; j > 0; j >>= 1) {
+            const E y = shfl_xor_any(other, j == h ? 2 * h - 1 : j);
+            other = (lane & j) == 0 ? (y < other ? y : other) : (y > other ? y : other);
+        }
+    }
+    const uint32_t below = (uint32_t)__popc(__ballot_sync(0xffffffffu, lane < n && other < v));
+    if (lane < n) a[lane < below ? lane : len - n + lane] = other;
+    __syncwarp();
+    return true;
+}
+
+// A whole CTA's sort of a[0..n) in shared memory, in time that hardly depends on
+// the keys: M of them, one drawn from each of M stretches, are put in order one
+// to a thread (shuffles up to 32 apart), every key finds its place among them --
+// equal to one, which needs no more order, or between two -- and a warp
+// finishes each gap.  (A bin of 5000 copies of a value and a few other keys:
+// 2^22 keys, nine in ten of them copies, 1.56 ms when the gap above a pivot held
+// the pivot's copies, too, and 0.41 by the cluster sort.)
 template <typename E, int T> struct BlockSort {
     static constexpr int M = T < 512 ? T : 512, ITEMS = T == 1024 ? 8 : 16, kMost = T * ITEMS;
     struct Smem {
@@ -228,8 +300,38 @@ template <typename E, int T> struct BlockSort {
         __syncthreads();
     }
 
+    // As warp_sort_mostly_one, by the CTA, with at most M other keys.
+    __device__ __noinline__ static bool mostly_one(Smem &sm, E *a, int n) {
+        const int t = threadIdx.x;
+        E v;
+        if (!common_key(a, (uint32_t)n, v)) return false;  // (every warp alike)
+        if (t == 0) sm.cnt[M] = 0;
+        __syncthreads();
+        for (int e = t; e < n; e += T)
+            if (a[e] != v) {
+                const uint32_t k = atomicAdd(&sm.cnt[M], 1u);
+                if (k < (uint32_t)M) {
+                    sm.piv[k] = a[e];
+                    sm.cnt[k] = (uint32_t)e;
+                }
+            }
+        __syncthreads();
+        const int c = (int)min(sm.cnt[M], (uint32_t)M + 1);
+        const E x = t < min(c, M) ? sm.piv[t] : all_ones<E>();
+        const uint32_t at = t < min(c, M) ? sm.cnt[t] : 0u;
+        __syncthreads();
+        if (c > M) return false;
+        if (c == 0) return true;
+        if (t < c) a[at] = v;
+        sort_pivots(sm.piv, x);
+        const int below = __syncthreads_count(t < c && sm.piv[t] < v);
+        if (t < c) a[t < below ? t : n - c + t] = sm.piv[t];
+        __syncthreads();
+        return true;
+    }
+
     __device__ __noinline__ static void run(Smem &sm, E *a, int n) {
-        const int t = threadIdx.x, warp = t >> 5;
+        const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
         if (n <= M) {
             sort_pivots(sm.piv, t < n ? a[t] : all_ones<E>());
             if (t < n) a[t] = sm.piv[t];
@@ -245,30 +347,45 @@ template <typename E, int T> struct BlockSort {
         if (t < M) x = a[(uint32_t)t * stretch + __umulhi((uint32_t)t * 0x9e3779b1u, stretch)];
         for (int i = t; i < M + 4; i += T) sm.cnt[i] = 0;
         sort_pivots(sm.piv, x);
+        // bin b, the keys with b pivots (of the first M - 1) at or below them:
+        // copies of the last of those (count in the low half), then the others
         E k[ITEMS];
-        uint32_t br[ITEMS];
+        uint32_t br[ITEMS];  // bin << 16 | copy << 15 | place among its kind
+        static_assert(kMost <= 0x7fff + 1, "places of 15 bits");
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
             const int e = i * T + t;
             if (e < n) {
                 k[i] = a[e];
-                uint32_t b = 0;  // pivots 0 .. M - 2 at or below the key
+                uint32_t b = 0;
 #pragma unroll
                 for (int w = M / 2; w > 0; w >>= 1)
                     if (!(k[i] < sm.piv[b + w - 1])) b += w;
-                br[i] = b << 16 | atomicAdd(&sm.cnt[b], 1u);
+                const bool copy = b > 0 && !(sm.piv[b - 1] < k[i]);
+                const uint32_t old = atomicAdd(&sm.cnt[b], copy ? 1u : 0x10000u);
+                br[i] = b << 16 | (copy ? 0x8000u | (old & 0xffffu) : old >> 16);
             }
         }
         __syncthreads();
-        const uint32_t total = block_excl_scan_smem<T>(sm.cnt, M, sm.tmp);
-        if (t == 0) sm.cnt[M] = total;
+        // each bin's first place and its copies
+        const uint32_t c = t < M ? sm.cnt[t] : 0u;
+        uint32_t tot;
+        uint32_t first = warp_excl_scan((c & 0xffffu) + (c >> 16), &tot);
+        if (lane == 31) sm.tmp[warp] = tot;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) first += sm.tmp[w];
+        if (t < M) sm.cnt[t] = first | c << 16;
+        if (t == 0) sm.cnt[M] = (uint32_t)n;
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i)
-            if (i * T + t < n) a[sm.cnt[br[i] >> 16] + (br[i] & 0xffffu)] = k[i];
+            if (i * T + t < n) {
+                const uint32_t w = sm.cnt[br[i] >> 16];
+                a[(w & 0xffffu) + ((br[i] & 0x8000u) ? 0u : w >> 16) + (br[i] & 0x7fffu)] = k[i];
+            }
         __syncthreads();
         for (int b = warp; b < M; b += T / 32) {
-            const uint32_t at = sm.cnt[b], len = sm.cnt[b + 1] - at;
+            const uint32_t at = (sm.cnt[b] & 0xffffu) + (sm.cnt[b] >> 16), len = (sm.cnt[b + 1] & 0xffffu) - at;
             if (len >= 2) warp_sort(a + at, len);
         }
         __syncthreads();
@@ -408,7 +525,8 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     static constexpr int kPer = kWin / 32;           // keys of a window per lane
     static constexpr int kLongMax = NBMAX / 16;      // listed long bins
     static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp,
-    static constexpr int kWarpMany = 1024;           // up to this where there are many
+    static constexpr int kWarpMany = 1024;           // up to this where there are many, and nearly
+    static constexpr int kWarpMost = 8192;           // one value up to this
     static constexpr int kPartsMax = 32;
     static constexpr int kUnits = 256;               // units of a narrow stage
     static constexpr int kTodo = 16;                 // crowded ranges waiting
@@ -440,8 +558,9 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
 
     // The long bins inside bins [b0, b0 + bn), each unsorted in the len slots
     // that end at its cursor (the first bin's start at slot pad).  A warp sorts a
-    // bin of up to kWarpBin keys, or up to kWarpMany where there are bins for half
-    // of the warps, and the CTA the others one after the other.
+    // bin of up to kWarpBin keys, up to kWarpMany where there are bins for half
+    // of the warps, and up to kWarpMost of nearly one value; the CTA takes the
+    // others one after the other.
     template <typename E>
     __device__ __noinline__ static void sort_long(Smem &sm, E *stage, uint32_t b0, uint32_t bn, uint32_t pad,
                                                    const uint32_t *cnt, uint32_t wmask, uint32_t half) {
@@ -454,8 +573,14 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             for (uint32_t i = warp; i < nl; i += W) {
                 const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
                 if (b - b0 >= bn) continue;
-                if (len <= (uint32_t)kWarpBin) warp_sort(stage + (end_of(b) - len), len);
-                else if (lane == 0) atomicAdd(&sm.nbig, 1u);
+                E *a = stage + (end_of(b) - len);
+                if (len <= (uint32_t)kWarpBin) {
+                    warp_sort(a, len);
+                } else if (len <= (uint32_t)kWarpMost && warp_sort_mostly_one(a, len)) {
+                    if (lane == 0) sm.longs[i] = 0;  // done
+                } else if (lane == 0) {
+                    atomicAdd(&sm.nbig, 1u);
+                }
             }
         } else {
             // more than the list holds (values of a few dozen copies each, say):
@@ -466,7 +591,9 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
                     const int l = __ffs(m) - 1;
                     const uint32_t n = __shfl_sync(0xffffffffu, len, l), at = __shfl_sync(0xffffffffu, end, l) - n;
                     if (n <= (uint32_t)kWarpBin) warp_sort(stage + at, n);
-                    else if (lane == 0) sm.longs[atomicAdd(&sm.nbig, 1u)] = (b0 + c + l) | n << 16;
+                    else if (n > (uint32_t)kWarpMost || !warp_sort_mostly_one(stage + at, n)) {
+                        if (lane == 0) sm.longs[atomicAdd(&sm.nbig, 1u)] = (b0 + c + l) | n << 16;
+                    }
                 }
             }
         }
@@ -488,10 +615,9 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             for (uint32_t m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
                 const uint32_t w = __shfl_sync(0xffffffffu, mine, __ffs(m) - 1), len = w >> 16;
                 E *a = stage + (end_of(w & 0xffffu) - len);
-                bool differ = false;
-                const E first = a[0];
-                for (uint32_t e = tid; e < len; e += T) differ |= a[e] != first;
-                if (__syncthreads_or(differ)) BlockSort<E, T>::run(*reinterpret_cast<typename BlockSort<E, T>::Smem *>(sm.sort), a, (int)len);
+                using BS = BlockSort<E, T>;
+                typename BS::Smem &bs = *reinterpret_cast<typename BS::Smem *>(sm.sort);
+                if (!BS::mostly_one(bs, a, (int)len)) BS::run(bs, a, (int)len);
             }
         }
     }

@@ -72,3 +72,18 @@ def test_many_listed_bins(c):
     some, base = phase_us(copies(n, c), p, [SORT])[0], phase_us(uniform(n), p, [SORT])[0]
     print(f"bucket sort: {c} copies of every key {some:.0f} us, uniform {base:.0f} us")
     assert some <= 3 * base, (some, base)
+
+
+def heavy(n, c, share, seed=3):
+    """Distinct keys, and a share of the keys on values of about c copies each."""
+    rng = np.random.default_rng(seed)
+    return np.where(rng.random(n) < share, copies(n, c, seed + 1), uniform(n, seed + 2))
+
+
+# values with thousands of copies, each sharing its bin with a few other keys
+@pytest.mark.parametrize("c, share", [(5000, 0.3), (5000, 0.9), (40_000, 0.5)])
+def test_heavy_values_among_distinct_keys(c, share):
+    n, p = 1 << 24, 256
+    some, base = phase_us(heavy(n, c, share), p, [SORT])[0], phase_us(uniform(n), p, [SORT])[0]
+    print(f"bucket sort: {share} of the keys on values of {c} copies {some:.0f} us, uniform {base:.0f} us")
+    assert some <= 6 * base, (some, base)
