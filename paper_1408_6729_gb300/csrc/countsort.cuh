@@ -180,15 +180,23 @@ template <typename E, int R> __device__ __forceinline__ void warp_sort_regs(E *a
     for (int r = 0; r < R; ++r)
         if (r * 32 + lane < len) a[r * 32 + lane] = x[r];
 }
-// ... of more than 32 keys: runs of 256 in registers, those merged where they lie.
+// ... of more than 32 keys: runs of 256 in registers, those merged where they
+// lie (128-bit words, which would fill the registers, all where they lie).
 template <typename E> __device__ __noinline__ void warp_sort_more(E *a, uint32_t len) {
-    if (len <= 64) {
-        warp_sort_regs<E, 2>(a, len);
-        return;
+    const int lane = (int)(threadIdx.x & 31);
+    if constexpr (sizeof(E) <= 8) {
+        if (len <= 64) {
+            warp_sort_regs<E, 2>(a, len);
+        } else if (len <= 128) {
+            warp_sort_regs<E, 4>(a, len);
+        } else {
+            for (uint32_t r = 0; r < len; r += 256) warp_sort_regs<E, 8>(a + r, len - r < 256 ? len - r : 256);
+            __syncwarp();
+            if (len > 256) bitonic(a, (int)len, lane, 32, [] { __syncwarp(); }, 256);
+        }
+    } else {
+        bitonic(a, (int)len, lane, 32, [] { __syncwarp(); });
     }
-    for (uint32_t r = 0; r < len; r += 256) warp_sort_regs<E, 8>(a + r, len - r < 256 ? len - r : 256);
-    __syncwarp();
-    if (len > 256) bitonic(a, (int)len, (int)(threadIdx.x & 31), 32, [] { __syncwarp(); }, 256);
 }
 // One warp's sort of a[0..len): nothing when all keys are equal.
 template <typename E> __device__ __forceinline__ void warp_sort(E *a, uint32_t len) {
@@ -525,7 +533,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
     static constexpr int kPer = kWin / 32;           // keys of a window per lane
     static constexpr int kLongMax = NBMAX / 16;      // listed long bins
     static constexpr int kWarpBin = 256;             // long bins up to this size are sorted by one warp,
-    static constexpr int kWarpMany = 1024;           // up to this where there are many, and nearly
+    static constexpr int kWarpMany = T < 1024 ? kWarpBin : 1024;  // up to this where there are many, and nearly
     static constexpr int kWarpMost = 8192;           // one value up to this
     static constexpr int kPartsMax = 32;
     static constexpr int kUnits = 256;               // units of a narrow stage
@@ -602,7 +610,7 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
         if (nbig == 0) return;
         if (nl > (uint32_t)kLongMax) nl = nbig;
         uint32_t warps_take = kWarpBin;
-        if (nbig >= (uint32_t)W / 2) {
+        if (kWarpMany > kWarpBin && nbig >= (uint32_t)W / 2) {
             warps_take = kWarpMany;
             for (uint32_t i = warp; i < nl; i += W) {
                 const uint32_t b = sm.longs[i] & 0xffffu, len = sm.longs[i] >> 16;
@@ -860,6 +868,10 @@ template <typename K, int T, int NBMAX, int STAGE> struct CountSort {
             if (threadIdx.x == 0) sm.ntodo = t - 1;
             K lo, hi;  // of the keys themselves: what crowds may be far narrower than its bins
             bounds(smem, in, n, lo, hi);
+            if (lo == hi) {  // copies of one value: no need to count them
+                for (uint32_t e = g * T + threadIdx.x; e < keys; e += G * T) sink.one((int64_t)at + e, lo);
+                continue;
+            }
             if (!run_range(smem, in, n, keys, lo, hi, at, sink, g, G)) return false;
         }
     }

@@ -87,3 +87,11 @@ def test_heavy_values_among_distinct_keys(c, share):
     some, base = phase_us(heavy(n, c, share), p, [SORT])[0], phase_us(uniform(n), p, [SORT])[0]
     print(f"bucket sort: {share} of the keys on values of {c} copies {some:.0f} us, uniform {base:.0f} us")
     assert some <= 6 * base, (some, base)
+
+
+# a few values a bucket, of tens of thousands of copies each: every range of bins that holds one is crowded
+def test_few_values_a_bucket():
+    n, p = 1 << 24, 256
+    some, base = phase_us(copies(n, 30_000).astype(np.float64), p, [SORT])[0], phase_us(uniform(n).astype(np.float64), p, [SORT])[0]
+    print(f"bucket sort: values of 30000 copies {some:.0f} us, uniform {base:.0f} us")
+    assert some <= 1.5 * base, (some, base)
