@@ -287,6 +287,7 @@ static int kernels_per_call(const Ctx &c) {
     if (pl.merge) return k + 3;                  // partition, bucket offsets, merge
     k += 2;                                      // routing (partition and segment copy: one more), bucket offsets
     if (pl.seg_route) k += 1;
+    if (c.both_routes) k += 2;                   // the look-back route and its cluster sort
     k += 3;                                      // copy or keys-only tier, cluster sort, out-of-core sort
     if (pl.classify == BSPS_LEARNED) k += mlp_train_kernels();  // training set, start, Adam steps, tables, index
     return k;
@@ -354,6 +355,20 @@ static bool output_on_input(const Ctx &c) {
     return written(c.keys_in, kb) || (c.pl.pairs && written(c.vals_in, vb));
 }
 
+// Whether pairs that can move as words are queued on the look-back route, too,
+// and the device takes that where the sample's keys repeat.  As words the
+// payloads are gathered by position at the end, and the words of one key value
+// are sorted by position; the look-back route carries payloads along in input
+// order, so sub-buckets of one value are copied.  Times in us, words / look-back
+// route: 2^26 uniform pairs in 65,536-pair buckets 3375 / 8541, of 256 Zipf
+// values 3550 / 2900; 2^24 in 4096-pair buckets 1062 / 1510 and 1260 / 1185; 2^22
+// pairs in 65,536-pair buckets 247 / 774 and 664 / 575, in 8192-pair buckets 264
+// / 558 and 483 / 555.  Below that the words are faster for any keys, and the
+// second route's launches (about 5 us) are left out.
+static bool pairs_on_both_routes(const Plan &p) {
+    return p.sample_size >= 64 && p.n >= (1 << 16) && (p.n >= ((int64_t)1 << 23) || p.n / p.P >= 24576);
+}
+
 // Random sampling, keys only, n >= 1: the whole path, for one call or for all
 // the calls of a batch (mark(i): phase boundary i).
 template <typename Mark> static int run_keys(Exec &x, Mark mark) {
@@ -408,7 +423,8 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
         }
         // (the test hook of the bounded waits stalls a tile of the look-back routing)
         const bool words = c.pl.pair_words && !on_input && c.dbg.stall_tile == 0;
-        if (c.pl.pairs && !c.pl.keep_runs && !words)
+        c.both_routes = words && pairs_on_both_routes(c.pl);
+        if (c.pl.pairs && !c.pl.keep_runs && (!words || (c.both_routes && !random)))  // (else the random sample clears it)
             BSPS_CUDA(cudaMemsetAsync(c.ly.state, 0, (size_t)c.pl.tiles * c.pl.P * 4, c.stream));
         BSPS_CUDA(mark(0));
         BSPS_CUDA(random ? launch_sample_random(x) : launch_sample(c));
@@ -442,6 +458,7 @@ static int run(const void *keys_in, const uint32_t *vals_in, void *keys_out, uin
                                             c.stream));
         } else {
             BSPS_CUDA(words ? launch_route_words(x) : c.pl.pairs ? launch_route(c) : launch_route_keys(x));
+            if (c.both_routes) BSPS_CUDA(launch_route(c));
             BSPS_CUDA(launch_bucket_finish(x));
             BSPS_CUDA(mark(4));
             BSPS_CUDA(words ? launch_pair_words(x) : bucket_sort());

@@ -19,6 +19,17 @@ cudaError_t launch_bucket_keys(Exec &x) {
     }
 }
 
+template <int DT> static cudaError_t launch_pairs_cluster(Exec &x) {
+    constexpr int IT = sizeof(typename KeyTraits<DT>::T) == 8 ? kPairItems64 : kPairItems32;
+    switch (x.calls[0].pl.bucket_cl) {
+    case 1: return launch_cluster<DT, true, 1, IT>(x);
+    case 2: return launch_cluster<DT, true, 2, IT>(x);
+    case 4: return launch_cluster<DT, true, 4, IT>(x);
+    case 8: return launch_cluster<DT, true, 8, IT>(x);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 template <int DT> static cudaError_t launch_bucket_pairs_t(Exec &x) {
     using K = typename KeyTraits<DT>::T;
     const Ctx &c = x.calls[0];
@@ -29,14 +40,7 @@ template <int DT> static cudaError_t launch_bucket_pairs_t(Exec &x) {
         a, c.ly.retry_list, &c.ly.status->retry_count);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    constexpr int IT = sizeof(K) == 8 ? kPairItems64 : kPairItems32;
-    switch (c.pl.bucket_cl) {
-    case 1: e = launch_cluster<DT, true, 1, IT>(x); break;
-    case 2: e = launch_cluster<DT, true, 2, IT>(x); break;
-    case 4: e = launch_cluster<DT, true, 4, IT>(x); break;
-    case 8: e = launch_cluster<DT, true, 8, IT>(x); break;
-    default: return cudaErrorInvalidValue;
-    }
+    e = launch_pairs_cluster<DT>(x);
     return e != cudaSuccess ? e : launch_slow<DT, true>(x);
 }
 
@@ -46,6 +50,17 @@ cudaError_t launch_bucket_pairs(Exec &x) {
     case BSPS_I32: return launch_bucket_pairs_t<BSPS_I32>(x);
     case BSPS_F32: return launch_bucket_pairs_t<BSPS_F32>(x);
     default: return launch_bucket_pairs_t<BSPS_F64>(x);
+    }
+}
+
+// The stable cluster sort alone, of the sub-buckets that pairs.cu lists when the
+// keys repeat.
+cudaError_t launch_repeats_cluster(Exec &x) {
+    switch (x.calls[0].pl.dtype) {
+    case BSPS_U32: return launch_pairs_cluster<BSPS_U32>(x);
+    case BSPS_I32: return launch_pairs_cluster<BSPS_I32>(x);
+    case BSPS_F32: return launch_pairs_cluster<BSPS_F32>(x);
+    default: return cudaErrorInvalidValue;
     }
 }
 

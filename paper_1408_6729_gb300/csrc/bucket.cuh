@@ -35,6 +35,8 @@ template <typename K> struct BucketArgs {
     int64_t slow_above;       // keys a cluster of the stable sort holds
     int one_value_done;       // sub-buckets of one key value are already in the output
     int G;                    // tier 1: CTAs per sub-bucket
+    int only_repeats;         // pairs queued on both routes: this one runs if the sample's keys repeat
+    uint32_t few_above;       // ... more often than this
     K *reg_keys_rw;           // tier 3 sorts between the regions and the output
     uint32_t *reg_vals_rw;
 };
@@ -65,6 +67,8 @@ bucket_sort_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
         if (!__syncthreads_or(any)) return;  // (every CTA of the grid alike)
     }
     each_call<MANY>(many, [&](const BucketArgs<K> &a) {
+    if constexpr (PAIRS)
+        if (a.only_repeats && a.st->repeats <= a.few_above) return;
     const int64_t nitems = *a.only_count, clusters = gridDim.x / CL;
     for (int64_t it = blockIdx.x / CL; it < nitems; it += clusters) {
         const int64_t v = a.only[it];
@@ -286,6 +290,8 @@ template <int DT> static void bucket_args(const Ctx &c, BucketArgs<typename KeyT
     a.only_count = &c.ly.status->retry_count;
     a.slow_above = (int64_t)8 * 1024 * (sizeof(K) == 8 ? kBucketItems64 : kBucketItems32);
     a.one_value_done = c.pl.seg_route;
+    a.only_repeats = c.both_routes;
+    a.few_above = repeats_above(c.pl);
     a.reg_keys_rw = (K *)c.ly.reg_keys;
     a.reg_vals_rw = c.ly.reg_vals;
 }

@@ -65,7 +65,8 @@ struct DevStatus {
     uint32_t run_too_big;       // a block of the regular sample did not fit on chip
     int32_t retry_count;        // sub-buckets for the stable cluster sort (keys only: given back)
     int32_t slow_count;         // entries of the out-of-core list
-    uint32_t pad_[4];
+    uint32_t repeats;           // of kRepeatProbes neighbours in the sorted sample, those of equal phi
+    uint32_t pad_[3];
 };
 
 __device__ __forceinline__ void set_error(DevStatus *st, int code) {

@@ -381,7 +381,9 @@ template <typename E, int T> struct BlockSort {
         uint32_t first = warp_excl_scan((c & 0xffffu) + (c >> 16), &tot);
         if (lane == 31) sm.tmp[warp] = tot;
         __syncthreads();
-        for (int w = 0; w < warp; ++w) first += sm.tmp[w];
+        uint32_t all;
+        const uint32_t before = warp_excl_scan(lane < T / 32 ? sm.tmp[lane] : 0u, &all);
+        first += __shfl_sync(0xffffffffu, before, warp);
         if (t < M) sm.cnt[t] = first | c << 16;
         if (t == 0) sm.cnt[M] = (uint32_t)n;
         __syncthreads();
@@ -392,9 +394,23 @@ template <typename E, int T> struct BlockSort {
                 a[(w & 0xffffu) + ((br[i] & 0x8000u) ? 0u : w >> 16) + (br[i] & 0x7fffu)] = k[i];
             }
         __syncthreads();
+        // the gaps: a few keys by one thread, more by a warp
+        constexpr uint32_t kByThread = 4;
+        if (t < M) {
+            const uint32_t at = (sm.cnt[t] & 0xffffu) + (sm.cnt[t] >> 16), end = sm.cnt[t + 1] & 0xffffu;
+            if (end - at <= kByThread)
+                for (uint32_t i = at + 1; i < end; ++i) {
+                    const E y = a[i];
+                    uint32_t j = i;
+                    for (; j > at && y < a[j - 1]; --j) a[j] = a[j - 1];
+                    a[j] = y;
+                }
+        }
         for (int b = warp; b < M; b += T / 32) {
             const uint32_t at = (sm.cnt[b] & 0xffffu) + (sm.cnt[b] >> 16), len = (sm.cnt[b + 1] & 0xffffu) - at;
-            if (len >= 2) warp_sort(a + at, len);
+            if (len <= kByThread) continue;
+            if (len <= 32) warp_sort_regs<E, 1>(a + at, len);
+            else warp_sort_more(a + at, len);
         }
         __syncthreads();
     }

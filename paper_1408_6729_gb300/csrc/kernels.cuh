@@ -131,6 +131,7 @@ struct Ctx {
     int64_t *bucket_sizes;
     bsps_debug dbg;
     cudaStream_t stream;
+    int both_routes;     // pairs: as words, or by the look-back route if the sample's keys repeat
 };
 
 // Internal record tag: the input position g for a key, n + k*M + j for the
@@ -159,6 +160,18 @@ cudaError_t launch_merge_buckets(const Ctx &c);   // gather + stable merge per b
 int merge_cluster(const Plan &pl);                // CTAs per bucket for a bound pl.cap (0: too large)
 int64_t merge_capacity(int cl);                   // keys a cluster of cl CTAs merges
 int64_t merge_runs_max();                         // largest R
+// Pairs whose keys repeat are not routed as words where both routes are queued:
+// the device leaves the work to the one that its sample names.  Neighbours in
+// the sorted sample are compared; where at least half are equal, those that are
+// not count the values, and the keys repeat if there are fewer than one for 400
+// keys (2^24 pairs: of 300 copies 1764 us as words and 1981 by the look-back
+// route, of 3000 copies 2274 and 1375).
+constexpr int kRepeatProbes = 4096;
+inline uint32_t repeat_probes(const Plan &p) { return (uint32_t)imax64(0, imin64(kRepeatProbes, p.sample_size - 1)); }
+inline uint32_t repeats_above(const Plan &p) {
+    const int64_t q = repeat_probes(p);
+    return (uint32_t)imax64(q / 2, q - (int64_t)((double)q * p.n / (400.0 * p.sample_size)));
+}
 constexpr int64_t kPairWordsMax = 8192;           // largest P of pairs as words (index, splitters and a chunk on chip)
 constexpr int64_t kSegRouteRunsMax = 16384;       // largest R of the segment-copy route (shared memory)
 size_t route_keys_smem_bytes(const Plan &pl);

@@ -131,6 +131,7 @@ cudaError_t launch_bucket_keys(Exec &x);
 cudaError_t launch_route_words(Exec &x);     // single calls of 4-byte keys with payloads, as words
 cudaError_t launch_pair_words(Exec &x);      // ... and their final step (pairs.cu)
 cudaError_t launch_bucket_pairs(Exec &x);    // single calls
+cudaError_t launch_repeats_cluster(Exec &x); // single calls of 4-byte keys with payloads, on both routes
 
 // api.cu: a call's plan, checks and layout, and the path above for calls that
 // are ready (random sampling, keys only, at least one key each)

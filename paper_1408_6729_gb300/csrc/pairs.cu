@@ -32,6 +32,9 @@ struct PairArgs {
     DevStatus *st;
     int64_t slow_above;        // keys a cluster of the stable sort held
     uint64_t *words_rw;
+    uint32_t few_above;        // the sample's keys repeat more often: the look-back route was taken
+    uint32_t *reg_keys, *reg_vals;  // ... whose regions these are
+    __device__ bool repeats() const { return st->repeats > few_above; }
 };
 
 template <int DT> struct PairSink {
@@ -74,6 +77,20 @@ __global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
     const int g = (int)(blockIdx.x % a.G);
     const int64_t cnt = a.vsize[v];
     if (cnt == 0) return;
+    if (a.repeats()) {  // in input order by sub-bucket: those of one value are copied, the others listed (bucket.cuh)
+        if (v > 0 && v < a.P - 1 && a.vphi[v - 1] == a.vphi[v]) {
+            const uint32_t key = KeyTraits<DT>::inv(a.vphi[v]), *vals = a.reg_vals + v * a.cap;
+            uint32_t *out_k = a.out_keys + a.voff[v], *out_v = a.out_vals + a.voff[v];
+#pragma unroll 8
+            for (int64_t e = g * blockDim.x + threadIdx.x; e < cnt; e += a.G * blockDim.x) {
+                out_k[e] = key;
+                out_v[e] = vals[e];
+            }
+        } else if (g == 0 && threadIdx.x == 0) {
+            a.retry_list[atomicAdd(&a.st->retry_count, 1)] = (uint32_t)v;
+        }
+        return;
+    }
     auto same = [](uint64_t w) { return w; };
     const KeySource<uint64_t, CountShape<SIZE>::T, decltype(same)> src{a.words + v * a.cap, same};
     // between two splitters; exact where one side has none or only positions differ
@@ -98,6 +115,7 @@ __global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
 template <int DT>
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024, 1) pair_listed_kernel(const Many<PairArgs> many) {
     const PairArgs &a = many.one;
+    if (a.repeats()) return;
     using SS = SegSort<uint64_t, false, 8, kBucketItems64>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typename SS::Smem &sm = *reinterpret_cast<typename SS::Smem *>(smem_raw);
@@ -118,7 +136,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024, 1) pair_listed
 }
 
 // Tier 3: one CTA sorts one oversized sub-bucket by LSD passes between its
-// region and its output, where a word lies as its two halves.
+// region and its output, where a word lies as its two halves (key and payload,
+// in input order and sorted by key, after the look-back route).
 template <int DT> __global__ void __launch_bounds__(kSlowThreads) pair_slow_kernel(const Many<PairArgs> many) {
     const PairArgs &a = many.one;
     using Rank = BlockRank<kSlowThreads, kSlowItems, 8>;
@@ -131,13 +150,17 @@ template <int DT> __global__ void __launch_bounds__(kSlowThreads) pair_slow_kern
         const int64_t v = a.slow_list[idx], cnt = a.vsize[v], off = (int64_t)a.voff[v];
         uint64_t *reg = a.words_rw + v * a.cap;
         uint32_t *ok = a.out_keys + off, *ov = a.out_vals + off;
-        auto get = [&](int buf, int64_t e) { return buf == 0 ? reg[e] : (uint64_t)ok[e] << 32 | ov[e]; };
+        const bool rep = a.repeats();
+        uint32_t *rk = a.reg_keys + v * a.cap, *rv = a.reg_vals + v * a.cap;
+        auto get = [&](int buf, int64_t e) {
+            return buf == 0 && !rep ? reg[e] : (uint64_t)(buf ? ok : rk)[e] << 32 | (buf ? ov : rv)[e];
+        };
         auto put = [&](int buf, int64_t e, uint64_t w) {
-            if (buf == 0) {
+            if (buf == 0 && !rep) {
                 reg[e] = w;
             } else {
-                ok[e] = (uint32_t)(w >> 32);
-                ov[e] = (uint32_t)w;
+                (buf ? ok : rk)[e] = (uint32_t)(w >> 32);
+                (buf ? ov : rv)[e] = (uint32_t)w;
             }
         };
         if (threadIdx.x == 0) {
@@ -154,10 +177,10 @@ template <int DT> __global__ void __launch_bounds__(kSlowThreads) pair_slow_kern
         atomicMin(&red[0], (unsigned long long)mn);
         atomicMax(&red[1], (unsigned long long)mx);
         __syncthreads();
-        const uint64_t base = red[0];
+        const uint64_t base = rep ? red[0] >> 32 << 32 : red[0];
         const int bits = bit_length<uint64_t>(red[1] - base);
         int cur = 0;
-        for (int shift = 0; shift < bits; shift += 8) {
+        for (int shift = rep ? 32 : 0; shift < bits; shift += 8) {
             for (int i = threadIdx.x; i < 256; i += kSlowThreads) hist[i] = 0;
             __syncthreads();
             for (int64_t e = threadIdx.x; e < cnt; e += kSlowThreads)
@@ -189,7 +212,15 @@ template <int DT> __global__ void __launch_bounds__(kSlowThreads) pair_slow_kern
             cur = 1 - cur;
         }
         const PairSink<DT> sink{ok, ov, a.vals_in, a.last};
-        for (int64_t e = threadIdx.x; e < cnt; e += kSlowThreads) sink.one(e, get(cur, e));
+        for (int64_t e = threadIdx.x; e < cnt; e += kSlowThreads) {
+            const uint64_t w = get(cur, e);
+            if (rep) {
+                ok[e] = KeyTraits<DT>::inv((uint32_t)(w >> 32));
+                ov[e] = (uint32_t)w;
+            } else {
+                sink.one(e, w);
+            }
+        }
         __syncthreads();
     }
 }
@@ -210,6 +241,9 @@ static void pair_args(const Ctx &c, PairArgs &a) {
     a.retry_list = c.ly.retry_list;
     a.slow_list = c.ly.slow_list;
     a.st = c.ly.status;
+    a.few_above = c.both_routes ? repeats_above(c.pl) : 0xffffffffu;
+    a.reg_keys = (uint32_t *)c.ly.reg_keys;
+    a.reg_vals = c.ly.reg_vals;
     a.slow_above = (int64_t)c.pl.bucket_cl * 1024 * kPairItems32;
 }
 
@@ -238,6 +272,7 @@ template <int DT> static cudaError_t launch_t(Exec &x) {
     auto listed = pair_listed_kernel<DT>;
     if (e == cudaSuccess)
         e = launch_calls<PairArgs>(x, listed, listed, 1024, SegSort<uint64_t, false, 8, kBucketItems64>::smem_bytes(), all(16 * 8));
+    if (e == cudaSuccess && x.calls[0].both_routes) e = launch_repeats_cluster(x);
     auto slow = pair_slow_kernel<DT>;
     if (e == cudaSuccess) e = launch_calls<PairArgs>(x, slow, slow, kSlowThreads, 0, all(64));
     return e;

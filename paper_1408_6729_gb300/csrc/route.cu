@@ -45,6 +45,8 @@ template <typename K> struct RouteArgs {
     int64_t stall_tile;          // test hook: tile stall_tile - 1 never publishes (0: none)
     uint32_t spin_limit;         // polls of one bounded wait
     uint32_t tag_floor;          // a key's tag is max(position, tag_floor): n - 1 drops the tie-break
+    int32_t only_repeats;        // queued beside the route as words: runs if the sample's keys repeat
+    uint32_t few_above;          // ... more often than this
 };
 
 template <typename K> struct RouteFixed {
@@ -98,6 +100,7 @@ __global__ void __launch_bounds__(kRouteThreads, 1) route_kernel(const RouteArgs
     constexpr int TH = kRouteThreads;
     constexpr int CH = route_chunk<K>();
     using Rank = BlockRank<TH, IT, 8>;
+    if (a.only_repeats && a.st->repeats <= a.few_above) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RouteSmemLayout<K, LEARNED> L(a.P);
     MlpTables *mt = reinterpret_cast<MlpTables *>(smem_raw + L.mlp);
@@ -436,6 +439,8 @@ template <int DT, bool LEARNED> static cudaError_t launch_route_t(const Ctx &c) 
     a.stall_tile = c.dbg.stall_tile;
     a.spin_limit = c.dbg.wait_polls ? c.dbg.wait_polls : kSpinLimit;
     a.tag_floor = c.pl.dup_off ? (uint32_t)(c.pl.n - 1) : 0u;
+    a.only_repeats = c.both_routes;
+    a.few_above = repeats_above(p);
     const DynSmem smem(RouteSmemLayout<K, LEARNED>((uint32_t)p.P).total, 227 * 1024);  // (make_plan's bound)
     auto kern = route_kernel<DT, LEARNED>;
     cudaError_t e = smem.allow(kern);

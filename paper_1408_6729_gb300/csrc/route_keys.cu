@@ -77,6 +77,7 @@ template <typename K> struct RouteKeysArgs {
     const uint16_t *ylut;         // ... and the index over its output
     int lut_bits;                 // cells of `lut`
     uint32_t tag_floor;           // a key's tag is max(position, tag_floor): n - 1 drops the tie-break
+    uint32_t few_above;           // PAIRS: left to the look-back route if the sample's keys repeat more often
 };
 
 // Shared memory: the radix index (with the learned classifier: the index over
@@ -152,6 +153,8 @@ __global__ void __launch_bounds__(kRkThreads, 1) route_keys_kernel(const Many<Ro
     using K = typename KeyTraits<DT>::T;
     const Pick<MANY, RouteKeysArgs<K>> pk(many);
     const RouteKeysArgs<K> &a = pk.a;
+    if constexpr (PAIRS)
+        if (a.st->repeats > a.few_above) return;
     constexpr int T = kRkThreads, IT = rk_items<K, LEARNED, PAIRS>(), CH = rk_chunk<K, LEARNED, PAIRS>(),
                   V = 16 / (int)sizeof(K);
     using Word = typename std::conditional<PAIRS, uint64_t, K>::type;  // what moves
@@ -486,6 +489,7 @@ template <int DT, bool LEARNED, bool PAIRS = false> static cudaError_t launch_t(
         a.ylut = c.ly.ylut;
         a.lut_bits = LEARNED ? kLutBits : p.lut_bits;
         a.tag_floor = p.dup_off ? (uint32_t)(p.n - 1) : 0u;
+        a.few_above = c.both_routes ? repeats_above(p) : 0xffffffffu;
         // one CTA per SM; of a batch's CTAs (each loads the index first) every
         // call gets its share of two waves
         const int64_t share = all <= 2 * sms ? a.chunks : imax64(1, 2 * sms * a.chunks / all);

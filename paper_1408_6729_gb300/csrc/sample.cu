@@ -24,6 +24,8 @@ template <typename K> struct SampleArgs {
     DevStatus *st;          // cleared here, before anything of the call uses them
     uint32_t *cursor, *retry_flag;
     int64_t P;
+    uint32_t *state;        // the look-back route's, where both routes of pairs are queued
+    int64_t state_words;
 };
 template <int DT, bool MANY>
 __global__ void __launch_bounds__(256) sample_random_kernel(const Many<SampleArgs<typename KeyTraits<DT>::T>> many) {
@@ -35,6 +37,7 @@ __global__ void __launch_bounds__(256) sample_random_kernel(const Many<SampleArg
         a.cursor[v] = 0;
         a.retry_flag[v] = 0;
     }
+    for (int64_t w = blk; w < a.state_words; w += (int64_t)pk.blocks * blockDim.x) a.state[w] = 0;
     const int64_t j0 = blk * 4;
     if (j0 >= a.S) return;
     uint64_t c[4] = {(uint64_t)blk, 0, 0, 0};
@@ -717,7 +720,10 @@ template <typename K> struct SplitterArgs {
     uint32_t *vtag;
     LutParams<K> *lutp;
     uint16_t *lut;
-    int lut_bits, pad_;
+    int lut_bits;
+    uint32_t probes;        // neighbours in the sample compared, counted in *repeats
+    int64_t S;
+    uint32_t *repeats;
 };
 template <typename K, bool MANY>
 __global__ void __launch_bounds__(256) splitter_kernel(const Many<SplitterArgs<K>> many) {
@@ -746,6 +752,15 @@ __global__ void __launch_bounds__(256) splitter_kernel(const Many<SplitterArgs<K
     } else if (t == P - 1) {  // above every key, for comparisons without a bounds check
         vphi[t] = all_ones<K>();
         vtag[t] = 0xffffffffu;
+    }
+    if (pk.a.probes > 0) {
+        bool same = false;
+        if (t < pk.a.probes) {
+            const int64_t r = t * (pk.a.S - 1) / pk.a.probes;
+            same = phi[r] == phi[r + 1];
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, same);
+        if (m && (threadIdx.x & 31) == 0) atomicAdd(pk.a.repeats, (uint32_t)__popc(m));
     }
     // the radix index, from the sorted sample itself
     if (t <= (1 << lut_bits))
@@ -972,7 +987,7 @@ template <int DT> static cudaError_t launch_sample_random_t(Exec &x) {
                                        [](const Ctx &c, SampleArgs<K> &a) {
         const Plan &p = c.pl;
         a = {(const K *)c.keys_in, p.n, p.sample_size, p.seed, (K *)c.ly.sphi[0], c.ly.stag[0], c.ly.status, c.ly.cursor,
-             c.ly.retry_flag, p.P};
+             c.ly.retry_flag, p.P, c.ly.state, c.both_routes ? p.tiles * p.P : 0};
         return (uint32_t)imax64(1, (p.sample_size + 1023) / 1024);
     });
 }
@@ -1010,7 +1025,9 @@ template <typename K> static cudaError_t launch_splitters_t(Exec &x) {
         const Plan &p = c.pl;
         const RecordBuffers<K> b = buffers_of<K>(c);
         const int fin = sample_final(p);
-        a = {b.phi[fin], b.tag[fin], p.P, p.Q, p.B, (K *)c.ly.vphi, c.ly.vtag, (LutParams<K> *)c.ly.lutp, c.ly.lut, p.lut_bits, 0};
+        a = {b.phi[fin], b.tag[fin], p.P, p.Q, p.B, (K *)c.ly.vphi, c.ly.vtag, (LutParams<K> *)c.ly.lutp, c.ly.lut, p.lut_bits,
+             c.both_routes ? repeat_probes(p) : 0u, p.sample_size, &c.ly.status->repeats};
+        static_assert(kRepeatProbes <= kLutCells, "a thread for each probe");
         return (uint32_t)((imax64(p.P, (1 << p.lut_bits) + 1) + 255) / 256);
     });
 }

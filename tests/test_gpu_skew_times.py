@@ -43,9 +43,10 @@ def copies(n, c, seed=2):
 
 
 # every key equals splitters, whose tags are then searched: log2 of their number more reads a key
+# (pairs at a size that only moves as words)
 @pytest.mark.parametrize("pairs", [False, True], ids=["keys", "pairs"])
 def test_routing_few_values(pairs):
-    n, p = 1 << 25, 1024
+    n, p = (1 << 22, 1024) if pairs else (1 << 25, 1024)
     few, base = phase_us(copies(n, n // 100), p, [ROUTE], pairs)[0], phase_us(uniform(n), p, [ROUTE], pairs)[0]
     print(f"routing: few values {few:.0f} us, uniform {base:.0f} us")
     assert few <= 2.5 * base, (few, base)
@@ -95,3 +96,12 @@ def test_few_values_a_bucket():
     some, base = phase_us(copies(n, 30_000).astype(np.float64), p, [SORT])[0], phase_us(uniform(n).astype(np.float64), p, [SORT])[0]
     print(f"bucket sort: values of 30000 copies {some:.0f} us, uniform {base:.0f} us")
     assert some <= 1.5 * base, (some, base)
+
+
+# pairs of few values: the payloads travel along and one-value buckets are copied, where distinct keys' payloads are gathered
+def test_pairs_of_few_values():
+    n, p = 1 << 26, 1024
+    phases = [ROUTE, SORT]
+    few, base = phase_us(copies(n, n // 256), p, phases, pairs=True)[0], phase_us(uniform(n), p, phases, pairs=True)[0]
+    print(f"routing and bucket sort of pairs: 256 values {few:.0f} us, uniform {base:.0f} us")
+    assert few <= 0.95 * base, (few, base)
