@@ -394,21 +394,20 @@ template <typename E, int T> struct BlockSort {
                 a[(w & 0xffffu) + ((br[i] & 0x8000u) ? 0u : w >> 16) + (br[i] & 0x7fffu)] = k[i];
             }
         __syncthreads();
-        // the gaps: a few keys by one thread, more by a warp
-        constexpr uint32_t kByThread = 4;
+        // the gaps: two keys by one thread, more by a warp
         if (t < M) {
             const uint32_t at = (sm.cnt[t] & 0xffffu) + (sm.cnt[t] >> 16), end = sm.cnt[t + 1] & 0xffffu;
-            if (end - at <= kByThread)
-                for (uint32_t i = at + 1; i < end; ++i) {
-                    const E y = a[i];
-                    uint32_t j = i;
-                    for (; j > at && y < a[j - 1]; --j) a[j] = a[j - 1];
-                    a[j] = y;
+            if (end - at == 2) {
+                const E u = a[at], v = a[at + 1];
+                if (v < u) {
+                    a[at] = v;
+                    a[at + 1] = u;
                 }
+            }
         }
         for (int b = warp; b < M; b += T / 32) {
             const uint32_t at = (sm.cnt[b] & 0xffffu) + (sm.cnt[b] >> 16), len = (sm.cnt[b + 1] & 0xffffu) - at;
-            if (len <= kByThread) continue;
+            if (len <= 2) continue;
             if (len <= 32) warp_sort_regs<E, 1>(a + at, len);
             else warp_sort_more(a + at, len);
         }
