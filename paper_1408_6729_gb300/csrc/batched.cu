@@ -6,8 +6,8 @@
 // (small.cu), in one launch per shape.  The larger ones, with random sampling,
 // run the single-call kernels together: every step of the path is one launch
 // for all of them (many.cuh), in waves that reuse one workspace.  With regular
-// sampling they run the single-call pipeline on several streams, recorded into one CUDA graph that later calls with the same
-// arguments relaunch.
+// sampling they run the single-call pipeline on several streams, recorded into
+// one CUDA graph that later calls with the same arguments relaunch.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -203,7 +203,8 @@ static int lanes_for_device(LaneSet *&L) {
     return BSPS_OK;
 }
 
-// Everything the call queues, on `stream` and the lanes forked from it.
+// Everything a call with regular sampling queues, on `stream` and the lanes
+// forked from it.
 static int enqueue_batch(const BatchPlan &bp, const void *in, void *out, int32_t dtype, int64_t *bsz,
                          unsigned char *ws, cudaStream_t stream, LaneSet *L) {
 #define BSPS_CK(call)                                    \
@@ -211,20 +212,14 @@ static int enqueue_batch(const BatchPlan &bp, const void *in, void *out, int32_t
         if ((call) != cudaSuccess) return BSPS_ERR_CUDA; \
     } while (0)
     DevStatus *bst = (DevStatus *)ws;
-    const SmallJob *djobs = (const SmallJob *)(ws + ((sizeof(DevStatus) + 255) & ~size_t(255)));
     unsigned char *lane_ws = ws + ((sizeof(DevStatus) + 255) & ~size_t(255)) + bp.jobs_bytes + bp.tables_bytes + bp.wave_ws;
     BSPS_CK(cudaMemsetAsync(bst, 0, sizeof(DevStatus), stream));
     const int nl = bp.lane_ws ? bp.lanes : 0;
     BSPS_CK(cudaEventRecord(L->fork, stream));
     for (int l = 0; l < nl; ++l) BSPS_CK(cudaStreamWaitEvent(L->s[l], L->fork, 0));
-    for (int size = 2; size >= 0; --size) {  // the largest first
-        const int first = bp.first[size], count = bp.first[size + 1] - first;
-        if (count > 0) BSPS_CK(launch_small_jobs(dtype, size, in, out, djobs + first, count, bsz, stream));
-    }
     int l = 0;
     for (size_t i = 0; i < bp.inst.size(); ++i) {
-        const Instance &I = bp.inst[i];
-        if (I.small) continue;
+        const Instance &I = bp.inst[i];  // (with regular sampling none runs on chip)
         unsigned char *w = lane_ws + (size_t)l * bp.lane_ws;
         const size_t kb = dtype == BSPS_F64 ? 8 : 4;
         const int rc = bsps_sort_keys((const unsigned char *)in + I.off * kb, (unsigned char *)out + I.off * kb, I.n,
@@ -256,9 +251,47 @@ static cudaError_t upload(void *to, const void *from, size_t bytes, cudaStream_t
     return cudaSuccess;
 }
 
-// The on-chip instances in one launch per shape and, wave by wave, the larger
-// ones in one launch per step (random sampling).  The argument tables are
-// gathered first and uploaded; nothing is kept between calls.
+static int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(sms, 1);
+}
+
+// The on-chip instances; their first launch clears the batch's status.  No more
+// of them than SMs: one launch, an SM and its largest CTA to each, which ends
+// first (8 instances of 2^8 to 2^12 keys 23 us, with CTAs of 256 threads 30), and
+// launches of several shapes would run one after the other on a mostly idle GPU
+// (10 instances of 2^8 to 2^14 keys: 51 + 46 + 46 us in three).  More: a launch
+// per shape, several CTAs of the smaller shapes to an SM.  Short lists of jobs go
+// with the launch, longer ones are uploaded to `djobs`.
+static int run_on_chip(const BatchPlan &bp, const void *in, void *out, int32_t dtype, int64_t *bsz, DevStatus *bst,
+                       SmallJob *djobs, cudaStream_t stream) {
+    const int njobs = (int)bp.jobs.size();
+    bool uploaded = false;
+    DevStatus *clear = bst;
+    auto launch = [&](int size, int first, int count) {
+        if (count == 0) return cudaSuccess;
+        const bool listed = count <= kSmallListed;
+        if (!listed && !uploaded) {
+            const cudaError_t e = upload(djobs, bp.jobs.data(), sizeof(SmallJob) * njobs, stream);
+            if (e != cudaSuccess) return e;
+            uploaded = true;
+        }
+        const cudaError_t e = launch_small_jobs(dtype, size, in, out, listed ? nullptr : djobs + first, &bp.jobs[first], count, bsz,
+                                                clear, stream);
+        clear = nullptr;
+        return e;
+    };
+    if (njobs <= sm_count()) return launch(2, 0, njobs) == cudaSuccess ? BSPS_OK : BSPS_ERR_CUDA;
+    for (int size = 2; size >= 0; --size)  // the largest first
+        if (launch(size, bp.first[size], bp.first[size + 1] - bp.first[size]) != cudaSuccess) return BSPS_ERR_CUDA;
+    return BSPS_OK;
+}
+
+// The on-chip instances and, wave by wave, the larger ones in one launch per
+// step (random sampling).  The argument tables are gathered first and uploaded;
+// nothing is kept between calls.
 static int run_grouped(const BatchPlan &bp, const void *in, void *out, int32_t dtype, int64_t *bsz, unsigned char *ws,
                        cudaStream_t stream) {
 #define BSPS_CK(call)                                    \
@@ -267,7 +300,6 @@ static int run_grouped(const BatchPlan &bp, const void *in, void *out, int32_t d
     } while (0)
     DevStatus *bst = (DevStatus *)ws;
     const size_t at_jobs = (sizeof(DevStatus) + 255) & ~size_t(255);
-    const SmallJob *djobs = (const SmallJob *)(ws + at_jobs);
     unsigned char *tables_at = ws + at_jobs + bp.jobs_bytes, *wave_ws = tables_at + bp.tables_bytes;
     const size_t kb = dtype == BSPS_F64 ? 8 : 4;
     std::vector<unsigned char> tables;
@@ -295,15 +327,13 @@ static int run_grouped(const BatchPlan &bp, const void *in, void *out, int32_t d
         });
     }
     if (tables.size() > bp.tables_bytes) return BSPS_ERR_WORKSPACE_TOO_SMALL;
-    BSPS_CK(cudaMemsetAsync(bst, 0, sizeof(DevStatus), stream));
-    if (!bp.jobs.empty())
-        BSPS_CK(upload(ws + at_jobs, bp.jobs.data(), bp.jobs.size() * sizeof(SmallJob), stream));
-    if (!tables.empty())
-        BSPS_CK(upload(tables_at, tables.data(), tables.size(), stream));
-    for (int size = 2; size >= 0; --size) {  // the largest first
-        const int first = bp.first[size], count = bp.first[size + 1] - first;
-        if (count > 0) BSPS_CK(launch_small_jobs(dtype, size, in, out, djobs + first, count, bsz, stream));
+    if (bp.jobs.empty()) {
+        BSPS_CK(cudaMemsetAsync(bst, 0, sizeof(DevStatus), stream));
+    } else {
+        const int rc = run_on_chip(bp, in, out, dtype, bsz, bst, (SmallJob *)(ws + at_jobs), stream);
+        if (rc) return rc;
     }
+    BSPS_CK(upload(tables_at, tables.data(), tables.size(), stream));
     for (const auto &f : later) BSPS_CK(f());
     for (size_t i = 0; i < bp.inst.size(); ++i)  // empty instances that are not on chip
         if (bp.inst[i].n == 0 && !bp.inst[i].small && bsz)
@@ -373,12 +403,6 @@ int bsps_sort_batched(const void *d_keys_in, void *d_keys_out, const int64_t *h_
     std::lock_guard<std::mutex> lock(g_mu);
     LaneSet *L = nullptr;
     if ((rc = lanes_for_device(L))) return rc;
-    // the on-chip instances' table, uploaded on every call (from pageable
-    // memory: the copy has read it when cudaMemcpyAsync returns)
-    if (!bp.jobs.empty() &&
-        cudaMemcpyAsync(ws + ((sizeof(DevStatus) + 255) & ~size_t(255)), bp.jobs.data(),
-                        bp.jobs.size() * sizeof(SmallJob), cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return BSPS_ERR_CUDA;
 
     // graph key: every argument the recorded work depends on
     std::vector<unsigned char> key;
@@ -514,7 +538,7 @@ int bsps_autotune_batched(int32_t dtype, const bsps_params *prm, int32_t max_log
                 if (bsps_batch_workspace_size(off.data(), cnt, dtype, prm, &tt, &w) || w > bws_bytes) continue;
                 float ms[3];
                 bool ok = true;
-                for (int r = -1; r < 3 && ok; ++r) {  // one untimed call records the graph
+                for (int r = -1; r < 3 && ok; ++r) {  // one untimed call first
                     if (r >= 0 && cudaEventRecord(e0, st) != cudaSuccess) ok = false;
                     if (ok && bsps_sort_batched(kin, kout, off.data(), cnt, dtype, prm, &tt, nullptr, bws, bws_bytes, st))
                         ok = false;

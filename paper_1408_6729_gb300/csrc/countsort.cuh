@@ -284,10 +284,11 @@ template <typename E, int T> struct BlockSort {
         uint32_t cnt[M + 4];
         uint32_t tmp[40];
     };
-    // the M keys at sm.piv (threads < M hold one each) in ascending order
-    __device__ static void sort_pivots(E *piv, E x) {
+    // the keys of threads < m (a power of two, at most M) in ascending order at
+    // piv[0..m); what the threads past them hold ends past those
+    __device__ static void sort_pivots(E *piv, E x, int m = M) {
         const int t = threadIdx.x;
-        for (int h = 1; h < M; h <<= 1) {
+        for (int h = 1; h < m; h <<= 1) {
             for (int j = h; j > 0; j >>= 1) {
                 // the first step of a merge pairs mirrored positions
                 const int o = j == h ? 2 * h - 1 : j;

@@ -3,7 +3,7 @@
 
 namespace bsps {
 
-template cudaError_t launch_small_keys_t<BSPS_I32>(int, const void *, void *, const SmallJob *, int, const SmallJob &,
+template cudaError_t launch_small_keys_t<BSPS_I32>(int, const void *, void *, const SmallJob *, int, const SmallList &, bool,
                                                      int64_t *, DevStatus *, cudaStream_t);
 template cudaError_t launch_small_pairs_t<BSPS_I32>(const Ctx &, const SmallJob &);
 

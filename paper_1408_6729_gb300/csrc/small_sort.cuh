@@ -90,22 +90,34 @@ template <int SIZE> struct SmallKeysShape {
 template <int DT, int SIZE>
 __global__ void __launch_bounds__(SmallKeysShape<SIZE>::T, SmallKeysShape<SIZE>::kPerSm)
 small_keys_kernel(const uint32_t *__restrict__ keys_in, uint32_t *keys_out, const SmallJob *__restrict__ jobs,
-                  const SmallJob single, int64_t *bucket_sizes, DevStatus *st) {
+                  const __grid_constant__ SmallList list, bool batch, int64_t *bucket_sizes, DevStatus *st) {
     using Sh = SmallKeysShape<SIZE>;
     using CS = typename Sh::Sort;
     constexpr int T = Sh::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typename Sh::Extra &ex = *reinterpret_cast<typename Sh::Extra *>(smem_raw + Sh::kExtra);
     const int tid = threadIdx.x, lane = tid & 31;
-    const SmallJob J = jobs ? jobs[blockIdx.x] : single;
+    const SmallJob J = jobs ? jobs[blockIdx.x] : list.job[blockIdx.x];
+    if (batch && st && blockIdx.x == 0 && tid == 0) *st = DevStatus{};
     const int n = J.n, p = J.p;
     const uint32_t *in = keys_in + J.off;
     auto phi = [](uint32_t k) { return KeyTraits<DT>::phi(k); };
     auto inv = [](uint32_t k) { return KeyTraits<DT>::inv(k); };
-    const KeySource<uint32_t, T, decltype(phi)> src{in, phi};
-    uint32_t lo, hi;
-    CS::bounds(smem_raw, src, n, lo, hi);
-    CS::run(smem_raw, src, n, lo, hi, KeySink<uint32_t, decltype(inv)>{keys_out + J.off, inv}, 0, 1);
+    using Few = BlockSort<uint32_t, T>;
+    if (n <= Few::M) {
+        // one key to a thread (a batch of one instance of 447 keys takes 18 us
+        // when they are counted)
+        uint32_t *piv = reinterpret_cast<uint32_t *>(smem_raw);
+        int m = 1;
+        while (m < n) m <<= 1;
+        Few::sort_pivots(piv, tid < n ? phi(in[tid]) : 0xffffffffu, m);
+        if (tid < n) keys_out[J.off + tid] = inv(piv[tid]);
+    } else {
+        const KeySource<uint32_t, T, decltype(phi)> src{in, phi};
+        uint32_t lo, hi;
+        CS::bounds(smem_raw, src, n, lo, hi);
+        CS::run(smem_raw, src, n, lo, hi, KeySink<uint32_t, decltype(inv)>{keys_out + J.off, inv}, 0, 1);
+    }
     uint32_t most = (uint32_t)n;
     if (p > 1) {
         __syncthreads();
@@ -151,7 +163,7 @@ small_keys_kernel(const uint32_t *__restrict__ keys_in, uint32_t *keys_out, cons
     }
     if (bucket_sizes)
         for (int b = tid; b < p; b += T) bucket_sizes[J.bbase + b] = p > 1 ? ex.hist[b] : (uint32_t)n;
-    if (!jobs) small_status<T>(most, ex.tmp, J.cap, st);
+    if (!batch) small_status<T>(most, ex.tmp, J.cap, st);
 }
 
 // ---- keys with payloads ----
@@ -272,13 +284,13 @@ small_pairs_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restr
 
 // ---- host side ----
 template <int DT, int SIZE>
-static cudaError_t launch_keys_t(const void *in, void *out, const SmallJob *jobs, int njobs, const SmallJob &one, int64_t *bsz,
-                                 DevStatus *st, cudaStream_t stream) {
+static cudaError_t launch_keys_t(const void *in, void *out, const SmallJob *jobs, int njobs, const SmallList &list, bool batch,
+                                 int64_t *bsz, DevStatus *st, cudaStream_t stream) {
     using Sh = SmallKeysShape<SIZE>;
     auto kern = small_keys_kernel<DT, SIZE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem());
     if (e != cudaSuccess) return e;
-    kern<<<jobs ? njobs : 1, Sh::T, Sh::smem(), stream>>>((const uint32_t *)in, (uint32_t *)out, jobs, one, bsz, st);
+    kern<<<njobs, Sh::T, Sh::smem(), stream>>>((const uint32_t *)in, (uint32_t *)out, jobs, list, batch, bsz, st);
     return cudaGetLastError();
 }
 
@@ -294,12 +306,12 @@ static cudaError_t launch_pairs_t(const Ctx &c, const SmallJob &J) {
 }
 
 template <int DT>
-cudaError_t launch_small_keys_t(int size, const void *in, void *out, const SmallJob *jobs, int njobs, const SmallJob &one,
-                                 int64_t *bsz, DevStatus *st, cudaStream_t stream) {
+cudaError_t launch_small_keys_t(int size, const void *in, void *out, const SmallJob *jobs, int njobs, const SmallList &list,
+                                bool batch, int64_t *bsz, DevStatus *st, cudaStream_t stream) {
     switch (size) {
-    case kCountSmall: return launch_keys_t<DT, kCountSmall>(in, out, jobs, njobs, one, bsz, st, stream);
-    case kCountMedium: return launch_keys_t<DT, kCountMedium>(in, out, jobs, njobs, one, bsz, st, stream);
-    default: return launch_keys_t<DT, kCountLarge>(in, out, jobs, njobs, one, bsz, st, stream);
+    case kCountSmall: return launch_keys_t<DT, kCountSmall>(in, out, jobs, njobs, list, batch, bsz, st, stream);
+    case kCountMedium: return launch_keys_t<DT, kCountMedium>(in, out, jobs, njobs, list, batch, bsz, st, stream);
+    default: return launch_keys_t<DT, kCountLarge>(in, out, jobs, njobs, list, batch, bsz, st, stream);
     }
 }
 
