@@ -459,12 +459,11 @@ template <typename K, int T, typename Xf> struct KeySource {
     }
 };
 
-// Records (phi, tag) of two arrays as single words, every stride-th of them.
+// Records (phi, tag) of two arrays as single words.
 template <typename P, int T> struct RecordSource {
     using K = typename std::conditional<sizeof(P) == 8, u128, uint64_t>::type;
     const P *__restrict__ phi;
     const uint32_t *__restrict__ tag;
-    int64_t stride;
     template <typename F> __device__ void each(int n, F f) const {
         int e = threadIdx.x;
         for (; e + 3 * T < n; e += 4 * T) {
@@ -472,13 +471,13 @@ template <typename P, int T> struct RecordSource {
             uint32_t b[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                a[j] = phi[(e + j * T) * stride];
-                b[j] = tag[(e + j * T) * stride];
+                a[j] = phi[e + j * T];
+                b[j] = tag[e + j * T];
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) f((K)a[j] << 32 | b[j]);
         }
-        for (; e < n; e += T) f((K)phi[e * stride] << 32 | tag[e * stride]);
+        for (; e < n; e += T) f((K)phi[e] << 32 | tag[e]);
     }
 };
 

@@ -339,10 +339,111 @@ __global__ void __launch_bounds__(kPivotThreads) sample_scatter_kernel(const Man
     }
 }
 
-// One bin per CTA, from buffer 1 into its place in buffer 0.  A bin that the
-// counting sort gives back (a run of its bins above the stage: the pivots keep
-// bins near their mean, so this is out of reach in practice) is put in order
-// where it lies by a bitonic network.
+// A bin's records in order by stable radix passes over the bytes in which they
+// differ (none: a copy), from buffer 1 to buffer 0 and back, by T threads.
+template <typename P, int T> struct RadixBin {
+    static constexpr int ITEMS = 8, CH = T * ITEMS;
+    using Rank = BlockRank<T, ITEMS, 8>;
+    struct Smem {
+        typename Rank::Smem rank;
+        uint32_t run[256], tmp[40], any[3], all[3];  // any, all: of the tags and the halves of the phi
+    };
+    __device__ static void run(Smem &sm, const RecordBuffers<P> &b, int64_t at, int n) {
+        const int tid = threadIdx.x;
+        if (tid < 3) {
+            sm.any[tid] = 0u;
+            sm.all[tid] = 0xffffffffu;
+        }
+        __syncthreads();
+        uint32_t any[3] = {}, all[3] = {~0u, ~0u, ~0u};
+#pragma unroll 8
+        for (int i = tid; i < n; i += T) {
+            const P f = b.phi[1][at + i];
+            const uint32_t w[3] = {b.tag[1][at + i], (uint32_t)f, (uint32_t)((uint64_t)f >> 32)};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                any[k] |= w[k];
+                all[k] &= w[k];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t x = __reduce_or_sync(0xffffffffu, any[k]), y = __reduce_and_sync(0xffffffffu, all[k]);
+            if ((tid & 31) == 0) {
+                atomicOr(&sm.any[k], x);
+                atomicAnd(&sm.all[k], y);
+            }
+        }
+        __syncthreads();
+        int cur = 1;
+        for (int pass = 0; pass < 4 + (int)sizeof(P); ++pass) {
+            const int shift = pass * 8 % 32;
+            if (((sm.any[pass / 4] ^ sm.all[pass / 4]) >> shift & 255u) == 0) continue;
+            const P *sf = b.phi[cur] + at;
+            const uint32_t *st = b.tag[cur] + at;
+            P *df = b.phi[1 - cur] + at;
+            uint32_t *dt = b.tag[1 - cur] + at;
+            auto digit = [&](P f, uint32_t t) {
+                return (pass < 4 ? t >> shift : (uint32_t)(f >> (pass * 8 - 32))) & 255u;
+            };
+            for (int i = tid; i < 256; i += T) sm.run[i] = 0;
+            __syncthreads();
+#pragma unroll 4
+            for (int i = tid; i < n; i += T) atomicAdd(&sm.run[pass < 4 ? digit(0, st[i]) : digit(sf[i], 0u)], 1u);
+            __syncthreads();
+            digit_excl_scan<T, 256>(sm.run, sm.tmp);
+            for (int c = 0; c < n; c += CH) {
+                P f[ITEMS];
+                uint32_t t[ITEMS], d[ITEMS], rk[ITEMS];
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    const int e = c + striped_slot<T, ITEMS>(i);
+                    if (e < n) {
+                        f[i] = sf[e];
+                        t[i] = st[e];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)  // past the end: after every record of digit 255
+                    d[i] = c + striped_slot<T, ITEMS>(i) < n ? digit(f[i], t[i]) : 255u;
+                Rank::rank(sm.rank, d, rk);
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    if (c + striped_slot<T, ITEMS>(i) < n) {
+                        const uint32_t o = sm.run[d[i]] + rk[i];
+                        df[o] = f[i];
+                        dt[o] = t[i];
+                    }
+                __syncthreads();
+                for (int i = tid; i < 256; i += T) sm.run[i] += sm.rank.digit_tot[i];
+                __syncthreads();
+            }
+            cur = 1 - cur;
+        }
+        if (cur == 1) {
+#pragma unroll 8
+            for (int i = tid; i < n; i += T) {
+                b.phi[0][at + i] = b.phi[1][at + i];
+                b.tag[0][at + i] = b.tag[1][at + i];
+            }
+        }
+    }
+};
+
+// Bins too large for the counting sort (radix_bins), one per CTA.
+constexpr int kRadixThreads = 512;
+template <typename P, bool MANY>
+__global__ void __launch_bounds__(kRadixThreads, 2) sample_radix_kernel(const Many<SortArgs<P>> many) {
+    const Pick<MANY, SortArgs<P>> pk(many);
+    __shared__ typename RadixBin<P, kRadixThreads>::Smem sm;
+    const uint32_t at = pk.a.sc.start[pk.block];
+    const int n = (int)(pk.a.sc.start[pk.block + 1] - at);
+    if (n > 0) RadixBin<P, kRadixThreads>::run(sm, pk.a.b, at, n);
+}
+
+// One bin per CTA, from buffer 1 into its place in buffer 0.  A bin of one
+// record (a sample of many more draws than keys) is copied; what the counting
+// sort gives back is sorted by radix passes.
 template <typename P, int SIZE, bool MANY>
 __global__ void __launch_bounds__(CountShape<SIZE>::T, CountShape<SIZE>::kPerSm)
 sample_bins_kernel(const Many<SortArgs<P>> many) {
@@ -356,45 +457,14 @@ sample_bins_kernel(const Many<SortArgs<P>> many) {
     const uint32_t at = sc.start[pk.block];
     const int n = (int)(sc.start[pk.block + 1] - at);
     if (n == 0) return;
-    P *f = b.phi[1] + at;
-    uint32_t *t = b.tag[1] + at;
-    const RecordSource<P, T> src{f, t, 1};
+    const RecordSource<P, T> src{b.phi[1] + at, b.tag[1] + at};
     K lo, hi;
     CS::bounds(smem_raw, src, n, lo, hi);
-    if (CS::run(smem_raw, src, n, lo, hi, RecordSink<P>{b.phi[0], b.tag[0], (int64_t)at}, 0, 1)) return;
+    if (lo != hi && CS::run(smem_raw, src, n, lo, hi, RecordSink<P>{b.phi[0], b.tag[0], (int64_t)at}, 0, 1)) return;
     __syncthreads();
-    int n2 = 1;
-    while (n2 < n) n2 <<= 1;
-    auto step = [&](int i, int l) {
-        if (l < n) {
-            const P x = f[i], y = f[l];
-            const uint32_t u = t[i], v = t[l];
-            if (x > y || (x == y && u > v)) {
-                f[i] = y;
-                f[l] = x;
-                t[i] = v;
-                t[l] = u;
-            }
-        }
-    };
-    for (int h = 1; h < n2; h <<= 1) {
-        for (int q = threadIdx.x; q < n2 / 2; q += T) {
-            const int c = (q & ~(h - 1)) * 2, o = q & (h - 1);
-            step(c + o, c + 2 * h - 1 - o);
-        }
-        __syncthreads();
-        for (int j = h >> 1; j > 0; j >>= 1) {
-            for (int q = threadIdx.x; q < n2 / 2; q += T) {
-                const int i = 2 * q - (q & (j - 1));
-                step(i, i + j);
-            }
-            __syncthreads();
-        }
-    }
-    for (int i = threadIdx.x; i < n; i += T) {
-        b.phi[0][at + i] = f[i];
-        b.tag[0][at + i] = t[i];
-    }
+    using Radix = RadixBin<P, T>;
+    static_assert(sizeof(typename Radix::Smem) <= CS::smem_bytes(), "in the counting sort's place");
+    Radix::run(*reinterpret_cast<typename Radix::Smem *>(smem_raw), b, at, n);
 }
 
 static int sm_count() {
@@ -429,13 +499,20 @@ static int bins_shape(int64_t S, int key_bytes) {
     const int64_t half = S / pivot_bins(S);
     return half <= 700 ? kCountSmall : half <= 2000 ? kCountMedium : kCountLarge;
 }
+// Bins past this mean take radix passes: the counting sort reads a bin again for
+// every part of it (a stage holds 5112 records of doubles, 18,680 of 4-byte keys).
+static bool radix_bins(int64_t S, int key_bytes) {
+    return 2 * S / pivot_bins(S) > (key_bytes == 8 ? 12288 : 65536);
+}
 static int scatter_items(int64_t S) { return S < (1 << 20) ? 4 : 8; }
 
 template <typename K, int SIZE> static cudaError_t launch_sample_bins(Exec &x) {
     using CS = typename CountShape<SIZE>::template Sort<typename RecordSink<K>::K>;
     return launch_calls<SortArgs<K>>(x, sample_bins_kernel<K, SIZE, false>, sample_bins_kernel<K, SIZE, true>,
                                      CountShape<SIZE>::T, CS::smem_bytes(), [](const Ctx &c, SortArgs<K> &a) {
-        if (c.pl.sample_size <= kOneSample || bins_shape(c.pl.sample_size, sizeof(K)) != SIZE) return 0u;
+        if (c.pl.sample_size <= kOneSample || bins_shape(c.pl.sample_size, sizeof(K)) != SIZE ||
+            radix_bins(c.pl.sample_size, sizeof(K)))
+            return 0u;
         sort_args(c, a);
         return (uint32_t)a.bins;
     });
@@ -489,6 +566,13 @@ template <typename K> static cudaError_t launch_sample_sort_t(Exec &x) {
     });
     if (e == cudaSuccess) e = launch_sample_scatter<K, 4>(x, bins);
     if (e == cudaSuccess) e = launch_sample_scatter<K, 8>(x, bins);
+    if (e == cudaSuccess)
+        e = launch_calls<SortArgs<K>>(x, sample_radix_kernel<K, false>, sample_radix_kernel<K, true>, kRadixThreads, 0,
+                                      [](const Ctx &c, SortArgs<K> &a) {
+            if (c.pl.sample_size <= kOneSample || !radix_bins(c.pl.sample_size, sizeof(K))) return 0u;
+            sort_args(c, a);
+            return (uint32_t)a.bins;
+        });
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(K) == 8) {
         return launch_sample_bins<K, kCountRecord>(x);

@@ -46,3 +46,14 @@ def test_sample_of_repeated_records(n, p, s):
     keys = np.random.default_rng(n).integers(0, 2**31, n).astype(np.int32)
     ref = oracle.sort(keys, p, s, 0, oracle.RANDOM, seed=3, want_sample=True)
     assert_same(run_gpu(keys, p, s, 0, oracle.RANDOM, 3), ref)
+
+
+# ... of far more draws than keys, bins of one record and of several past 65,535 copies, and bins that take radix passes
+@pytest.mark.parametrize("n, p, s, dt", [(10, 2, 1_000_000, np.int32), (10, 2, 1_000_000, np.float64), (40, 1, 8_000_000, np.int32),
+                                         (3000, 16, 100_000, np.int32), (3000, 16, 100_000, np.float64), (700, 2, 13_000_000, np.float64)])
+def test_sample_much_larger_than_the_input(n, p, s, dt):
+    keys = np.random.default_rng(n).integers(-2**31, 2**31, n).astype(dt)
+    keys[: n // 3] = keys[0]
+    ref = oracle.sort(keys, p, s, 0, oracle.RANDOM, seed=3, want_sample=False)
+    got = run_gpu(keys, p, s, 0, oracle.RANDOM, 3, debug=False)
+    assert got.keys.tobytes() == ref.keys.tobytes() and np.array_equal(got.bucket_sizes, ref.bucket_sizes)

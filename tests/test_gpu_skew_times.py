@@ -105,3 +105,12 @@ def test_pairs_of_few_values():
     few, base = phase_us(copies(n, n // 256), p, phases, pairs=True)[0], phase_us(uniform(n), p, phases, pairs=True)[0]
     print(f"routing and bucket sort of pairs: 256 values {few:.0f} us, uniform {base:.0f} us")
     assert few <= 0.95 * base, (few, base)
+
+
+# large samples of doubles, whose 128-bit records fill a stage sooner
+def test_sample_sort_of_many_doubles():
+    n, p, s = 1 << 22, 1024, 1 << 16
+    k = uniform(n)
+    wide, base = phase_us(k.astype(np.float64), p, [SAMPLE_SORT], s=s)[0], phase_us(k, p, [SAMPLE_SORT], s=s)[0]
+    print(f"sample sort of 2^26 records: doubles {wide:.0f} us, int32 {base:.0f} us")
+    assert wide <= 4 * base, (wide, base)
