@@ -144,7 +144,7 @@ typedef struct {
     int64_t vbuckets;        /* p * refine */
     int64_t capacity;        /* keys per sub-bucket region */
     int32_t run_cluster;     /* CTAs per block sort (regular mode) */
-    int32_t bucket_cluster;  /* CTAs per sub-bucket sort */
+    int32_t bucket_cluster;  /* CTAs per sub-bucket of the stable cluster sort (keys alone: for which sub-buckets are sized) */
     int64_t route_tiles;
     size_t workspace_bytes;
 } bsps_plan;
@@ -154,7 +154,8 @@ typedef struct {
     int32_t status;          /* BSPS_OK or the first device-side error */
     int32_t overflow;        /* nonzero if a bucket exceeded its region */
     int32_t timeouts;        /* bounded waits that expired */
-    int32_t slow_buckets;    /* sub-buckets sorted by the out-of-core path */
+    int32_t slow_buckets;    /* sub-buckets sorted out of core: larger than a cluster's shared memory and
+                                sorted in parts, or by radix passes through global memory */
     int64_t max_bucket;      /* largest bucket, real keys only */
     int64_t max_vbucket;     /* largest sub-bucket */
     int64_t mispredicted;    /* learned classifier: keys whose prediction was corrected */
@@ -169,7 +170,8 @@ typedef struct {
  *     routing, after the bucket sort.
  *   launches: HOST int32 that receives the number of kernels the call launched.
  *   stall_tile, wait_polls: test hooks of the bounded waits (Sec. 5.1: the
- *     prefix step depends on every earlier processor).  With payloads,
+ *     prefix step depends on every earlier processor).  With payloads (4-byte
+ *     keys then take the look-back route, too),
  *     routing tile stall_tile - 1 never publishes its per-bucket counts
  *     (0: every tile publishes), so the later tiles' look-back waits on it
  *     expire; wait_polls bounds the polls of one wait (0: the default bound,

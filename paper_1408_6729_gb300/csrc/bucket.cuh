@@ -32,7 +32,7 @@ template <typename K> struct BucketArgs {
     uint32_t *retry_list;
     const uint32_t *only;     // tier 2 over a list (nullable: every sub-bucket)
     const int32_t *only_count;
-    int64_t slow_above;       // keys a cluster of the stable sort holds
+    int64_t slow_above;       // a larger sub-bucket, sorted in several parts, counts as out of core
     int one_value_done;       // sub-buckets of one key value are already in the output
     int G;                    // tier 1: CTAs per sub-bucket
     int only_repeats;         // pairs queued on both routes: this one runs if the sample's keys repeat
@@ -156,7 +156,7 @@ bucket_count_kernel(const Many<BucketArgs<typename KeyTraits<DT>::T>> many) {
         for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) out_k[e] = x;
     } else {
         done = CS::run(smem_raw, src, (int)cnt, lo, hi, KeySink<K, decltype(inv)>{out_k, inv}, g, G);
-        // larger than a cluster of the stable sort holds: sorted out of core, part by part
+        // larger than a cluster's shared memory: sorted out of core, part by part
         if (done && cnt > a.slow_above && g == 0 && threadIdx.x == 0) atomicAdd(&a.st->slow_buckets, 1);
     }
     if (!done && threadIdx.x == 0 && atomicExch(&a.retry_flag[v], 1u) == 0u)

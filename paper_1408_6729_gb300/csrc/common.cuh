@@ -56,7 +56,7 @@ struct DevStatus {
     int32_t error;        // first device-side error code (0 = none)
     int32_t overflow;     // a bucket region overflowed
     int32_t timeouts;     // bounded waits that expired
-    int32_t slow_buckets; // sub-buckets handled by the out-of-core path
+    int32_t slow_buckets; // sub-buckets sorted out of core, in parts or by radix passes
     unsigned long long max_bucket;
     unsigned long long max_vbucket;
     unsigned long long mispredicted;

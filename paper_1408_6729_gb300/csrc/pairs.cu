@@ -30,7 +30,7 @@ struct PairArgs {
     uint32_t *out_keys, *out_vals;
     uint32_t *retry_flag, *retry_list, *slow_list;
     DevStatus *st;
-    int64_t slow_above;        // keys a cluster of the stable sort held
+    int64_t slow_above;        // a larger sub-bucket, sorted in several parts, counts as out of core
     uint64_t *words_rw;
     uint32_t few_above;        // the sample's keys repeat more often: the look-back route was taken
     uint32_t *reg_keys, *reg_vals;  // ... whose regions these are
@@ -244,7 +244,7 @@ static void pair_args(const Ctx &c, PairArgs &a) {
     a.few_above = c.both_routes ? repeats_above(c.pl) : 0xffffffffu;
     a.reg_keys = (uint32_t *)c.ly.reg_keys;
     a.reg_vals = c.ly.reg_vals;
-    a.slow_above = (int64_t)c.pl.bucket_cl * 1024 * kPairItems32;
+    a.slow_above = (int64_t)8 * 1024 * kPairItems32;
 }
 
 template <int DT, int SIZE> static cudaError_t launch_count(Exec &x) {
