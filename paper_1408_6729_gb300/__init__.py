@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libbspsort.so")
@@ -255,9 +256,9 @@ def bsps_mlp_predict(params, x, m, y, workspace, stream=None) -> int:
 def _offsets(offsets):
     """Host int64 offsets as an argument: a contiguous numpy int64 array where it
     lies, any other sequence as a ctypes array."""
-    flags = getattr(offsets, "flags", None)
-    if flags is not None and getattr(offsets, "ndim", 0) == 1 and offsets.dtype == "int64" and flags.c_contiguous \
-            and flags.aligned and offsets.dtype.isnative and len(offsets):
+    numpy = sys.modules.get("numpy")
+    if numpy is not None and isinstance(offsets, numpy.ndarray) and offsets.ndim == 1 and offsets.dtype == numpy.int64 \
+            and offsets.dtype.isnative and offsets.flags.c_contiguous and offsets.flags.aligned and len(offsets):
         return offsets.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), len(offsets) - 1
     vals = [int(v) for v in offsets]
     return (ctypes.c_int64 * max(1, len(vals)))(*vals), len(vals) - 1
