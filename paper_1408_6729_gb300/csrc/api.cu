@@ -19,7 +19,8 @@ static bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
 static int64_t align_up(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
 
-// keys one CTA of the sub-bucket sort holds
+// an eighth of what a sub-bucket is sized for: with payloads what one CTA of
+// the stable cluster sort holds
 static int64_t cta_capacity(int key_bytes, bool slot) {
     if (slot) return (int64_t)kSortThreads * (key_bytes == 8 ? kPairItems64 : kPairItems32);
     return (int64_t)512 * (key_bytes == 8 ? kKeysItems64 : kKeysItems32);
@@ -289,7 +290,7 @@ static int kernels_per_call(const Ctx &c) {
     if (pl.seg_route) k += 1;
     if (c.both_routes) k += 2;                   // the look-back route and its cluster sort
     k += 3;                                      // copy or keys-only tier, cluster sort, out-of-core sort
-    if (pl.classify == BSPS_LEARNED) k += mlp_train_kernels();  // training set, start, Adam steps, tables, index
+    if (pl.classify == BSPS_LEARNED) k += mlp_train_kernels();  // training set, start, descent steps, tables, index
     return k;
 }
 

@@ -30,8 +30,9 @@ constexpr int kBucketItems32 = 14;     // sub-bucket sort, keys only, 4-byte key
 constexpr int kBucketItems64 = 10;     // ... 8-byte keys
 constexpr int kPairItems32 = 12;       // sub-bucket sort with payload slots, 4-byte keys
 constexpr int kPairItems64 = 8;        // ... 8-byte keys
-constexpr int kKeysItems32 = 20;       // throughput keys-only sort: 512 threads x 20 = 10240 keys per CTA
-constexpr int kKeysItems64 = 10;       // ... 8-byte keys
+constexpr int kKeysItems32 = 20;       // sizing of sub-buckets without payloads: 8 * 512 x 20 = 81,920 keys at most
+constexpr int kKeysItems64 = 10;       // ... 8-byte keys (the counting sort takes any size; its stage holds 74,744 half
+                                       // words of 4-byte keys, 37,368 of 8-byte keys, so this is about one or two parts)
 constexpr int kSlowThreads = 512;      // out-of-core sort of an oversized sub-bucket
 constexpr int kSlowItems = 8;
 

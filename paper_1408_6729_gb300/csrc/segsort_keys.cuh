@@ -1,15 +1,15 @@
-// segsort_keys.cuh -- the keys-only bucket sort (Fig. 2 step 12), tuned for
-// throughput: equal keys cannot be told apart, so no ranking needs to be
-// stable and every rank comes from shared-memory atomics.
+// segsort_keys.cuh -- the sort of unique words by a cluster, for the blocks of
+// the regular sample that carry payloads (Fig. 1 step 3; words phi << 32 |
+// position): equal words cannot occur, so no ranking needs to be stable and
+// every rank comes from shared-memory atomics.
 //
 // With MINMAX the split also records every bin's smallest and largest key,
 // which the caller's give_up predicate reads; without it a bin only keeps one
 // of its keys and a flag for any other value, enough to find bins of one
 // distinct key.
 //
-// A cluster of CL CTAs (512 threads, two per SM) sorts one sub-bucket whose
-// keys lie in [lo, hi] (bounds from the splitters).  Each CTA loads its share
-// into registers with 16-byte loads and ranks its keys per split bin (the top
+// A cluster of CL CTAs (512 threads, two per SM) sorts one block whose keys lie
+// in [lo, hi].  Each CTA loads its share into registers and ranks its keys per split bin (the top
 // bits of key - lo), grouping them by bin in a local stage buffer.  The bin
 // counts are read across the cluster through distributed shared memory; bins
 // holding one distinct key are written out directly, every other bin is given
@@ -22,7 +22,7 @@
 // popcounts of the masks below its value plus its occurrence index.  Keys of
 // other bins are placed by comparison.  A bin too large for one CTA,
 // or count bins longer than kBinMax that need comparisons, make the cluster
-// give the sub-bucket back (returns false) to the stable cluster sort of
+// give the block back (returns false) to the stable cluster sort of
 // segsort.cuh.
 #pragma once
 
@@ -98,25 +98,6 @@ struct SegSortKeys {
         } else {
             atomicMin((unsigned *)mn, (unsigned)v);
             atomicMax((unsigned *)mx, (unsigned)v);
-        }
-    }
-
-    // n keys from global memory (16-byte aligned; reading up to the next
-    // multiple of V keys stays inside the caller's region) into registers
-    __device__ static void load(K (&k)[ITEMS], const K *__restrict__ src, int n) {
-        const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
-#pragma unroll
-        for (int j = 0; j < ITEMS / V; ++j) {
-            const int q = j * T + (int)threadIdx.x;
-            if (q * V < n) {
-                const uint4 w = __ldg(s4 + q);
-                if constexpr (sizeof(K) == 4) {
-                    k[j * V + 0] = w.x; k[j * V + 1] = w.y; k[j * V + 2] = w.z; k[j * V + 3] = w.w;
-                } else {
-                    k[j * V + 0] = ((uint64_t)w.y << 32) | w.x;
-                    k[j * V + 1] = ((uint64_t)w.w << 32) | w.z;
-                }
-            }
         }
     }
 
@@ -296,24 +277,14 @@ struct SegSortKeys {
         return true;
     }
 
-    // Sorts the cnt keys at gsrc (bounds lo <= key <= hi) and calls
-    // emit(position, key) for each.  Returns false when the sub-bucket does not
-    // fit this cluster or its bins are too uneven; the caller then hands it to
-    // the stable sort, which rewrites every position (keys already emitted are
-    // rewritten with the same values).  smem holds Smem, then the stage and the
-    // receive buffer (CAP keys each).
-    template <typename Emit>
-    __device__ static bool run(unsigned char *smem, const K *__restrict__ gsrc, int64_t cnt, K lo, K hi, Emit emit) {
-        auto from_global = [&](K (&k)[ITEMS], int64_t e0, int n) { load(k, gsrc + e0, n); };
-        auto never = [](K, K) { return false; };
-        return run_load(smem, cnt, lo, hi, from_global, emit, never);
-    }
-
-    // As run(), with the keys of positions [e0, e0 + n) produced by
-    // load(k, e0, n) into register i of each thread for position e0 + lidx(i).
-    // give_up(min, max) marks split bins the caller expects to be slow here;
-    // when they hold more than a quarter of the keys the sub-bucket is given
-    // back right after the split.
+    // Sorts cnt keys (lo <= key <= hi), those of positions [e0, e0 + n) produced
+    // by load(k, e0, n) into register i of each thread for position e0 +
+    // lidx(i), and calls emit(position, key) for each.  Returns false when they
+    // do not fit this cluster or its bins are too uneven; the caller then hands
+    // them to the stable sort, which rewrites every position.  smem holds Smem,
+    // then the stage and the receive buffer (CAP keys each).  give_up(min, max)
+    // marks split bins the caller expects to be slow here; when they hold more
+    // than a quarter of the keys, all are given back right after the split.
     template <typename Load, typename Emit, typename GiveUp>
     __device__ static bool run_load(unsigned char *smem, int64_t cnt, K lo, K hi, Load loadf, Emit emit,
                                     GiveUp give_up) {
