@@ -491,13 +491,14 @@ template <typename K> static void sort_args(const Ctx &c, SortArgs<K> &a) {
     a.sc = PivotScratch<K>(c.ly.pivots, a.bins);
 }
 
-// The shape that sorts a bin (its mean is 2 S / bins records, twice that fits
-// the stage), and the tiles of the scatter: 2K records until there are enough
+// The shape that sorts a bin (its mean is 2 S / bins records; the stages hold
+// 3832, 8696 and 18,680 of them, and two CTAs of 512 threads on an SM beat one of
+// 1024 while a bin fits: 8.4M records 344 us and 383), and the tiles of the scatter: 2K records until there are enough
 // of 4K to fill the GPU.
 static int bins_shape(int64_t S, int key_bytes) {
     if (key_bytes == 8) return kCountRecord;
     const int64_t half = S / pivot_bins(S);
-    return half <= 700 ? kCountSmall : half <= 2000 ? kCountMedium : kCountLarge;
+    return half <= 700 ? kCountSmall : half <= 3000 ? kCountMedium : kCountLarge;
 }
 // Bins past this mean take radix passes: the counting sort reads a bin again for
 // every part of it (a stage holds 5112 records of doubles, 18,680 of 4-byte keys).
