@@ -363,6 +363,7 @@ template <typename E, int T> struct BlockSort {
         static_assert(kMost <= 0x7fff + 1, "places of 15 bits");
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
+            if (i * T >= n) break;  // (the code of the rest is not even fetched: few keys, one CTA)
             const int e = i * T + t;
             if (e < n) {
                 k[i] = a[e];
@@ -389,11 +390,13 @@ template <typename E, int T> struct BlockSort {
         if (t == 0) sm.cnt[M] = (uint32_t)n;
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i)
+        for (int i = 0; i < ITEMS; ++i) {
+            if (i * T >= n) break;
             if (i * T + t < n) {
                 const uint32_t w = sm.cnt[br[i] >> 16];
                 a[(w & 0xffffu) + ((br[i] & 0x8000u) ? 0u : w >> 16) + (br[i] & 0x7fffu)] = k[i];
             }
+        }
         __syncthreads();
         // the gaps: two keys by one thread, more by a warp
         if (t < M) {
