@@ -105,29 +105,32 @@ METRIC = "keys/sec and % HBM roofline, 2^28 int32; learned/batched vs plain, bit
 PHASES = ["sample", "sample_sort", "splitters", "route", "bucket_sort"]
 PHASE_KERNEL = {("route", False): "route_keys_kernel", ("bucket_sort", False): "bucket_count_kernel",
                 ("route", True): "route_kernel", ("bucket_sort", True): "bucket_sort_kernel"}
-PHASE_KERNEL_F64 = {"bucket_sort": "bucket_count_kernel"}
+# random pairs of 4-byte keys move as words up to this many sub-buckets (distinct keys; few values: as the other pairs)
+PAIR_WORDS_MAX = 8192
+PHASE_KERNEL_WORDS = {"route": "route_keys_kernel", "bucket_sort": "pair_count_kernel"}
 # the variant timed beside a workload: (label, the parameters that change)
 COMPARE = {"tree": ("tree", dict(classify=0)), "sort": ("bucket_sort_final_step", dict(final_step=0)),
            "tags": ("with_duplicate_handling", dict(duplicates=0))}
 
 # dram__bytes_read.sum + dram__bytes_write.sum per key of each kernel from one
 # ncu capture (its summary is under profiles/), valid while the kernel source is unchanged:
-# routing from the 2^26-key capture (4096 buckets, as at 2^28); the kernel
-# streams every key once, so bytes per key carry over to 2^28
+# routing from the 2^26-key capture (4096 buckets, as at 2^28), the bucket sort
+# from the 2^27-key capture on [0, 2^30) (65,536-key buckets over 2^19 values, as
+# at 2^28); both stream every key once, so bytes per key carry over to 2^28
 # (bytes per key, source hash, payloads) of each capture; the segment copy's
 # from the 2^26-pair Zipf capture (4096 buckets of 16-key segments, as at 2^28)
-NCU_TRAFFIC = {"route_keys_kernel": ((271.608576e6 + 223.674880e6) / (1 << 26), "8baca4c618da453f", False),
-               "segment_copy_kernel": ((617.909248e6 + 494.979328e6) / (1 << 26), "333c4e171f9cd65e", True)}
-KERNEL_SOURCE = {"route_kernel": ["paper_1408_6729_gb300/csrc/route.cu"],
-                 "segment_copy_kernel": ["paper_1408_6729_gb300/csrc/merge.cu"],
-                 "route_keys_kernel": ["paper_1408_6729_gb300/csrc/route_keys.cu",
-                                       "paper_1408_6729_gb300/csrc/classify.cuh",
-                                       "paper_1408_6729_gb300/csrc/kernels.cuh"],
-                 "bucket_sort_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
-                                        "paper_1408_6729_gb300/csrc/segsort.cuh"],
-                 "bucket_count_kernel": ["paper_1408_6729_gb300/csrc/bucket.cu",
-                                         "paper_1408_6729_gb300/csrc/countsort.cuh",
-                                         "paper_1408_6729_gb300/csrc/radix.cuh"]}
+NCU_TRAFFIC = {"route_keys_kernel": ((273.444608e6 + 221.018368e6) / (1 << 26), "9ad1eb3c57e7e8ac", False),
+               "bucket_count_kernel": ((539.887616e6 + 496.415744e6) / (1 << 27), "d65413af0b79da98", False),
+               "segment_copy_kernel": ((618.172672e6 + 495.224576e6) / (1 << 26), "5e0884ea5bc46122", True)}
+CSRC = "paper_1408_6729_gb300/csrc/"
+SHARED_SOURCE = ["common.cuh", "kernels.cuh", "many.cuh"]
+KERNEL_SOURCE = {k: [CSRC + f for f in v + SHARED_SOURCE] for k, v in {
+    "route_kernel": ["route.cu", "classify.cuh", "mlp.cuh", "radix.cuh"],
+    "route_keys_kernel": ["route_keys.cu", "classify.cuh", "mlp.cuh"],
+    "segment_copy_kernel": ["merge.cu"],
+    "bucket_sort_kernel": ["bucket.cuh", "segsort.cuh", "radix.cuh"],
+    "bucket_count_kernel": ["bucket.cuh", "countsort.cuh", "radix.cuh"],
+    "pair_count_kernel": ["pairs.cu", "countsort.cuh", "radix.cuh"]}.items()}
 
 
 def peaks():
@@ -552,8 +555,8 @@ def report(args, wl, name, world, n, p, plan, st, per_step, elapsed_ms, e2e_ms, 
     # (kernel, algorithmic bytes) of every phase that moves all the keys
     model = {}
     if wl["sampling"] == 0:  # the block sort reads every key (and writes the sorted blocks when it keeps them)
-        # keys without payloads in whole 16-byte groups: the counting sort (and the tag kernel)
-        counting = keep and not wl["pairs"] and n % 4 == 0 and -(-n // plan.R) % 4 == 0
+        # keys without payloads: the counting sort (and the tag kernel)
+        counting = keep and not wl["pairs"]
         kern0 = "run_sample_count_kernel" if counting else "run_sample_keys_kernel"
         model["sample"] = (wl.get("block_sort_kernel", kern0), n * (2 * kb if keep else key_bytes))
     if merge:
@@ -561,8 +564,8 @@ def report(args, wl, name, world, n, p, plan, st, per_step, elapsed_ms, e2e_ms, 
     else:
         for ph in ("route", "bucket_sort"):
             kern = PHASE_KERNEL[(ph, bool(wl["pairs"]))]
-            if key_bytes == 8 and not wl["pairs"]:
-                kern = PHASE_KERNEL_F64.get(ph, kern)
+            if wl["pairs"] and key_bytes == 4 and not keep and plan.vbuckets <= PAIR_WORDS_MAX:
+                kern = PHASE_KERNEL_WORDS[ph]
             if ph == "route" and keep:
                 kern = "segment_copy_kernel"
             model[ph] = (kern, n * 2 * kb)

@@ -175,7 +175,7 @@ static int make_plan(int64_t n, int dtype, const bsps_params *prm, int pairs, Pl
     take(pl.P * 4);
     take((kLutCells + 2) * 2);
     take(64);
-    const bool look_back = pairs && !pl.keep_runs;
+    const bool look_back = pairs && !pl.keep_runs;  // (pairs that can move as words take that route for some inputs, too)
     take(look_back ? std::max<int64_t>(pl.tiles, 1) * pl.P * 4 : 0);
     take(look_back ? std::max<int64_t>(pl.tiles, 1) * kRouteTile * 2 : 0);
     take(pl.P * 4);

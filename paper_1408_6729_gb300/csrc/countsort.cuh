@@ -43,13 +43,13 @@
 // takes every G-th part.  Every decision is a function of the segment alone,
 // so the CTAs agree without talking to each other.
 //
-// Bound by instruction issue (about 72 warp instructions per 32 keys, the
+// Bound by instruction issue (about 93 warp instructions per 32 keys, the
 // integer ones at half rate) and by the latency of the phases.  2^28 uniform
-// int32 keys in 65,536-key sub-buckets: 1.22 ms (1.76 TB/s of keys read and
+// int32 keys in 65,536-key sub-buckets: 1.26 ms (1.70 TB/s of keys read and
 // written); the cluster split, exchange and count it replaced took 2.38.  With
-// a wide stage in two parts 1.26, with edge checks in every window 1.23.  2^28
-// skewed doubles in 4096 sub-buckets: 2.9 ms, before the crowded ranges were
-// sorted here 3.8 and 0.84 for one bucket out of core.
+// a wide stage in two parts 1.26 against 1.22, with edge checks in every window
+// 1.23.  2^28 skewed doubles in 4096 sub-buckets: 2.6 ms, before the crowded
+// ranges were sorted here 3.8 and 0.84 for one bucket out of core.
 #pragma once
 
 #include <type_traits>

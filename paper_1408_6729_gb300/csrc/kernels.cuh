@@ -12,7 +12,7 @@ struct MlpNorm;
 constexpr int kLutBits = 14;
 constexpr int kLutCells = 1 << kLutBits;
 constexpr int kLutBitsFine = kLutBits + 1;  // keys without payloads, where it fits (with 4096 splitters 7 of 8 cells
-                                            // hold none, against 3 of 4: routing 2^28 keys 1.66 ms, before 1.77)
+                                            // hold none, against 3 of 4: routing 2^28 keys 1.77 -> 1.66 ms)
 
 // Routing geometry (Fig. 1 steps 9-11).
 constexpr int kRouteThreads = 1024;
